@@ -1404,6 +1404,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
             p2[DIM + 1] = pp[DIM + 1];
           }
         }
+        if (!neu) __syncthreads();   // (the - side's rows are read by other threads than wrote them)
         eval_uvalues_block<DIM, T>(a, npt, sPt, sM, sU);
         for (int ql = 0; ql < nq; ++ql) {
           if (base + ql < f0 || base + ql >= f1) continue;   // another CTA's Gram points
@@ -2173,6 +2174,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
                 sGdd[id * nrhs + r] = gD != nullptr ? sw * gD[(long long)r * a.n_bnd + goff] : 0.0;
             }
           }
+          if (ifc) __syncthreads();   // (the - side's rows are read by other threads than wrote them)
           eval_uvalues_block<DIM, T>(a, ifc ? 2 * nq : nq, sPt, sM, sU);
           for (int id = tid; id < nq * nrhs; id += blockDim.x) {
             const int ql = id / nrhs, r = id % nrhs;
@@ -2401,6 +2403,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
                 sGdd[id * nrhs + r] = gD != nullptr ? sw * gD[(long long)r * a.n_bnd + goff] : 0.0;
             }
           }
+          if (ifc) __syncthreads();   // (the - side's rows are read by other threads than wrote them)
           eval_uvalues_block<DIM, T>(a, ifc ? 2 * nq : nq, sPt, sM, sU);
           for (int id = tid; id < nq * nrhs; id += blockDim.x) {
             const int ql = id / nrhs, r = id % nrhs, q = base + ql;
