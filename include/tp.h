@@ -70,7 +70,7 @@ typedef struct tp_mesh_desc {
  * 0.5); kappa: pitching slope factor (edge-slope limit delta_e = kappa l_e /
  * c_e); T: final time; precision: TP_FP64 (every step in binary64) or
  * TP_MIXED (assembly, residual and outflow in float-float on the binary32
- * pipes, binary32 inverse of the equilibrated local matrix, iterative
+ * pipes; both precisions: float-float inverse of the equilibrated local matrix, iterative
  * refinement to float-float accuracy; a tent whose refinement does not
  * settle is solved by a direct binary64 LU instead);
  * nrhs: right-hand sides advanced together (same tents, same matrices;

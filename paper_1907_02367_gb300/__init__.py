@@ -103,7 +103,7 @@ class Solver:
 
     precision "fp64": assembly, residual and outflow in binary64.  "mixed":
     the same in float-float on the binary32 pipes.  Both invert the
-    equilibrated local matrix in binary32 and refine the solution in their
+    equilibrated local matrix in float-float and refine the solution in their
     own precision (a direct binary64 LU where the refinement does not settle).
     alpha, beta: the penalties of eq. (2.5) (Dirichlet, interface and Neumann
     facets).  bnd_type: optional (n_elem, dim+1) array, 1 marks the boundary

@@ -16,7 +16,7 @@
 //   bottom data (RHS):  b_i += w_q [ (c^-2 v_b - s_b.g_b) v_i + (s_b - v_b g_b).s_i + U_b U_i ];
 //   Dirichlet vertical faces (eq. 4.1):
 //     A_ij += w (s_j.n + alpha v_j) v_i,  b_i += w g_D (alpha v_i - s_i.n).
-// Then the local solve (a binary32 inverse of the equilibrated matrix and
+// Then the local solve (a float-float inverse of the equilibrated matrix and
 // refinement in the path's precision, a direct binary64 LU as fallback), and
 // (U, v, sigma) at the top points overwrite the front (Section 4.1: only the
 // latest values are stored).
@@ -166,10 +166,11 @@ struct tp_ctx {
   long long* d_info = nullptr;
   cudaStream_t cap_stream = nullptr;
   cudaStream_t last_stream = nullptr;
-  int n_sm = 152, max_cs = 1;
+  int n_sm = 152, max_cs = 1, flow_cs = 1;   // largest cluster of a launch per level; cluster of the dataflow sweep
   // right-hand sides split over the CTAs of a tent's cluster (1: not split)
   int rsplit_cs = 1;
   bool tc_used = false;   // tensor-core moments and outflow in the forward sweep
+  bool wide = false;      // one CTA per SM (its shared-memory plan does not leave room for two): twice the threads
   bool mixed = false;
   // persistent dataflow sweep
   bool persistent = true;
@@ -179,8 +180,7 @@ struct tp_ctx {
   int* d_queue = nullptr;
   int* d_done = nullptr;
   int* d_tent_vert = nullptr;
-  // dependency lists of the dataflow sweep kept on the host (tp_inject_wait)
-  std::vector<int32_t> dep_ptr_h, dep_need_h;
+  std::vector<int32_t> tent_level_h;   // levels of the tents (tp_inject_wait)
   // vertex stars in the record order (grouped by material) and the tents'
   // vertices and top times (point outputs are assigned to tents on the host)
   std::vector<int> star_sorted;
@@ -190,7 +190,7 @@ struct tp_ctx {
   int n_probe = 0, n_probe_t = 0;
   double* d_probe_out = nullptr;
   std::vector<void*> probe_allocs;
-  int* d_dep_need = nullptr;
+  int* d_inject = nullptr;
   unsigned long long* d_stats = nullptr;   // solve statistics (kMaxRefine + 2 counters)
   std::map<std::pair<int, int>, cudaGraphExec_t> graphs;
   int device = 0;
@@ -205,49 +205,73 @@ int ctx_upload(tp_ctx* ctx, T** d, const std::vector<T>& h) {
   return rc;
 }
 
-constexpr size_t kTwoPerSmSmem = 95 * 1024;  // plan that leaves room for two CTAs per SM
+// the launchers of each (space dimension, kind of sweep, Neumann facets)
+struct Launchers {
+  decltype(&tp::layer_attrs_d10_n0) attrs;
+  decltype(&tp::layer_static_smem_d10_n0) static_smem;
+  decltype(&tp::launch_layer_d10_n0) launch;
+  decltype(&tp::max_clusters_d10_n0) max_clusters;
+};
+#define TP_ROW(D, K, N)                                                                                              \
+  {                                                                                                                  \
+    tp::layer_attrs_d##D##K##_n##N, tp::layer_static_smem_d##D##K##_n##N, tp::launch_layer_d##D##K##_n##N,           \
+        tp::max_clusters_d##D##K##_n##N                                                                              \
+  }
+#define TP_KIND_ROWS(D, K) { TP_ROW(D, K, 0), TP_ROW(D, K, 1) }
+#define TP_DIM_ROWS(D) { TP_KIND_ROWS(D, 0), TP_KIND_ROWS(D, 1), TP_KIND_ROWS(D, 2), TP_KIND_ROWS(D, 3) }
+const Launchers kLaunchers[3][4][2] = {TP_DIM_ROWS(1), TP_DIM_ROWS(2), TP_DIM_ROWS(3)};
+#undef TP_DIM_ROWS
+#undef TP_KIND_ROWS
+#undef TP_ROW
+enum { kForward64 = 0, kForwardMixed = 1, kAdjoint64 = 2, kForwardTc = 3 };
 
-// cap of the shared-memory plan: the device's per-block limit less the
-// kernel's static shared memory; the attribute is set to it, so contexts of
-// any size can share the kernel
-int max_dyn_smem(int dim, size_t* cap) {
-  int dev = 0, optin = 0;
+int static_smem(int dim, size_t* bytes) {
+  *bytes = 0;
+  for (const auto& kind : kLaunchers[dim - 1])
+    for (const Launchers& l : kind) {
+      size_t b = 0;
+      TP_CUDA_OK(l.static_smem(&b));
+      *bytes = std::max(*bytes, b);
+    }
+  return TP_OK;
+}
+
+// caps of the shared-memory plan: the device's per-block limit less the
+// kernel's static shared memory (the attribute is set to it, so contexts of
+// any size can share the kernel), and what leaves room for two CTAs per SM
+// (each with 1 KB that the system reserves)
+int max_dyn_smem(int dim, size_t* cap, size_t* two_per_sm) {
+  int dev = 0, optin = 0, sm = 0;
   size_t stat = 0;
   TP_CUDA_OK(cudaGetDevice(&dev));
   TP_CUDA_OK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  TP_CUDA_OK(dim == 1 ? tp::layer_static_smem_d1(&stat) : dim == 2 ? tp::layer_static_smem_d2(&stat)
-                                                                     : tp::layer_static_smem_d3(&stat));
-  if ((size_t)optin <= stat + kTwoPerSmSmem) {
-    *cap = kTwoPerSmSmem;
-  } else {
-    *cap = ((size_t)optin - stat) & ~(size_t)1023;
-  }
+  TP_CUDA_OK(cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+  const int rc = static_smem(dim, &stat);
+  if (rc != TP_OK) return rc;
+  *cap = ((size_t)optin - stat) & ~(size_t)1023;
+  *two_per_sm = std::min(*cap, ((size_t)sm / 2 - 1024 - stat) & ~(size_t)127);
   return TP_OK;
 }
 
 int set_smem_attr(int dim, size_t cap) {
-  cudaError_t e = dim == 1 ? tp::layer_attrs_d1(cap) : dim == 2 ? tp::layer_attrs_d2(cap) : tp::layer_attrs_d3(cap);
-  TP_CUDA_OK(e);
+  for (const auto& kind : kLaunchers[dim - 1])
+    for (const Launchers& l : kind) TP_CUDA_OK(l.attrs(cap));
   return TP_OK;
 }
 
-cudaError_t launch_layer(tp_ctx* ctx, const KArgs& a, int n_cluster, int cs, int t0, cudaStream_t st, int mode,
+// the kind of kernel that runs this context's forward sweep
+int forward_kind(const tp_ctx* ctx) { return ctx->tc_used ? kForwardTc : ctx->mixed ? kForwardMixed : kForward64; }
+
+cudaError_t launch_layer(tp_ctx* ctx, const KArgs& a, int n_cluster, int cs, int t0, cudaStream_t st, int kind,
                          bool persistent) {
-  if (ctx->neumann) mode |= 4;   // the kernel variant with the Neumann facet code
-  switch (ctx->dim) {
-    case 1: return tp::launch_layer_d1(a, n_cluster, cs, t0, ctx->smem_bytes, st, mode, persistent);
-    case 2: return tp::launch_layer_d2(a, n_cluster, cs, t0, ctx->smem_bytes, st, mode, persistent);
-    default: return tp::launch_layer_d3(a, n_cluster, cs, t0, ctx->smem_bytes, st, mode, persistent);
-  }
+  return kLaunchers[ctx->dim - 1][kind][ctx->neumann].launch(a, n_cluster, cs, t0, ctx->smem_bytes, st, persistent, ctx->wide);
 }
 
 // resident clusters of the persistent kernel for cluster size cs
 int set_persist_cs(tp_ctx* ctx, int cs) {
   int nclu = 0;
-  const int mode = (ctx->mixed ? 1 : 0) | (ctx->neumann ? 4 : 0);
-  cudaError_t e = ctx->dim == 1 ? tp::max_clusters_d1(cs, ctx->smem_bytes, mode, &nclu)
-                : ctx->dim == 2 ? tp::max_clusters_d2(cs, ctx->smem_bytes, mode, &nclu)
-                                : tp::max_clusters_d3(cs, ctx->smem_bytes, mode, &nclu);
+  cudaError_t e = kLaunchers[ctx->dim - 1][forward_kind(ctx)][ctx->neumann].max_clusters(
+      cs, ctx->smem_bytes, ctx->rsplit_cs > 1, ctx->wide, &nclu);
   if (e != cudaSuccess || nclu < 1) {
     cudaGetLastError();
     return TP_ERR_UNSUPPORTED;
@@ -296,7 +320,7 @@ int launch_level(tp_ctx* ctx, int32_t L, cudaStream_t st, bool adj = false, int 
   if (t1 <= t0) return TP_OK;
   const int nt = (int)(t1 - t0);
   const int cs = level_cluster_size(ctx, nt);
-  const int mode = adj ? 2 : (ctx->mixed ? 1 : 0);
+  const int mode = adj ? kAdjoint64 : forward_kind(ctx);
   double* tau = adj ? ctx->d_tau_adj : ctx->d_tau;
   const int k0 = group < 0 ? 0 : group, k1 = group < 0 ? ctx->rhs_groups : group + 1;
   const bool restore = group < 0 && ctx->rhs_groups > 1;
@@ -316,7 +340,7 @@ int launch_level_with(tp_ctx* ctx, int32_t L, cudaStream_t st, bool adj, const K
   const int64_t t0 = ctx->level_ptr[L - 1], t1 = ctx->level_ptr[L];
   if (t1 <= t0) return TP_OK;
   const int nt = (int)(t1 - t0);
-  TP_CUDA_OK(launch_layer(ctx, a, nt, level_cluster_size(ctx, nt), (int)t0, st, adj ? 2 : (ctx->mixed ? 1 : 0), false));
+  TP_CUDA_OK(launch_layer(ctx, a, nt, level_cluster_size(ctx, nt), (int)t0, st, adj ? kAdjoint64 : forward_kind(ctx), false));
   TP_CUDA_OK(cudaGetLastError());
   return TP_OK;
 }
@@ -364,11 +388,13 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   ctx->level_ptr = tents->level_ptr;
   ctx->neumann = std::find(T.facet_kind.begin(), T.facet_kind.end(), (int8_t)1) != T.facet_kind.end();
   // patch checks: size limits; materials (distinct wave speeds) per tent
-  int ngmax = 1, pmax = 1;
+  int ngmax = 1, pmax = 1, fmax = 1, nmax = 1;
   std::vector<std::array<int, 4>> facet_mix;   // distinct (materials, Dirichlet, interface, Neumann facets)
   for (int64_t v = 0; v < T.nv; ++v) {
     const int p0 = T.star_ptr[v], p1 = T.star_ptr[v + 1];
     pmax = std::max(pmax, p1 - p0);
+    fmax = std::max(fmax, (T.vfac_ptr[v + 1] - T.vfac_ptr[v]) + (T.ifac_ptr[v + 1] - T.ifac_ptr[v]));
+    nmax = std::max(nmax, 1 + T.nbr_ptr[v + 1] - T.nbr_ptr[v]);
     if ((T.vfac_ptr[v + 1] - T.vfac_ptr[v]) + (T.ifac_ptr[v + 1] - T.ifac_ptr[v]) > tp::kMaxFacets) {
       tp::set_error("tp_create: vertex " + std::to_string(v) + " lies on more than 16 boundary or interface facets");
       return fail(TP_ERR_UNSUPPORTED);
@@ -453,25 +479,37 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   ctx->n_bnd = gdoff[ctx->ntents];
   gdoff.pop_back();
 
-  // dependencies of the dataflow sweep: tent (v, L) waits until every vertex w
-  // of {v} and its neighbours has completed its tents of level < L
-  std::vector<int32_t> dep_ptr(ctx->ntents + 1, 0), dep_vert, dep_need;
+  // dependencies of the dataflow sweep: tent (v, L) waits until v and every
+  // neighbour w have completed their tents of level < L; the counts in the
+  // order (v, neighbours).  And the front times of w after 0, 1, .. of its
+  // tents, so that the kernel finds the times a tent starts from
+  std::vector<int32_t> dep_ptr(ctx->ntents + 1, 0), dep_need, vt_ptr(T.nv + 1, 0);
+  std::vector<double> vt_tau((size_t)T.nv + ctx->ntents, 0.0);
+  std::vector<int32_t> tents_at(ctx->ntents);   // per vertex, its tents in order
   {
-    std::vector<std::vector<int32_t>> lev_at(T.nv);
-    for (int64_t it = 0; it < ctx->ntents; ++it) lev_at[tents->vert[it]].push_back(tents->level[it]);
+    std::vector<int32_t> cnt(T.nv, 0);
+    for (int64_t it = 0; it < ctx->ntents; ++it) ++cnt[tents->vert[it]];
+    for (int64_t v = 0; v < T.nv; ++v) vt_ptr[v + 1] = vt_ptr[v] + cnt[v] + 1;
+    std::fill(cnt.begin(), cnt.end(), 0);
+    size_t total = 0;
+    for (int64_t it = 0; it < ctx->ntents; ++it) total += 1 + (size_t)(T.nbr_ptr[tents->vert[it] + 1] - T.nbr_ptr[tents->vert[it]]);
+    if (total > 0x7fffffff) {
+      tp::set_error("tp_create: too many tents");
+      return fail(TP_ERR_UNSUPPORTED);
+    }
+    dep_need.reserve(total);
+    int64_t l0 = 0;   // first tent of the level being counted
     for (int64_t it = 0; it < ctx->ntents; ++it) {
-      const int v = tents->vert[it], L = tents->level[it];
-      auto add = [&](int w) {
-        const auto& lv = lev_at[w];
-        const int need = (int)(std::lower_bound(lv.begin(), lv.end(), L) - lv.begin());
-        if (need > 0) {
-          dep_vert.push_back(w);
-          dep_need.push_back(need);
-        }
-      };
-      add(v);
-      for (int e = T.nbr_ptr[v]; e < T.nbr_ptr[v + 1]; ++e) add(T.nbr[e]);
-      dep_ptr[it + 1] = (int32_t)dep_vert.size();
+      if (it > 0 && tents->level[it] != tents->level[it - 1]) {   // the level before is complete
+        for (int64_t j = l0; j < it; ++j) ++cnt[tents->vert[j]];
+        l0 = it;
+      }
+      const int v = tents->vert[it];
+      dep_need.push_back(cnt[v]);
+      for (int e = T.nbr_ptr[v]; e < T.nbr_ptr[v + 1]; ++e) dep_need.push_back(cnt[T.nbr[e]]);
+      dep_ptr[it + 1] = (int32_t)dep_need.size();
+      vt_tau[(size_t)vt_ptr[v] + 1 + cnt[v]] = tents->t_top[it];
+      tents_at[(size_t)vt_ptr[v] - v + cnt[v]] = (int32_t)it;
     }
   }
   // dataflow queue order: level by level (every awaited tent is earlier in the
@@ -480,18 +518,20 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   // critical path.  Work of a tent: 1, +0.2 with Dirichlet or interface facets.
   std::vector<int32_t> queue_tent(ctx->ntents);
   {
-    std::vector<std::vector<int32_t>> tents_at(T.nv);
-    for (int64_t it = 0; it < ctx->ntents; ++it) tents_at[tents->vert[it]].push_back((int32_t)it);
-    std::vector<std::vector<int32_t>> succ(ctx->ntents);
-    for (int64_t it = 0; it < ctx->ntents; ++it)
-      for (int e = dep_ptr[it]; e < dep_ptr[it + 1]; ++e) succ[tents_at[dep_vert[e]][dep_need[e] - 1]].push_back((int32_t)it);
-    std::vector<double> height(ctx->ntents, 0.0);
+    // the longest chain of work after each tent, from the last tent back: a
+    // tent's height goes to the last earlier tent of v and of each neighbour
+    std::vector<float> height(ctx->ntents, 0.f);
     for (int64_t it = ctx->ntents - 1; it >= 0; --it) {   // tents are sorted by level
       const int v = tents->vert[it];
-      double h = 0.0;
-      for (int32_t sc : succ[it]) h = std::max(h, height[sc]);
       const bool extra = (T.vfac_ptr[v + 1] > T.vfac_ptr[v]) || (T.ifac_ptr[v + 1] > T.ifac_ptr[v]);
-      height[it] = h + (extra ? 1.2 : 1.0);
+      height[it] += extra ? 1.2f : 1.f;   // (holds the largest height of its successors)
+      const int32_t* need = &dep_need[dep_ptr[it]];
+      for (int e = -1; e < T.nbr_ptr[v + 1] - T.nbr_ptr[v]; ++e) {
+        const int w = e < 0 ? v : T.nbr[T.nbr_ptr[v] + e], c = need[e + 1];
+        if (c == 0) continue;
+        float& hw = height[tents_at[(size_t)vt_ptr[w] - w + c - 1]];
+        hw = std::max(hw, height[it]);
+      }
     }
     for (int64_t it = 0; it < ctx->ntents; ++it) queue_tent[it] = (int32_t)it;
     for (int L = 0; L < tents->n_levels; ++L) {
@@ -506,7 +546,8 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   KArgs& a = ctx->args;
   double *dX, *dc, *dbary, *dw, *dsqw, *dttop, *dspc;
   int *del, *dtv, *dspp, *dspm, *dpar, *dvar, *drp, *drs, *dtp, *dtd;
-  int *ddp, *ddv, *ddn, *dqt;
+  int *ddp, *ddn, *dqt, *dvtp, *dinj;
+  double* dvtt;
   double *drf, *dtf;
   float2* dcdd;
   float2* dsqwff = nullptr;
@@ -624,11 +665,12 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     return fail(rc);
   // per vertex: one record with all of its star that does not depend on the
   // sweep, so that a tent reads it in one round of loads.
-  //   ints:    per element (el, material, vertex ids[n+1]); per facet (Dirichlet
-  //            first, then interface, then Neumann): (elements of the + and -
-  //            sides in slots 0, 1, vertex ids other than v in slots 2..n,
-  //            material of the + element, of the - element, position among the
-  //            vertex's boundary facets = block of its boundary data)
+  //   ints:    per element (el, material, its n+1 vertices as places in the list
+  //            (v, neighbours)); per facet (Dirichlet first, then interface, then
+  //            Neumann): (elements of the + and - sides in slots 0, 1, places of
+  //            the vertices other than v in slots 2..n, material of the +
+  //            element, of the - element, position among the vertex's boundary
+  //            facets = block of its boundary data); v and its neighbours' ids
   //   doubles: x_v[n], speeds[kMaxGroups], their 1/c^2 [kMaxGroups]; per element its vertex coordinates
   //            [(n+1) n]; per facet its normal [n] and vertex coordinates [(n+1) n]
   // per tent: (v, int offset, double offset, elements, Dirichlet facets,
@@ -638,6 +680,12 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   std::vector<int> vrec_i(T.nv), vrec_d(T.nv);
   {
     const int NVn = n + 1;
+    // place of vertex w in the list of v and its neighbours
+    auto place_of = [&](int64_t v, int w) {
+      if (w == v) return 0;
+      const auto b = T.nbr.begin() + T.nbr_ptr[v], e = T.nbr.begin() + T.nbr_ptr[v + 1];
+      return 1 + (int)(std::lower_bound(b, e, w) - b);
+    };
     auto grp_of = [&](int64_t v, double ck) {
       int g = 0;
       while (g < vert_ng[v] - 1 && vert_gc[(size_t)v * tp::kMaxGroups + g] != ck) ++g;
@@ -658,7 +706,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
         rec_i.push_back(star_grp[e]);
         for (int i = 0; i < NVn; ++i) {
           const int vi = T.elems[(size_t)el * NVn + i];
-          rec_i.push_back(vi);
+          rec_i.push_back(place_of(v, vi));
           for (int d = 0; d < n; ++d) rec_d.push_back(T.X[(size_t)vi * n + d]);
         }
       }
@@ -689,7 +737,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
         // facet's other vertices
         rec_i.push_back(bnd ? T.facet_elem[fid] : T.ifac_kp[fid]);
         rec_i.push_back(bnd ? T.facet_elem[fid] : T.ifac_km[fid]);
-        for (int i = 2; i < NVn; ++i) rec_i.push_back(w_[i]);
+        for (int i = 2; i < NVn; ++i) rec_i.push_back(place_of(v, w_[i]));
         rec_i.push_back(grp_of(v, T.c[bnd ? T.facet_elem[fid] : T.ifac_kp[fid]]));
         rec_i.push_back(grp_of(v, T.c[bnd ? T.facet_elem[fid] : T.ifac_km[fid]]));
         rec_i.push_back(fo[2]);
@@ -697,6 +745,8 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
         for (int i = 0; i < NVn; ++i)
           for (int d = 0; d < n; ++d) rec_d.push_back(w_[i] >= 0 ? T.X[(size_t)w_[i] * n + d] : 0.0);
       }
+      rec_i.push_back((int)v);
+      for (int e = T.nbr_ptr[v]; e < T.nbr_ptr[v + 1]; ++e) rec_i.push_back(T.nbr[e]);
     }
     for (int64_t it = 0; it < ctx->ntents; ++it) {
       const int v = tents->vert[it];
@@ -722,7 +772,8 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     return fail(rc);
   if ((rc = ctx_upload(ctx, &dX, T.X)) || (rc = ctx_upload(ctx, &dc, T.c)) ||
       (rc = ctx_upload(ctx, &del, T.elems)) || (rc = ctx_upload(ctx, &dbary, ctx->rule.bary)) ||
-      (rc = ctx_upload(ctx, &ddp, dep_ptr)) || (rc = ctx_upload(ctx, &ddv, dep_vert)) ||
+      (rc = ctx_upload(ctx, &ddp, dep_ptr)) || (rc = ctx_upload(ctx, &dvtp, vt_ptr)) ||
+      (rc = ctx_upload(ctx, &dvtt, vt_tau)) || (rc = ctx_upload(ctx, &dinj, std::vector<int>{-1, 0})) ||
       (rc = ctx_upload(ctx, &ddn, dep_need)) || (rc = ctx_upload(ctx, &dqt, queue_tent)) ||
       (rc = ctx_upload(ctx, &dw, ctx->rule.w)) || (rc = ctx_upload(ctx, &dsqw, sqw)) ||
       (rc = ctx_upload(ctx, &dtv, tv)) || (rc = ctx_upload(ctx, &dttop, ttop)) ||
@@ -828,11 +879,12 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   a.beta = prm->beta;
   a.ngmax = ngmax;
   a.dep_ptr = ddp;
-  a.dep_vert = ddv;
   a.dep_need = ddn;
-  ctx->d_dep_need = ddn;
-  ctx->dep_ptr_h = dep_ptr;
-  ctx->dep_need_h = dep_need;
+  a.vt_ptr = dvtp;
+  a.vt_tau = dvtt;
+  a.inject = dinj;
+  ctx->d_inject = dinj;
+  ctx->tent_level_h = tents->level;
   a.max_spin = tp::kMaxSpin;
   a.max_refine = tp::kMaxRefine;
   if (cudaMalloc(&ctx->d_stats, (tp::kMaxRefine + 2) * sizeof(unsigned long long)) != cudaSuccess) {
@@ -866,6 +918,24 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   a.elem_sdet = desdet;
   a.elem_isdet = deisdet;
   a.isqw = disqw;
+  {   // the rule of the face integrals
+    const tp::FaceRule& fr = tp::face_rule(n, basis->p, ctx->rule);
+    a.S = fr.S;
+    a.tf_stride = fr.stride;
+    std::vector<double> tf(fr.to_points);
+    tf.insert(tf.end(), fr.to_front.begin(), fr.to_front.end());
+    std::vector<float> tff(fr.to_points_ff);
+    tff.insert(tff.end(), fr.to_front_ff.begin(), fr.to_front_ff.end());
+    double *dsb = nullptr, *dss = nullptr, *dtf_ = nullptr;
+    float* dtff_ = nullptr;
+    if ((rc = ctx_upload(ctx, &dsb, fr.bary)) || (rc = ctx_upload(ctx, &dss, fr.sqw)) || (rc = ctx_upload(ctx, &dtf_, tf)) ||
+        (rc = ctx_upload(ctx, &dtff_, tff)))
+      return fail(rc);
+    a.s_bary = dsb;
+    a.s_sqw = dss;
+    a.tf = dtf_;
+    a.tf_dd = reinterpret_cast<const float2*>(dtff_);
+  }
   a.bary = dbary;
   a.wref = dw;
   a.sqw = dsqw;
@@ -904,7 +974,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   // shared-memory plan: the largest chunk of points that fits
   const int nb = ctx->nb, C = ctx->C;
   const int npair = nb * (nb + 1) / 2;
-  if (npair > kMaxPair * kThreads) {
+  if (npair > kMaxPairs) {
     tp::set_error("tp_create: dim U^p too large for this kernel (more than 38)");
     return fail(TP_ERR_UNSUPPORTED);
   }
@@ -916,42 +986,47 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   bool ifneu = false;   // some tent has interface or Neumann facets
   for (const auto& m : facet_mix) ifneu = ifneu || m[2] > 0 || m[3] > 0;
   bool tc_try = false;   // the plan with the tensor-core staging
-  auto plan = [&](int CH, int keep) {
+  // (CH: points per chunk; keep: points whose U-values a CTA keeps; rows: points
+  // evaluated at a time into them; rule: the S-point rule of the face integrals)
+  const int S_rule = a.S;
+  int rs = prm->rhs_split;
+  auto plan = [&](int CH, int keep, int rows, bool rule) {
     size_t off = 0;
+    a.S = rule ? S_rule : 0;
+    const int QK = a.S > 0 ? a.S : Q;
     auto take = [&](int* field, size_t count) {
       if (field) *field = (int)off;
       off += count;
     };
     const size_t nmom = (size_t)nrg * C * nb;
     const size_t NB = (size_t)ngmax * nb;          // unknowns of the largest tent
-    const size_t half_nb = (NB + 1) / 2, half_rb = ((size_t)nrg * NB + 1) / 2;
-    // region used in turn by the monomials (point phases 1, 2, 4) and by A, the
-    // summed Grams and the solve buffers (reduction to solve); A at offset 0
-    // (the binary32 sweep buffers of the solve reuse the summed Grams, dead after the congruence)
-    const size_t sg_al = std::max((size_t)ngmax * (n + 2) * npair, NB * NB);
-    // interface blocks (tents with interface facets) followed by the Dirichlet
-    // sums of every material (tents with Dirichlet facets), partials reduced in place
-    // (and for tents with Neumann facets the blocks plus a partial b)
+    const size_t half_nb = (NB + 1) / 2, rb = (size_t)nrg * NB;
+    // Dirichlet sums of every material (tents with Dirichlet facets), partials
+    // reduced in place, and a partial b (tents with Neumann facets)
     size_t pd = 0;
     for (const auto& m : facet_mix)
-      pd = std::max(pd, (m[2] > 0 || m[3] > 0 ? (size_t)m[0] * nb * m[0] * nb : 0) +
-                            (m[1] > 0 ? (size_t)m[0] * (n + 1) * (npair + (size_t)nrg * nb) : 0) +
+      pd = std::max(pd, (m[1] > 0 ? (size_t)m[0] * (n + 1) * (npair + (size_t)nrg * nb) : 0) +
                             (m[3] > 0 ? (size_t)nrg * m[0] * nb : 0));
-    const size_t solve_part = NB * NB + sg_al + (size_t)nrg * NB + half_rb;
-    const size_t mono_part = (size_t)2 * CH * a.mono_stride;
-    a.off_mono = 0;
     take(nullptr, NB * NB);                        // A
-    a.off_al = (int)off;                           // two binary32 N x N sweep buffers
-    take(&a.off_sg, sg_al);
-    take(&a.off_x, (size_t)nrg * NB);
-    take(&a.off_z, half_rb);
-    off = std::max(solve_part, mono_part);
-    take(&a.off_b, (size_t)nrg * NB);
-    take(&a.off_pg, (size_t)ngmax * npair);        // G, H_m, Gbot contiguous
-    take(&a.off_ph, (size_t)ngmax * n * npair);
-    take(&a.off_pgb, (size_t)ngmax * npair);
+    take(&a.off_x, rb);
+    take(&a.off_z, rb);
+    take(&a.off_b, rb);
+    // one region in turn: facet Grams of interface and Neumann facets, the
+    // Grams G, H_m, Gbot (contiguous), the float-float inverse
+    // (right-hand sides split: the facet Grams have a region of their own)
+    const size_t fg = ifneu ? (size_t)2 * npair + nb * nb : 0;
+    a.off_f = (int)off;
+    a.off_f2 = a.off_f + npair;
+    a.off_fpm = a.off_f2 + npair;
+    if (rs > 1) off += fg;
+    a.off_pg = (int)off;
+    a.off_ph = a.off_pg + ngmax * npair;
+    a.off_pgb = a.off_ph + ngmax * n * npair;
+    take(nullptr, std::max({(size_t)ngmax * (n + 2) * npair, NB * NB, fg}));
     take(&a.off_pm, (size_t)ngmax * nmom);        // moments: partials, summed in place, then the outflow vectors
     a.off_sm = a.off_y = a.off_pm;
+    a.ev_rows = std::max(2 * CH, rows);
+    take(&a.off_mono, (size_t)a.ev_rows * a.mono_stride);
     // tensor-core staging (bf16 digit planes), in the region of the facet
     // sums (dead during the point passes before phase 2 and during the
     // outflow): the moments' A (rows of data coefficients x CH points) and B
@@ -969,31 +1044,43 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     off += off & 1;                                // 16-byte alignment of the staging
     a.off_tc = (int)off;
     take(&a.off_pd, std::max(pd, tcd));
-    // facet Grams of interface and Neumann facets (none on meshes without them)
-    take(&a.off_f, ifneu ? npair : 0);
-    take(&a.off_f2, ifneu ? npair : 0);
-    take(&a.off_fpm, ifneu ? (size_t)nb * nb : 0);
     take(&a.off_del, (size_t)nrg * nb);
     take(&a.off_u, (size_t)2 * CH * (nb | 1));
-    take(&a.off_pt, (size_t)2 * CH * (n + 2));
-    take(&a.off_cb, (size_t)(CH + 1) * nrg * C);   // data coefficients, rows of CH + 1
+    take(&a.off_pt, (size_t)a.ev_rows * (n + 2));
+    // data coefficients, a row per right-hand side and component: of a chunk
+    // of points; under the S-point rule of raw_el elements' points (with kept
+    // U-values and few right-hand sides of all of the CTA's), and these
+    // elements' data at the front's points
+    a.raw_el = a.S == 0 || rs > 1 ? 0 : keep > 0 && nrg <= 4 ? keep / QK : std::max(1, (keep > 0 ? CH : 2 * CH) / QK);
+    a.cb_pts = std::max({CH, a.raw_el * QK, keep > 0 && nrg <= 4 ? keep : 0});
+    take(&a.off_cb, (size_t)(a.cb_pts | 1) * nrg * C);
+    take(&a.off_raw, (size_t)a.raw_el * Q * nrg * C);
+    take(&a.off_tf, rs > 1 ? 0 : (size_t)2 * a.S * a.tf_stride);
     take(&a.off_gd, (size_t)CH * nrg);
     take(&a.off_rd, NB);
+    take(&a.off_rc, NB > 32 ? 4 * NB : 0);
     take(&a.off_eq, half_nb);
-    take(&a.off_keep, (size_t)keep * nb);          // top U-values of the CTA's slice, kept for the outflow
-    take(&a.off_keepw, (size_t)keep);
+    take(&a.off_keep, (size_t)2 * keep * (nb | 1));   // U-values of the CTA's slice on both faces
+    {   // the patch (Geo)
+      const size_t NVg = n + 1, P_ = pmax, F_ = fmax, M_ = nmax;
+      const size_t dbl[] = {P_ * NVg * n, P_ * NVg, P_ * NVg, P_ * n, P_ * n, P_, P_, P_, P_ * NVg,
+                            F_ * NVg * NVg, F_, F_ * n, M_};
+      const size_t ints[] = {P_, P_, P_ * NVg, F_ * NVg, F_, F_, M_};
+      int g = 0;
+      for (size_t c : dbl) take(&a.geo[g++], c);
+      for (size_t c : ints) take(&a.geo[g++], (c + 1) / 2);
+    }
     // wave-speed gradient (reverse sweep): y(x), y(x'), y(mu') per material and the forward solution
     take(&a.off_yg, prm->ckpt_stride > 0 ? 3 * (size_t)ngmax * nmom + (size_t)nrg * NB : 0);
     return off * sizeof(double);
   };
   int CH = 0;
   size_t bytes = 0, cap_used = 0;
-  size_t max_dyn = 0;
-  if ((rc = max_dyn_smem(n, &max_dyn)) != TP_OK) return fail(rc);
+  size_t max_dyn = 0, two_per_sm = 0;
+  if ((rc = max_dyn_smem(n, &max_dyn, &two_per_sm)) != TP_OK) return fail(rc);
   // right-hand sides split over the cluster: rs CTAs, each owning a slice of
   // every group's right-hand sides (automatic: 16 or more per CTA; at 3D
   // p = 3 with 64 right-hand sides, 4 CTAs of 16 sweep 1.6x faster than 8 of 8)
-  int rs = prm->rhs_split;
   if (rs == 0) {
     rs = 1;
     for (int r : {8, 4, 2})
@@ -1018,20 +1105,25 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   size_t stat_smem = 0;
   TP_CUDA_OK(cudaGetDevice(&dev_));
   TP_CUDA_OK(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev_));
-  TP_CUDA_OK(n == 1 ? tp::layer_static_smem_d1(&stat_smem) : n == 2 ? tp::layer_static_smem_d2(&stat_smem)
-                                                                     : tp::layer_static_smem_d3(&stat_smem));
+  if ((rc = static_smem(n, &stat_smem)) != TP_OK) return fail(rc);
   const bool tc_want = prm->tensor_cores >= 0 && ctx->mixed && rs > 1 && nb <= 32 &&
                        (ctx->nrhs / rs) * C <= 96;
-  for (int pass = 0; pass < 2 && CH == 0; ++pass) {
+  // (the S-point rule where its points fit the evaluation buffer; right-hand
+  // sides not split: U-values evaluated again need whole elements in it)
+  // (split right-hand sides keep the front rule, whose U-values their moments and outflow take)
+  bool rule = false;
+  for (int pass = 0; pass < 3 && CH == 0; ++pass) {
     tc_try = tc_want && pass == 0;
     if (!tc_want && pass == 0) continue;
+    rule = S_rule > 0 && rs == 1 && pass < 2;
+    if (pass == 2 && (S_rule == 0 || rs > 1)) continue;
     for (grp = ctx->nrhs; grp >= 1 && CH == 0; --grp) {
       if (ctx->nrhs % grp || grp % rs) continue;
       nrg = grp / rs;
       if (tc_try && nrg * C > 96) continue;
-      for (size_t cap : {kTwoPerSmSmem, max_dyn}) {
+      for (size_t cap : {two_per_sm, max_dyn}) {
         for (int ch : {48, 32, 16, 8}) {
-          if (CH != 0 || plan(ch, 0) > cap) continue;
+          if (CH != 0 || (rule && 2 * ch < S_rule) || plan(ch, 0, 0, rule) > cap) continue;
           if (tc_try && (ch % 16 != 0 || ch * tp::kTcSlices * 65536 >= (1 << 24))) continue;
           CH = ch;
         }
@@ -1047,15 +1139,32 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     tp::set_error("tp_create: shared-memory plan does not fit (nb/nrhs too large)");
     return fail(TP_ERR_UNSUPPORTED);
   }
-  // the rest of the budget keeps the top U-values of up to `keep` points per
-  // CTA (a slice that fits skips their second evaluation in the outflow)
-  // (split right-hand sides evaluate the top U-values of every point again: no keep buffer)
-  int keep = rs > 1 ? 0 : (int)std::min<size_t>((cap_used - plan(CH, 0)) / ((size_t)(nb + 1) * sizeof(double)),
-                                                (size_t)pmax * Q);
-  while (keep > 0 && plan(CH, keep) > cap_used) --keep;
-  bytes = plan(CH, keep);
+  // U-values kept by the CTAs of a tent (right-hand sides not split), so that
+  // nothing is evaluated after the wait.  The smallest cluster for which the
+  // slices of the largest patch fit, with two CTAs per SM if any does; the
+  // chunks of the other passes shrink for it.
+  int keep = 0, rows = 0, keep_cs = 0;
+  if (rs == 1) {
+    const int QK = rule ? S_rule : Q;
+    static const int kChunks[][2] = {{48, 96}, {32, 96}, {16, 96}, {16, 64}, {8, 64}, {8, 32}};   // (chunk, rows)
+    for (size_t cap : {two_per_sm, max_dyn})
+      for (int cs : {1, 2, 4, 8})
+        for (const auto& c : kChunks) {
+          const int want = (pmax + cs - 1) / cs * QK;
+          if (keep_cs != 0 || (rule && 2 * c[0] < S_rule) || plan(c[0], want, c[1], rule) > cap) continue;
+          CH = c[0];
+          rows = c[1];
+          keep = want;
+          keep_cs = cs;
+        }
+  }
+  bytes = plan(CH, keep, rows, rule);
+  ctx->wide = bytes > two_per_sm;
   // one CTA per SM with the tensor-core contractions (it holds all 512 columns)
-  if (tc_try) bytes = std::max(bytes, std::min(max_dyn, (size_t)smem_sm / 2 + 1024 - stat_smem));
+  if (tc_try) {
+    bytes = std::max(bytes, std::min(max_dyn, (size_t)smem_sm / 2 + 1024 - stat_smem));
+    ctx->wide = true;
+  }
   a.CH = CH;
   a.keep_pts = keep;
   a.nrhs = nrg;
@@ -1085,7 +1194,14 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     const double avg_pts = (double)T.star_el.size() / (double)T.nv * Q;
     int cs = 1;
     while (cs < 8 && avg_pts / (2.0 * cs) >= 32.0) cs *= 2;
-    ctx->max_cs = cs;
+    ctx->max_cs = std::max(cs, keep_cs);
+    // dataflow sweep, right-hand sides not split: the smallest cluster that
+    // keeps its U-values, doubled while a third of the resident CTAs holds a
+    // level's tents (the others then work ahead) and a CTA keeps 5/4 elements
+    const double width = (double)ctx->ntents / std::max(1, ctx->n_levels), star = (double)T.star_el.size() / (double)T.nv;
+    cs = std::max(1, keep_cs);
+    while (cs < 8 && 2.0 * cs * width <= (ctx->wide ? 1 : 2) * ctx->n_sm / 3.0 && star / (2.0 * cs) >= 1.25) cs *= 2;
+    ctx->flow_cs = cs;
   }
   {
     const double avg_star = (double)T.star_el.size() / (double)T.nv;
@@ -1093,7 +1209,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     std::copy(key, key + 5, ctx->tune_key);
   }
   if (ctx->persistent) {
-    int cs = ctx->max_cs;
+    int cs = ctx->flow_cs;
     bool sched_dataflow = true;
     if (tuned_lookup(ctx->tune_key, &cs, &sched_dataflow)) ctx->persistent = sched_dataflow;
     if (rs > 1) cs = rs;   // the cluster is the right-hand-side split
@@ -1411,14 +1527,14 @@ extern "C" int tp_inject_wait(tp_ctx* ctx, int64_t tent, int32_t extra) {
     tp::set_error("tp_inject_wait: invalid argument");
     return TP_ERR_ARG;
   }
-  const int d0 = ctx->dep_ptr_h[tent], d1 = ctx->dep_ptr_h[tent + 1];
-  if (d1 <= d0) {
+  // (a tent of level 1 follows no tent at its vertex or neighbours, one of a
+  // later level follows at least one)
+  if (ctx->tent_level_h[tent] <= 1) {
     tp::set_error("tp_inject_wait: tent " + std::to_string(tent) + " waits for no earlier tent");
     return TP_ERR_ARG;
   }
-  std::vector<int32_t> need(ctx->dep_need_h.begin() + d0, ctx->dep_need_h.begin() + d1);
-  for (auto& x : need) x += extra;
-  TP_CUDA_OK(cudaMemcpy(ctx->d_dep_need + d0, need.data(), need.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+  const int h[2] = {extra > 0 ? (int)tent : -1, extra};
+  TP_CUDA_OK(cudaMemcpy(ctx->d_inject, h, sizeof(h), cudaMemcpyHostToDevice));
   return TP_OK;
 }
 
@@ -1492,7 +1608,7 @@ extern "C" int tp_advance(tp_ctx* ctx, int32_t level_begin, int32_t level_end, v
           e = cudaGetLastError();
         }
         if (e == cudaSuccess)
-          e = launch_layer(ctx, a, ctx->persist_clusters, ctx->persist_cs, 0, ctx->cap_stream, ctx->mixed ? 1 : 0, true);
+          e = launch_layer(ctx, a, ctx->persist_clusters, ctx->persist_cs, 0, ctx->cap_stream, forward_kind(ctx), true);
         if (e != cudaSuccess) {
           tp::set_error(std::string("tp_advance: CUDA error ") + cudaGetErrorString(e));
           rc = TP_ERR_CUDA;

@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstdio>
 #include <map>
+#include <mutex>
 #include <numeric>
 #include <string>
 #include <vector>
@@ -293,6 +294,167 @@ SimplexRule simplex_rule(int n, int m) {
     for (int d = 0; d < n; ++d) R.bary[q * (n + 1) + 1 + d] = pt[d];
   }
   return R;
+}
+
+namespace {
+
+// Fully symmetric rules with positive weights and interior points, as orbits of
+// barycentric coordinates under permutation: found from random starts by
+// Gauss-Newton on the moment equations of degree 2p (5 for the 14 points) and
+// polished to 45 digits there.  kind: digits = how often each value repeats
+// (3 or 4: the centroid); weights sum to 1 over the rule.
+struct Orbit {
+  int kind;
+  double w, a, b;
+};
+const std::vector<Orbit>& face_orbits(int n, int p) {
+  static const std::vector<Orbit> none;
+  static const std::vector<Orbit> d2[6] = {
+      {},
+      {{21, 0.33333333333333333333, 0.16666666666666666667, 0}},
+      {{21, 0.10995174365532186764, 0.09157621350977074346, 0}, {21, 0.2233815896780114657, 0.44594849091596488632, 0}},
+      {{21, 0.08073108959303097831, 0.48013796411221504403, 0},
+       {21, 0.17133312415298103012, 0.21942998254978296, 0},
+       {111, 0.040634559793660662452, 0.01937172436124078838, 0.14161901592396815841}},
+      {{3, 0.14431560767778716825, 0, 0},
+       {21, 0.095091634267284624794, 0.45929258829272315603, 0},
+       {21, 0.10321737053471825028, 0.17056930775176020662, 0},
+       {21, 0.032458497623198080311, 0.050547228317030975458, 0},
+       {111, 0.027230314174434994265, 0.26311282963463811342, 0.0083947774099576053372}},
+      {{3, 0.090817990382753580095, 0, 0},
+       {21, 0.045321059435527934783, 0.1094815754850370548, 0},
+       {21, 0.036725957756466704717, 0.48557763338365737737, 0},
+       {111, 0.028327242531057484837, 0.025003534762686386074, 0.72832390459741092001},
+       {111, 0.072757916845420108604, 0.55035294182099909508, 0.14170721941487995476},
+       {111, 0.0094216669637328234599, 0.92365593358750027665, 0.0095408154002994575802}}};
+  static const std::vector<Orbit> d3[4] = {
+      {},
+      {{31, 0.25, 0.13819660112501051518, 0}},
+      {{31, 0.073493043116361949544, 0.092735250310891226402, 0},
+       {31, 0.1126879257180158508, 0.3108859192633006098, 0},
+       {22, 0.042546020777081466438, 0.45449629587435035051, 0}},
+      {{31, 0.055357181543654722095, 0.32233789014227551034, 0},
+       {31, 0.010077211055320642948, 0.040673958534611353116, 0},
+       {31, 0.0399227502581674921, 0.21460287125915202929, 0},
+       {211, 0.048214285714285714286, 0.063661001875017525299, 0.26967233145831580803}}};
+  if (n == 2 && p <= 5) return d2[p];
+  if (n == 3 && p <= 3) return d3[p];
+  return none;
+}
+
+}  // namespace
+
+static FaceRule make_face_rule(int n, int p, const SimplexRule& front) {
+  FaceRule R;
+  for (const Orbit& o : face_orbits(n, p)) {
+    std::array<double, 4> v{};
+    std::array<int, 4> id{};
+    switch (o.kind) {
+      case 21: v = {o.a, 1.0 - 2.0 * o.a}; id = {0, 0, 1}; break;
+      case 111: v = {o.a, o.b, 1.0 - o.a - o.b}; id = {0, 1, 2}; break;
+      case 31: v = {o.a, 1.0 - 3.0 * o.a}; id = {0, 0, 0, 1}; break;
+      case 22: v = {o.a, 0.5 - o.a}; id = {0, 0, 1, 1}; break;
+      case 211: v = {o.a, o.b, 1.0 - 2.0 * o.a - o.b}; id = {0, 0, 1, 2}; break;
+      default: v = {1.0 / (n + 1)}; break;
+    }
+    do {
+      for (int i = 0; i <= n; ++i) R.bary.push_back(v[id[i]]);
+      R.sqw.push_back(std::sqrt(o.w / (n == 2 ? 2.0 : 6.0)));
+      ++R.S;
+    } while (std::next_permutation(id.begin(), id.begin() + n + 1));
+  }
+  if (R.S == 0 || R.S >= front.Q) return FaceRule();
+  // orthonormal bases of P_p in the inner products of the two rules: monomials
+  // in the barycentric coordinates, Gram-Schmidt twice, carried on the values
+  // at this rule's points and the front's points together
+  const int Q = front.Q, M = R.S + Q;
+  std::vector<long double> w(R.S);
+  for (int i = 0; i < R.S; ++i) w[i] = (long double)R.sqw[i] * R.sqw[i];
+  auto lam = [&](int i, int d) { return (long double)(i < R.S ? R.bary[i * (n + 1) + d] : front.bary[(i - R.S) * (n + 1) + d]); };
+  using Values = std::vector<std::vector<long double>>;
+  auto basis = [&](bool own) {
+    Values phi;
+    auto dot = [&](const std::vector<long double>& f, const std::vector<long double>& g) {
+      long double s = 0.0L;
+      if (own)
+        for (int i = 0; i < R.S; ++i) s += w[i] * f[i] * g[i];
+      else
+        for (int q = 0; q < Q; ++q) s += front.w[q] * f[R.S + q] * g[R.S + q];
+      return s;
+    };
+    for (int e0 = 0; e0 <= p; ++e0)
+      for (int e1 = 0; e0 + e1 <= p; ++e1)
+        for (int e2 = 0; e2 <= (n == 3 ? p - e0 - e1 : 0); ++e2) {
+          std::vector<long double> f(M, 1.0L);
+          for (int i = 0; i < M; ++i) {
+            for (int k = 0; k < e0; ++k) f[i] *= lam(i, 1) - 0.25L;
+            for (int k = 0; k < e1; ++k) f[i] *= lam(i, 2) - 0.25L;
+            for (int k = 0; k < e2; ++k) f[i] *= lam(i, 3) - 0.25L;
+          }
+          for (int pass = 0; pass < 2; ++pass) {
+            for (const auto& g : phi) {
+              const long double s = dot(f, g);
+              for (int i = 0; i < M; ++i) f[i] -= s * g[i];
+            }
+            const long double s = std::sqrt(dot(f, f));
+            for (int i = 0; i < M; ++i) f[i] /= s;
+          }
+          phi.push_back(f);
+        }
+    return phi;
+  };
+  R.stride = Q | 1;
+  const size_t len = (size_t)R.S * R.stride;
+  for (auto* t : {&R.to_points, &R.to_front}) t->assign(len, 0.0);
+  for (auto* t : {&R.to_points_ff, &R.to_front_ff}) t->assign(2 * len, 0.f);
+  auto kernel = [&](const Values& phi) {   // sqw_s K(X_s, x_q)
+    std::vector<long double> k(len, 0.0L);
+    for (int i = 0; i < R.S; ++i)
+      for (int q = 0; q < Q; ++q)
+        for (const auto& g : phi) k[(size_t)i * R.stride + q] += R.sqw[i] * g[i] * g[R.S + q];
+    return k;
+  };
+  const std::vector<long double> kq = kernel(basis(false)), ks = kernel(basis(true));
+  // a row of entries (at[e], value, weight in the constant's sum) rounded one
+  // after the other, largest first, each taking the weighted error so far
+  struct Entry {
+    size_t at;
+    long double value, weight;
+  };
+  auto round_row = [&](std::vector<Entry> row, std::vector<double>& t, std::vector<float>& ff) {
+    std::stable_sort(row.begin(), row.end(), [](const Entry& x, const Entry& y) { return fabsl(x.value) > fabsl(y.value); });
+    long double c = 0.0L, cf = 0.0L;
+    for (const Entry& e : row) {
+      long double v = e.value + c / e.weight;
+      t[e.at] = (double)v;
+      c = (v - t[e.at]) * e.weight;
+      v = e.value + cf / e.weight;
+      const float hi = (float)v, lo = (float)(v - hi);
+      ff[2 * e.at] = hi;
+      ff[2 * e.at + 1] = lo;
+      cf = (v - hi - lo) * e.weight;
+    }
+  };
+  for (int i = 0; i < R.S; ++i) {
+    std::vector<Entry> row;
+    for (int q = 0; q < Q; ++q) row.push_back({(size_t)i * R.stride + q, kq[(size_t)i * R.stride + q] * front.w[q], 1.0L});
+    round_row(row, R.to_points, R.to_points_ff);
+  }
+  for (int q = 0; q < Q; ++q) {
+    std::vector<Entry> row;
+    for (int i = 0; i < R.S; ++i) row.push_back({(size_t)i * R.stride + q, ks[(size_t)i * R.stride + q], (long double)R.sqw[i]});
+    round_row(row, R.to_front, R.to_front_ff);
+  }
+  return R;
+}
+
+const FaceRule& face_rule(int n, int p, const SimplexRule& front) {
+  static std::mutex mu;
+  static std::map<std::pair<int, int>, FaceRule> made;   // at most one per supported (n, p)
+  std::lock_guard<std::mutex> lk(mu);
+  auto it = made.find({n, p});
+  if (it == made.end()) it = made.emplace(std::make_pair(n, p), make_face_rule(n, p, front)).first;
+  return it->second;
 }
 
 }  // namespace tp

@@ -56,6 +56,30 @@ struct SimplexRule {
 };
 SimplexRule simplex_rule(int n, int m);
 
+// The S-point rule of the tent matrix's face integrals, exact to degree 2p
+// with about the fewest points known (2D p = 4: 16 instead of the front rule's
+// 25; 3D p = 3: 24 instead of 64).  U^p restricted to a face is in P_p, so its
+// values at these points carry all of it.  With K the reproducing kernel of P_p
+// in a rule's inner product (K_S: this rule's, K_Q: the front rule's), u(x) =
+// sum_s w_s K_S(X_s, x) u(X_s), w_s = sqw_s^2.  Between the points (values scaled
+// by sqw) and the front's points:
+//   to_points[s * stride + q] = sqw_s w_q K_Q(X_s, x_q)   (sums with weights: moments of front data)
+//   to_front[s * stride + q]  = sqw_s K_S(X_s, x_q)       (values)
+// Both are exact on P_p whatever the rounding of the rules' points and weights,
+// so that the data a tent leaves are the data the next one integrates.
+// Rounded so that a constant passes with an error far below one rounding
+// (each row's rounding errors are carried into its next entries): the same
+// table serves every tent of a sweep, and its errors would add up.
+// S = 0 where the front rule itself is as small (1D).
+struct FaceRule {
+  int S = 0, stride = 0;
+  std::vector<double> bary, sqw;     // S * (n+1); S, square roots of the weights
+  std::vector<double> to_points, to_front;
+  std::vector<float> to_points_ff, to_front_ff;   // the same as float-float pairs
+};
+// (made once per process for each (n, p); front: simplex_rule(n, p + 1))
+const FaceRule& face_rule(int n, int p, const SimplexRule& front);
+
 }  // namespace tp
 
 // ---------------------------------------------------------------------------

@@ -17,8 +17,9 @@ namespace cg = cooperative_groups;
 
 namespace tp {
 
-constexpr int kThreads = 256;
-constexpr int kMaxPair = 3;      // Gram pairs per thread (nb (nb+1)/2 <= 3 * 256: dim U^p <= 38)
+constexpr int kThreads = 256;      // of a CTA where two share an SM
+constexpr int kThreadsWide = 512;  // where one CTA fills the SM's shared memory (16 warps hide more latency than 8)
+constexpr int kMaxPairs = 768;   // Gram pairs nb (nb+1)/2 (dim U^p <= 38)
 constexpr int kMaxRefine = 40;   // refinement steps of the mixed path
 constexpr long long kMaxSpin = 1LL << 20;   // bounded dependency wait: 2^20 polls (well under a second), then TP_ERR_TIMEOUT
 
@@ -31,7 +32,13 @@ __device__ __forceinline__ void red_release_add(int* p, int v) {
   asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// arrays of a tent's patch in shared memory (KArgs::geo: offsets in doubles)
+struct Geo {
+  enum { X, TB, TT, GB, GT, SDET, ISDET, GEL, GBF, FP, FSQ, FN, NTAU, EL, GRP, VID, FW, FG, FG2, NID, COUNT };
+};
+
 struct KArgs {
+  int geo[Geo::COUNT];
   int nb, nmono, Q, nrhs, CH, mono_stride, ngmax;
   int ustride;                    // row stride of the U-values of a point in shared memory (nb rounded up to odd)
   // right-hand sides split over the cluster: CTA r of a tent's cluster owns
@@ -118,13 +125,15 @@ struct KArgs {
   int* status;
   long long* status_info;
   // persistent sweep: tent queue, completed tents per vertex, dependencies
-  // (for tent t: vertices w of its star with the number of their tents that
-  // must be complete, [dep_ptr[t], dep_ptr[t+1]))
+  // (for tent t at v, [dep_ptr[t], dep_ptr[t+1]): how many tents of v and of
+  // each of its neighbours, in the order of the star record, precede it)
   int* queue;
   int* done;
   const int* dep_ptr;
-  const int* dep_vert;
   const int* dep_need;
+  const int* vt_ptr;          // per vertex w: its front times after 0, 1, .. of its tents, vt_tau[vt_ptr[w] ..]
+  const double* vt_tau;
+  const int* inject;          // (tent, extra): that tent waits for `extra` completions more (tp_inject_wait)
   const int* queue_tent;      // tent at each queue position (level order, critical chains first)
   int tent_end;
   // shared-memory carve (offsets in doubles)
@@ -136,10 +145,20 @@ struct KArgs {
   const double* relT_fac;
   const float* rel_facf;      // relation factors (small integers) in binary32
   const float* relT_facf;
-  int off_al, off_eq, off_z, off_x;             // solve: binary32 inverse and refinement
+  int off_eq, off_z, off_x;                     // solve: scales, scaled residual, iterate
   int off_pt;                                   // per-point (that, xhat, scale) of the block-wide evaluation
-  int keep_pts, off_keep, off_keepw;            // kept top U-values (scaled) and 1/sqrt(w) of a CTA's slice
-  int off_b, off_pg, off_ph, off_pgb, off_pm, off_pd, off_sg, off_sm, off_f, off_f2, off_fpm, off_del,
+  int keep_pts, off_keep;                       // kept U-values (scaled, both faces) of a CTA's slice
+  int cb_pts;                                   // points of the data-coefficient buffer
+  int ev_rows;                                  // points evaluated at a time into the kept rows
+  // kept tents: the S-point rule of the face integrals (0: the front rule) and
+  // the tables between its points and the front's (FaceRule: to_points, then
+  // to_front), in shared memory at off_tf; raw_el elements' front data at a
+  // time at off_raw
+  int S, tf_stride, off_tf, raw_el, off_raw;
+  const double *s_bary, *s_sqw, *tf;
+  const float2* tf_dd;
+  int off_rc;                                   // pivot row and column of the shared-memory elimination (two of each)
+  int off_b, off_pg, off_ph, off_pgb, off_pm, off_pd, off_sm, off_f, off_f2, off_fpm, off_del,
       off_u, off_mono, off_cb, off_gd, off_y, off_rd;
   // tensor-core contractions (mixed forward sweep with split right-hand
   // sides, single-material tents): the data moments and the outflow run as
@@ -271,6 +290,15 @@ __device__ __forceinline__ dd dd_split(double x) {
   return {__uint_as_float(hb), lo};
 }
 
+// 1/x of a float-float value: Newton step r + r (1 - x r) from the binary32
+// reciprocal of the leading part (24 -> 48 bits)
+__device__ __forceinline__ dd dd_rcp(dd x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x.hi));
+  const float e = fmaf(-x.lo, r, fmaf(-x.hi, r, 1.f));
+  return fast_two_sum(r, __fmul_rn(r, e));
+}
+
 template <typename T>
 struct Ar;
 
@@ -294,6 +322,9 @@ struct Ar<double> {
   static __device__ __forceinline__ double accn(double s, double a, double b) { return ::fma(-a, b, s); }
   static __device__ __forceinline__ double norm(double s) { return s; }
   static __device__ __forceinline__ double fma(double a, double b, double c) { return ::fma(a, b, c); }
+  // x s as a float-float pair for a power of two s, and back
+  static __device__ __forceinline__ dd scaled(double x, float s) { return dd_split(x * (double)s); }
+  static __device__ __forceinline__ double of(dd x) { return (double)x.hi + (double)x.lo; }
   static __device__ __forceinline__ double coef(const KArgs& a, int e);
 };
 
@@ -341,6 +372,8 @@ struct Ar<dd> {
   static __device__ __forceinline__ dd accn(dd s, dd a, dd b) { return acc(s, {-a.hi, -a.lo}, b); }   // s -= a b
   static __device__ __forceinline__ dd norm(dd s) { return fast_two_sum(s.hi, s.lo); }
   static __device__ __forceinline__ dd fma(dd a, dd b, dd c) { return dd_add(dd_mul(a, b), c); }
+  static __device__ __forceinline__ dd scaled(dd x, float s) { return {__fmul_rn(x.hi, s), __fmul_rn(x.lo, s)}; }
+  static __device__ __forceinline__ dd of(dd x) { return x; }
   static __device__ __forceinline__ dd coef(const KArgs& a, int e);
 };
 
@@ -489,13 +522,18 @@ __device__ __forceinline__ T relT_apply(const KArgs& a, int k, int var, const T*
 }
 
 // binary32 reciprocal of the hardware's approximate reciprocal instruction
-// (about 1 ulp): the binary32 inverse of the solve is refined against A, so its
-// last bit does not matter, and the correctly rounded reciprocal costs several
-// times as long on the critical path of the elimination
+// (about 1 ulp): the inverse of the solve is refined against A, so its last
+// bits do not matter, and the correctly rounded reciprocal costs several times
+// as long in the elimination's chain of pivots
 __device__ __forceinline__ float rcp_fast(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
+}
+// power of two nearest below 1 / sqrt(d) (within a factor of two; exact scaling)
+__device__ __forceinline__ float pow2_rsqrt(float d) {
+  const int e = (int)((__float_as_uint(d) >> 23) & 0xFF) - 127;
+  return __uint_as_float((unsigned int)(127 - (e >> 1)) << 23);
 }
 
 // 1/x by two Newton-Raphson steps r <- r + r (1 - x r) from the binary32
@@ -587,10 +625,10 @@ __device__ __forceinline__ void iface_terms(const KArgs& a, int i, int j, const 
 // solves, and writes the outflow of its slice.
 //
 // MIXED = false: assembly, residual and outflow in binary64; MIXED = true:
-// in float-float.  Both: A is equilibrated (D A D, D = |diag A|^-1/2),
-// inverted in binary32 and the solution refined against A in the path's
-// precision until the correction stops shrinking; a refinement that does not
-// settle falls back to a direct binary64 LU.
+// in float-float.  Both: A is equilibrated (D A D, D powers of two near
+// |diag A|^-1/2), inverted in float-float and the solution refined against A in
+// the path's precision until the correction stops shrinking; a refinement that
+// does not settle falls back to a direct binary64 LU.
 //
 // ADJ = true: the adjoint tent map (reverse sweep).  With g_D = 0 a tent maps
 // its bottom values linearly to its top values, b = B f_bot, A x = b,
@@ -609,8 +647,20 @@ __device__ __forceinline__ void iface_terms(const KArgs& a, int i, int j, const 
 // awaited tent is held by a running cluster: no launch per level, and a tent
 // starts as soon as its own inputs are ready.  The front and the front times
 // are read through L2 (ld.global.cg) so that no stale L1 line is used.
-template <int DIM, bool MIXED, bool ADJ, bool PERSIST, bool NEU>
-__global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int tent0) {
+//
+// What bounds a sweep with few right-hand sides is the chain of dependent
+// tents (levels times what a tent does between its wait and its publication)
+// or, on wide levels, the work of all tents over the resident CTAs.  The tent
+// matrix depends on the front times alone, which the tents fix, so the
+// geometry, the U-values, A and its inverse come before the wait: the chain
+// keeps the moments, b, the solve and the outflow.  2D p = 4, 968 triangles,
+// one column: 18.5 -> 10.4 ms binary64, 26.9 -> 8.6 ms mixed (with the S-point
+// rule and the float-float inverse below).
+template <int DIM, bool MIXED, bool ADJ, bool PERSIST, bool NEU, bool SPLIT, bool TC, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) k_layer(const KArgs a, const int tent0) {
+  static_assert(!TC || (MIXED && !ADJ && SPLIT), "tensor-core contractions: mixed forward sweep, split right-hand sides");
+  constexpr int NT = WIDE ? kThreadsWide : kThreads, NW = NT / 32;   // threads and warps of a CTA
+  constexpr int kMaxPair = (kMaxPairs + NT - 1) / NT;            // Gram pairs per thread
   using T = typename std::conditional<MIXED, dd, double>::type;
   using R = Ar<T>;
   constexpr int NV = DIM + 1;   // vertices per element
@@ -620,58 +670,90 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
   __shared__ double s_ttop, s_tbot, s_tc, s_ih;
   __shared__ double s_gc[tp::kMaxGroups], s_gic2[tp::kMaxGroups];   // speeds and 1/c^2 of the materials
   __shared__ double s_xv[DIM];
-  __shared__ int s_el[tp::kMaxPatch], s_grp[tp::kMaxPatch];
-  // vertex ids of elements; of facets (slots 2..): for boundary facets slot 0
-  // holds the block of their data among the vertex's boundary facets
-  __shared__ int s_vid[tp::kMaxPatch][NV], s_fw[tp::kMaxFacets][NV];
-  __shared__ double s_X[tp::kMaxPatch][NV][DIM];
-  __shared__ double s_tb[tp::kMaxPatch][NV], s_tt[tp::kMaxPatch][NV];
-  __shared__ double s_gb[tp::kMaxPatch][DIM], s_gt[tp::kMaxPatch][DIM];
-  __shared__ double s_sdet[tp::kMaxPatch], s_isdet[tp::kMaxPatch];
-  // mixed path: g_bot (DIM) and sqrt|det| (slot DIM) of each element and c^-2 of each material as float-float pairs
-  __shared__ float2 s_gbf[MIXED ? tp::kMaxPatch : 1][DIM + 1];
-  __shared__ float2 s_gic2f[tp::kMaxGroups];
-  __shared__ double s_fP[tp::kMaxFacets][NV][DIM + 1];   // vertical face simplices (x, t)
-  __shared__ double s_fsq[tp::kMaxFacets], s_fn[tp::kMaxFacets][DIM];   // sqrt(n! volume), normal
-  __shared__ int s_fg[tp::kMaxFacets], s_fg2[tp::kMaxFacets];   // groups (Dirichlet: one; interface: +, -)
-  __shared__ int s_pgrp[2 * 64];
-  __shared__ double s_gel[tp::kMaxPatch];   // wave-speed gradient of the tent per patch element
+  // the patch, in dynamic shared memory sized for the context's largest star
+  // (off_geo, in the order of Geo): per element its vertices' coordinates,
+  // bottom and top times, front gradients, sqrt|det| and its reciprocal, the
+  // tent's wave-speed gradient and, mixed path, g_bot (DIM) and sqrt|det| (slot
+  // DIM) as float-float pairs; per facet its simplex (x, t), sqrt(n! volume)
+  // and normal; the front times of v and its neighbours; then integers: element
+  // id and material, the place of each of its vertices in the list of v and its
+  // neighbours; of a facet the same (slots 2..; for boundary facets slot 0
+  // holds the block of their data among the vertex's boundary facets) and its
+  // groups (Dirichlet: one; interface: +, -); the neighbour list's vertex ids
+  double(*const s_X)[NV][DIM] = reinterpret_cast<double(*)[NV][DIM]>(sm + a.geo[Geo::X]);
+  double(*const s_tb)[NV] = reinterpret_cast<double(*)[NV]>(sm + a.geo[Geo::TB]);
+  double(*const s_tt)[NV] = reinterpret_cast<double(*)[NV]>(sm + a.geo[Geo::TT]);
+  double(*const s_gb)[DIM] = reinterpret_cast<double(*)[DIM]>(sm + a.geo[Geo::GB]);
+  double(*const s_gt)[DIM] = reinterpret_cast<double(*)[DIM]>(sm + a.geo[Geo::GT]);
+  double* const s_sdet = sm + a.geo[Geo::SDET];
+  double* const s_isdet = sm + a.geo[Geo::ISDET];
+  double* const s_gel = sm + a.geo[Geo::GEL];
+  float2(*const s_gbf)[DIM + 1] = reinterpret_cast<float2(*)[DIM + 1]>(sm + a.geo[Geo::GBF]);
+  double(*const s_fP)[NV][DIM + 1] = reinterpret_cast<double(*)[NV][DIM + 1]>(sm + a.geo[Geo::FP]);
+  double* const s_fsq = sm + a.geo[Geo::FSQ];
+  double(*const s_fn)[DIM] = reinterpret_cast<double(*)[DIM]>(sm + a.geo[Geo::FN]);
+  double* const s_ntau = sm + a.geo[Geo::NTAU];
+  int* const s_el = reinterpret_cast<int*>(sm + a.geo[Geo::EL]);
+  int* const s_grp = reinterpret_cast<int*>(sm + a.geo[Geo::GRP]);
+  int(*const s_vid)[NV] = reinterpret_cast<int(*)[NV]>(sm + a.geo[Geo::VID]);
+  int(*const s_fw)[NV] = reinterpret_cast<int(*)[NV]>(sm + a.geo[Geo::FW]);
+  int* const s_fg = reinterpret_cast<int*>(sm + a.geo[Geo::FG]);
+  int* const s_fg2 = reinterpret_cast<int*>(sm + a.geo[Geo::FG2]);
+  int* const s_nid = reinterpret_cast<int*>(sm + a.geo[Geo::NID]);
+  __shared__ float2 s_gic2f[tp::kMaxGroups];   // mixed path: c^-2 of each material as a float-float pair
+  __shared__ int s_ge0[tp::kMaxGroups + 1];   // elements of material g: [s_ge0[g], s_ge0[g + 1])
   __shared__ int s_piv;
-  __shared__ float s_pb[2][4][32];   // register sweeps: the pivot rows of a block of four steps
-  __shared__ float s_red[2][kThreads / 32];
+  __shared__ dd s_pb[2][4][32];   // register elimination: the pivot rows of a block of four steps
+  __shared__ float s_red[2][NW];
 
-  __shared__ int s_tent;
+  __shared__ int s_tent, s_bad;
   // tensor-core contractions: tensor-memory base, completion barrier of the
   // MMAs, binary exponents of the rows of A (0) and the columns of B (1)
   __shared__ uint32_t s_tmem;
   __shared__ __align__(8) uint64_t s_tcbar;
-  __shared__ int s_tce[2][tc::kMaxM];
+  __shared__ int s_tce[2][TC ? tc::kMaxM : 1];
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
   const int CS = (int)cluster.num_blocks();
   const int tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
-  constexpr bool kTC = MIXED && !ADJ;   // the tensor-core path exists for the mixed forward sweep
+  constexpr bool kTC = TC;
   uint32_t tc_phase = 0;                // parity of the next completion of s_tcbar
-  if (kTC && a.tc) {
+  if constexpr (kTC) {
     if (warp == 0) tc::tmem_alloc(&s_tmem, a.tc_cols);
     if (tid == 0) tc::mbar_init(&s_tcbar, 1);
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
   }
+  if (!SPLIT && a.S > 0) {   // (ordered before its first use by the first tent's barriers)
+    T* sTF = reinterpret_cast<T*>(sm + a.off_tf);
+    for (int id = tid; id < 2 * a.S * a.tf_stride; id += NT) {
+      if constexpr (MIXED) sTF[id] = {a.tf_dd[id].x, a.tf_dd[id].y};
+      else sTF[id] = a.tf[id];
+    }
+  }
+  // barrier of the cluster (a cluster of one CTA: the block's)
+  auto csync = [&]() {
+    if (CS > 1) cluster.sync();
+    else __syncthreads();
+  };
   for (;;) {
   int tent;
   if constexpr (PERSIST) {
     // rank 0 takes the next tent and stores its index into every CTA of the
     // cluster (each CTA read its copy of the previous index several cluster
     // barriers ago)
+    if (tid == 0) s_bad = 0;
     if (rank == 0 && tid == 0) {
       const int pos = atomicAdd(a.queue, 1);
       const int t_ = pos < a.tent_end ? __ldg(a.queue_tent + pos) : a.tent_end;
-      for (int r = 0; r < CS; ++r) *cluster.map_shared_rank(&s_tent, r) = t_;
+      if (CS > 1)
+        for (int r = 0; r < CS; ++r) *cluster.map_shared_rank(&s_tent, r) = t_;
+      else
+        s_tent = t_;
     }
-    cluster.sync();
+    csync();
     tent = s_tent;
     if (tent >= a.tent_end) break;
   } else {
@@ -680,7 +762,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
   const int nb = a.nb, Q = a.Q, nrhs = a.nrhs, CH = a.CH, NG = a.ngmax;
   const int us = a.ustride;   // row stride of the U-values in shared memory (odd: no bank conflicts between points)
   // this CTA's right-hand sides (all of the group unless they are split over the cluster)
-  const bool rsplit = a.rsplit != 0;
+  constexpr bool rsplit = SPLIT;
   double* const front = a.front + (rsplit ? (size_t)rank * nrhs * a.ne * Q * C : 0);
   const double* const gD = a.gD != nullptr ? a.gD + (rsplit ? (size_t)rank * nrhs * a.n_bnd : 0) : nullptr;
   const int npair = nb * (nb + 1) / 2;
@@ -691,8 +773,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
   T* sPH = reinterpret_cast<T*>(sm + a.off_ph);      // NG*DIM*npair  H_m
   T* sPGb = reinterpret_cast<T*>(sm + a.off_pgb);    // NG*npair   G (bottom, recovery)
   T* sPM = reinterpret_cast<T*>(sm + a.off_pm);      // NG*nmom    moments (gamma, alpha, beta_m) per rhs, this CTA
-  T* sPD = reinterpret_cast<T*>(sm + a.off_pd);      // N*N        interface blocks (tents with interface facets)
-  T* sSG = reinterpret_cast<T*>(sm + a.off_sg);      // NG*(DIM+2)*npair  summed G, H_m, Gbot
+  T* sSG = sPG;                                      // the same summed over the cluster, in place
   T* sSM = reinterpret_cast<T*>(sm + a.off_sm);      // NG*nmom    summed moments (in place of sPM)
   T* sF = reinterpret_cast<T*>(sm + a.off_f);        // npair      facet Gram (+ side)
   T* sF2 = reinterpret_cast<T*>(sm + a.off_f2);      // npair      facet Gram (- side)
@@ -702,7 +783,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
   T* sPt = reinterpret_cast<T*>(sm + a.off_pt);      // 2*CH*(DIM+2)  (that, xhat, scale) per point
   T* sM = reinterpret_cast<T*>(sm + a.off_mono);     // 2*CH*mono_stride
   T* sCB = reinterpret_cast<T*>(sm + a.off_cb);      // nrhs*C*(CH+1) data coefficients, point fastest
-  const int cbs = CH + 1;                            // their row stride (odd: no bank conflicts along a row)
+  const int cbs = a.cb_pts | 1;                      // their row stride (odd: no bank conflicts along a row)
   T* sGd = reinterpret_cast<T*>(sm + a.off_gd);      // CH*nrhs    Dirichlet data coefficients
   T* sY = reinterpret_cast<T*>(sm + a.off_y);        // NG*nmom    outflow coefficient vectors (sPM, dead after the congruence)
   double* sRD = sm + a.off_rd;                       // N          reciprocal pivots (binary64 path)
@@ -725,8 +806,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
     s_ng = ng;
     s_nneu = h1.w;
   }
-  for (int id = tid; id < NG * nmom; id += blockDim.x) sPM[id] = R::zero();
-  for (int id = tid; id < NG * (DIM + 2) * npair; id += blockDim.x) sPG[id] = R::zero();   // PG, PH, PGb contiguous
   const int N = ng * nb;
   const bool extra = (nfac > 0 || nif > 0 || (NEU && h1.w > 0));
   {
@@ -744,7 +823,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
     const double* rX = rd + DIM + 2 * tp::kMaxGroups;
     for (int k = tid; k < P; k += blockDim.x) {
       s_el[k] = __ldg(ri + k * (2 + NV));
-      s_grp[k] = __ldg(ri + k * (2 + NV) + 1);
+      const int gk = __ldg(ri + k * (2 + NV) + 1);   // (elements are sorted by material)
+      s_grp[k] = gk;
+      if (k == 0 || __ldg(ri + (k - 1) * (2 + NV) + 1) != gk) s_ge0[gk] = k;
       for (int i = 0; i < NV; ++i) {
         s_vid[k][i] = __ldg(ri + k * (2 + NV) + 2 + i);
         for (int d = 0; d < DIM; ++d) s_X[k][i][d] = __ldg(rX + (k * NV + i) * DIM + d);
@@ -753,6 +834,14 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
     // vertical face simplices (x_v, t_bot), (x_v, t_top), (x_w, tau_w): Dirichlet
     // facets first, then the time-like interface facets, then Neumann facets
     const int* rfi = ri + P * (2 + NV);
+    const int nfa = nfac + nif + h1.w, d0 = __ldg(a.dep_ptr + tent), nn = __ldg(a.dep_ptr + tent + 1) - d0;
+    for (int e = tid; e < nn; e += blockDim.x) {
+      const int w = __ldg(rfi + nfa * (NV + 3) + e);
+      s_nid[e] = w;
+      // the front time of w when this tent's turn comes: fixed by the tents alone
+      if (PERSIST) s_ntau[e] = __ldg(a.vt_tau + __ldg(a.vt_ptr + w) + __ldg(a.dep_need + d0 + e));
+    }
+    if (tid < ng + 1 && tid == ng) s_ge0[ng] = P;
     const double* rfd = rX + P * NV * DIM;
     for (int f = tid; f < nfac + nif + (NEU ? h1.w : 0); f += blockDim.x) {
       for (int i = 2; i < NV; ++i) s_fw[f][i] = __ldg(rfi + f * (NV + 3) + i);
@@ -765,15 +854,18 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
         for (int d = 0; d < DIM; ++d) s_fP[f][i][d] = __ldg(fd + DIM + i * DIM + d);
     }
   }
-  if constexpr (PERSIST) {
-    // the earlier tents of this vertex and its neighbours must be complete:
-    // every CTA of a tent publishes its own completion, so a vertex whose
-    // first `need` tents are done has a count of need * CS; each CTA waits
-    // for (and acquires) the counts itself
-    {
-      const int d0 = a.dep_ptr[tent], d1 = a.dep_ptr[tent + 1];
-      for (int e = d0 + tid; e < d1; e += blockDim.x) {
-        const int w = a.dep_vert[e], need = a.dep_need[e] * CS;
+  const int d0_ = __ldg(a.dep_ptr + tent), nn_ = __ldg(a.dep_ptr + tent + 1) - d0_;
+  // the earlier tents of this vertex and its neighbours must be complete:
+  // every CTA of a tent publishes its own completion, so a vertex whose
+  // first `need` tents are done has a count of need * CS; each CTA waits
+  // for (and acquires) the counts itself
+  auto wait_deps = [&]() {
+    if constexpr (PERSIST) {
+      const int extra_ = __ldg(a.inject) == tent ? __ldg(a.inject + 1) : 0;
+      for (int e = tid; e < nn_; e += blockDim.x) {
+        const int before = __ldg(a.dep_need + d0_ + e);
+        if (before == 0) continue;
+        const int w = s_nid[e], need = (before + extra_) * CS;
         long long spins = 0;
         while (ld_acquire(a.done + w) < need) {
           if (++spins > a.max_spin) {
@@ -786,178 +878,96 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
           __nanosleep(32);
         }
       }
+      __syncthreads();
     }
-    __syncthreads();
-  } else {
-    __syncthreads();
-  }
-  // (b) the front times: bottom and top fronts over every element, causality
-  const double tbot = ADJ ? a.tent_tbot[tent] : __ldcg(a.tau + v);
-  if (tid == 0) {
-    s_tbot = tbot;
-    s_tc = 0.5 * (tbot + s_ttop);
-  }
-  for (int k = tid; k < P; k += blockDim.x) {
-    for (int i = 0; i < NV; ++i) {
-      const int vi = s_vid[k][i];
-      const double tv = (vi == v) ? tbot : __ldcg(a.tau + vi);
-      s_tb[k][i] = tv;
-      s_tt[k][i] = (vi == v) ? s_ttop : tv;
-    }
-    // gradients of the linear fronts: g = e^-1 (tau_i - tau_0), e from the host
-    const int el = s_el[k];
-    double db[DIM], dt[DIM];
-    for (int i = 0; i < DIM; ++i) {
-      db[i] = s_tb[k][i + 1] - s_tb[k][0];
-      dt[i] = s_tt[k][i + 1] - s_tt[k][0];
-    }
-    double g2 = 0.0;
-    for (int d = 0; d < DIM; ++d) {
-      double gb = 0.0, gt = 0.0;
-      for (int i = 0; i < DIM; ++i) {
-        const double ei = __ldg(a.elem_einv + ((int64_t)el * DIM + d) * DIM + i);
-        gb = fma(ei, db[i], gb);
-        gt = fma(ei, dt[i], gt);
-      }
-      s_gb[k][d] = gb;
-      s_gt[k][d] = gt;
-      g2 = fma(gt, gt, g2);
-    }
-    s_sdet[k] = __ldg(a.elem_sdet + el);
-    s_isdet[k] = __ldg(a.elem_isdet + el);
-    if constexpr (MIXED) {
-      for (int d = 0; d < DIM; ++d) {
-        const dd gf = dd_split(s_gb[k][d]);
-        s_gbf[k][d] = make_float2(gf.hi, gf.lo);
-      }
-      const dd sf = dd_split(s_sdet[k]);
-      s_gbf[k][DIM] = make_float2(sf.hi, sf.lo);
-    }
-    const double ck = s_gc[s_grp[k]];
-    if (!(ck * ck * g2 < 1.0)) flag_error(a, TP_ERR_CAUSALITY, tent);   // space-like top face: c |g| < 1
-  }
-  for (int f = tid; f < nfac + nif + (NEU ? s_nneu : 0); f += blockDim.x) {
-    s_fP[f][0][DIM] = tbot;
-    s_fP[f][1][DIM] = s_ttop;
-    for (int c2 = 2; c2 <= DIM; ++c2) s_fP[f][c2][DIM] = __ldcg(a.tau + s_fw[f][c2]);
-    // n! * n-volume = sqrt(det(E^T E)), E = [P_i - P_0] ((n+1) x n)
-    double G[DIM][DIM];
-    for (int i = 0; i < DIM; ++i)
-      for (int j = 0; j < DIM; ++j) {
-        double s_ = 0.0;
-        for (int d = 0; d <= DIM; ++d) s_ += (s_fP[f][i + 1][d] - s_fP[f][0][d]) * (s_fP[f][j + 1][d] - s_fP[f][0][d]);
-        G[i][j] = s_;
-      }
-    // sqrt(w) = sqrt(w_ref) sqrt(n! volume) at the facet's points
-    s_fsq[f] = sqrt(sqrt(fabs(small_det<DIM>(G))));
-  }
-  // Gram pairs owned by this thread (upper triangle, i <= j, row-major order)
-  int pi[kMaxPair], pj[kMaxPair];
-  T aK[kMaxPair], aG[kMaxPair], aH[kMaxPair][DIM], aB[kMaxPair];
-#pragma unroll
-  for (int s = 0; s < kMaxPair; ++s) {
-    const int id = tid + s * kThreads;
-    int i = 0, j = 0;
-    if (id < npair) {
-      int rem = id;
-      while (rem >= nb - i) {
-        rem -= nb - i;
-        ++i;
-      }
-      j = i + rem;
-    }
-    pi[s] = i;
-    pj[s] = j;
-    aK[s] = aG[s] = aB[s] = R::zero();
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) aH[s][d] = R::zero();
-  }
+  };
+  // The tent matrix depends on the front times only, and those are fixed by
+  // the tents: in the dataflow sweep a tent is assembled and inverted from
+  // the tabulated times while the tents it waits for still run, and only the
+  // data of the bottom front, the solve and the outflow follow the wait.  A
+  // front whose times are not the tabulated ones (tp_set_front with others)
+  // is found after the wait, and the tent assembled again from its own.
+  // (`real`: the times are those of the front)
+  const int slice_el = (P + CS - 1) / CS;   // a CTA's share of the patch: whole elements
+  const int QK = a.S > 0 ? a.S : Q;         // points per element of a kept tent
+  const bool kept = !SPLIT && slice_el * QK <= a.keep_pts;
+  bool real = !PERSIST;
   __syncthreads();
-
-  // tensor-core contractions for this tent (single material, split right-hand sides)
-  const bool tc_on = kTC && a.tc && ng == 1;
-  // ---------------- phase 1: this CTA's slice of the patch points ----------------
-  const int NP = P * Q;
-  const int slice = (NP + CS - 1) / CS;
-  const int q0 = min(NP, rank * slice), q1 = min(NP, q0 + slice);
-  const double ih = s_ih, tc = s_tc;
-  int curk = q0 / Q, kend = (curk + 1) * Q;
-  int curg = (q1 > q0) ? s_grp[curk] : 0;
-  // forward sweep: the top U-values of a slice that fits the keep buffer are
-  // kept for the outflow instead of being evaluated a second time
-  const bool keep = !ADJ && !rsplit && (q1 - q0) <= a.keep_pts;
-  T* sKeep = reinterpret_cast<T*>(sm + a.off_keep);   // keep_pts*nb  sqrt(w)-scaled top U-values
-  double* sKeepW = sm + a.off_keepw;                   // keep_pts     1 / sqrt(w)
-  // element flush: G += G_K, H_m += g_{K,m} G_K;  group flush: publish G, H, Gbot of the group
-  auto flush_element = [&](int k) {
-    T g[DIM];
-    for (int d = 0; d < DIM; ++d) g[d] = R::from(s_gt[k][d]);
-#pragma unroll
-    for (int s = 0; s < kMaxPair; ++s) {
-      const T k_ = R::norm(aK[s]);
-      aG[s] = R::add(aG[s], k_);
-#pragma unroll
-      for (int d = 0; d < DIM; ++d) aH[s][d] = R::fma(g[d], k_, aH[s][d]);
-      aK[s] = R::zero();
-    }
-  };
-  auto flush_group = [&](int g) {
-#pragma unroll
-    for (int s = 0; s < kMaxPair; ++s) {
-      const int id = tid + s * kThreads;
-      if (id < npair) {
-        sPG[g * npair + id] = R::add(sPG[g * npair + id], aG[s]);
-#pragma unroll
-        for (int d = 0; d < DIM; ++d)
-          sPH[(g * DIM + d) * npair + id] = R::add(sPH[(g * DIM + d) * npair + id], aH[s][d]);
-        sPGb[g * npair + id] = R::add(sPGb[g * npair + id], R::norm(aB[s]));
+  // after the wait: s_bad of every CTA of the cluster is set where a time
+  // used is not the front's (read after the next cluster barrier, so that the
+  // CTAs decide alike)
+  auto check_times = [&]() {
+    if constexpr (PERSIST) {
+      for (int e = tid; e < nn_; e += blockDim.x) {
+        if (__ldcg(a.tau + s_nid[e]) == s_ntau[e]) continue;
+        if (CS == 1) s_bad = 1;
+        else
+          for (int r = 0; r < CS; ++r) *cluster.map_shared_rank(&s_bad, r) = 1;
       }
-      aG[s] = aB[s] = R::zero();
-#pragma unroll
-      for (int d = 0; d < DIM; ++d) aH[s][d] = R::zero();
     }
   };
+  // tensor-core contractions for this tent (single material, split right-hand sides)
+  const bool tc_on = kTC && ng == 1;
+  const int NP = P * Q;
+  // this CTA's points of the patch for the Grams (split right-hand sides: even
+  // shares of the points; else whole elements, whose data and outflow are this CTA's too)
+  const int slice = (P * QK + CS - 1) / CS;
+  const int e0 = P * rank / CS, e1 = P * (rank + 1) / CS;
+  const int q0 = SPLIT ? min(P * QK, rank * slice) : e0 * Q;
+  const int q1 = SPLIT ? min(P * QK, q0 + slice) : e1 * Q;
+  const int np = (e1 - e0) * QK;           // points of the slice in the rule of the face integrals
+  // elements whose data are taken at a time (their points fit sU where the rows are not kept)
+  const int EC = kept || a.S == 0 ? a.raw_el : min(a.raw_el, 2 * CH / QK);
+  const double *bary_ = a.S > 0 ? a.s_bary : a.bary, *sqw_ = a.S > 0 ? a.s_sqw : a.sqw;
+  double ih = 0.0, tc = 0.0;
+  T* sKeep = reinterpret_cast<T*>(sm + a.off_keep);   // kept slice: its top U-values, then its bottom U-values
+  T* sKB = sKeep + (size_t)np * us;
+  const T* sTP = reinterpret_cast<const T*>(sm + a.off_tf);   // data to the rule's points, values to the front's
+  const T* sTF = sTP + a.S * a.tf_stride;
+  T* sRaw = reinterpret_cast<T*>(sm + a.off_raw);
   // a patch point q of element k mapped to the tent's reference coordinates
   // (Remark 3.1) on the top (TOP) or bottom face, with sqrt(w) as the scale of
-  // its U-values; returns sqrt(w)
-  auto map_point = [&](T* pp, int k, int q, bool top) {
+  // its U-values
+  // (point q of the front rule; of the rule of bary_, sqw_)
+  auto map_point_of = [&](T* pp, int k, int q, bool top, const double* bary_, const double* sqw_) {
     const double cg = s_gc[s_grp[k]];
     double x[DIM], tt = 0.0;
     for (int d = 0; d < DIM; ++d) x[d] = 0.0;
     for (int i = 0; i < NV; ++i) {
-      const double l = __ldg(a.bary + q * NV + i);
+      const double l = __ldg(bary_ + q * NV + i);
       for (int d = 0; d < DIM; ++d) x[d] = fma(l, s_X[k][i][d], x[d]);
       tt = fma(l, top ? s_tt[k][i] : s_tb[k][i], tt);
     }
     pp[0] = R::from(cg * (tt - tc) * ih);
     for (int d = 0; d < DIM; ++d) pp[1 + d] = R::from((x[d] - s_xv[d]) * ih);
-    const double sw = __ldg(a.sqw + q) * s_sdet[k];
-    pp[DIM + 1] = R::from(sw);
-    return sw;
+    pp[DIM + 1] = R::from(__ldg(sqw_ + q) * s_sdet[k]);
   };
+  auto map_point = [&](T* pp, int k, int q, bool top) { map_point_of(pp, k, q, top, a.bary, a.sqw); };
   // data coefficients of the points base .. base + nq - 1 (patch point
   // numbering) for every right-hand side, one (point, right-hand side) per
   // thread so that the front loads of a chunk are all in flight at once:
   // forward, the bottom values in the form of the moments (gamma, alpha,
-  // beta_m); adjoint, lambda at the top point
-  auto data_coefs = [&](int base, int nq) {
+  // beta_m); adjoint, lambda at the top point; component cc of point ql and
+  // right-hand side r at dst[(r * C + cc) * stride + ql], for the U-values
+  // scaled by sqrt(w) (RAW: without weights)
+  auto data_coefs = [&](int base, int nq, T* dst, int stride, bool raw) {
     for (int id = tid; id < nq * nrhs; id += blockDim.x) {   // (consecutive threads: consecutive points)
       const int r = id / nq, ql = id % nq, qg = base + ql, k = qg / Q, q = qg % Q;
       const double* f = front + (((int64_t)r * a.ne + s_el[k]) * Q + q) * C;
       double fv[C];
 #pragma unroll
       for (int cc = 0; cc < C; ++cc) fv[cc] = __ldcg(f + cc);
-      T* cb = sCB + (size_t)r * C * cbs + ql;   // component cc at cb[cc * cbs]
+      T* cb = dst + (size_t)r * C * stride + ql;
       if constexpr (ADJ) {
         // adjoint: zeta = sum_q lambda_q u_q over the top points
-        const double isw = __ldg(a.isqw + q) * s_isdet[k];
+        const double isw = raw ? 1.0 : __ldg(a.isqw + q) * s_isdet[k];
 #pragma unroll
-        for (int cc = 0; cc < C; ++cc) cb[cc * cbs] = R::from(fv[cc] * isw);
+        for (int cc = 0; cc < C; ++cc) cb[cc * stride] = R::from(fv[cc] * isw);
       } else if constexpr (MIXED) {
         // the same coefficients in float-float, the stored values split by
         // integer operations (no binary64 arithmetic per point and column)
         const float2 w2 = __ldg(a.sqw_dd + q), d2 = s_gbf[k][DIM], c2 = s_gic2f[s_grp[k]];
-        const dd sw = dd_mul({w2.x, w2.y}, {d2.x, d2.y});
+        const dd sw = raw ? dd{1.f, 0.f} : dd_mul({w2.x, w2.y}, {d2.x, d2.y});
         dd f[C];
 #pragma unroll
         for (int cc = 0; cc < C; ++cc) f[cc] = dd_split(fv[cc]);
@@ -968,17 +978,17 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
 #pragma unroll
         for (int d = 1; d < DIM; ++d) sg = dd_add(sg, dd_mul(f[2 + d], gb[d]));
         cb[0] = dd_mul(sw, f[0]);                                                     // gamma
-        cb[cbs] = dd_mul(sw, R::sub(dd_mul({c2.x, c2.y}, f[1]), sg));                   // alpha
+        cb[stride] = dd_mul(sw, R::sub(dd_mul({c2.x, c2.y}, f[1]), sg));                   // alpha
 #pragma unroll
-        for (int d = 0; d < DIM; ++d) cb[(2 + d) * cbs] = dd_mul(sw, R::sub(f[2 + d], dd_mul(f[1], gb[d])));   // beta_m
+        for (int d = 0; d < DIM; ++d) cb[(2 + d) * stride] = dd_mul(sw, R::sub(f[2 + d], dd_mul(f[1], gb[d])));   // beta_m
       } else {
-        const double sw = __ldg(a.sqw + q) * s_sdet[k], ic2 = s_gic2[s_grp[k]];
+        const double sw = raw ? 1.0 : __ldg(a.sqw + q) * s_sdet[k], ic2 = s_gic2[s_grp[k]];
         const double Ub = fv[0], vb = fv[1];
         double sg = 0.0;
         for (int d = 0; d < DIM; ++d) sg = fma(fv[2 + d], s_gb[k][d], sg);
         cb[0] = R::from(sw * Ub);                       // gamma
-        cb[cbs] = R::from(sw * (ic2 * vb - sg));          // alpha
-        for (int d = 0; d < DIM; ++d) cb[(2 + d) * cbs] = R::from(sw * (fv[2 + d] - vb * s_gb[k][d]));   // beta_m
+        cb[stride] = R::from(sw * (ic2 * vb - sg));          // alpha
+        for (int d = 0; d < DIM; ++d) cb[(2 + d) * stride] = R::from(sw * (fv[2 + d] - vb * s_gb[k][d]));   // beta_m
       }
     }
   };
@@ -992,28 +1002,30 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
       asm volatile("prefetch.global.L2 [%0];" ::"l"(f + C - 1));
     }
   };
-  // moments of the data of nq points whose U-values are rows prow.. of sU, per
-  // material: one (material, right-hand side, basis function) per group of
+  // moments of the data of the points base .. base + nq - 1 whose U-values are
+  // the rows of U, per material (whose elements, of QE points each, are
+  // consecutive): one (material, right-hand side, basis function) per group of
   // ps lanes with its C components as independent sums; the lanes of a group
   // take every ps-th point and are added by butterfly shuffles (a fixed order)
-  auto data_moments = [&](int nq, int prow) {
+  auto data_moments = [&](int base, int nq, const T* U, int QE) {
     const int nitem = ng * nrhs * nb;
     int ps = 1;
-    while (ps < 8 && nitem * ps * 2 <= (int)blockDim.x) ps *= 2;
+    while (ps < 8 && nitem * ps * 2 <= NT) ps *= 2;
     for (int id0 = 0; id0 < nitem * ps; id0 += blockDim.x) {
       const int id = id0 + tid, item = id / ps, part = id % ps;
       const int g = item / (nrhs * nb), rest = item % (nrhs * nb), r = rest / nb, i = rest % nb;
       T t[C];
 #pragma unroll
       for (int cc = 0; cc < C; ++cc) t[cc] = R::zero();
-      if (item < nitem)
-        for (int ql = part; ql < nq; ql += ps)
-          if (s_pgrp[ql] == g) {
-            const T u = sU[(size_t)(prow + ql) * us + i];
-            const T* cb = sCB + (size_t)r * C * cbs + ql;
+      if (item < nitem) {
+        const int l0 = max(0, s_ge0[g] * QE - base), l1 = min(nq, s_ge0[g + 1] * QE - base);
+        const T* cb = sCB + (size_t)r * C * cbs;
+        for (int ql = l0 + part; ql < l1; ql += ps) {
+          const T u = U[(size_t)ql * us + i];
 #pragma unroll
-            for (int cc = 0; cc < C; ++cc) t[cc] = R::acc(t[cc], cb[cc * cbs], u);
-          }
+          for (int cc = 0; cc < C; ++cc) t[cc] = R::acc(t[cc], cb[cc * cbs + ql], u);
+        }
+      }
 #pragma unroll
       for (int cc = 0; cc < C; ++cc) t[cc] = R::norm(t[cc]);
       for (int o = 1; o < ps; o <<= 1)
@@ -1098,17 +1110,19 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
       uint16_t* sTB = sTA + tc::kSlices * planeA + 512;
       int* eA = s_tce[0];
       int* eB = s_tce[1];
-      // two threads per row (M + nb <= 128 rows, so every thread takes part
-      // once and the pair's maxima meet by one shuffle)
+      // TPR threads per row (M + nb <= 128 rows, so every thread takes part
+      // once and a row's maxima meet by shuffles)
       {
-        const int m = tid >> 1, part = tid & 1;
+        constexpr int TPR = NT / 128;
+        const int m = tid / TPR, part = tid % TPR;
         float mx = 0.f;
         if (m < M) {
-          for (int ql = part; ql < nq; ql += 2) mx = fmaxf(mx, fabsf(sCB[(size_t)m * cbs + ql].hi));
+          for (int ql = part; ql < nq; ql += TPR) mx = fmaxf(mx, fabsf(sCB[(size_t)m * cbs + ql].hi));
         } else if (m < M + nb) {
-          for (int ql = part; ql < nq; ql += 2) mx = fmaxf(mx, fabsf(sU[(size_t)ql * us + (m - M)].hi));
+          for (int ql = part; ql < nq; ql += TPR) mx = fmaxf(mx, fabsf(sU[(size_t)ql * us + (m - M)].hi));
         }
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+#pragma unroll
+        for (int o = 1; o < TPR; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         if (part == 0 && m < M) eA[m] = tc::scale_exp(mx);
         if (part == 0 && m >= M && m < M + nb) eB[m - M] = tc::scale_exp(mx);
       }
@@ -1143,20 +1157,21 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
       const int* eB = s_tce[1];
       const bool ok = tc_wait();
       // levels -> float-float moments: warp w reads rows 32 (w % 4) .. + 31,
-      // basis functions 16 (w / 4) .. + 15
+      // basis functions CW (w / 4) .. + CW - 1
+      constexpr int CW = 32 / (NW / 4);
       const int q4 = warp & 3, h = warp >> 2;
       if (ok && 32 * q4 < M) {
         const int m = 32 * q4 + lane;
-        for (int c8 = 0; c8 < 2; ++c8) {
+        for (int c8 = 0; c8 < CW / 8; ++c8) {
           float lv[tc::kSlices][8];
 #pragma unroll
           for (int l = 0; l < tc::kSlices; ++l)
-            tc::ld8(s_tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(l * 32 + 16 * h + 8 * c8), lv[l]);
+            tc::ld8(s_tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(l * 32 + CW * h + 8 * c8), lv[l]);
           tc::wait_ld();
           if (m < M) {
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-              const int i = 16 * h + 8 * c8 + j;
+              const int i = CW * h + 8 * c8 + j;
               if (i >= nb) continue;
               float acc[tc::kSlices];
 #pragma unroll
@@ -1174,99 +1189,153 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
       __syncthreads();   // the exponents and columns read above are rewritten by the next chunk
     }
   };
-  for (int base = q0; base < q1; base += CH) {
-    const int nq = min(CH, q1 - base);
-    // (a) one thread per (side, point): mapped coordinates, sqrt(w), data
-    // coefficients; then the U-values of all 2 nq points with the whole block
-    // (point q = side * nq + ql)
-    const int npt = 2 * nq;
-    for (int id = tid; id < npt; id += blockDim.x) {
-      const int side = id / nq, ql = id % nq, qg = base + ql;
-      const int k = qg / Q, q = qg % Q;
-      if (side == 0) s_pgrp[ql] = s_grp[k];
-      map_point(sPt + id * (DIM + 2), k, q, side == 0);
-      if (keep && side == 0) sKeepW[base - q0 + ql] = __ldg(a.isqw + q) * s_isdet[k];
-    }
-    // (with the right-hand sides split over the cluster the moments take a pass of their own)
-    if (!rsplit) data_coefs(base, nq);
-    eval_uvalues_block<DIM, T>(a, npt, sPt, sM, sU);
-    if (keep)
-      for (int id = tid; id < nq * nb; id += blockDim.x) sKeep[(size_t)(base - q0) * nb + id] = sU[(id / nb) * us + id % nb];
-    // (b) Grams of U-values: top per element (flushed into G and H_m), bottom; per material
-    for (int ql = 0; ql < nq; ++ql) {
-      if (base + ql >= kend) {   // the next element's points start
-        const int k = (base + ql) / Q;
-        flush_element(curk);
-        if (s_grp[k] != curg) {
-          flush_group(curg);
-          curg = s_grp[k];
-        }
-        curk = k;
-        kend = (k + 1) * Q;
-      }
-      const T* ut = sU + (size_t)ql * us;
-      const T* ub = sU + (size_t)(nq + ql) * us;
+  const int nneu = NEU ? s_nneu : 0;   // (kernels for meshes without Neumann facets leave out their code)
+  const bool pblk = nif > 0 || nneu > 0;
+  T* sFD = reinterpret_cast<T*>(sm + a.off_pd);      // Dirichlet sums (Grams, then data moments), then Neumann data
+  T* sDD = sFD + (size_t)ng * (DIM + 1) * npair;
+  const int nfd = nfac > 0 ? ng * (DIM + 1) * (npair + nrhs * nb) : 0;
+  T* sPBN = sFD + nfd;
+  unsigned gdir = 0;   // materials with Dirichlet facets
+  for (int f = 0; f < nfac; ++f) gdir |= 1u << s_fg[f];
+  T* A0 = CS > 1 ? cluster.map_shared_rank(sA, 0) : sA;
+  dd* sF_ = reinterpret_cast<dd*>(sm + a.off_pg);         // N*N     inverse of the equilibrated matrix (the Grams are dead by then)
+  float* sEq = reinterpret_cast<float*>(sm + a.off_eq);   // N       equilibration scales (powers of two)
+  // ---------------- cluster reduction (rank order) ----------------
+  // every CTA sums every CTA's partials in rank order (all remote loads of an
+  // entry are issued before the additions)
+  auto cluster_sum = [&](T* src, int id) {
+    T t = R::zero();
+    for (int r0 = 0; r0 < CS; r0 += 4) {
+      T v[4];
 #pragma unroll
-      for (int s = 0; s < kMaxPair; ++s) {
-        if (tid + s * kThreads < npair) {
-          aK[s] = R::acc(aK[s], ut[pi[s]], ut[pj[s]]);
-          aB[s] = R::acc(aB[s], ub[pi[s]], ub[pj[s]]);
-        }
-      }
+      for (int u = 0; u < 4; ++u)
+        if (r0 + u < CS) v[u] = cluster.map_shared_rank(src, r0 + u)[id];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (r0 + u < CS) t = R::add(t, v[u]);
     }
-    // (c) moments of the data (forward: bottom points; adjoint: top points), per material
-    if (!rsplit) data_moments(nq, ADJ ? 0 : nq);
+    return t;
+  };
+  // reduce-scatter: rank r sums its share of every array over the cluster and
+  // stores the sums into every CTA's copy
+  auto cluster_reduce = [&](T* part, T* sum, int n) {
+    if (CS == 1) {
+      if (sum != part)
+        for (int id = tid; id < n; id += blockDim.x) sum[id] = part[id];
+      return;
+    }
+    const int lo = (n * rank) / CS, hi = (n * (rank + 1)) / CS;
+    for (int id = lo + tid; id < hi; id += blockDim.x) {
+      const T t = cluster_sum(part, id);
+      for (int rr = 0; rr < CS; ++rr) cluster.map_shared_rank(sum, rr)[id] = t;
+    }
+  };
+  for (;;) {   // assembly and inverse (a second time only where the front's times are not the tabulated ones)
+  // (b) the front times: bottom and top fronts over every element, causality
+  if (real) {
+    for (int e = tid; e < nn_; e += blockDim.x) s_ntau[e] = ADJ && e == 0 ? a.tent_tbot[tent] : __ldcg(a.tau + s_nid[e]);
     __syncthreads();
   }
-  if (q1 > q0) {
-    flush_element(curk);
-    flush_group(curg);
+  const double tbot = s_ntau[0];
+  if (tid == 0) {
+    s_tbot = tbot;
+    s_tc = 0.5 * (tbot + s_ttop);
   }
-  if (rsplit) {
-    // this CTA's right-hand sides at every point of the patch (forward: the
-    // bottom points; adjoint: the top points): the moments are complete in
-    // this CTA and take no cluster reduction
-    prefetch_front(0, min(CH, NP));
-    for (int base = 0; base < NP; base += CH) {
-      const int nq = min(CH, NP - base);
-      for (int id = tid; id < nq; id += blockDim.x) {
-        const int qg = base + id, k = qg / Q, q = qg % Q;
-        s_pgrp[id] = s_grp[k];
-        map_point(sPt + id * (DIM + 2), k, q, ADJ);
-      }
-      data_coefs(base, nq);
-      if (base + CH < NP) prefetch_front(base + CH, min(CH, NP - base - CH));
-      eval_uvalues_block<DIM, T>(a, nq, sPt, sM, sU);
-      if (tc_on) {
-        if (base > 0) tc_mom_finish();   // the previous chunk's products ran meanwhile
-        tc_mom_start(nq);                // (its issue barrier orders this chunk's reads before the next writes)
-      } else {
-        data_moments(nq, 0);
-        __syncthreads();
-      }
+  for (int id = tid; id < NG * nmom; id += blockDim.x) sPM[id] = R::zero();
+  for (int id = tid; id < N * N; id += blockDim.x) sA[id] = R::zero();
+  for (int k = tid; k < P; k += blockDim.x) {
+    for (int i = 0; i < NV; ++i) {
+      const int e = s_vid[k][i];
+      s_tb[k][i] = s_ntau[e];
+      s_tt[k][i] = e == 0 ? s_ttop : s_ntau[e];
     }
-    if (tc_on && NP > 0) tc_mom_finish();
+    // gradients of the linear fronts: g = e^-1 (tau_i - tau_0), e from the host
+    const int el = s_el[k];
+    double db[DIM], dt[DIM];
+    for (int i = 0; i < DIM; ++i) {
+      db[i] = s_tb[k][i + 1] - s_tb[k][0];
+      dt[i] = s_tt[k][i + 1] - s_tt[k][0];
+    }
+    double g2 = 0.0;
+    for (int d = 0; d < DIM; ++d) {
+      double gb = 0.0, gt = 0.0;
+      for (int i = 0; i < DIM; ++i) {
+        const double ei = __ldg(a.elem_einv + ((int64_t)el * DIM + d) * DIM + i);
+        gb = fma(ei, db[i], gb);
+        gt = fma(ei, dt[i], gt);
+      }
+      s_gb[k][d] = gb;
+      s_gt[k][d] = gt;
+      g2 = fma(gt, gt, g2);
+    }
+    s_sdet[k] = __ldg(a.elem_sdet + el);
+    s_isdet[k] = __ldg(a.elem_isdet + el);
+    if constexpr (MIXED) {
+      for (int d = 0; d < DIM; ++d) {
+        const dd gf = dd_split(s_gb[k][d]);
+        s_gbf[k][d] = make_float2(gf.hi, gf.lo);
+      }
+      const dd sf = dd_split(s_sdet[k]);
+      s_gbf[k][DIM] = make_float2(sf.hi, sf.lo);
+    }
+    const double ck = s_gc[s_grp[k]];
+    if (!(ck * ck * g2 < 1.0)) flag_error(a, TP_ERR_CAUSALITY, tent);   // space-like top face: c |g| < 1
   }
+  for (int f = tid; f < nfac + nif + (NEU ? s_nneu : 0); f += blockDim.x) {
+    s_fP[f][0][DIM] = tbot;
+    s_fP[f][1][DIM] = s_ttop;
+    for (int c2 = 2; c2 <= DIM; ++c2) s_fP[f][c2][DIM] = s_ntau[s_fw[f][c2]];
+    // n! * n-volume = sqrt(det(E^T E)), E = [P_i - P_0] ((n+1) x n)
+    double G[DIM][DIM];
+    for (int i = 0; i < DIM; ++i)
+      for (int j = 0; j < DIM; ++j) {
+        double s_ = 0.0;
+        for (int d = 0; d <= DIM; ++d) s_ += (s_fP[f][i + 1][d] - s_fP[f][0][d]) * (s_fP[f][j + 1][d] - s_fP[f][0][d]);
+        G[i][j] = s_;
+      }
+    // sqrt(w) = sqrt(w_ref) sqrt(n! volume) at the facet's points
+    s_fsq[f] = sqrt(sqrt(fabs(small_det<DIM>(G))));
+  }
+  // Gram pairs owned by this thread (upper triangle, i <= j, row-major order)
+  int pi[kMaxPair], pj[kMaxPair];
+  T aK[kMaxPair], aG[kMaxPair], aH[kMaxPair][DIM], aB[kMaxPair];
+#pragma unroll
+  for (int s = 0; s < kMaxPair; ++s) {
+    const int id = tid + s * NT;
+    int i = 0, j = 0;
+    if (id < npair) {
+      int rem = id;
+      while (rem >= nb - i) {
+        rem -= nb - i;
+        ++i;
+      }
+      j = i + rem;
+    }
+    pi[s] = i;
+    pj[s] = j;
+    aK[s] = aG[s] = aB[s] = R::zero();
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) aH[s][d] = R::zero();
+  }
+  __syncthreads();
+  ih = s_ih;
+  tc = s_tc;
 
-  // ---------------- phase 2: vertical faces ----------------
+  // ---------------- vertical faces ----------------
+  // (before the Grams, whose region the facet Grams share; with split
+  // right-hand sides after the moments, whose tensor-core staging shares the
+  // region of the Dirichlet sums)
   // Dirichlet facets, per material g, after the interface blocks: the facet
   // Grams summed over g's facets, G_g, and weighted by the facets' normals,
   // Gn_g[d] = sum_f n_f[d] F_f (layout [G_g | Gn_g[0..DIM)] of npair each),
   // then the data moments in the same arrangement (nrhs*nb each).  The
   // congruences with the derivative maps are linear, so these sums carry all
   // a tent needs; they are formed after the cluster reduction.
-  // Interface and Neumann facets add their blocks to the partial A (N*N)
+  // Interface and Neumann facets add their blocks to this CTA's partial A
   // at once; Neumann facets also to a partial b (nrhs*N, after the
   // Dirichlet sums).
-  const int nneu = NEU ? s_nneu : 0;   // (kernels for meshes without Neumann facets leave out their code)
-  const bool pblk = nif > 0 || nneu > 0;
-  T* sFD = sPD + (pblk ? (size_t)N * N : 0);
-  T* sDD = sFD + (size_t)ng * (DIM + 1) * npair;
-  const int nfd = nfac > 0 ? ng * (DIM + 1) * (npair + nrhs * nb) : 0;
-  T* sPBN = sFD + nfd;
+  auto facet_phase = [&]() {
   if (extra) {
-    if (pblk)
-      for (int id = tid; id < N * N; id += blockDim.x) sPD[id] = R::zero();
     for (int id = tid; id < nfd; id += blockDim.x) sFD[id] = R::zero();
     if (nneu > 0)
       for (int id = tid; id < nrhs * N; id += blockDim.x) sPBN[id] = R::zero();
@@ -1291,8 +1360,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
         T* Fg = sFD + (size_t)s_fg[f] * (DIM + 1) * npair;
 #pragma unroll
         for (int s = 0; s < kMaxPair; ++s)
-          if (tid + s * kThreads < npair) {
-            const int q = tid + s * kThreads;
+          if (tid + s * NT < npair) {
+            const int q = tid + s * NT;
             Fg[q] = R::add(Fg[q], aF[s]);
             for (int d = 0; d < DIM; ++d)
               Fg[(1 + d) * npair + q] = R::fma(R::from(s_fn[f][d]), aF[s], Fg[(1 + d) * npair + q]);
@@ -1335,7 +1404,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
           const T* u = sU + (size_t)ql * us;
 #pragma unroll
           for (int s = 0; s < kMaxPair; ++s)
-            if (tid + s * kThreads < npair) aF[s] = R::fma(u[pi[s]], u[pj[s]], aF[s]);
+            if (tid + s * NT < npair) aF[s] = R::fma(u[pi[s]], u[pj[s]], aF[s]);
         }
         for (int id = tid; id < nrhs * nb; id += blockDim.x) {
           const int r = id / nb, i = id % nb;
@@ -1412,7 +1481,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
           const T* u2 = sU + (size_t)(nq + ql) * us;
 #pragma unroll
           for (int s = 0; s < kMaxPair; ++s)
-            if (tid + s * kThreads < npair) {
+            if (tid + s * NT < npair) {
               aF[s] = R::fma(u[pi[s]], u[pj[s]], aF[s]);
               if (!neu) aF2[s] = R::fma(u2[pi[s]], u2[pj[s]], aF2[s]);
             }
@@ -1436,9 +1505,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
       }
 #pragma unroll
       for (int s = 0; s < kMaxPair; ++s)
-        if (tid + s * kThreads < npair) {
-          sF[tid + s * kThreads] = aF[s];
-          sF2[tid + s * kThreads] = aF2[s];
+        if (tid + s * NT < npair) {
+          sF[tid + s * NT] = aF[s];
+          sF2[tid + s * NT] = aF2[s];
         }
       __syncthreads();
       T nrm[DIM];
@@ -1450,7 +1519,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
           T tt_, nt_, tn_, nn_;
           iface_terms<DIM, T, 0>(a, i, j, sF, nb, nrm, &tt_, &nt_, &tn_, &nn_);
           const T t = R::fma(R::from(-cp * ih2), nt_, R::mul(R::from(a.beta * ih2), nn_));
-          T* dst = sPD + (size_t)(gp * nb + i) * N + gp * nb + j;
+          T* dst = sA + (size_t)(gp * nb + i) * N + gp * nb + j;
           *dst = R::add(*dst, t);
         }
         for (int id = tid; id < nrhs * nb; id += blockDim.x) {
@@ -1487,7 +1556,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
           t = R::fma(R::from(st * ss * a.alpha * cs * ct * ih2), tt_, t);
           t = R::fma(R::from(st * ss * a.beta * ih2), nn_, t);
           const int gr = tside ? gm : gp, gcl = sside ? gm : gp;
-          T* dst = sPD + (size_t)(gr * nb + i) * N + gcl * nb + j;
+          T* dst = sA + (size_t)(gr * nb + i) * N + gcl * nb + j;
           *dst = R::add(*dst, t);
         }
       }
@@ -1496,41 +1565,137 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
       __syncthreads();
     }
   }
+  };
+  if constexpr (!SPLIT) facet_phase();
+  // (the facets' Grams shared this region)
+  for (int id = tid; id < NG * (DIM + 2) * npair; id += blockDim.x) sPG[id] = R::zero();   // PG, PH, PGb contiguous
+  if (extra || np == 0) __syncthreads();
 
-  // ---------------- cluster reduction (rank order) ----------------
-  // every CTA sums every CTA's partials in rank order (all remote loads of an
-  // entry are issued before the additions)
-  auto cluster_sum = [&](T* src, int id) {
-    T t = R::zero();
-    for (int r0 = 0; r0 < CS; r0 += 4) {
-      T v[4];
+  // ---------------- Grams over this CTA's points ----------------
+  int curk = SPLIT ? q0 / QK : e0, kend = (curk + 1) * QK;
+  int curg = (q1 > q0) ? s_grp[curk] : 0;
+  // element flush: G += G_K, H_m += g_{K,m} G_K;  group flush: publish G, H, Gbot of the group
+  auto flush_element = [&](int k) {
+    T g[DIM];
+    for (int d = 0; d < DIM; ++d) g[d] = R::from(s_gt[k][d]);
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (r0 + u < CS) v[u] = cluster.map_shared_rank(src, r0 + u)[id];
+    for (int s = 0; s < kMaxPair; ++s) {
+      const T k_ = R::norm(aK[s]);
+      aG[s] = R::add(aG[s], k_);
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (r0 + u < CS) t = R::add(t, v[u]);
-    }
-    return t;
-  };
-  // reduce-scatter: rank r sums its share of every array over the cluster and
-  // stores the sums into every CTA's copy
-  auto cluster_reduce = [&](T* part, T* sum, int n) {
-    const int lo = (n * rank) / CS, hi = (n * (rank + 1)) / CS;
-    for (int id = lo + tid; id < hi; id += blockDim.x) {
-      const T t = cluster_sum(part, id);
-      for (int rr = 0; rr < CS; ++rr) cluster.map_shared_rank(sum, rr)[id] = t;
+      for (int d = 0; d < DIM; ++d) aH[s][d] = R::fma(g[d], k_, aH[s][d]);
+      aK[s] = R::zero();
     }
   };
-  cluster.sync();
+  auto flush_group = [&](int g) {
+#pragma unroll
+    for (int s = 0; s < kMaxPair; ++s) {
+      const int id = tid + s * NT;
+      if (id < npair) {
+        sPG[g * npair + id] = R::add(sPG[g * npair + id], aG[s]);
+#pragma unroll
+        for (int d = 0; d < DIM; ++d)
+          sPH[(g * DIM + d) * npair + id] = R::add(sPH[(g * DIM + d) * npair + id], aH[s][d]);
+        sPGb[g * npair + id] = R::add(sPGb[g * npair + id], R::norm(aB[s]));
+      }
+      aG[s] = aB[s] = R::zero();
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) aH[s][d] = R::zero();
+    }
+  };
+  // one point (U-values ut at the top, ub at the bottom) of the slice added to the Grams
+  auto gram_point = [&](int pt, const T* ut, const T* ub) {
+    if (pt >= kend) {   // the next element's points start
+      const int k = SPLIT ? pt / QK : curk + 1;
+      flush_element(curk);
+      if (s_grp[k] != curg) {
+        flush_group(curg);
+        curg = s_grp[k];
+      }
+      curk = k;
+      kend = (k + 1) * QK;
+    }
+#pragma unroll
+    for (int s = 0; s < kMaxPair; ++s) {
+      if (tid + s * NT < npair) {
+        aK[s] = R::acc(aK[s], ut[pi[s]], ut[pj[s]]);
+        aB[s] = R::acc(aB[s], ub[pi[s]], ub[pj[s]]);
+      }
+    }
+  };
+  if (kept) {
+    // every U-value of the slice first (rows: its top points, then its bottom
+    // points), kept for the data moments and the outflow
+    for (int base = 0; base < 2 * np; base += a.ev_rows) {
+      const int n = min(a.ev_rows, 2 * np - base);
+      for (int id = tid; id < n; id += blockDim.x) {
+        const int row = base + id;
+        const bool top = row < np;
+        const int pt = top ? row : row - np, k = pt / QK;
+        map_point_of(sPt + id * (DIM + 2), e0 + k, pt - k * QK, top, bary_, sqw_);
+      }
+      eval_uvalues_block<DIM, T>(a, n, sPt, sM, sKeep + (size_t)base * us);
+    }
+    for (int pt = 0; pt < np; ++pt) gram_point(e0 * QK + pt, sKeep + (size_t)pt * us, sKB + (size_t)pt * us);
+  } else {
+    // chunks of points: U-values at the top, then at the bottom
+    const int p0 = SPLIT ? q0 : e0 * QK, p1 = SPLIT ? q1 : e1 * QK;
+    for (int base = p0; base < p1; base += CH) {
+      const int nq = min(CH, p1 - base);
+      for (int id = tid; id < 2 * nq; id += blockDim.x) {
+        const int side = id / nq, pt = base + id - side * nq, k = pt / QK;
+        map_point_of(sPt + id * (DIM + 2), k, pt - k * QK, side == 0, bary_, sqw_);
+      }
+      eval_uvalues_block<DIM, T>(a, 2 * nq, sPt, sM, sU);
+      for (int ql = 0; ql < nq; ++ql) gram_point(base + ql, sU + (size_t)ql * us, sU + (size_t)(nq + ql) * us);
+      __syncthreads();
+    }
+  }
+  if (q1 > q0) {
+    flush_element(curk);
+    flush_group(curg);
+  }
+  if constexpr (SPLIT) {
+    if (!real) {
+      wait_deps();
+      check_times();
+    }
+    // this CTA's right-hand sides at every point of the patch (forward: the
+    // bottom points; adjoint: the top points): the moments are complete in
+    // this CTA and take no cluster reduction
+    prefetch_front(0, min(CH, NP));
+    for (int base = 0; base < NP; base += CH) {
+      const int nq = min(CH, NP - base);
+      for (int id = tid; id < nq; id += blockDim.x) {
+        const int qg = base + id, k = qg / Q, q = qg % Q;
+        map_point(sPt + id * (DIM + 2), k, q, ADJ);
+      }
+      data_coefs(base, nq, sCB, cbs, false);
+      if (base + CH < NP) prefetch_front(base + CH, min(CH, NP - base - CH));
+      eval_uvalues_block<DIM, T>(a, nq, sPt, sM, sU);
+      if (tc_on) {
+        if (base > 0) tc_mom_finish();   // the previous chunk's products ran meanwhile
+        tc_mom_start(nq);                // (its issue barrier orders this chunk's reads before the next writes)
+      } else {
+        data_moments(base, nq, sU, Q);
+        __syncthreads();
+      }
+    }
+    if (tc_on && NP > 0) tc_mom_finish();
+  }
+
+  if constexpr (SPLIT) facet_phase();
+  csync();
+  if (SPLIT && !real) {
+    real = true;
+    if (s_bad) continue;
+  }
   // layout [G (NG*npair) | H_m (NG*DIM*npair) | Gbot (NG*npair)]; unused groups hold zeros
-  cluster_reduce(sPG, sSG, NG * (DIM + 2) * npair);
+  if (CS > 1) cluster_reduce(sPG, sPG, NG * (DIM + 2) * npair);
   // (split right-hand sides: each CTA's moments, Dirichlet data sums and
   // Neumann partial b already cover every point for its own right-hand sides)
-  if (!rsplit) cluster_reduce(sPM, sSM, ng * nmom);   // in place (sSM == sPM): each entry has one owner
-  if (pblk) cluster_reduce(sPD, sA, N * N);   // interface and Neumann blocks
-  else
-    for (int id = tid; id < N * N; id += blockDim.x) sA[id] = R::zero();
+  // (in place: each entry is read and rewritten by the one thread that owns it)
+  if (pblk && CS > 1) cluster_reduce(sA, sA, N * N);   // interface and Neumann blocks
   if (NEU && s_nneu > 0) {   // Neumann data (after the Dirichlet sums)
     if (rsplit)
       for (int id = tid; id < nrhs * N; id += blockDim.x) sb[id] = sFD[nfd + id];
@@ -1539,15 +1704,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
   } else {
     for (int id = tid; id < nrhs * N; id += blockDim.x) sb[id] = R::zero();
   }
-  // in place: each entry is read and rewritten by the one thread that owns it
   if (nfac > 0) cluster_reduce(sFD, sFD, rsplit ? ng * (DIM + 1) * npair : nfd);
-  cluster.sync();   // no CTA leaves or reuses its partials while another still reads them
-  // congruence: rank r forms rows [N r / CS, N (r + 1) / CS) of A and b and
-  // stores them into rank 0's A and b; rank 0 alone solves.  Every CTA holds
-  // the same summed partials, so the rows do not depend on which rank forms them.
-  T* A0 = cluster.map_shared_rank(sA, 0);
-  T* b0 = cluster.map_shared_rank(sb, 0);
-  const int row0 = (N * rank) / CS, nrow = (N * (rank + 1)) / CS - row0;
+  csync();   // no CTA leaves or reuses its partials while another still reads them
+  // congruence: the ranks form shares of A's entries and store them into rank
+  // 0's A; rank 0 alone inverts and solves.  Every CTA holds the same summed
+  // partials, so an entry does not depend on which rank forms it.  (The
+  // adjoint solves with A^T: it is stored transposed.)
   {
     const T ih2 = R::from(ih * ih), mih = R::from(-ih);
     // top-face form of every material block by the merged tables: entries
@@ -1555,8 +1717,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
     // is stored with its mirror (the form is symmetric, the Dirichlet and
     // interface parts already in A are not)
     const int nent = ng * npair, ent0 = (nent * rank) / CS, ent1 = (nent * (rank + 1)) / CS;
-    unsigned gdir = 0;   // materials with Dirichlet facets
-    for (int f = 0; f < nfac; ++f) gdir |= 1u << s_fg[f];
     if (nfac > 0) {
       // Dirichlet facets, A_D = (c/h) D_t F E^T with E = alpha (c/h) D_t - (1/h) D_n
       // summed over the material's facets, from G_g and Gn_g, added into this
@@ -1626,11 +1786,237 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
         A0[o2] = R::add(sA[o2], val);
       }
     }
-    // (split right-hand sides: every row of this CTA's own b, kept in this CTA)
-    const int brow0 = rsplit ? 0 : row0, bnrow = rsplit ? N : nrow;
-    T* const bdst = rsplit ? sb : b0;
-    for (int id = tid; id < nrhs * bnrow; id += blockDim.x) {
-      const int r = id / bnrow, Rw = brow0 + id % bnrow;
+  }
+  csync();   // rank 0 holds the assembled A
+  if constexpr (SPLIT) {
+    // every CTA solves for its own right-hand sides with its own copy of A
+    if (rank != 0)
+      for (int id = tid; id < N * N; id += blockDim.x) sA[id] = A0[id];
+    csync();   // rank 0's A is read before any CTA's solve overwrites its own
+  }
+  if (rank == 0 || SPLIT) {
+    if constexpr (ADJ) {   // solve with A^T
+      for (int id = tid; id < N * N; id += blockDim.x) {
+        const int i = id / N, j = id % N;
+        if (i < j) {
+          const T t = sA[id];
+          sA[id] = sA[j * N + i];
+          sA[j * N + i] = t;
+        }
+      }
+      __syncthreads();
+    }
+    // ---------------- inverse of the equilibrated matrix ----------------
+    // Both precisions: F = (D A D)^-1, D powers of two near |diag A|^-1/2
+    // (exact scaling), by Gauss-Jordan in float-float without row
+    // interchanges.  With ~48 bits F's error in the refinement below is
+    // kappa(A) 2^-46 per step: one or two steps instead of the 3 to 40 that
+    // a binary32 inverse took at p = 4, 5, and the direct LU is rarely
+    // needed.  The inverse costs more than a binary32 one, but it is formed
+    // before the wait, off the chain of dependent tents.
+    // Every tent matrix has a positive definite symmetric part (testing the
+    // tent system with V = U_h gives x^T A x = 1/2 int_top Q_g(u) + 1/2 int_bot
+    // Q_g(u_b) + int_bot U^2 + the dissipative boundary and interface terms > 0),
+    // and so has each of its Schur complements: elimination without
+    // interchanges does not break down.  The direct LU of the fallback keeps
+    // partial pivoting on Dirichlet and interface tents.
+    for (int i = tid; i < N; i += blockDim.x) {
+      const float d = fabsf(R::hi(sA[i * N + i]));
+      sEq[i] = (d > 0.f && isfinite(d)) ? pow2_rsqrt(d) : 1.f;
+    }
+    __syncthreads();
+    auto bad_pivot = [&](float pv) {
+      // binary64: the refinement then fails and the direct LU decides
+      if (!(fabsf(pv) > 0.f) || !isfinite(pv)) {
+        if (MIXED && lane == 0) flag_error(a, TP_ERR_SINGULAR, tent);
+        return true;
+      }
+      return false;
+    };
+    if (N <= 32) {
+      // register path: row warp + NW s of the matrix in gr[s], column = lane.
+      // Blocks of four steps K = {k..k+3} per barrier: with S_K the block's
+      // pivot rows at its start, every warp reduces S_K by the four steps
+      // itself (P = [S_KK^-1 | S_KK^-1 S_KJ] in the pivot and the other
+      // columns), and a row i outside K becomes
+      //   (columns of K set to 0, the others kept) - sum_b s_{i,k+b} P_b,
+      // which is the four single steps taken at once (block Gauss-Jordan).
+      constexpr int NS = 32 / NW;
+      dd gr[NS];
+#pragma unroll
+      for (int s_ = 0; s_ < NS; ++s_) {
+        const int i = warp + NW * s_;
+        gr[s_] = {0.f, 0.f};
+        if (i < N && lane < N) gr[s_] = R::scaled(sA[i * N + lane], sEq[i] * sEq[lane]);
+      }
+      for (int k = 0, blk = 0; k < N; k += 4, ++blk) {
+        const int kb = min(4, N - k);
+        dd(*pb)[32] = s_pb[blk & 1];
+        // the owners publish the block's pivot rows (rows k..k+3 are on warps
+        // k % NW .. k % NW + 3, slot k / NW)
+        if (warp >= k % NW && warp < k % NW + kb) {
+#pragma unroll
+          for (int s_ = 0; s_ < NS; ++s_)
+            if (s_ == k / NW) pb[warp - k % NW][lane] = gr[s_];
+        }
+        // this warp's rows in the pivot columns (block-start values)
+        dd ml[NS][4];
+#pragma unroll
+        for (int s_ = 0; s_ < NS; ++s_)
+#pragma unroll
+          for (int b = 0; b < 4; ++b)
+            ml[s_][b] = {-__shfl_sync(0xffffffffu, gr[s_].hi, k + b), -__shfl_sync(0xffffffffu, gr[s_].lo, k + b)};
+        __syncthreads();
+        dd Pr[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          Pr[b] = {0.f, 0.f};
+          if (b < kb) Pr[b] = pb[b][lane];
+        }
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          if (b >= kb) break;
+          const int kc = k + b;
+          dd mm[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            mm[c] = {__shfl_sync(0xffffffffu, Pr[c].hi, kc), __shfl_sync(0xffffffffu, Pr[c].lo, kc)};
+          dd pv = mm[b];
+          if (bad_pivot(pv.hi)) pv = {1.f, 0.f};
+          const dd rp = dd_rcp(pv);
+          const dd pn = (lane == kc) ? rp : dd_mul(Pr[b], rp);
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (c != b) {
+              const dd x0 = lane == kc ? dd{0.f, 0.f} : Pr[c];
+              Pr[c] = Ar<dd>::norm(Ar<dd>::accn(x0, mm[c], pn));
+            }
+          Pr[b] = pn;
+        }
+        const bool kcol = lane >= k && lane < k + kb;
+#pragma unroll
+        for (int s_ = 0; s_ < NS; ++s_) {
+          const int i = warp + NW * s_, bi = i - k;
+          if (bi >= 0 && bi < kb) {
+            gr[s_] = bi == 0 ? Pr[0] : bi == 1 ? Pr[1] : bi == 2 ? Pr[2] : Pr[3];
+          } else {
+            dd x = kcol ? dd{0.f, 0.f} : gr[s_];
+#pragma unroll
+            for (int b = 0; b < 4; ++b) x = Ar<dd>::acc(x, ml[s_][b], Pr[b]);
+            gr[s_] = Ar<dd>::norm(x);
+          }
+        }
+      }
+#pragma unroll
+      for (int s_ = 0; s_ < NS; ++s_) {
+        const int i = warp + NW * s_;
+        if (i < N && lane < N) sF_[i * N + lane] = gr[s_];
+      }
+    } else {
+      // shared-memory path, one step per barrier: every entry belongs to one
+      // thread (rows over warps, columns over lanes), which also writes the
+      // next pivot row and column into a second buffer
+      dd* rowb = reinterpret_cast<dd*>(sm + a.off_rc);   // 2 x N pivot rows, 2 x N pivot columns
+      dd* colb = rowb + 2 * N;
+      for (int i = warp; i < N; i += NW)
+        for (int j = lane; j < N; j += 32) {
+          const dd x = R::scaled(sA[i * N + j], sEq[i] * sEq[j]);
+          sF_[i * N + j] = x;
+          if (i == 0) rowb[j] = x;
+          if (j == 0) colb[i] = x;
+        }
+      __syncthreads();
+      for (int k = 0; k < N; ++k) {
+        const dd *pr = rowb + (k & 1) * N, *pc = colb + (k & 1) * N;
+        dd *nr = rowb + ((k + 1) & 1) * N, *nc = colb + ((k + 1) & 1) * N;
+        dd pv = pr[k];
+        if (bad_pivot(pv.hi)) pv = {1.f, 0.f};
+        const dd rp = dd_rcp(pv);
+        for (int i = warp; i < N; i += NW) {
+          const dd l0 = dd_mul(pc[i], rp), l = {-l0.hi, -l0.lo};
+          for (int j = lane; j < N; j += 32) {
+            dd x;
+            if (i == k) x = j == k ? rp : dd_mul(pr[j], rp);
+            else if (j == k) x = l;
+            else x = Ar<dd>::norm(Ar<dd>::acc(sF_[i * N + j], l, pr[j]));
+            sF_[i * N + j] = x;
+            if (i == k + 1) nr[j] = x;
+            if (j == k + 1) nc[i] = x;
+          }
+        }
+        __syncthreads();
+      }
+    }
+  }
+  if (!real) {
+    wait_deps();
+    check_times();
+  }
+  // ---------------- the data of the bottom front (adjoint: of the top) ----------------
+  if constexpr (!SPLIT) {
+    const T* U = ADJ ? sKeep : sKB;
+    if (!kept && a.S == 0) {
+      for (int base = q0; base < q1; base += CH) {
+        const int nq = min(CH, q1 - base);
+        for (int id = tid; id < nq; id += blockDim.x) map_point(sPt + id * (DIM + 2), (base + id) / Q, (base + id) % Q, ADJ);
+        data_coefs(base, nq, sCB, cbs, false);
+        eval_uvalues_block<DIM, T>(a, nq, sPt, sM, sU);
+        data_moments(base, nq, sU, Q);
+        __syncthreads();
+      }
+    } else if (a.S > 0) {
+      // U on a face is in P_p, so sum_q w_q f(q) u(q) = sum_s u(X_s) [sum_q w_q w_s K(X_s, x_q) f(q)]
+      // (FaceRule): the data go to the rule's points, a few elements at a time
+      const int S = a.S, raws = a.raw_el * Q;
+      for (int eb = e0; eb < e1; eb += EC) {
+        const int ne = min(EC, e1 - eb);
+        if (eb > e0) __syncthreads();
+        data_coefs(eb * Q, ne * Q, sRaw, raws, true);
+        __syncthreads();
+        for (int id = tid; id < nrhs * C * ne * S; id += blockDim.x) {
+          const int rc = id / (ne * S), pt = id - rc * (ne * S), k = pt / S, q_ = pt - k * S;
+          const T *f = sRaw + (size_t)rc * raws + k * Q, *w = (ADJ ? sTF : sTP) + q_ * a.tf_stride;
+          T t0 = R::zero(), t1 = R::zero();
+          int q = 0;
+          for (; q + 1 < Q; q += 2) {
+            t0 = R::acc(t0, w[q], f[q]);
+            t1 = R::acc(t1, w[q + 1], f[q + 1]);
+          }
+          if (q < Q) t0 = R::acc(t0, w[q], f[q]);
+          sCB[(size_t)rc * cbs + pt] = R::mul(R::from(ADJ ? s_isdet[eb + k] : s_sdet[eb + k]), R::add(R::norm(t0), R::norm(t1)));
+        }
+        __syncthreads();
+        if (!kept) {
+          for (int id = tid; id < ne * S; id += blockDim.x)
+            map_point_of(sPt + id * (DIM + 2), eb + id / S, id % S, ADJ, bary_, sqw_);
+          eval_uvalues_block<DIM, T>(a, ne * S, sPt, sM, sU);
+        }
+        data_moments(eb * S, ne * S, kept ? U + (size_t)(eb - e0) * S * us : sU, S);
+      }
+    } else {
+      for (int base = 0; base < np; base += a.cb_pts) {
+        const int nq = min(a.cb_pts, np - base);
+        if (base > 0) __syncthreads();
+        data_coefs(q0 + base, nq, sCB, cbs, false);
+        __syncthreads();
+        data_moments(q0 + base, nq, U + (size_t)base * us, Q);
+      }
+    }
+  }
+  csync();
+  if (real || !s_bad) break;
+  real = true;
+  }   // assembly
+  if (rank == 0 || SPLIT) {
+  // (rank 0 sums the partial moments; the others keep theirs until its b is solved)
+  if (!SPLIT && CS > 1) {
+    for (int id = tid; id < ng * nmom; id += blockDim.x) sPM[id] = cluster_sum(sPM, id);
+    __syncthreads();
+  }
+  {
+    const T mih = R::from(-ih);
+    for (int id = tid; id < nrhs * N; id += blockDim.x) {
+      const int r = id / N, Rw = id % N;
       const int g = Rw / nb, i = Rw % nb;
       const T* M = sSM + (size_t)g * nmom + (size_t)r * C * nb;   // gamma, alpha, beta_1..beta_n
       T t = R::fma(R::from(s_gc[g] * ih), rel_apply<DIM, T>(a, i, 0, M + nb), M[i]);
@@ -1645,265 +2031,80 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
         t = R::add(t, R::fma(R::from(ih), dn, R::mul(ac, rel_apply<DIM, T>(a, i, 0, Dg))));
       }
       const size_t o = (size_t)r * N + Rw;
-      bdst[o] = R::add(sb[o], t);
+      sb[o] = R::add(sb[o], t);
     }
   }
-  cluster.sync();   // rank 0 holds the assembled A and b
-  if (rsplit) {
-    // every CTA solves for its own right-hand sides with its own copy of A
-    if (rank != 0)
-      for (int id = tid; id < N * N; id += blockDim.x) sA[id] = A0[id];
-    cluster.sync();   // rank 0's A is read before any CTA's solve overwrites its own
-  }
-  if (rank == 0 || rsplit) {
-  if constexpr (ADJ) {   // solve with A^T
-    for (int id = tid; id < N * N; id += blockDim.x) {
-      const int i = id / N, j = id % N;
-      if (i < j) {
-        const T t = sA[id];
-        sA[id] = sA[j * N + i];
-        sA[j * N + i] = t;
-      }
-    }
-    __syncthreads();
-  }
+  __syncthreads();
 
   // ---------------- phase 3: solve ----------------
-  // Both precisions: the equilibrated matrix D A D (D = |diag A|^-1/2) is
-  // inverted in binary32 by Gauss-Jordan without row interchanges, then
-  // x += D F D (b - A x) with the residual in the path's precision (binary64,
-  // or float-float for MIXED) until the correction stops shrinking; a
-  // refinement that does not settle falls back to a direct binary64 LU.
-  // Every tent matrix has a positive definite symmetric part (testing the
-  // tent system with V = U_h gives x^T A x = 1/2 int_top Q_g(u) + 1/2 int_bot
-  // Q_g(u_b) + int_bot U^2 + the dissipative boundary and interface terms > 0),
-  // and so has each of its Schur complements: elimination without
-  // interchanges does not break down.  The direct LU of the fallback keeps
-  // partial pivoting on Dirichlet and interface tents.
+  // x = D F D b, then x += D F D (b - A x) with the residual in the path's
+  // precision (binary64, or float-float for MIXED) until the correction stops
+  // shrinking; a refinement that does not settle falls back to a direct
+  // binary64 LU.
   const bool lu_pivoting = extra || ng > 1;
   bool refined = false;
   {
-    float* sG = reinterpret_cast<float*>(sm + a.off_al);    // 2*N*N   ping-pong sweep buffers
-    float* sEq = reinterpret_cast<float*>(sm + a.off_eq);   // N       equilibration scales
-    float* sZ = reinterpret_cast<float*>(sm + a.off_z);     // nrhs*N  scaled residual (binary32)
+    dd* sZ = reinterpret_cast<dd*>(sm + a.off_z);           // nrhs*N  scaled residual
     T* sX = reinterpret_cast<T*>(sm + a.off_x);             // nrhs*N  iterate
-    // register path with room for the right-hand sides: D b rides along as
-    // extra columns (lanes N .. N + nrhs - 1) and the elimination leaves the
-    // first iterate (D A D)^-1 D b in them
-    const bool regs = N <= 32, aug = regs && N + nrhs <= 32;
-    for (int i = tid; i < N; i += blockDim.x) {
-      const float d = fabsf(R::hi(sA[i * N + i]));
-      sEq[i] = (d > 0.f && isfinite(d)) ? rsqrtf(d) : 1.f;
-    }
-    // (items from warp 1 on, beside warp 0's scales)
-    for (int id = (tid + kThreads - 32) % kThreads; id < nrhs * N; id += blockDim.x) {
-      sX[id] = R::zero();
-      if (aug) {   // the same scale as sEq, formed here so that one barrier suffices
-        const float d = fabsf(R::hi(sA[(id % N) * (N + 1)]));
-        sZ[id] = ((d > 0.f && isfinite(d)) ? rsqrtf(d) : 1.f) * R::hi(sb[id]);
-      }
-    }
-    __syncthreads();
-    auto bad_pivot = [&](float pv) {
-      // binary64: the refinement then fails and the direct LU decides
-      if (!(fabsf(pv) > 0.f) || !isfinite(pv)) {
-        if (MIXED && lane == 0) flag_error(a, TP_ERR_SINGULAR, tent);
-        return true;
-      }
-      return false;
-    };
-    // register path (N <= 32): row warp + 8 s of the sweep matrix in gr[s],
-    // column = lane.  Blocks of four steps K = {k..k+3} per barrier: with S_K
-    // the block's pivot rows at its start, every warp reduces S_K by the four
-    // steps itself (P = [S_KK^-1 | S_KK^-1 S_KJ] in the pivot and the other
-    // columns), and a row i outside K becomes
-    //   (columns of K set to 0, the others kept) - sum_b s_{i,k+b} P_b,
-    // which is the four single steps taken at once (block Gauss-Jordan).
-    float gr[4] = {0.f, 0.f, 0.f, 0.f};
-    if (regs) {
-#pragma unroll
-      for (int s_ = 0; s_ < 4; ++s_) {
-        const int i = warp + 8 * s_;
-        if (i < N && lane < N) gr[s_] = R::hi(sA[i * N + lane]) * sEq[i] * sEq[lane];
-        else if (aug && i < N && lane < N + nrhs) gr[s_] = sZ[(lane - N) * N + i];
-      }
-      for (int k = 0, blk = 0; k < N; k += 4, ++blk) {
-        const int kb = min(4, N - k);
-        float(*pb)[32] = s_pb[blk & 1];
-        // the owners publish the block's pivot rows (rows k..k+3 are on warps
-        // (k & 7) .. (k & 7) + 3, slot k >> 3)
-        if (warp >= (k & 7) && warp < (k & 7) + kb) {
-          const int s_ = k >> 3;
-          pb[warp - (k & 7)][lane] = s_ == 0 ? gr[0] : s_ == 1 ? gr[1] : s_ == 2 ? gr[2] : gr[3];
-        }
-        // this warp's rows in the pivot columns (block-start values)
-        float ml[4][4];
-#pragma unroll
-        for (int s_ = 0; s_ < 4; ++s_)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) ml[s_][b] = __shfl_sync(0xffffffffu, gr[s_], k + b);
-        __syncthreads();
-        float P[4];
-#pragma unroll
-        for (int b = 0; b < 4; ++b) P[b] = b < kb ? pb[b][lane] : 0.f;
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          if (b >= kb) break;
-          const int kc = k + b;
-          float mm[4];
-#pragma unroll
-          for (int c = 0; c < 4; ++c) mm[c] = __shfl_sync(0xffffffffu, P[c], kc);
-          float pv = mm[b];
-          if (bad_pivot(pv)) pv = 1.f;
-          const float rp = rcp_fast(pv);
-          const float pn = (lane == kc) ? rp : P[b] * rp;
-#pragma unroll
-          for (int c = 0; c < 4; ++c)
-            if (c != b) P[c] = fmaf(-mm[c], pn, lane == kc ? 0.f : P[c]);
-          P[b] = pn;
-        }
-        const bool kcol = lane >= k && lane < k + kb;
-#pragma unroll
-        for (int s_ = 0; s_ < 4; ++s_) {
-          const int i = warp + 8 * s_;
-          const int bi = i - k;
-          if (bi >= 0 && bi < kb) {
-            gr[s_] = bi == 0 ? P[0] : bi == 1 ? P[1] : bi == 2 ? P[2] : P[3];
-          } else {
-            float x = kcol ? 0.f : gr[s_];
-#pragma unroll
-            for (int b = 0; b < 4; ++b) x = fmaf(-ml[s_][b], P[b], x);
-            gr[s_] = x;
-          }
-        }
-      }
-    } else {
-      for (int id = tid; id < N * N; id += blockDim.x) sG[id] = R::hi(sA[id]) * sEq[id / N] * sEq[id % N];
-      __syncthreads();
-      // Gauss-Jordan sweeps: step k reads buffer k % 2 and writes buffer
-      // (k + 1) % 2; the final buffer holds F = (D A D)^-1
-      for (int k = 0; k < N; ++k) {
-        const float* S = sG + (size_t)(k & 1) * N * N;
-        float* Gn = sG + (size_t)((k + 1) & 1) * N * N;
-        float pv = S[k * N + k];
-        if (bad_pivot(pv)) pv = 1.f;
-        const float rp = rcp_fast(pv);
-        for (int i = warp; i < N; i += kThreads / 32) {   // rows over warps, columns over lanes
-          const float lik = -S[i * N + k] * rp;
-          for (int j = lane; j < N; j += 32) {
-            float g;
-            if (i == k) g = (j == k) ? rp : S[k * N + j] * rp;
-            else if (j == k) g = lik;
-            else g = fmaf(lik, S[k * N + j], S[i * N + j]);
-            Gn[i * N + j] = g;
-          }
-        }
-        __syncthreads();
-      }
-    }
-    const float* F = sG + (size_t)(N & 1) * N * N;
-    __syncthreads();
-    // refinement
-    float prev = 3.4e38f;
+    float prev = 0.f;
     const int maxit = min(a.max_refine, kMaxRefine);
     for (int it = 0; it < maxit; ++it) {
-      // residual b - A x, each row split over 8 lanes of one warp; stored
-      // scaled by D in binary32 (the first iterate is x = 0: the residual is b)
-      if (it == 0 && aug) {
-        // the first iterate from the extra columns: x = D (D A D)^-1 D b
-#pragma unroll
-        for (int s_ = 0; s_ < 4; ++s_) {
-          const int i = warp + 8 * s_;
-          if (i < N && lane >= N && lane < N + nrhs) sZ[(lane - N) * N + i] = sEq[i] * gr[s_];
-        }
-        __syncthreads();
-        float dmax = 0.f;
-        for (int id = tid; id < nrhs * N; id += blockDim.x) {
-          const float dx = sZ[id];
-          sX[id] = R::addf(sX[id], dx);
-          dmax = fmaxf(dmax, fabsf(dx));
-        }
-        for (int o = 16; o > 0; o >>= 1) dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-        if (lane == 0) s_red[1][warp] = dmax;
-        __syncthreads();
-        continue;
-      }
-      if (it == 0)
-        for (int id = tid; id < nrhs * N; id += blockDim.x) sZ[id] = sEq[id % N] * R::hi(sb[id]);
-      for (int base4 = 0; base4 < (it == 0 ? 0 : nrhs * N * 4); base4 += blockDim.x) {
-        const int id = base4 + tid, item = id >> 2, sub = id & 3;
-        T t = R::zero();
-        if (item < nrhs * N) {
-          const int r = item / N, i = item % N;
-          const T* xr = sX + (size_t)r * N;
-          for (int j = sub; j < N; j += 4) t = R::accn(t, sA[i * N + j], xr[j]);
-          t = R::norm(t);
-        }
-        for (int o = 2; o > 0; o >>= 1) {
-          T u;
-          if constexpr (MIXED) {
-            u.hi = __shfl_xor_sync(0xffffffffu, t.hi, o);
-            u.lo = __shfl_xor_sync(0xffffffffu, t.lo, o);
-          } else {
-            u = __shfl_xor_sync(0xffffffffu, t, o);
+      // residual b - A x scaled by D (the first iterate is x = 0: the residual
+      // is b), each row split over 8 lanes of one warp
+      if (it == 0) {
+        for (int id = tid; id < nrhs * N; id += blockDim.x) sZ[id] = R::scaled(sb[id], sEq[id % N]);
+      } else {
+        for (int base8 = 0; base8 < nrhs * N * 8; base8 += blockDim.x) {
+          const int id = base8 + tid, item = id >> 3, sub = id & 7;
+          T t = R::zero();
+          if (item < nrhs * N) {
+            const int r = item / N, i = item % N;
+            const T* xr = sX + (size_t)r * N;
+            for (int j = sub; j < N; j += 8) t = R::accn(t, sA[i * N + j], xr[j]);
+            t = R::norm(t);
           }
-          t = R::add(t, u);
+          for (int o = 4; o > 0; o >>= 1) t = R::add(t, shfl_xor_t(t, o));
+          if (sub == 0 && item < nrhs * N) sZ[item] = R::scaled(R::add(sb[item], t), sEq[item % N]);
         }
-        if (sub == 0 && item < nrhs * N) sZ[item] = sEq[item % N] * R::hi(R::add(sb[item], t));
       }
       __syncthreads();
-      // x += D F r: register path, one row per (warp, slot), summed over lanes
+      // x += D F z, each row split over 8 lanes
       // (the scale |x| of the stop test is taken from the first iterate)
       float dmax = 0.f;
-      if (regs) {
-        for (int r = 0; r < nrhs; ++r) {
-          const float vj = (lane < N) ? sZ[(size_t)r * N + lane] : 0.f;
-          float zs = 0.f;   // lane s_ < 4 ends with the sum of slot s_
-#pragma unroll
-          for (int s_ = 0; s_ < 4; ++s_) {
-            float z = gr[s_] * vj;
-            for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-            if (lane == s_) zs = z;
-          }
-          // one update instruction per warp for its (up to) four rows
-          const int i = warp + 8 * lane;
-          if (lane < 4 && i < N) {
-            const float dx = sEq[i] * zs;
-            const size_t o_ = (size_t)r * N + i;
-            sX[o_] = R::addf(sX[o_], dx);
-            dmax = fmaxf(dmax, fabsf(dx));
-          }
-        }
-      }
-      // shared-memory path: each row split over 8 lanes
-      for (int base8 = 0; base8 < (regs ? 0 : nrhs * N * 8); base8 += blockDim.x) {
+      for (int base8 = 0; base8 < nrhs * N * 8; base8 += blockDim.x) {
         const int id = base8 + tid, item = id >> 3, sub = id & 7;
-        float z = 0.f;
+        dd z = {0.f, 0.f};
         if (item < nrhs * N) {
           const int r = item / N, i = item % N;
-          const float* zr = sZ + (size_t)r * N;
-          for (int j = sub; j < N; j += 8) z = fmaf(F[i * N + j], zr[j], z);
+          const dd* zr = sZ + (size_t)r * N;
+          for (int j = sub; j < N; j += 8) z = Ar<dd>::acc(z, sF_[i * N + j], zr[j]);
+          z = Ar<dd>::norm(z);
         }
-        for (int o = 4; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+        for (int o = 4; o > 0; o >>= 1) z = dd_add(z, shfl_xor_t(z, o));
         if (sub == 0 && item < nrhs * N) {
-          const float dx = sEq[item % N] * z;
-          sX[item] = R::addf(sX[item], dx);
-          dmax = fmaxf(dmax, fabsf(dx));
+          const float e = sEq[item % N];
+          const dd dx = {__fmul_rn(z.hi, e), __fmul_rn(z.lo, e)};
+          sX[item] = it == 0 ? R::of(dx) : R::add(sX[item], R::of(dx));
+          dmax = fmaxf(dmax, fabsf(dx.hi));
+          if (!isfinite(dx.hi)) dmax = dx.hi;
         }
       }
-      for (int o = 16; o > 0; o >>= 1) dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-      if (it == 0) {   // the first correction is the whole binary32 solution: no test
-        if (lane == 0) s_red[1][warp] = dmax;
-        __syncthreads();
-        continue;
+      for (int o = 16; o > 0; o >>= 1) {
+        const float other = __shfl_xor_sync(0xffffffffu, dmax, o);
+        dmax = (isfinite(dmax) && !(other <= dmax)) ? other : dmax;   // (the larger; a non-finite one stays)
       }
-      if (lane == 0) s_red[0][warp] = dmax;
+      if (lane == 0) s_red[it == 0][warp] = dmax;
       __syncthreads();
+      if (it == 0) continue;
       float dm = 0.f, xm = 0.f;
-      for (int w = 0; w < kThreads / 32; ++w) {
+      bool fin = true;
+      for (int w = 0; w < NW; ++w) {
         dm = fmaxf(dm, s_red[0][w]);
         xm = fmaxf(xm, s_red[1][w]);
+        fin = fin && isfinite(s_red[0][w]) && isfinite(s_red[1][w]);
       }
+      if (!fin) break;   // the direct LU decides
+      if (it == 1) prev = xm;   // the first iterate counts as the correction of x = 0
       // stop once the correction is at the resolution of the residual's
       // precision, or once it stops shrinking at a small level (the residual's
       // rounding then limits the accuracy)
@@ -1911,11 +2112,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
       // convergence in kMaxRefine steps, sends the tent to the direct LU)
       const float tiny = MIXED ? 4e-15f : 2.5e-16f, floor_ = MIXED ? 1e-10f : 1e-12f;
       const float stall = 0.5f;
-      if (!(isfinite(dm) && isfinite(xm))) break;   // the direct LU decides
       // (the next correction is predicted as dm * (dm / prev) once the
       // corrections shrink fast; stop when that is below the resolution too)
       const bool done = dm <= tiny * xm || (it >= 2 && dm > stall * prev && dm <= floor_ * xm) ||
-                        (it >= 2 && dm <= 0.01f * prev && 4.f * dm * (dm / prev) <= tiny * xm);
+                        (dm <= 0.01f * prev && 4.f * dm * (dm / prev) <= tiny * xm);
       prev = dm;
       if (done) {
         refined = true;
@@ -1925,7 +2125,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
       // (the next iteration writes s_red only after its first barrier)
     }
     if (refined) {
-      __syncthreads();
       for (int id = tid; id < nrhs * N; id += blockDim.x) sb[id] = sX[id];
       __syncthreads();
     }
@@ -2059,9 +2258,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
     }
   }
   }   // rank 0 (every rank with split right-hand sides)
-  cluster.sync();   // the solution is in rank 0's b (split right-hand sides: in each CTA's own)
-  if (rank != 0 && !rsplit)
+  csync();   // the solution is in rank 0's b (split right-hand sides: in each CTA's own)
+  if (rank != 0 && !rsplit) {
+    const T* b0 = cluster.map_shared_rank(sb, 0);
     for (int id = tid; id < nrhs * N; id += blockDim.x) sb[id] = b0[id];
+  }
   if constexpr (!ADJ) {
     // the forward solution kept for the reverse sweep of the wave-speed gradient
     if (a.xsave != nullptr && (rank == 0 || rsplit)) {
@@ -2509,8 +2710,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
       const bool ok = tc_product(tc::smem_addr(sTA), (uint32_t)planeU * 2, (uint32_t)RGU * 128,
                                  tc::smem_addr(sTB), (uint32_t)planeY * 2, (uint32_t)(NY >> 3) * 128, 2, NY, cstride);
       // levels -> binary64 front values: the thread of lane l of warp w holds
-      // point 32 (w % 4) + l and the rows (r, c) of half w / 4
-      const int q4 = warp & 3, h = warp >> 2, half = NY >> 1;
+      // point 32 (w % 4) + l and every (NW / 4)th group of 8 rows (r, c)
+      const int q4 = warp & 3;
       if (ok && 32 * q4 < nq) {
         const int ql = 32 * q4 + lane;
         const bool live = ql < nq;
@@ -2522,7 +2723,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
           ep = eU[ql] - 16;
         }
         const int64_t rstride = (int64_t)a.ne * Q * C;
-        for (int c0 = h * half; c0 < (h + 1) * half; c0 += 8) {
+        for (int c0 = 8 * (warp >> 2); c0 < NY; c0 += 2 * NW) {
           float lv[tc::kSlices][8];
 #pragma unroll
           for (int l = 0; l < tc::kSlices; ++l)
@@ -2552,9 +2753,76 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
       __syncthreads();
     }
   };
-  for (int base = o0; base < o1; base += 2 * CH) {
-    const int nq = min(2 * CH, o1 - base);
-    if (!keep) {
+  // the outflow's point formula of the adjoint: fields sv of mu at point q of
+  // element k to lambda_bot = w (s0, c^-2 s_t - g_b.s, s_m - g_b,m s_t)
+  auto store_adjoint = [&](int r, int k, int q, const double* sv) {
+    const double cg = s_gc[s_grp[k]];
+    const double sq = __ldg(a.sqw + q) * s_sdet[k];
+    const double w = sq * sq;
+    double gs = 0.0;
+    for (int d = 0; d < DIM; ++d) gs = fma(s_gb[k][d], sv[2 + d], gs);
+    double* f = front + (((int64_t)r * a.ne + s_el[k]) * Q + q) * C;
+    f[0] = w * sv[0];
+    f[1] = w * (sv[1] / (cg * cg) - gs);
+    for (int d = 0; d < DIM; ++d) f[2 + d] = w * (sv[2 + d] - s_gb[k][d] * sv[1]);
+  };
+  if (!SPLIT && a.S > 0) {
+    // the fields at the rule's points, then through the table to the front's
+    const int S = a.S;
+    const T* U = ADJ ? sKB : sKeep;
+    for (int eb = e0; eb < e1; eb += EC) {
+      const int ne = min(EC, e1 - eb);
+      if (eb > e0) __syncthreads();
+      if (!kept) {
+        for (int id = tid; id < ne * S; id += blockDim.x)
+          map_point_of(sPt + id * (DIM + 2), eb + id / S, id % S, !ADJ, bary_, sqw_);
+        eval_uvalues_block<DIM, T>(a, ne * S, sPt, sM, sU);
+      }
+      const T* Ue = kept ? U + (size_t)(eb - e0) * S * us : sU;
+      for (int id = tid; id < nrhs * C * ne * S; id += blockDim.x) {
+        const int rc = id / (ne * S), pt = id - rc * (ne * S), k = eb + pt / S;
+        const T *u = Ue + (size_t)pt * us, *y = sY + (size_t)s_grp[k] * nmom + (size_t)rc * nb;
+        T t0 = R::zero(), t1 = R::zero();
+        int j = 0;
+        for (; j + 1 < nb; j += 2) {
+          t0 = R::acc(t0, y[j], u[j]);
+          t1 = R::acc(t1, y[j + 1], u[j + 1]);
+        }
+        if (j < nb) t0 = R::acc(t0, y[j], u[j]);
+        sCB[(size_t)rc * cbs + pt] = R::add(R::norm(t0), R::norm(t1));
+      }
+      __syncthreads();
+      auto at_front = [&](int rc, int k, int q) {   // component at front point q of element eb + k
+        const T *F = sCB + (size_t)rc * cbs + k * S, *w = sTF + q;
+        T t0 = R::zero(), t1 = R::zero();
+        int s_ = 0;
+        for (; s_ + 1 < S; s_ += 2) {
+          t0 = R::acc(t0, w[s_ * a.tf_stride], F[s_]);
+          t1 = R::acc(t1, w[(s_ + 1) * a.tf_stride], F[s_ + 1]);
+        }
+        if (s_ < S) t0 = R::acc(t0, w[s_ * a.tf_stride], F[s_]);
+        return R::to(R::add(R::norm(t0), R::norm(t1))) * s_isdet[eb + k];
+      };
+      if constexpr (!ADJ) {
+        for (int id = tid; id < nrhs * ne * Q * C; id += blockDim.x) {
+          const int cc = id % C, rq = id / C, r = rq / (ne * Q), ql = rq - r * (ne * Q), k = ql / Q, q = ql - k * Q;
+          front[(((int64_t)r * a.ne + s_el[eb + k]) * Q + q) * C + cc] = at_front(r * C + cc, k, q);
+        }
+      } else {
+        for (int id = tid; id < nrhs * ne * Q; id += blockDim.x) {
+          const int r = id / (ne * Q), ql = id - r * (ne * Q), k = ql / Q, q = ql - k * Q;
+          double sv[C];
+#pragma unroll
+          for (int cc = 0; cc < C; ++cc) sv[cc] = at_front(r * C + cc, k, q);
+          store_adjoint(r, eb + k, q, sv);
+        }
+      }
+    }
+    __syncthreads();
+  } else
+  for (int base = o0; base < o1; base += kept ? NP : 2 * CH) {   // (kept U-values: one pass)
+    const int nq = min(kept ? NP : 2 * CH, o1 - base);
+    if (!kept) {
     for (int id = tid; id < nq; id += blockDim.x) {
       const int qg = base + id, k = qg / Q, q = qg % Q;
       const double cg = s_gc[s_grp[k]];
@@ -2582,12 +2850,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
         for (int id = tid; id < nq * nrhs * C; id += blockDim.x) {
           const int cc = id % C, rq = id / C, r = rq / nq, ql = rq % nq;
           const int qg = base + ql, k = qg / Q, q = qg % Q;
-          const T* u = keep ? sKeep + (size_t)(base - q0 + ql) * nb : sU + (size_t)ql * us;
+          const T* u = kept ? sKeep + (size_t)(base - q0 + ql) * us : sU + (size_t)ql * us;
           const T* y = sY + (size_t)s_grp[k] * nmom + ((size_t)r * C + cc) * nb;
           T t = R::zero();
           for (int j = 0; j < nb; ++j) t = R::acc(t, y[j], u[j]);
           const double val = R::to(R::norm(t));
-          front[(((int64_t)r * a.ne + s_el[k]) * Q + q) * C + cc] = keep ? val * sKeepW[base - q0 + ql] : val;
+          front[(((int64_t)r * a.ne + s_el[k]) * Q + q) * C + cc] = kept ? val * (__ldg(a.isqw + q) * s_isdet[k]) : val;
         }
       } else
       // one (point, right-hand side) per thread, its C components as
@@ -2595,7 +2863,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
       for (int id = tid; id < nq * nrhs; id += blockDim.x) {
         const int r = id / nq, ql = id % nq;
         const int qg = base + ql, k = qg / Q, q = qg % Q;
-        const T* u = keep ? sKeep + (size_t)(base - q0 + ql) * nb : sU + (size_t)ql * us;
+        const T* u = kept ? sKeep + (size_t)(base - q0 + ql) * us : sU + (size_t)ql * us;
         const T* y = sY + (size_t)s_grp[k] * nmom + (size_t)r * C * nb;
         T t[C];
 #pragma unroll
@@ -2606,8 +2874,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
           for (int cc = 0; cc < C; ++cc) t[cc] = R::acc(t[cc], y[cc * nb + j], uj);
         }
         double* f = front + (((int64_t)r * a.ne + s_el[k]) * Q + q) * C;
-        if (keep) {
-          const double sc = sKeepW[base - q0 + ql];
+        if (kept) {
+          const double sc = __ldg(a.isqw + q) * s_isdet[k];
 #pragma unroll
           for (int cc = 0; cc < C; ++cc) f[cc] = R::to(R::norm(t[cc])) * sc;
         } else {
@@ -2616,28 +2884,19 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
         }
       }
     } else {
-      // lambda_bot = w (s0, c^-2 s_t - g_b.s, s_m - g_b,m s_t)
       for (int id = tid; id < nq * nrhs; id += blockDim.x) {
         const int ql = id / nrhs, r = id % nrhs;
         const int qg = base + ql, k = qg / Q, q = qg % Q;
-        const T* u = sU + (size_t)ql * us;
+        const T* u = kept ? sKB + (size_t)(base - q0 + ql) * us : sU + (size_t)ql * us;
         double sv[C];
         for (int cc = 0; cc < C; ++cc) {
           const T* y = sY + (size_t)s_grp[k] * nmom + ((size_t)r * C + cc) * nb;
           T t = R::zero();
           for (int j = 0; j < nb; ++j) t = R::acc(t, y[j], u[j]);
           t = R::norm(t);
-          sv[cc] = R::to(t);
+          sv[cc] = kept ? R::to(t) * (__ldg(a.isqw + q) * s_isdet[k]) : R::to(t);
         }
-        const double cg = s_gc[s_grp[k]];
-        const double sq = __ldg(a.sqw + q) * s_sdet[k];
-        const double w = sq * sq;
-        double gs = 0.0;
-        for (int d = 0; d < DIM; ++d) gs = fma(s_gb[k][d], sv[2 + d], gs);
-        double* f = front + (((int64_t)r * a.ne + s_el[k]) * Q + q) * C;
-        f[0] = w * sv[0];
-        f[1] = w * (sv[1] / (cg * cg) - gs);
-        for (int d = 0; d < DIM; ++d) f[2 + d] = w * (sv[2 + d] - s_gb[k][d] * sv[1]);
+        store_adjoint(r, k, q, sv);
       }
     }
     __syncthreads();
@@ -2651,11 +2910,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
     __syncthreads();
     if (tid == 0) red_release_add(a.done + v, 1);
   } else {
-    cluster.sync();   // rank 0's b stays valid until every CTA has read the solution
+    csync();   // rank 0's b stays valid until every CTA has read the solution
     break;
   }
   }   // tent loop
-  if (kTC && a.tc) {
+  if constexpr (kTC) {
     tc::fence_before();
     __syncthreads();
     if (warp == 0) tc::tmem_free(s_tmem, a.tc_cols);
@@ -2663,19 +2922,24 @@ __global__ void __launch_bounds__(kThreads, 2) k_layer(const KArgs a, const int 
 }
 
 
-// launchers, one translation unit per space dimension (tp_layer_d<n>.cu)
-// mode: 0 forward binary64, 1 forward mixed, 2 adjoint binary64, plus 4 for
-// meshes with Neumann facets;
-// persistent: one resident grid of clusters pulling tents from a queue
-#define TP_DECLARE_LAUNCHERS(D)                                                                  \
-  cudaError_t layer_attrs_d##D(size_t smem);                                                      \
-  cudaError_t layer_static_smem_d##D(size_t* bytes);                                              \
-  cudaError_t launch_layer_d##D(const KArgs& a, int n_cluster, int cs, int t0, size_t smem,       \
-                                cudaStream_t st, int mode, bool persistent);                      \
-  cudaError_t max_clusters_d##D(int cs, size_t smem, int mode, int* n);
-TP_DECLARE_LAUNCHERS(1)
-TP_DECLARE_LAUNCHERS(2)
-TP_DECLARE_LAUNCHERS(3)
+// launchers, one translation unit per space dimension D, kind of sweep K (0
+// forward binary64, 1 forward mixed, 2 adjoint binary64, 3 forward mixed on the
+// tensor cores) and N = 1 for meshes with Neumann facets; persistent: one
+// resident grid of clusters pulling tents from a queue; wide: kThreadsWide
+// threads per CTA
+#define TP_DECLARE_LAUNCHERS(D, K, N)                                                                      \
+  cudaError_t layer_attrs_d##D##K##_n##N(size_t smem);                                                      \
+  cudaError_t layer_static_smem_d##D##K##_n##N(size_t* bytes);                                              \
+  cudaError_t launch_layer_d##D##K##_n##N(const KArgs& a, int n_cluster, int cs, int t0, size_t smem,       \
+                                          cudaStream_t st, bool persistent, bool wide);                     \
+  cudaError_t max_clusters_d##D##K##_n##N(int cs, size_t smem, bool split, bool wide, int* n);
+#define TP_DECLARE_KIND(D, K) TP_DECLARE_LAUNCHERS(D, K, 0) TP_DECLARE_LAUNCHERS(D, K, 1)
+#define TP_DECLARE_DIM(D) TP_DECLARE_KIND(D, 0) TP_DECLARE_KIND(D, 1) TP_DECLARE_KIND(D, 2) TP_DECLARE_KIND(D, 3)
+TP_DECLARE_DIM(1)
+TP_DECLARE_DIM(2)
+TP_DECLARE_DIM(3)
+#undef TP_DECLARE_DIM
+#undef TP_DECLARE_KIND
 #undef TP_DECLARE_LAUNCHERS
 
 }  // namespace tp

@@ -1,118 +1,97 @@
-// Instantiations and launchers of the tent kernel for one space dimension.
-// Compiled once per dimension with -DTP_DIM=1, 2 or 3 (the translation units
-// build in parallel).
+// Instantiations and launchers of the tent kernel for one space dimension, one
+// kind of sweep and meshes with or without Neumann facets.  Compiled once per
+// dimension (-DTP_DIM=1, 2 or 3), kind (-DTP_KIND=0 forward binary64, 1 forward
+// mixed, 2 adjoint binary64, 3 forward mixed on the tensor cores) and
+// -DTP_NEU=0 or 1, so that the translation units build in parallel.
 #include <algorithm>
+#include <utility>
 
 #include "tp_kernel.cuh"
 
-#ifndef TP_DIM
-#error "compile with -DTP_DIM=1, 2 or 3"
+#if !defined(TP_DIM) || !defined(TP_KIND) || !defined(TP_NEU)
+#error "compile with -DTP_DIM=1, 2 or 3, -DTP_KIND=0, 1, 2 or 3 and -DTP_NEU=0 or 1"
 #endif
 
-#define TP_CAT2(a, b) a##b
-#define TP_CAT(a, b) TP_CAT2(a, b)
+#define TP_CAT2(a, b, c, d, e) a##b##c##d##e
+#define TP_CAT(a, b, c, d, e) TP_CAT2(a, b, c, d, e)
+#define TP_NAME(a) TP_CAT(a, TP_DIM, TP_KIND, _n, TP_NEU)
 
 namespace tp {
 
 namespace {
 
-template <bool MIXED, bool ADJ, bool PERSIST>
-cudaError_t set_attr(size_t smem) {
-  cudaError_t e = cudaFuncSetAttribute(k_layer<TP_DIM, MIXED, ADJ, PERSIST, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_layer<TP_DIM, MIXED, ADJ, PERSIST, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)smem);
+constexpr bool kMixed = TP_KIND == 1 || TP_KIND == 3, kAdj = TP_KIND == 2, kTc = TP_KIND == 3;
+
+using Kernel = void (*)(const KArgs, const int);
+
+// the variant for (dataflow, split right-hand sides, wide CTAs); the adjoint
+// runs one launch per level, launches per level have narrow CTAs, the tensor
+// cores take split right-hand sides in wide CTAs
+constexpr int kVariants = 8;
+template <int I>
+Kernel variant() {
+  constexpr bool PERSIST = I & 4, SPLIT = I & 2, WIDE = I & 1;
+  if constexpr ((kAdj && PERSIST) || (kTc ? !(SPLIT && WIDE) : (WIDE && !PERSIST))) return nullptr;
+  else return k_layer<TP_DIM, kMixed, kAdj, PERSIST, TP_NEU != 0, SPLIT, kTc, WIDE>;
+}
+template <int... I>
+Kernel pick_of(int i, std::integer_sequence<int, I...>) {
+  static const Kernel k[kVariants] = {variant<I>()...};
+  return k[i];
+}
+Kernel pick(int i) { return pick_of(i, std::make_integer_sequence<int, kVariants>()); }
+Kernel pick(bool persistent, bool split, bool wide) {
+  return pick((persistent ? 4 : 0) + (split ? 2 : 0) + (wide ? 1 : 0));
 }
 
-template <bool MIXED, bool ADJ, bool PERSIST, bool NEU>
-cudaError_t launch(const KArgs& a, int n_cluster, int cs, int t0, size_t smem, cudaStream_t st) {
+cudaLaunchConfig_t config(int n_cluster, int cs, size_t smem, cudaStream_t st, bool wide, cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(n_cluster * cs));
-  cfg.blockDim = dim3(kThreads);
+  cfg.blockDim = dim3(wide ? kThreadsWide : kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)cs;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_layer<TP_DIM, MIXED, ADJ, PERSIST, NEU>, a, t0);
-}
-
-template <bool MIXED, bool ADJ, bool PERSIST, bool NEU>
-cudaError_t occupancy(int cs, size_t smem, int* n) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)cs);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)cs;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaOccupancyMaxActiveClusters(n, k_layer<TP_DIM, MIXED, ADJ, PERSIST, NEU>, &cfg);
+  return cfg;
 }
 
 }  // namespace
 
-// largest static shared memory of the instantiations (bytes)
-cudaError_t TP_CAT(layer_static_smem_d, TP_DIM)(size_t* bytes) {
-  size_t m = 0;
-  cudaFuncAttributes fa;
-  cudaError_t e;
-  const void* k[] = {
-      (const void*)k_layer<TP_DIM, false, false, false, false>, (const void*)k_layer<TP_DIM, true, false, false, false>,
-      (const void*)k_layer<TP_DIM, false, true, false, false>, (const void*)k_layer<TP_DIM, false, false, true, false>,
-      (const void*)k_layer<TP_DIM, true, false, true, false>, (const void*)k_layer<TP_DIM, false, false, false, true>,
-      (const void*)k_layer<TP_DIM, true, false, false, true>, (const void*)k_layer<TP_DIM, false, true, false, true>,
-      (const void*)k_layer<TP_DIM, false, false, true, true>, (const void*)k_layer<TP_DIM, true, false, true, true>};
-  for (const void* f : k) {
-    if ((e = cudaFuncGetAttributes(&fa, f)) != cudaSuccess) return e;
-    m = std::max(m, fa.sharedSizeBytes);
-  }
-  *bytes = m;
+// largest static shared memory of the instantiations (bytes), and the dynamic limit set on each
+cudaError_t TP_NAME(layer_static_smem_d)(size_t* bytes) {
+  *bytes = 0;
+  for (int i = 0; i < kVariants; ++i)
+    if (Kernel k = pick(i)) {
+      cudaFuncAttributes fa;
+      const cudaError_t e = cudaFuncGetAttributes(&fa, (const void*)k);
+      if (e != cudaSuccess) return e;
+      *bytes = std::max(*bytes, fa.sharedSizeBytes);
+    }
   return cudaSuccess;
 }
-
-cudaError_t TP_CAT(layer_attrs_d, TP_DIM)(size_t smem) {
-  cudaError_t e;
-  if ((e = set_attr<false, false, false>(smem)) != cudaSuccess) return e;
-  if ((e = set_attr<true, false, false>(smem)) != cudaSuccess) return e;
-  if ((e = set_attr<false, true, false>(smem)) != cudaSuccess) return e;
-  if ((e = set_attr<false, false, true>(smem)) != cudaSuccess) return e;
-  return set_attr<true, false, true>(smem);
+cudaError_t TP_NAME(layer_attrs_d)(size_t smem) {
+  for (int i = 0; i < kVariants; ++i)
+    if (Kernel k = pick(i)) {
+      const cudaError_t e = cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+    }
+  return cudaSuccess;
 }
-
-cudaError_t TP_CAT(launch_layer_d, TP_DIM)(const KArgs& a, int n_cluster, int cs, int t0, size_t smem,
-                                           cudaStream_t st, int mode, bool persistent) {
-  const bool neu = (mode & 4) != 0;
-  mode &= 3;
-  if (persistent) {
-    if (mode == 1)
-      return neu ? launch<true, false, true, true>(a, n_cluster, cs, t0, smem, st)
-                 : launch<true, false, true, false>(a, n_cluster, cs, t0, smem, st);
-    return neu ? launch<false, false, true, true>(a, n_cluster, cs, t0, smem, st)
-               : launch<false, false, true, false>(a, n_cluster, cs, t0, smem, st);
-  }
-  if (mode == 2)
-    return neu ? launch<false, true, false, true>(a, n_cluster, cs, t0, smem, st)
-               : launch<false, true, false, false>(a, n_cluster, cs, t0, smem, st);
-  if (mode == 1)
-    return neu ? launch<true, false, false, true>(a, n_cluster, cs, t0, smem, st)
-               : launch<true, false, false, false>(a, n_cluster, cs, t0, smem, st);
-  return neu ? launch<false, false, false, true>(a, n_cluster, cs, t0, smem, st)
-             : launch<false, false, false, false>(a, n_cluster, cs, t0, smem, st);
+cudaError_t TP_NAME(launch_layer_d)(const KArgs& a, int n_cluster, int cs, int t0, size_t smem, cudaStream_t st,
+                                    bool persistent, bool wide) {
+  cudaLaunchAttribute attr[1];
+  if (!kTc && !persistent) wide = false;
+  const cudaLaunchConfig_t cfg = config(n_cluster, cs, smem, st, wide, attr);
+  return cudaLaunchKernelEx(&cfg, pick(persistent, a.rsplit != 0, wide), a, t0);
 }
-
-cudaError_t TP_CAT(max_clusters_d, TP_DIM)(int cs, size_t smem, int mode, int* n) {
-  const bool neu = (mode & 4) != 0;
-  if ((mode & 3) == 1) return neu ? occupancy<true, false, true, true>(cs, smem, n) : occupancy<true, false, true, false>(cs, smem, n);
-  return neu ? occupancy<false, false, true, true>(cs, smem, n) : occupancy<false, false, true, false>(cs, smem, n);
+cudaError_t TP_NAME(max_clusters_d)(int cs, size_t smem, bool split, bool wide, int* n) {
+  cudaLaunchAttribute attr[1];
+  const cudaLaunchConfig_t cfg = config(1, cs, smem, nullptr, wide, attr);
+  return cudaOccupancyMaxActiveClusters(n, pick(!kAdj, split, wide), &cfg);
 }
 
 }  // namespace tp
