@@ -170,6 +170,7 @@ struct tp_ctx {
   // right-hand sides split over the CTAs of a tent's cluster (1: not split)
   int rsplit_cs = 1;
   bool tc_used = false;   // tensor-core moments and outflow in the forward sweep
+  int min_cs = 1;         // smallest cluster whose CTAs keep their U-values (every tent's: the plan counts on it)
   bool wide = false;      // one CTA per SM (its shared-memory plan does not leave room for two): twice the threads
   bool mixed = false;
   // persistent dataflow sweep
@@ -269,6 +270,7 @@ cudaError_t launch_layer(tp_ctx* ctx, const KArgs& a, int n_cluster, int cs, int
 
 // resident clusters of the persistent kernel for cluster size cs
 int set_persist_cs(tp_ctx* ctx, int cs) {
+  if (cs < ctx->min_cs) return TP_ERR_UNSUPPORTED;
   int nclu = 0;
   cudaError_t e = kLaunchers[ctx->dim - 1][forward_kind(ctx)][ctx->neumann].max_clusters(
       cs, ctx->smem_bytes, ctx->rsplit_cs > 1, ctx->wide, &nclu);
@@ -298,7 +300,7 @@ bool tuned_lookup(const int* key, int* cs, bool* dataflow) {
 // nt * cs <= 2 CTAs per SM
 int level_cluster_size(const tp_ctx* ctx, int64_t nt) {
   if (ctx->rsplit_cs > 1) return ctx->rsplit_cs;   // one CTA per slice of the right-hand sides
-  int cs = 1;
+  int cs = ctx->min_cs;
   while (cs * 2 <= ctx->max_cs && nt * cs * 2 <= 2LL * ctx->n_sm) cs *= 2;
   return cs;
 }
@@ -918,23 +920,32 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   a.elem_sdet = desdet;
   a.elem_isdet = deisdet;
   a.isqw = disqw;
-  {   // the rule of the face integrals
-    const tp::FaceRule& fr = tp::face_rule(n, basis->p, ctx->rule);
+  {   // tables in binary64 and float-float: the front rule, the rule of the face integrals
+    const tp::FaceRule fr = tp::face_rule(n, basis->p, ctx->rule);
     a.S = fr.S;
     a.tf_stride = fr.stride;
+    auto table = [&](RuleTab* t, const std::vector<double>& d, const std::vector<float>* ff) {
+      std::vector<float> f;
+      for (size_t i = 0; !ff && i < d.size(); ++i) {
+        const float h = (float)d[i];
+        f.push_back(h);
+        f.push_back((float)(d[i] - (double)h));
+      }
+      double* dd_ = nullptr;
+      float* df = nullptr;
+      int r = ctx_upload(ctx, &dd_, d);
+      if (r == TP_OK) r = ctx_upload(ctx, &df, ff ? *ff : f);
+      t->d = dd_;
+      t->ff = reinterpret_cast<const float2*>(df);
+      return r;
+    };
     std::vector<double> tf(fr.to_points);
     tf.insert(tf.end(), fr.to_front.begin(), fr.to_front.end());
     std::vector<float> tff(fr.to_points_ff);
     tff.insert(tff.end(), fr.to_front_ff.begin(), fr.to_front_ff.end());
-    double *dsb = nullptr, *dss = nullptr, *dtf_ = nullptr;
-    float* dtff_ = nullptr;
-    if ((rc = ctx_upload(ctx, &dsb, fr.bary)) || (rc = ctx_upload(ctx, &dss, fr.sqw)) || (rc = ctx_upload(ctx, &dtf_, tf)) ||
-        (rc = ctx_upload(ctx, &dtff_, tff)))
+    if ((rc = table(&a.tf, tf, &tff)) || (rc = table(&a.baryT, ctx->rule.bary, nullptr)) || (rc = table(&a.sqwT, sqw, nullptr)) ||
+        (rc = table(&a.s_baryT, fr.bary, nullptr)) || (rc = table(&a.s_sqwT, fr.sqw, nullptr)))
       return fail(rc);
-    a.s_bary = dsb;
-    a.s_sqw = dss;
-    a.tf = dtf_;
-    a.tf_dd = reinterpret_cast<const float2*>(dtff_);
   }
   a.bary = dbary;
   a.wref = dw;
@@ -990,8 +1001,13 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   // evaluated at a time into them; rule: the S-point rule of the face integrals)
   const int S_rule = a.S;
   int rs = prm->rhs_split;
+  // (with every tent's U-values kept, regions that are not in use together are
+  // shared: the evaluation's monomials with the Grams, the chunk of U-values of
+  // the facet, energy and probe passes with the end of the kept rows, whose
+  // owners, the moments' rows, are not yet or no longer needed in those passes)
   auto plan = [&](int CH, int keep, int rows, bool rule) {
     size_t off = 0;
+    const bool share_mono = keep > 0 && ngmax == 1 && !ifneu, share_u = keep >= 2 * CH;
     a.S = rule ? S_rule : 0;
     const int QK = a.S > 0 ? a.S : Q;
     auto take = [&](int* field, size_t count) {
@@ -1003,10 +1019,13 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     const size_t half_nb = (NB + 1) / 2, rb = (size_t)nrg * NB;
     // Dirichlet sums of every material (tents with Dirichlet facets), partials
     // reduced in place, and a partial b (tents with Neumann facets)
-    size_t pd = 0;
-    for (const auto& m : facet_mix)
-      pd = std::max(pd, (m[1] > 0 ? (size_t)m[0] * (n + 1) * (npair + (size_t)nrg * nb) : 0) +
-                            (m[3] > 0 ? (size_t)nrg * m[0] * nb : 0));
+    size_t pd = 0, pdd = 0;
+    for (const auto& m : facet_mix) {
+      pd = std::max(pd, m[1] > 0 ? (size_t)m[0] * (n + 1) * npair : 0);
+      pdd = std::max(pdd, (m[1] > 0 ? (size_t)m[0] * (n + 1) * nrg * nb : 0) + (m[3] > 0 ? (size_t)nrg * m[0] * nb : 0));
+    }
+    a.ev_rows = std::max(2 * CH, rows);
+    const size_t mono = (size_t)a.ev_rows * a.mono_stride;
     take(nullptr, NB * NB);                        // A
     take(&a.off_x, rb);
     take(&a.off_z, rb);
@@ -1022,11 +1041,11 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     a.off_pg = (int)off;
     a.off_ph = a.off_pg + ngmax * npair;
     a.off_pgb = a.off_ph + ngmax * n * npair;
-    take(nullptr, std::max({(size_t)ngmax * (n + 2) * npair, NB * NB, fg}));
+    a.off_mono = (int)off;
+    take(nullptr, std::max({(size_t)ngmax * (n + 2) * npair, NB * NB, fg, share_mono ? mono : 0}));
     take(&a.off_pm, (size_t)ngmax * nmom);        // moments: partials, summed in place, then the outflow vectors
     a.off_sm = a.off_y = a.off_pm;
-    a.ev_rows = std::max(2 * CH, rows);
-    take(&a.off_mono, (size_t)a.ev_rows * a.mono_stride);
+    if (!share_mono) take(&a.off_mono, mono);
     // tensor-core staging (bf16 digit planes), in the region of the facet
     // sums (dead during the point passes before phase 2 and during the
     // outflow): the moments' A (rows of data coefficients x CH points) and B
@@ -1043,27 +1062,31 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     }
     off += off & 1;                                // 16-byte alignment of the staging
     a.off_tc = (int)off;
-    take(&a.off_pd, std::max(pd, tcd));
+    // elements whose front data are taken at a time under the S-point rule (with
+    // kept U-values and few right-hand sides: all of the CTA's); the data share
+    // the region of the Dirichlet Grams
+    a.raw_el = a.S == 0 || rs > 1 ? 0 : keep > 0 && nrg <= 4 ? keep / QK : std::max(1, (keep > 0 ? CH : 2 * CH) / QK);
+    const size_t raw = (size_t)a.raw_el * Q * nrg * C;
+    a.off_raw = (int)off;
+    take(&a.off_pd, std::max({pd, raw, tcd > pdd ? tcd - pdd : 0}));
+    take(&a.off_dd, pdd);
     take(&a.off_del, (size_t)nrg * nb);
-    take(&a.off_u, (size_t)2 * CH * (nb | 1));
+    if (!share_u) take(&a.off_u, (size_t)2 * CH * (nb | 1));
     take(&a.off_pt, (size_t)a.ev_rows * (n + 2));
     // data coefficients, a row per right-hand side and component: of a chunk
-    // of points; under the S-point rule of raw_el elements' points (with kept
-    // U-values and few right-hand sides of all of the CTA's), and these
-    // elements' data at the front's points
-    a.raw_el = a.S == 0 || rs > 1 ? 0 : keep > 0 && nrg <= 4 ? keep / QK : std::max(1, (keep > 0 ? CH : 2 * CH) / QK);
+    // of points, or of those elements' points
     a.cb_pts = std::max({CH, a.raw_el * QK, keep > 0 && nrg <= 4 ? keep : 0});
     take(&a.off_cb, (size_t)(a.cb_pts | 1) * nrg * C);
-    take(&a.off_raw, (size_t)a.raw_el * Q * nrg * C);
     take(&a.off_tf, rs > 1 ? 0 : (size_t)2 * a.S * a.tf_stride);
     take(&a.off_gd, (size_t)CH * nrg);
     take(&a.off_rd, NB);
-    take(&a.off_rc, NB > 32 ? 4 * NB : 0);
+    take(&a.off_rc, NB > 96 ? 4 * NB : 8 * 32 * ((NB + 31) / 32));
     take(&a.off_eq, half_nb);
     take(&a.off_keep, (size_t)2 * keep * (nb | 1));   // U-values of the CTA's slice on both faces
+    if (share_u) a.off_u = a.off_keep + (2 * keep - 2 * CH) * (nb | 1);
     {   // the patch (Geo)
       const size_t NVg = n + 1, P_ = pmax, F_ = fmax, M_ = nmax;
-      const size_t dbl[] = {P_ * NVg * n, P_ * NVg, P_ * NVg, P_ * n, P_ * n, P_, P_, P_, P_ * NVg,
+      const size_t dbl[] = {P_ * NVg * n, P_ * NVg * (n + 2), P_ * NVg, P_ * NVg, P_ * n, P_ * n, P_, P_, P_, P_ * NVg,
                             F_ * NVg * NVg, F_, F_ * n, M_};
       const size_t ints[] = {P_, P_, P_ * NVg, F_ * NVg, F_, F_, M_};
       int g = 0;
@@ -1160,6 +1183,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   }
   bytes = plan(CH, keep, rows, rule);
   ctx->wide = bytes > two_per_sm;
+  ctx->min_cs = std::max(1, keep_cs);
   // one CTA per SM with the tensor-core contractions (it holds all 512 columns)
   if (tc_try) {
     bytes = std::max(bytes, std::min(max_dyn, (size_t)smem_sm / 2 + 1024 - stat_smem));
@@ -1212,6 +1236,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     int cs = ctx->flow_cs;
     bool sched_dataflow = true;
     if (tuned_lookup(ctx->tune_key, &cs, &sched_dataflow)) ctx->persistent = sched_dataflow;
+    cs = std::max(cs, ctx->min_cs);
     if (rs > 1) cs = rs;   // the cluster is the right-hand-side split
     if (ctx->persistent && set_persist_cs(ctx, cs) != TP_OK) ctx->persistent = false;   // one launch per level
   }

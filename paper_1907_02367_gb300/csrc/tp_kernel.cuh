@@ -34,7 +34,13 @@ __device__ __forceinline__ void red_release_add(int* p, int v) {
 
 // arrays of a tent's patch in shared memory (KArgs::geo: offsets in doubles)
 struct Geo {
-  enum { X, TB, TT, GB, GT, SDET, ISDET, GEL, GBF, FP, FSQ, FN, NTAU, EL, GRP, VID, FW, FG, FG2, NID, COUNT };
+  enum { X, XH, TB, TT, GB, GT, SDET, ISDET, GEL, GBF, FP, FSQ, FN, NTAU, EL, GRP, VID, FW, FG, FG2, NID, COUNT };
+};
+
+// a table in binary64 and as float-float pairs
+struct RuleTab {
+  const double* d;
+  const float2* ff;
 };
 
 struct KArgs {
@@ -155,10 +161,10 @@ struct KArgs {
   // to_front), in shared memory at off_tf; raw_el elements' front data at a
   // time at off_raw
   int S, tf_stride, off_tf, raw_el, off_raw;
-  const double *s_bary, *s_sqw, *tf;
-  const float2* tf_dd;
-  int off_rc;                                   // pivot row and column of the shared-memory elimination (two of each)
-  int off_b, off_pg, off_ph, off_pgb, off_pm, off_pd, off_sm, off_f, off_f2, off_fpm, off_del,
+  RuleTab tf;
+  RuleTab baryT, sqwT, s_baryT, s_sqwT;   // points (barycentric) and sqrt(w_ref) of the front rule and the S-point rule
+  int off_rc;                                   // pivot rows (and columns) of the elimination, two of each
+  int off_b, off_pg, off_ph, off_pgb, off_pm, off_pd, off_dd, off_sm, off_f, off_f2, off_fpm, off_del,
       off_u, off_mono, off_cb, off_gd, off_y, off_rd;
   // tensor-core contractions (mixed forward sweep with split right-hand
   // sides, single-material tents): the data moments and the outflow run as
@@ -447,6 +453,18 @@ __device__ __forceinline__ void eval_uvalues_block(const KArgs& a, int npt, cons
   __syncthreads();
 }
 
+// entry of a table in the path's arithmetic, and the table of a rule (KArgs: binary64, float-float)
+__device__ __forceinline__ double tab(const double* p) { return __ldg(p); }
+__device__ __forceinline__ dd tab(const dd* p) {
+  const float2 v = __ldg(reinterpret_cast<const float2*>(p));
+  return {v.x, v.y};
+}
+template <typename T>
+__device__ __forceinline__ const T* rule_tab(const RuleTab& t) {
+  if constexpr (std::is_same<T, dd>::value) return reinterpret_cast<const dd*>(t.ff);
+  else return t.d;
+}
+
 // s + y f for a factor f of a table of small exact numbers (derivative
 // relations, merged congruence tables): binary64 reads the table's binary64
 // copy and takes one fused multiply-add; float-float reads the binary32 copy
@@ -671,8 +689,8 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   __shared__ double s_gc[tp::kMaxGroups], s_gic2[tp::kMaxGroups];   // speeds and 1/c^2 of the materials
   __shared__ double s_xv[DIM];
   // the patch, in dynamic shared memory sized for the context's largest star
-  // (off_geo, in the order of Geo): per element its vertices' coordinates,
-  // bottom and top times, front gradients, sqrt|det| and its reciprocal, the
+  // (in the order of Geo): per element its vertices' coordinates, the same
+  // scaled to the tent's reference coordinates, bottom and top times, front gradients, sqrt|det| and its reciprocal, the
   // tent's wave-speed gradient and, mixed path, g_bot (DIM) and sqrt|det| (slot
   // DIM) as float-float pairs; per facet its simplex (x, t), sqrt(n! volume)
   // and normal; the front times of v and its neighbours; then integers: element
@@ -681,6 +699,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   // holds the block of their data among the vertex's boundary facets) and its
   // groups (Dirichlet: one; interface: +, -); the neighbour list's vertex ids
   double(*const s_X)[NV][DIM] = reinterpret_cast<double(*)[NV][DIM]>(sm + a.geo[Geo::X]);
+  T(*const s_xh)[NV][DIM + 2] = reinterpret_cast<T(*)[NV][DIM + 2]>(sm + a.geo[Geo::XH]);
   double(*const s_tb)[NV] = reinterpret_cast<double(*)[NV]>(sm + a.geo[Geo::TB]);
   double(*const s_tt)[NV] = reinterpret_cast<double(*)[NV]>(sm + a.geo[Geo::TT]);
   double(*const s_gb)[DIM] = reinterpret_cast<double(*)[DIM]>(sm + a.geo[Geo::GB]);
@@ -703,7 +722,6 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   __shared__ float2 s_gic2f[tp::kMaxGroups];   // mixed path: c^-2 of each material as a float-float pair
   __shared__ int s_ge0[tp::kMaxGroups + 1];   // elements of material g: [s_ge0[g], s_ge0[g + 1])
   __shared__ int s_piv;
-  __shared__ dd s_pb[2][4][32];   // register elimination: the pivot rows of a block of four steps
   __shared__ float s_red[2][NW];
 
   __shared__ int s_tent, s_bad;
@@ -729,8 +747,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   if (!SPLIT && a.S > 0) {   // (ordered before its first use by the first tent's barriers)
     T* sTF = reinterpret_cast<T*>(sm + a.off_tf);
     for (int id = tid; id < 2 * a.S * a.tf_stride; id += NT) {
-      if constexpr (MIXED) sTF[id] = {a.tf_dd[id].x, a.tf_dd[id].y};
-      else sTF[id] = a.tf[id];
+      sTF[id] = tab(rule_tab<T>(a.tf) + id);
     }
   }
   // barrier of the cluster (a cluster of one CTA: the block's)
@@ -918,31 +935,39 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   const int np = (e1 - e0) * QK;           // points of the slice in the rule of the face integrals
   // elements whose data are taken at a time (their points fit sU where the rows are not kept)
   const int EC = kept || a.S == 0 ? a.raw_el : min(a.raw_el, 2 * CH / QK);
-  const double *bary_ = a.S > 0 ? a.s_bary : a.bary, *sqw_ = a.S > 0 ? a.s_sqw : a.sqw;
   double ih = 0.0, tc = 0.0;
-  T* sKeep = reinterpret_cast<T*>(sm + a.off_keep);   // kept slice: its top U-values, then its bottom U-values
-  T* sKB = sKeep + (size_t)np * us;
+  // kept slice: the U-values of the outflow (forward: top points; adjoint:
+  // bottom), then those of the moments (the other face)
+  T* sKeep = reinterpret_cast<T*>(sm + a.off_keep);
+  T* sKI = sKeep + (size_t)np * us;
   const T* sTP = reinterpret_cast<const T*>(sm + a.off_tf);   // data to the rule's points, values to the front's
   const T* sTF = sTP + a.S * a.tf_stride;
   T* sRaw = reinterpret_cast<T*>(sm + a.off_raw);
   // a patch point q of element k mapped to the tent's reference coordinates
-  // (Remark 3.1) on the top (TOP) or bottom face, with sqrt(w) as the scale of
-  // its U-values
-  // (point q of the front rule; of the rule of bary_, sqw_)
-  auto map_point_of = [&](T* pp, int k, int q, bool top, const double* bary_, const double* sqw_) {
-    const double cg = s_gc[s_grp[k]];
-    double x[DIM], tt = 0.0;
-    for (int d = 0; d < DIM; ++d) x[d] = 0.0;
+  // (Remark 3.1) on the top (TOP) or bottom face: its barycentric coordinates
+  // (a rule's table) times the element's scaled vertices (s_xh), in the path's
+  // arithmetic; and sqrt(w) as the scale of its U-values (UNIT: 1)
+  auto map_with = [&](T* pp, int k, int q, bool top, const T* bary_, const T* sqw_, bool unit) {
+    T x[DIM + 1];
+#pragma unroll
+    for (int d = 0; d <= DIM; ++d) x[d] = R::zero();
+#pragma unroll
     for (int i = 0; i < NV; ++i) {
-      const double l = __ldg(bary_ + q * NV + i);
-      for (int d = 0; d < DIM; ++d) x[d] = fma(l, s_X[k][i][d], x[d]);
-      tt = fma(l, top ? s_tt[k][i] : s_tb[k][i], tt);
+      const T l = tab(bary_ + q * NV + i);
+      x[0] = R::acc(x[0], l, s_xh[k][i][top ? DIM + 1 : DIM]);
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) x[1 + d] = R::acc(x[1 + d], l, s_xh[k][i][d]);
     }
-    pp[0] = R::from(cg * (tt - tc) * ih);
-    for (int d = 0; d < DIM; ++d) pp[1 + d] = R::from((x[d] - s_xv[d]) * ih);
-    pp[DIM + 1] = R::from(__ldg(sqw_ + q) * s_sdet[k]);
+#pragma unroll
+    for (int d = 0; d <= DIM; ++d) pp[d] = R::norm(x[d]);
+    pp[DIM + 1] = unit ? R::one() : R::mul(tab(sqw_ + q), R::from(s_sdet[k]));
   };
-  auto map_point = [&](T* pp, int k, int q, bool top) { map_point_of(pp, k, q, top, a.bary, a.sqw); };
+  auto map_point = [&](T* pp, int k, int q, bool top) {   // of the front rule
+    map_with(pp, k, q, top, rule_tab<T>(a.baryT), rule_tab<T>(a.sqwT), false);
+  };
+  auto map_rule = [&](T* pp, int k, int q, bool top) {    // of the rule of the face integrals
+    map_with(pp, k, q, top, rule_tab<T>(a.S > 0 ? a.s_baryT : a.baryT), rule_tab<T>(a.S > 0 ? a.s_sqwT : a.sqwT), false);
+  };
   // data coefficients of the points base .. base + nq - 1 (patch point
   // numbering) for every right-hand side, one (point, right-hand side) per
   // thread so that the front loads of a chunk are all in flight at once:
@@ -1192,9 +1217,9 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   const int nneu = NEU ? s_nneu : 0;   // (kernels for meshes without Neumann facets leave out their code)
   const bool pblk = nif > 0 || nneu > 0;
   T* sFD = reinterpret_cast<T*>(sm + a.off_pd);      // Dirichlet sums (Grams, then data moments), then Neumann data
-  T* sDD = sFD + (size_t)ng * (DIM + 1) * npair;
-  const int nfd = nfac > 0 ? ng * (DIM + 1) * (npair + nrhs * nb) : 0;
-  T* sPBN = sFD + nfd;
+  T* sDD = reinterpret_cast<T*>(sm + a.off_dd);
+  const int nfg = nfac > 0 ? ng * (DIM + 1) * npair : 0, nfm = nfac > 0 ? ng * (DIM + 1) * nrhs * nb : 0;
+  T* sPBN = sDD + nfm;
   unsigned gdir = 0;   // materials with Dirichlet facets
   for (int f = 0; f < nfac; ++f) gdir |= 1u << s_fg[f];
   T* A0 = CS > 1 ? cluster.map_shared_rank(sA, 0) : sA;
@@ -1268,6 +1293,14 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       s_gt[k][d] = gt;
       g2 = fma(gt, gt, g2);
     }
+    {   // vertices in the tent's reference coordinates: xhat, then that on the bottom and the top
+      const double cg = s_gc[s_grp[k]], tcn = 0.5 * (tbot + s_ttop), ihn = s_ih;
+      for (int i = 0; i < NV; ++i) {
+        for (int d = 0; d < DIM; ++d) s_xh[k][i][d] = R::from((s_X[k][i][d] - s_xv[d]) * ihn);
+        s_xh[k][i][DIM] = R::from(cg * (s_tb[k][i] - tcn) * ihn);
+        s_xh[k][i][DIM + 1] = R::from(cg * (s_tt[k][i] - tcn) * ihn);
+      }
+    }
     s_sdet[k] = __ldg(a.elem_sdet + el);
     s_isdet[k] = __ldg(a.elem_isdet + el);
     if constexpr (MIXED) {
@@ -1336,7 +1369,8 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   // Dirichlet sums).
   auto facet_phase = [&]() {
   if (extra) {
-    for (int id = tid; id < nfd; id += blockDim.x) sFD[id] = R::zero();
+    for (int id = tid; id < nfg; id += blockDim.x) sFD[id] = R::zero();
+    for (int id = tid; id < nfm; id += blockDim.x) sDD[id] = R::zero();
     if (nneu > 0)
       for (int id = tid; id < nrhs * N; id += blockDim.x) sPBN[id] = R::zero();
     for (int id = tid; id < nrhs * nb; id += blockDim.x) sDel[id] = R::zero();
@@ -1567,9 +1601,10 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   }
   };
   if constexpr (!SPLIT) facet_phase();
-  // (the facets' Grams shared this region)
-  for (int id = tid; id < NG * (DIM + 2) * npair; id += blockDim.x) sPG[id] = R::zero();   // PG, PH, PGb contiguous
-  if (extra || np == 0) __syncthreads();
+  if (!kept) {   // (the facets' Grams shared this region)
+    for (int id = tid; id < NG * (DIM + 2) * npair; id += blockDim.x) sPG[id] = R::zero();
+    if (extra || np == 0) __syncthreads();
+  }
 
   // ---------------- Grams over this CTA's points ----------------
   int curk = SPLIT ? q0 / QK : e0, kend = (curk + 1) * QK;
@@ -1603,40 +1638,56 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       for (int d = 0; d < DIM; ++d) aH[s][d] = R::zero();
     }
   };
-  // one point (U-values ut at the top, ub at the bottom) of the slice added to the Grams
-  auto gram_point = [&](int pt, const T* ut, const T* ub) {
-    if (pt >= kend) {   // the next element's points start
-      const int k = SPLIT ? pt / QK : curk + 1;
-      flush_element(curk);
-      if (s_grp[k] != curg) {
-        flush_group(curg);
-        curg = s_grp[k];
+  // points pt .. end - 1 (rows of U-values ut at the top, ub at the bottom) added
+  // to the Grams, element by element so that the loads of several points are in
+  // flight (one point at a time exposed a shared-memory round trip per point)
+  auto gram_points = [&](int pt, int end, const T* ut, const T* ub) {
+    while (pt < end) {
+      if (pt >= kend) {   // the next element's points start
+        const int k = SPLIT ? pt / QK : curk + 1;
+        flush_element(curk);
+        if (s_grp[k] != curg) {
+          flush_group(curg);
+          curg = s_grp[k];
+        }
+        curk = k;
+        kend = (k + 1) * QK;
       }
-      curk = k;
-      kend = (k + 1) * QK;
-    }
+      const int n = min(end, kend) - pt;
 #pragma unroll
-    for (int s = 0; s < kMaxPair; ++s) {
-      if (tid + s * NT < npair) {
-        aK[s] = R::acc(aK[s], ut[pi[s]], ut[pj[s]]);
-        aB[s] = R::acc(aB[s], ub[pi[s]], ub[pj[s]]);
+      for (int s = 0; s < kMaxPair; ++s) {
+        if (tid + s * NT < npair) {
+          const T *ti = ut + pi[s], *tj = ut + pj[s], *bi = ub + pi[s], *bj = ub + pj[s];
+          T k_ = aK[s], b_ = aB[s];
+#pragma unroll 4
+          for (int q = 0; q < n; ++q) {
+            k_ = R::acc(k_, ti[q * us], tj[q * us]);
+            b_ = R::acc(b_, bi[q * us], bj[q * us]);
+          }
+          aK[s] = k_;
+          aB[s] = b_;
+        }
       }
+      pt += n;
+      ut += (size_t)n * us;
+      ub += (size_t)n * us;
     }
   };
   if (kept) {
-    // every U-value of the slice first (rows: its top points, then its bottom
-    // points), kept for the data moments and the outflow
+    // every U-value of the slice first, kept for the data moments and the outflow
     for (int base = 0; base < 2 * np; base += a.ev_rows) {
       const int n = min(a.ev_rows, 2 * np - base);
       for (int id = tid; id < n; id += blockDim.x) {
         const int row = base + id;
-        const bool top = row < np;
-        const int pt = top ? row : row - np, k = pt / QK;
-        map_point_of(sPt + id * (DIM + 2), e0 + k, pt - k * QK, top, bary_, sqw_);
+        const int pt = row < np ? row : row - np, k = pt / QK;
+        map_rule(sPt + id * (DIM + 2), e0 + k, pt - k * QK, (row < np) != ADJ);
       }
       eval_uvalues_block<DIM, T>(a, n, sPt, sM, sKeep + (size_t)base * us);
     }
-    for (int pt = 0; pt < np; ++pt) gram_point(e0 * QK + pt, sKeep + (size_t)pt * us, sKB + (size_t)pt * us);
+    // (the evaluation's buffer may share the Grams' region)
+    for (int id = tid; id < NG * (DIM + 2) * npair; id += blockDim.x) sPG[id] = R::zero();   // PG, PH, PGb contiguous
+    __syncthreads();
+    gram_points(e0 * QK, e1 * QK, ADJ ? sKI : sKeep, ADJ ? sKeep : sKI);
   } else {
     // chunks of points: U-values at the top, then at the bottom
     const int p0 = SPLIT ? q0 : e0 * QK, p1 = SPLIT ? q1 : e1 * QK;
@@ -1644,10 +1695,10 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       const int nq = min(CH, p1 - base);
       for (int id = tid; id < 2 * nq; id += blockDim.x) {
         const int side = id / nq, pt = base + id - side * nq, k = pt / QK;
-        map_point_of(sPt + id * (DIM + 2), k, pt - k * QK, side == 0, bary_, sqw_);
+        map_rule(sPt + id * (DIM + 2), k, pt - k * QK, side == 0);
       }
       eval_uvalues_block<DIM, T>(a, 2 * nq, sPt, sM, sU);
-      for (int ql = 0; ql < nq; ++ql) gram_point(base + ql, sU + (size_t)ql * us, sU + (size_t)(nq + ql) * us);
+      gram_points(base, base + nq, sU, sU + (size_t)nq * us);
       __syncthreads();
     }
   }
@@ -1698,13 +1749,16 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   if (pblk && CS > 1) cluster_reduce(sA, sA, N * N);   // interface and Neumann blocks
   if (NEU && s_nneu > 0) {   // Neumann data (after the Dirichlet sums)
     if (rsplit)
-      for (int id = tid; id < nrhs * N; id += blockDim.x) sb[id] = sFD[nfd + id];
+      for (int id = tid; id < nrhs * N; id += blockDim.x) sb[id] = sPBN[id];
     else
-      cluster_reduce(sFD + nfd, sb, nrhs * N);
+      cluster_reduce(sPBN, sb, nrhs * N);
   } else {
     for (int id = tid; id < nrhs * N; id += blockDim.x) sb[id] = R::zero();
   }
-  if (nfac > 0) cluster_reduce(sFD, sFD, rsplit ? ng * (DIM + 1) * npair : nfd);
+  if (nfac > 0) {
+    cluster_reduce(sFD, sFD, nfg);
+    if (!rsplit) cluster_reduce(sDD, sDD, nfm);
+  }
   csync();   // no CTA leaves or reuses its partials while another still reads them
   // congruence: the ranks form shares of A's entries and store them into rank
   // 0's A; rank 0 alone inverts and solves.  Every CTA holds the same summed
@@ -1833,85 +1887,118 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       }
       return false;
     };
-    if (N <= 32) {
-      // register path: row warp + NW s of the matrix in gr[s], column = lane.
-      // Blocks of four steps K = {k..k+3} per barrier: with S_K the block's
-      // pivot rows at its start, every warp reduces S_K by the four steps
-      // itself (P = [S_KK^-1 | S_KK^-1 S_KJ] in the pivot and the other
-      // columns), and a row i outside K becomes
-      //   (columns of K set to 0, the others kept) - sum_b s_{i,k+b} P_b,
-      // which is the four single steps taken at once (block Gauss-Jordan).
-      constexpr int NS = 32 / NW;
-      dd gr[NS];
+    // register path: row warp + NW s of the matrix in gr[s], columns lane + 32 c.
+    // Blocks of four steps K = {k..k+3} per barrier: with S_K the block's
+    // pivot rows at its start, every warp reduces S_K by the four steps
+    // itself (P = [S_KK^-1 | S_KK^-1 S_KJ] in the pivot and the other
+    // columns), and a row i outside K becomes
+    //   (columns of K set to 0, the others kept) - sum_b s_{i,k+b} P_b,
+    // which is the four single steps taken at once (block Gauss-Jordan).
+    // (Against one step per barrier in shared memory: 36 unknowns 40 us.)
+    auto invert_in_registers = [&](auto cols) {
+      constexpr int NC = decltype(cols)::value, NS = (32 * NC + NW - 1) / NW;
+      dd* pbuf = reinterpret_cast<dd*>(sm + a.off_rc);   // 2 x 4 pivot rows of 32 NC entries
+      dd gr[NS][NC];
 #pragma unroll
-      for (int s_ = 0; s_ < NS; ++s_) {
-        const int i = warp + NW * s_;
-        gr[s_] = {0.f, 0.f};
-        if (i < N && lane < N) gr[s_] = R::scaled(sA[i * N + lane], sEq[i] * sEq[lane]);
-      }
+      for (int s_ = 0; s_ < NS; ++s_)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          const int i = warp + NW * s_, j = lane + 32 * c;
+          gr[s_][c] = {0.f, 0.f};
+          if (i < N && j < N) gr[s_][c] = R::scaled(sA[i * N + j], sEq[i] * sEq[j]);
+        }
       for (int k = 0, blk = 0; k < N; k += 4, ++blk) {
-        const int kb = min(4, N - k);
-        dd(*pb)[32] = s_pb[blk & 1];
+        const int kb = min(4, N - k), kl = k & 31, kcw = k >> 5;   // (a block lies in one column group: 4 divides 32)
+        dd* pb = pbuf + (blk & 1) * 4 * 32 * NC;
         // the owners publish the block's pivot rows (rows k..k+3 are on warps
         // k % NW .. k % NW + 3, slot k / NW)
         if (warp >= k % NW && warp < k % NW + kb) {
 #pragma unroll
           for (int s_ = 0; s_ < NS; ++s_)
-            if (s_ == k / NW) pb[warp - k % NW][lane] = gr[s_];
+            if (s_ == k / NW) {
+#pragma unroll
+              for (int c = 0; c < NC; ++c) pb[(warp - k % NW) * 32 * NC + 32 * c + lane] = gr[s_][c];
+            }
         }
-        // this warp's rows in the pivot columns (block-start values)
-        dd ml[NS][4];
-#pragma unroll
-        for (int s_ = 0; s_ < NS; ++s_)
-#pragma unroll
-          for (int b = 0; b < 4; ++b)
-            ml[s_][b] = {-__shfl_sync(0xffffffffu, gr[s_].hi, k + b), -__shfl_sync(0xffffffffu, gr[s_].lo, k + b)};
         __syncthreads();
-        dd Pr[4];
+        dd Pr[4][NC];
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          Pr[b] = {0.f, 0.f};
-          if (b < kb) Pr[b] = pb[b][lane];
-        }
+        for (int b = 0; b < 4; ++b)
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+            Pr[b][c] = {0.f, 0.f};
+            if (b < kb) Pr[b][c] = pb[b * 32 * NC + 32 * c + lane];
+          }
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
           if (b >= kb) break;
-          const int kc = k + b;
+          const int kc = kl + b;
           dd mm[4];
 #pragma unroll
-          for (int c = 0; c < 4; ++c)
-            mm[c] = {__shfl_sync(0xffffffffu, Pr[c].hi, kc), __shfl_sync(0xffffffffu, Pr[c].lo, kc)};
+          for (int r = 0; r < 4; ++r) {
+            dd x = Pr[r][0];
+#pragma unroll
+            for (int c = 1; c < NC; ++c)
+              if (c == kcw) x = Pr[r][c];
+            mm[r] = {__shfl_sync(0xffffffffu, x.hi, kc), __shfl_sync(0xffffffffu, x.lo, kc)};
+          }
           dd pv = mm[b];
           if (bad_pivot(pv.hi)) pv = {1.f, 0.f};
           const dd rp = dd_rcp(pv);
-          const dd pn = (lane == kc) ? rp : dd_mul(Pr[b], rp);
 #pragma unroll
-          for (int c = 0; c < 4; ++c)
-            if (c != b) {
-              const dd x0 = lane == kc ? dd{0.f, 0.f} : Pr[c];
-              Pr[c] = Ar<dd>::norm(Ar<dd>::accn(x0, mm[c], pn));
-            }
-          Pr[b] = pn;
+          for (int c = 0; c < NC; ++c) {
+            const bool own = c == kcw && lane == kc;
+            const dd pn = own ? rp : dd_mul(Pr[b][c], rp);
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+              if (r != b) {
+                const dd x0 = own ? dd{0.f, 0.f} : Pr[r][c];
+                Pr[r][c] = Ar<dd>::norm(Ar<dd>::accn(x0, mm[r], pn));
+              }
+            Pr[b][c] = pn;
+          }
         }
-        const bool kcol = lane >= k && lane < k + kb;
+        const bool kcol = lane >= kl && lane < kl + kb;
 #pragma unroll
         for (int s_ = 0; s_ < NS; ++s_) {
           const int i = warp + NW * s_, bi = i - k;
-          if (bi >= 0 && bi < kb) {
-            gr[s_] = bi == 0 ? Pr[0] : bi == 1 ? Pr[1] : bi == 2 ? Pr[2] : Pr[3];
-          } else {
-            dd x = kcol ? dd{0.f, 0.f} : gr[s_];
+          if (i >= N) continue;
+          // this row in the pivot columns (block-start values)
+          dd x = gr[s_][0];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) x = Ar<dd>::acc(x, ml[s_][b], Pr[b]);
-            gr[s_] = Ar<dd>::norm(x);
+          for (int c = 1; c < NC; ++c)
+            if (c == kcw) x = gr[s_][c];
+          dd ml[4];
+#pragma unroll
+          for (int b = 0; b < 4; ++b)
+            ml[b] = {-__shfl_sync(0xffffffffu, x.hi, kl + b), -__shfl_sync(0xffffffffu, x.lo, kl + b)};
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+            if (bi >= 0 && bi < kb) {
+              gr[s_][c] = bi == 0 ? Pr[0][c] : bi == 1 ? Pr[1][c] : bi == 2 ? Pr[2][c] : Pr[3][c];
+            } else {
+              dd y = (c == kcw && kcol) ? dd{0.f, 0.f} : gr[s_][c];
+#pragma unroll
+              for (int b = 0; b < 4; ++b) y = Ar<dd>::acc(y, ml[b], Pr[b][c]);
+              gr[s_][c] = Ar<dd>::norm(y);
+            }
           }
         }
       }
 #pragma unroll
-      for (int s_ = 0; s_ < NS; ++s_) {
-        const int i = warp + NW * s_;
-        if (i < N && lane < N) sF_[i * N + lane] = gr[s_];
-      }
+      for (int s_ = 0; s_ < NS; ++s_)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          const int i = warp + NW * s_, j = lane + 32 * c;
+          if (i < N && j < N) sF_[i * N + j] = gr[s_][c];
+        }
+    };
+    if (N <= 32) {
+      invert_in_registers(std::integral_constant<int, 1>{});
+    } else if (N <= 64) {
+      invert_in_registers(std::integral_constant<int, 2>{});
+    } else if (WIDE && N <= 96) {
+      if constexpr (WIDE) invert_in_registers(std::integral_constant<int, 3>{});
     } else {
       // shared-memory path, one step per barrier: every entry belongs to one
       // thread (rows over warps, columns over lanes), which also writes the
@@ -1954,7 +2041,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   }
   // ---------------- the data of the bottom front (adjoint: of the top) ----------------
   if constexpr (!SPLIT) {
-    const T* U = ADJ ? sKeep : sKB;
+    const T* U = sKI;
     if (!kept && a.S == 0) {
       for (int base = q0; base < q1; base += CH) {
         const int nq = min(CH, q1 - base);
@@ -1988,7 +2075,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
         __syncthreads();
         if (!kept) {
           for (int id = tid; id < ne * S; id += blockDim.x)
-            map_point_of(sPt + id * (DIM + 2), eb + id / S, id % S, ADJ, bary_, sqw_);
+            map_rule(sPt + id * (DIM + 2), eb + id / S, id % S, ADJ);
           eval_uvalues_block<DIM, T>(a, ne * S, sPt, sM, sU);
         }
         data_moments(eb * S, ne * S, kept ? U + (size_t)(eb - e0) * S * us : sU, S);
@@ -2769,13 +2856,13 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   if (!SPLIT && a.S > 0) {
     // the fields at the rule's points, then through the table to the front's
     const int S = a.S;
-    const T* U = ADJ ? sKB : sKeep;
+    const T* U = sKeep;
     for (int eb = e0; eb < e1; eb += EC) {
       const int ne = min(EC, e1 - eb);
       if (eb > e0) __syncthreads();
       if (!kept) {
         for (int id = tid; id < ne * S; id += blockDim.x)
-          map_point_of(sPt + id * (DIM + 2), eb + id / S, id % S, !ADJ, bary_, sqw_);
+          map_rule(sPt + id * (DIM + 2), eb + id / S, id % S, !ADJ);
         eval_uvalues_block<DIM, T>(a, ne * S, sPt, sM, sU);
       }
       const T* Ue = kept ? U + (size_t)(eb - e0) * S * us : sU;
@@ -2824,19 +2911,8 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
     const int nq = min(kept ? NP : 2 * CH, o1 - base);
     if (!kept) {
     for (int id = tid; id < nq; id += blockDim.x) {
-      const int qg = base + id, k = qg / Q, q = qg % Q;
-      const double cg = s_gc[s_grp[k]];
-      double x[DIM], tt = 0.0;
-      for (int d = 0; d < DIM; ++d) x[d] = 0.0;
-      for (int i = 0; i < NV; ++i) {
-        const double l = __ldg(a.bary + q * NV + i);
-        for (int d = 0; d < DIM; ++d) x[d] = fma(l, s_X[k][i][d], x[d]);
-        tt = fma(l, ADJ ? s_tb[k][i] : s_tt[k][i], tt);
-      }
-      T* pp = sPt + id * (DIM + 2);
-      pp[0] = R::from(cg * (tt - tc) * ih);
-      for (int d = 0; d < DIM; ++d) pp[1 + d] = R::from((x[d] - s_xv[d]) * ih);
-      pp[DIM + 1] = R::one();
+      const int qg = base + id;
+      map_with(sPt + id * (DIM + 2), qg / Q, qg % Q, !ADJ, rule_tab<T>(a.baryT), rule_tab<T>(a.sqwT), true);
     }
     eval_uvalues_block<DIM, T, false>(a, nq, sPt, sM, sU);
     }
@@ -2887,7 +2963,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       for (int id = tid; id < nq * nrhs; id += blockDim.x) {
         const int ql = id / nrhs, r = id % nrhs;
         const int qg = base + ql, k = qg / Q, q = qg % Q;
-        const T* u = kept ? sKB + (size_t)(base - q0 + ql) * us : sU + (size_t)ql * us;
+        const T* u = kept ? sKeep + (size_t)(base - q0 + ql) * us : sU + (size_t)ql * us;
         double sv[C];
         for (int cc = 0; cc < C; ++cc) {
           const T* y = sY + (size_t)s_grp[k] * nmom + ((size_t)r * C + cc) * nb;
