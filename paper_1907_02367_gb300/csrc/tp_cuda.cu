@@ -159,7 +159,7 @@ struct tp_ctx {
   double* d_tau_work = nullptr;
   double* d_ckpt = nullptr;
   double* d_ckpt_tau = nullptr;
-  double* d_snap = nullptr;
+  double* d_fsave = nullptr;
   double* d_xsave = nullptr;
   long long xs_stride = 0, xsave_tents = 0;
   int* d_status = nullptr;
@@ -175,13 +175,16 @@ struct tp_ctx {
   bool mixed = false;
   // persistent dataflow sweep
   bool persistent = true;
-  int persist_clusters = 0;
+  int persist_clusters = 0, persist_clusters_adj = 0;
   int persist_cs = 1;
   int tune_key[5] = {0, 0, 0, 0, 0};   // (dim, p, nrhs, mixed, patch bucket) of the autotuner cache
   int* d_queue = nullptr;
   int* d_done = nullptr;
+  int* d_queue_adj = nullptr;   // of the reverse sweep and the gradient's forward sweeps (tp_adjoint)
+  int* d_done_adj = nullptr;
   int* d_tent_vert = nullptr;
   std::vector<int32_t> tent_level_h;   // levels of the tents (tp_inject_wait)
+  std::vector<long long> tent_el_h;    // elements of the patches of all tents before (ckpt_stride > 0)
   // vertex stars in the record order (grouped by material) and the tents'
   // vertices and top times (point outputs are assigned to tents on the host)
   std::vector<int> star_sorted;
@@ -271,15 +274,19 @@ cudaError_t launch_layer(tp_ctx* ctx, const KArgs& a, int n_cluster, int cs, int
 // resident clusters of the persistent kernel for cluster size cs
 int set_persist_cs(tp_ctx* ctx, int cs) {
   if (cs < ctx->min_cs) return TP_ERR_UNSUPPORTED;
-  int nclu = 0;
+  int nclu = 0, nadj = 0;
   cudaError_t e = kLaunchers[ctx->dim - 1][forward_kind(ctx)][ctx->neumann].max_clusters(
       cs, ctx->smem_bytes, ctx->rsplit_cs > 1, ctx->wide, &nclu);
-  if (e != cudaSuccess || nclu < 1) {
+  if (e == cudaSuccess)
+    e = kLaunchers[ctx->dim - 1][kAdjoint64][ctx->neumann].max_clusters(cs, ctx->smem_bytes, ctx->rsplit_cs > 1,
+                                                                        ctx->wide, &nadj);
+  if (e != cudaSuccess || nclu < 1 || nadj < 1) {
     cudaGetLastError();
     return TP_ERR_UNSUPPORTED;
   }
   ctx->persist_cs = cs;
   ctx->persist_clusters = nclu;
+  ctx->persist_clusters_adj = nadj;
   return TP_OK;
 }
 
@@ -315,6 +322,33 @@ KArgs group_args(const tp_ctx* ctx, KArgs a, int k) {
   return a;
 }
 
+__global__ void k_sweep_setup(const int* vert, int lo, int hi, int cs, int* done, int* queue, int head) {
+  // tents [lo, hi) complete before the range, per vertex (each tent counts once
+  // per CTA of its cluster); queue head at the range start
+  for (int t = lo + blockIdx.x * blockDim.x + threadIdx.x; t < hi; t += gridDim.x * blockDim.x)
+    atomicAdd(done + vert[t], cs);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *queue = head;
+}
+
+// the dataflow sweep over the tents of levels [level_begin, level_end), forward
+// or in reverse, with explicit kernel arguments
+cudaError_t launch_dataflow(tp_ctx* ctx, KArgs a, int32_t level_begin, int32_t level_end, bool adj, int* done, int* queue,
+                            cudaStream_t st) {
+  const int t0 = (int)ctx->level_ptr[level_begin - 1], t1 = (int)ctx->level_ptr[level_end - 1];
+  const int lo = adj ? t1 : 0, hi = adj ? (int)ctx->ntents : t0;
+  a.tent_beg = t0;
+  a.tent_end = t1;
+  a.done = done;
+  a.queue = queue;
+  cudaError_t e = cudaMemsetAsync(done, 0, ctx->nv * sizeof(int), st);
+  if (e != cudaSuccess) return e;
+  k_sweep_setup<<<std::max(1, std::min(1024, (hi - lo + 255) / 256)), 256, 0, st>>>(ctx->args.tent_v, lo, hi, ctx->persist_cs,
+                                                                                     done, queue, t0);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  return launch_layer(ctx, a, adj ? ctx->persist_clusters_adj : ctx->persist_clusters, ctx->persist_cs, 0, st,
+                      adj ? kAdjoint64 : forward_kind(ctx), true);
+}
+
 // one level; group < 0: every right-hand-side group, each from the front
 // times before the level (saved, and restored before every group after the first)
 int launch_level(tp_ctx* ctx, int32_t L, cudaStream_t st, bool adj = false, int group = -1) {
@@ -337,13 +371,21 @@ int launch_level(tp_ctx* ctx, int32_t L, cudaStream_t st, bool adj = false, int 
   return TP_OK;
 }
 
-// one level with explicit kernel arguments (one right-hand-side group)
-int launch_level_with(tp_ctx* ctx, int32_t L, cudaStream_t st, bool adj, const KArgs& a) {
-  const int64_t t0 = ctx->level_ptr[L - 1], t1 = ctx->level_ptr[L];
-  if (t1 <= t0) return TP_OK;
-  const int nt = (int)(t1 - t0);
-  TP_CUDA_OK(launch_layer(ctx, a, nt, level_cluster_size(ctx, nt), (int)t0, st, adj ? kAdjoint64 : forward_kind(ctx), false));
-  TP_CUDA_OK(cudaGetLastError());
+// levels [L0, L1) forward (or, adj, from L1 - 1 down) with explicit kernel
+// arguments (one right-hand-side group), by the context's schedule
+int launch_range_with(tp_ctx* ctx, int32_t L0, int32_t L1, cudaStream_t st, bool adj, const KArgs& a) {
+  if (ctx->persistent) {
+    TP_CUDA_OK(launch_dataflow(ctx, a, L0, L1, adj, ctx->d_done_adj, ctx->d_queue_adj, st));
+    return TP_OK;
+  }
+  for (int32_t i = L0; i < L1; ++i) {
+    const int32_t L = adj ? L1 - 1 - (i - L0) : i;
+    const int64_t t0 = ctx->level_ptr[L - 1], t1 = ctx->level_ptr[L];
+    if (t1 <= t0) continue;
+    const int nt = (int)(t1 - t0);
+    TP_CUDA_OK(launch_layer(ctx, a, nt, level_cluster_size(ctx, nt), (int)t0, st, adj ? kAdjoint64 : forward_kind(ctx), false));
+    TP_CUDA_OK(cudaGetLastError());
+  }
   return TP_OK;
 }
 
@@ -885,6 +927,16 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   a.vt_ptr = dvtp;
   a.vt_tau = dvtt;
   a.inject = dinj;
+  if (prm->ckpt_stride > 0) {
+    ctx->tent_el_h.assign(ctx->ntents + 1, 0);
+    for (int64_t it = 0; it < ctx->ntents; ++it) {
+      const int v = tents->vert[it];
+      ctx->tent_el_h[it + 1] = ctx->tent_el_h[it] + T.star_ptr[v + 1] - T.star_ptr[v];
+    }
+    long long* dte = nullptr;
+    if ((rc = ctx_upload(ctx, &dte, ctx->tent_el_h))) return fail(rc);
+    a.tent_el = dte;
+  }
   ctx->d_inject = dinj;
   ctx->tent_level_h = tents->level;
   a.max_spin = tp::kMaxSpin;
@@ -1586,16 +1638,6 @@ extern "C" int tp_solve_layer(tp_ctx* ctx, int32_t level, void* stream) {
   return launch_level(ctx, level, (cudaStream_t)stream);
 }
 
-namespace {
-__global__ void k_sweep_setup(const int* vert, int t_begin, int cs, int* done, int* queue) {
-  // completed tents before the range, per vertex (each tent counts once per
-  // CTA of its cluster); queue head at the range start
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < t_begin; t += gridDim.x * blockDim.x)
-    atomicAdd(done + vert[t], cs);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *queue = t_begin;
-}
-}  // namespace
-
 extern "C" int tp_advance(tp_ctx* ctx, int32_t level_begin, int32_t level_end, void* stream) {
   if (!ctx || level_begin < 1 || level_end > ctx->n_levels + 1 || level_end < level_begin) {
     tp::set_error("tp_advance: level range out of bounds");
@@ -1623,17 +1665,8 @@ extern "C" int tp_advance(tp_ctx* ctx, int32_t level_begin, int32_t level_end, v
         break;
       }
       if (ctx->persistent) {
-        const int t_begin = (int)ctx->level_ptr[level_begin - 1], t_end = (int)ctx->level_ptr[level_end - 1];
-        KArgs a = group_args(ctx, ctx->args, k);
-        a.tent_end = t_end;
-        cudaError_t e = cudaMemsetAsync(ctx->d_done, 0, ctx->nv * sizeof(int), ctx->cap_stream);
-        if (e == cudaSuccess) {
-          k_sweep_setup<<<std::max(1, std::min(1024, (t_begin + 255) / 256)), 256, 0, ctx->cap_stream>>>(
-              ctx->args.tent_v, t_begin, ctx->persist_cs, ctx->d_done, ctx->d_queue);
-          e = cudaGetLastError();
-        }
-        if (e == cudaSuccess)
-          e = launch_layer(ctx, a, ctx->persist_clusters, ctx->persist_cs, 0, ctx->cap_stream, forward_kind(ctx), true);
+        const cudaError_t e = launch_dataflow(ctx, group_args(ctx, ctx->args, k), level_begin, level_end, false, ctx->d_done,
+                                              ctx->d_queue, ctx->cap_stream);
         if (e != cudaSuccess) {
           tp::set_error(std::string("tp_advance: CUDA error ") + cudaGetErrorString(e));
           rc = TP_ERR_CUDA;
@@ -1674,10 +1707,11 @@ int grad_buffers(tp_ctx* ctx) {
   if (ctx->d_work) return TP_OK;
   const size_t nfront = (size_t)ctx->nrhs * ctx->ne * ctx->Q * ctx->C;
   const int S = ctx->ckpt_stride, nseg = (ctx->n_levels + S - 1) / S;
-  int64_t most = 0;   // tents of the largest segment
+  int64_t most = 0, mostel = 0;   // tents of the largest segment; elements of a segment's patches
   for (int sg = 0; sg < nseg; ++sg) {
     const int L0 = 1 + sg * S, L1 = std::min(L0 + S, ctx->n_levels + 1);
     most = std::max<int64_t>(most, ctx->level_ptr[L1 - 1] - ctx->level_ptr[L0 - 1]);
+    mostel = std::max<int64_t>(mostel, ctx->tent_el_h[ctx->level_ptr[L1 - 1]] - ctx->tent_el_h[ctx->level_ptr[L0 - 1]]);
   }
   ctx->xs_stride = (long long)ctx->nrhs * ctx->args.ngmax * ctx->nb;
   ctx->xsave_tents = most;
@@ -1685,9 +1719,9 @@ int grad_buffers(tp_ctx* ctx) {
       cudaMalloc(&ctx->d_tau_work, ctx->nv * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&ctx->d_ckpt, (size_t)nseg * nfront * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&ctx->d_ckpt_tau, (size_t)nseg * ctx->nv * sizeof(double)) != cudaSuccess ||
-      cudaMalloc(&ctx->d_snap, (size_t)S * nfront * sizeof(double)) != cudaSuccess ||
+      cudaMalloc(&ctx->d_fsave, (size_t)std::max<int64_t>(1, mostel) * ctx->nrhs * ctx->Q * ctx->C * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&ctx->d_xsave, (size_t)std::max<int64_t>(1, most) * ctx->xs_stride * sizeof(double)) != cudaSuccess) {
-    for (double** g : {&ctx->d_work, &ctx->d_tau_work, &ctx->d_ckpt, &ctx->d_ckpt_tau, &ctx->d_snap, &ctx->d_xsave}) {
+    for (double** g : {&ctx->d_work, &ctx->d_tau_work, &ctx->d_ckpt, &ctx->d_ckpt_tau, &ctx->d_fsave, &ctx->d_xsave}) {
       cudaFree(*g);
       *g = nullptr;
     }
@@ -1701,9 +1735,9 @@ int grad_buffers(tp_ctx* ctx) {
 // reverse sweep with the wave-speed gradient: forward from the initial state
 // of the last tp_set_state keeping a checkpoint (front and times) at the start
 // of every segment of ckpt_stride levels; then segment by segment from the
-// last: forward again from its checkpoint keeping the front before each level
-// and every tent's solution, and the reverse levels of the segment, each
-// adding its tents' dJ/dc
+// last: forward again from its checkpoint keeping every tent's bottom front
+// and solution, and the reverse levels of the segment, each adding its tents'
+// dJ/dc
 int adjoint_with_gradient(tp_ctx* ctx, double* d_dJ_dc, cudaStream_t st) {
   const size_t nfront = (size_t)ctx->nrhs * ctx->ne * ctx->Q * ctx->C;
   const size_t fb = nfront * sizeof(double), tb = ctx->nv * sizeof(double);
@@ -1722,8 +1756,8 @@ int adjoint_with_gradient(tp_ctx* ctx, double* d_dJ_dc, cudaStream_t st) {
     const int L0 = 1 + sg * S, L1 = std::min(L0 + S, ctx->n_levels + 1);
     TP_CUDA_OK(cudaMemcpyAsync(ctx->d_ckpt + (size_t)sg * nfront, ctx->d_work, fb, cudaMemcpyDeviceToDevice, st));
     TP_CUDA_OK(cudaMemcpyAsync(ctx->d_ckpt_tau + (size_t)sg * ctx->nv, ctx->d_tau_work, tb, cudaMemcpyDeviceToDevice, st));
-    for (int L = L0; L < L1; ++L)
-      if ((rc = launch_level_with(ctx, L, st, false, af)) != TP_OK) return rc;
+    // (the last segment is swept below)
+    if (sg + 1 < nseg && (rc = launch_range_with(ctx, L0, L1, st, false, af)) != TP_OK) return rc;
   }
   KArgs aa = ctx->args_adj;   // reverse, with the forward boundary data and the gradient
   aa.gD = ctx->args.gD;
@@ -1732,19 +1766,15 @@ int adjoint_with_gradient(tp_ctx* ctx, double* d_dJ_dc, cudaStream_t st) {
   aa.xs_stride = ctx->xs_stride;
   af.xsave = ctx->d_xsave;
   af.xs_stride = ctx->xs_stride;
+  af.fsave = aa.fsave = ctx->d_fsave;
   for (int sg = nseg - 1; sg >= 0; --sg) {
     const int L0 = 1 + sg * S, L1 = std::min(L0 + S, ctx->n_levels + 1);
     af.xbase = aa.xbase = ctx->level_ptr[L0 - 1];
+    af.fbase = aa.fbase = ctx->tent_el_h[af.xbase];
     TP_CUDA_OK(cudaMemcpyAsync(ctx->d_work, ctx->d_ckpt + (size_t)sg * nfront, fb, cudaMemcpyDeviceToDevice, st));
     TP_CUDA_OK(cudaMemcpyAsync(ctx->d_tau_work, ctx->d_ckpt_tau + (size_t)sg * ctx->nv, tb, cudaMemcpyDeviceToDevice, st));
-    for (int L = L0; L < L1; ++L) {
-      TP_CUDA_OK(cudaMemcpyAsync(ctx->d_snap + (size_t)(L - L0) * nfront, ctx->d_work, fb, cudaMemcpyDeviceToDevice, st));
-      if ((rc = launch_level_with(ctx, L, st, false, af)) != TP_OK) return rc;
-    }
-    for (int L = L1 - 1; L >= L0; --L) {
-      aa.front_fwd = ctx->d_snap + (size_t)(L - L0) * nfront;
-      if ((rc = launch_level_with(ctx, L, st, true, aa)) != TP_OK) return rc;
-    }
+    if ((rc = launch_range_with(ctx, L0, L1, st, false, af)) != TP_OK) return rc;
+    if ((rc = launch_range_with(ctx, L0, L1, st, true, aa)) != TP_OK) return rc;
   }
   return TP_OK;
 }
@@ -1769,9 +1799,14 @@ extern "C" int tp_adjoint(tp_ctx* ctx, const double* d_lambda_T, double* d_dJ_dc
   const size_t nfront = (size_t)ctx->nrhs * ctx->ne * ctx->Q * ctx->C;
   if (!ctx->d_adj) {   // the adjoint state, on first use
     if (cudaMalloc(&ctx->d_adj, nfront * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&ctx->d_tau_adj, ctx->nv * sizeof(double)) != cudaSuccess) {
+        cudaMalloc(&ctx->d_tau_adj, ctx->nv * sizeof(double)) != cudaSuccess ||
+        cudaMalloc(&ctx->d_queue_adj, sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&ctx->d_done_adj, ctx->nv * sizeof(int)) != cudaSuccess) {
       cudaFree(ctx->d_adj);
-      ctx->d_adj = nullptr;
+      cudaFree(ctx->d_tau_adj);
+      cudaFree(ctx->d_queue_adj);
+      ctx->d_adj = ctx->d_tau_adj = nullptr;
+      ctx->d_queue_adj = nullptr;
       cudaGetLastError();
       tp::set_error("tp_adjoint: device allocation of the adjoint state failed");
       return TP_ERR_OOM;
@@ -1798,6 +1833,12 @@ extern "C" int tp_adjoint(tp_ctx* ctx, const double* d_lambda_T, double* d_dJ_dc
           k_fill<<<(unsigned)std::min<int64_t>(1024, (ctx->nv + 255) / 256), 256, 0, ctx->cap_stream>>>(
               ctx->d_tau_adj, ctx->nv, ctx->T_final);
           if (cudaGetLastError() != cudaSuccess) rc = TP_ERR_CUDA;
+        }
+        if (ctx->persistent) {
+          if (rc == TP_OK && launch_dataflow(ctx, group_args(ctx, ctx->args_adj, k), 1, ctx->n_levels + 1, true, ctx->d_done_adj,
+                                             ctx->d_queue_adj, ctx->cap_stream) != cudaSuccess)
+            rc = TP_ERR_CUDA;
+          continue;
         }
         for (int32_t L = ctx->n_levels; L >= 1 && rc == TP_OK; --L) rc = launch_level(ctx, L, ctx->cap_stream, true, k);
       }
@@ -1950,11 +1991,13 @@ extern "C" void tp_destroy_ctx(tp_ctx* ctx) {
   cudaFree(ctx->d_diss);
   cudaFree(ctx->d_stats);
   for (void* g : ctx->probe_allocs) cudaFree(g);
-  for (double* g : {ctx->d_front0, ctx->d_work, ctx->d_tau_work, ctx->d_ckpt, ctx->d_ckpt_tau, ctx->d_snap, ctx->d_xsave})
+  for (double* g : {ctx->d_front0, ctx->d_work, ctx->d_tau_work, ctx->d_ckpt, ctx->d_ckpt_tau, ctx->d_fsave, ctx->d_xsave})
     cudaFree(g);
   cudaFree(ctx->d_adj);
   cudaFree(ctx->d_queue);
   cudaFree(ctx->d_done);
+  cudaFree(ctx->d_queue_adj);
+  cudaFree(ctx->d_done_adj);
   cudaFree(ctx->d_tau_adj);
   cudaFree(ctx->d_tau_save);
   if (ctx->adj_graph) cudaGraphExecDestroy(ctx->adj_graph);

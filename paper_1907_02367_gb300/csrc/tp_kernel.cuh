@@ -101,11 +101,15 @@ struct KArgs {
   // wave-speed gradient: the forward sweep stores each tent's solution
   // (xsave[(tent - xbase) * xs_stride + r * ngmax * nb + row], r over the
   // group's right-hand sides) when xsave is set; the reverse sweep reads it
-  // back with the forward front before the level (front_fwd) and adds
-  // dJ/dc per element into dJdc when dJdc is set
+  // back and adds dJ/dc per element into dJdc when dJdc is set; so with the
+  // bottom front of each tent, fsave[((tent_el[tent] - fbase) * R + r * P) * Q C ..]
+  // (tent_el: elements of the patches of all tents before; R, r: over the
+  // group's right-hand sides)
   double* xsave;
   long long xbase, xs_stride;
-  const double* front_fwd;
+  double* fsave;
+  long long fbase;
+  const long long* tent_el;
   double* dJdc;
   int off_yg;                 // shared memory of the gradient: y(x), y(x'), y(mu') and x
   // bounded waits and the solve's refinement: the dependency wait gives up
@@ -140,6 +144,7 @@ struct KArgs {
   const int* vt_ptr;          // per vertex w: its front times after 0, 1, .. of its tents, vt_tau[vt_ptr[w] ..]
   const double* vt_tau;
   const int* inject;          // (tent, extra): that tent waits for `extra` completions more (tp_inject_wait)
+  int tent_beg;               // tents of the sweep's range: [tent_beg, tent_end)
   const int* queue_tent;      // tent at each queue position (level order, critical chains first)
   int tent_end;
   // shared-memory carve (offsets in doubles)
@@ -764,7 +769,8 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
     if (tid == 0) s_bad = 0;
     if (rank == 0 && tid == 0) {
       const int pos = atomicAdd(a.queue, 1);
-      const int t_ = pos < a.tent_end ? __ldg(a.queue_tent + pos) : a.tent_end;
+      // (the reverse sweep takes the positions from the end)
+      const int t_ = pos < a.tent_end ? __ldg(a.queue_tent + (ADJ ? a.tent_beg + a.tent_end - 1 - pos : pos)) : a.tent_end;
       if (CS > 1)
         for (int r = 0; r < CS; ++r) *cluster.map_shared_rank(&s_tent, r) = t_;
       else
@@ -878,11 +884,14 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   // for (and acquires) the counts itself
   auto wait_deps = [&]() {
     if constexpr (PERSIST) {
-      const int extra_ = __ldg(a.inject) == tent ? __ldg(a.inject + 1) : 0;
+      const int extra_ = !ADJ && __ldg(a.inject) == tent ? __ldg(a.inject + 1) : 0;
       for (int e = tid; e < nn_; e += blockDim.x) {
-        const int before = __ldg(a.dep_need + d0_ + e);
+        const int w = s_nid[e];
+        int before = __ldg(a.dep_need + d0_ + e);
+        if constexpr (ADJ)   // the reverse sweep waits for the tents of w that follow this one
+          before = __ldg(a.vt_ptr + w + 1) - __ldg(a.vt_ptr + w) - 1 - before - (e == 0 ? 1 : 0);
         if (before == 0) continue;
-        const int w = s_nid[e], need = (before + extra_) * CS;
+        const int need = (before + extra_) * CS;
         long long spins = 0;
         while (ld_acquire(a.done + w) < need) {
           if (++spins > a.max_spin) {
@@ -916,7 +925,8 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   auto check_times = [&]() {
     if constexpr (PERSIST) {
       for (int e = tid; e < nn_; e += blockDim.x) {
-        if (__ldcg(a.tau + s_nid[e]) == s_ntau[e]) continue;
+        // (the reverse sweep finds v at the tent's top)
+        if (__ldcg(a.tau + s_nid[e]) == (ADJ && e == 0 ? s_ttop : s_ntau[e])) continue;
         if (CS == 1) s_bad = 1;
         else
           for (int r = 0; r < CS; ++r) *cluster.map_shared_rank(&s_bad, r) = 1;
@@ -2375,6 +2385,20 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   // the points whose front values this CTA overwrites (split right-hand
   // sides: this CTA's own right-hand sides at every point)
   const int o0 = rsplit ? 0 : q0, o1 = rsplit ? NP : q1;
+  // this tent's bottom front, for the reverse sweep of the wave-speed gradient
+  auto saved_front = [&](int r) {
+    return a.fsave + ((size_t)(__ldg(a.tent_el + tent) - a.fbase) * (SPLIT ? CS * nrhs : nrhs) +
+                      (size_t)((SPLIT ? rank * nrhs : 0) + r) * P) * Q * C;
+  };
+  if constexpr (!ADJ) {
+    if (a.fsave != nullptr) {
+      for (int id = tid; id < nrhs * (o1 - o0) * C; id += blockDim.x) {
+        const int r = id / ((o1 - o0) * C), qc = o0 * C + id - r * ((o1 - o0) * C), k = qc / (Q * C);
+        saved_front(r)[qc] = __ldcg(front + ((int64_t)r * a.ne + s_el[k]) * Q * C + (qc - k * Q * C));
+      }
+      __syncthreads();
+    }
+  }
   // ---------------- energy lost in the tent (forward sweep, when tracked) ----------------
   // Testing the tent system with V = U_h and using d/dt e + div(v sigma) = 0
   // inside the Trefftz tent: 1/2 int_top Q_{g_t}(u) = 1/2 int_bot Q_{g_b}(u_b) - D,
@@ -2599,6 +2623,15 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
         dFx[1] += Fx[1] / cg;
         dFm[1] += Fm[1] / cg;
       };
+      // contributions val[id], id = point * nrhs + right-hand side, added to an
+      // element by one warp in a fixed order
+      double* sVal = reinterpret_cast<double*>(sCB);   // 2 CH nrhs values (sCB is dead)
+      auto add_range = [&](int k, int lo, int hi) {
+        double t_ = 0.0;
+        for (int id = lo + lane; id < hi; id += 32) t_ += sVal[id];
+        for (int o = 16; o > 0; o >>= 1) t_ += __shfl_xor_sync(0xffffffffu, t_, o);
+        if (lane == 0) s_gel[k] += t_;
+      };
       // (a) top points (the map E and the top form) and bottom points (the
       // bottom form of b and the recovery terms), this CTA's points
       for (int side = 0; side < 2; ++side) {
@@ -2636,13 +2669,16 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
               val = e - (Qf(dFx, Fm) + Qf(Fx, dFm) + dic2 * Fx[1] * Fm[1]);
             } else {
               const double sw = __ldg(a.sqw + q) * s_sdet[k];
-              const double* f0 = a.front_fwd + (((int64_t)(rg0 + r) * a.ne + s_el[k]) * Q + q) * C;
+              const double* f0 = saved_front(r) + (size_t)qg * C;
               double fb[C];
               for (int cc = 0; cc < C; ++cc) fb[cc] = sw * __ldcg(f0 + cc);
               val = Qf(fb, dFm) + dic2 * fb[1] * Fm[1] + fb[0] * dFm[0] - (dFx[0] * Fm[0] + Fx[0] * dFm[0]);
             }
-            atomicAdd(s_gel + k, val);
+            sVal[id] = val;
           }
+          __syncthreads();
+          for (int k = base / Q + warp; k * Q < base + nq; k += NW)
+            add_range(k, max(0, k * Q - base) * nrhs, min(nq, (k + 1) * Q - base) * nrhs);
           __syncthreads();
         }
       }
@@ -2714,8 +2750,8 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
                 return 0.5 * (jm * (Xp[1] + Xm[1]) + dv * (sn(Xp) + sn(Xm))) + a.alpha * dv * (Xp[1] - Xm[1]) +
                        a.beta * jm * (sn(Xp) - sn(Xm));
               };
-              atomicAdd(s_gel + kp, -(I(dFx, Z, Fm, Gm) + I(Fx, Gx, dFm, Z)));
-              atomicAdd(s_gel + km, -(I(Z, dGx, Fm, Gm) + I(Fx, Gx, Z, dGm)));
+              sVal[id] = -(I(dFx, Z, Fm, Gm) + I(Fx, Gx, dFm, Z));
+              sVal[nq * nrhs + id] = -(I(Z, dGx, Fm, Gm) + I(Fx, Gx, Z, dGm));
             } else {
               const double gv = sGdd[id];
               double val;
@@ -2726,8 +2762,13 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
                 val = gv * (a.alpha * dFm[1] - sn(dFm)) -
                       ((sn(dFx) + a.alpha * dFx[1]) * Fm[1] + (sn(Fx) + a.alpha * Fx[1]) * dFm[1]);
               }
-              atomicAdd(s_gel + kp, val);
+              sVal[id] = val;
             }
+          }
+          __syncthreads();
+          if (warp == 0) {   // (the - side's follow the + side's)
+            add_range(kp, 0, nq * nrhs);
+            if (ifc) add_range(km, nq * nrhs, 2 * nq * nrhs);
           }
           __syncthreads();
         }

@@ -24,14 +24,14 @@ constexpr bool kMixed = TP_KIND == 1 || TP_KIND == 3, kAdj = TP_KIND == 2, kTc =
 
 using Kernel = void (*)(const KArgs, const int);
 
-// the variant for (dataflow, split right-hand sides, wide CTAs); the adjoint
-// runs one launch per level, launches per level have narrow CTAs, the tensor
-// cores take split right-hand sides in wide CTAs
+// the variant for (dataflow, split right-hand sides, wide CTAs); launches per
+// level have narrow CTAs, the tensor cores take split right-hand sides in wide
+// CTAs
 constexpr int kVariants = 8;
 template <int I>
 Kernel variant() {
   constexpr bool PERSIST = I & 4, SPLIT = I & 2, WIDE = I & 1;
-  if constexpr ((kAdj && PERSIST) || (kTc ? !(SPLIT && WIDE) : (WIDE && !PERSIST))) return nullptr;
+  if constexpr (kTc ? !(SPLIT && WIDE) : (WIDE && !PERSIST)) return nullptr;
   else return k_layer<TP_DIM, kMixed, kAdj, PERSIST, TP_NEU != 0, SPLIT, kTc, WIDE>;
 }
 template <int... I>
@@ -91,7 +91,7 @@ cudaError_t TP_NAME(launch_layer_d)(const KArgs& a, int n_cluster, int cs, int t
 cudaError_t TP_NAME(max_clusters_d)(int cs, size_t smem, bool split, bool wide, int* n) {
   cudaLaunchAttribute attr[1];
   const cudaLaunchConfig_t cfg = config(1, cs, smem, nullptr, wide, attr);
-  return cudaOccupancyMaxActiveClusters(n, pick(!kAdj, split, wide), &cfg);
+  return cudaOccupancyMaxActiveClusters(n, pick(true, split, wide), &cfg);
 }
 
 }  // namespace tp
