@@ -1085,7 +1085,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     // one region in turn: facet Grams of interface and Neumann facets, the
     // Grams G, H_m, Gbot (contiguous), the float-float inverse
     // (right-hand sides split: the facet Grams have a region of their own)
-    const size_t fg = ifneu ? (size_t)2 * npair + nb * nb : 0;
+    const size_t fg = ifneu ? (size_t)2 * npair + 3 * nb * nb : 0;   // (and two nb x nb products)
     a.off_f = (int)off;
     a.off_f2 = a.off_f + npair;
     a.off_fpm = a.off_f2 + npair;

@@ -507,25 +507,6 @@ __device__ __forceinline__ int pair_index(int i, int j, int nb) {
   return lo * nb - lo * (lo - 1) / 2 + (hi - lo);
 }
 
-// (D_va X D_vb^T)_ij for a packed symmetric X, D_var given by the relation
-// table: (D_var u)_j = sum over entries e of (j, var) of fac_e u[src_e]
-// (the factors are small integers, exact in binary32)
-template <int DIM, typename T>
-__device__ __forceinline__ T congruence(const KArgs& a, int i, int va, int j, int vb, const T* X, int nb) {
-  constexpr int NVAR = DIM + 1;
-  const int a0 = __ldg(a.rel_ptr + i * NVAR + va), a1 = __ldg(a.rel_ptr + i * NVAR + va + 1);
-  const int b0 = __ldg(a.rel_ptr + j * NVAR + vb), b1 = __ldg(a.rel_ptr + j * NVAR + vb + 1);
-  T s = Ar<T>::zero();
-  for (int e = a0; e < a1; ++e) {
-    const int si = __ldg(a.rel_src + e);
-    T t = Ar<T>::zero();
-    for (int f = b0; f < b1; ++f)
-      t = Fac<T>::add(t, X[pair_index(si, __ldg(a.rel_src + f), nb)], a.rel_facf, a.rel_fac, f);
-    s = Fac<T>::add(s, t, a.rel_facf, a.rel_fac, e);
-  }
-  return s;
-}
-
 // (D_var y)_i for a vector y
 template <int DIM, typename T>
 __device__ __forceinline__ T rel_apply(const KArgs& a, int i, int var, const T* y) {
@@ -570,50 +551,6 @@ __device__ __forceinline__ double recip(double x) {
   r = fma(r, e, r);
   e = fma(-x, r, 1.0);
   return fma(r, e, r);
-}
-
-// (D_va X D_vb^T)_ij for a full row-major nb x nb X (or X^T when TR)
-template <int DIM, typename T, bool TR>
-__device__ __forceinline__ T congruence_full(const KArgs& a, int i, int va, int j, int vb, const T* X, int nb) {
-  constexpr int NVAR = DIM + 1;
-  const int a0 = __ldg(a.rel_ptr + i * NVAR + va), a1 = __ldg(a.rel_ptr + i * NVAR + va + 1);
-  const int b0 = __ldg(a.rel_ptr + j * NVAR + vb), b1 = __ldg(a.rel_ptr + j * NVAR + vb + 1);
-  T s = Ar<T>::zero();
-  for (int e = a0; e < a1; ++e) {
-    const int si = __ldg(a.rel_src + e);
-    T t = Ar<T>::zero();
-    for (int f = b0; f < b1; ++f) {
-      const int sj = __ldg(a.rel_src + f);
-      t = Fac<T>::add(t, TR ? X[sj * nb + si] : X[si * nb + sj], a.rel_facf, a.rel_fac, f);
-    }
-    s = Fac<T>::add(s, t, a.rel_facf, a.rel_fac, e);
-  }
-  return s;
-}
-
-// n-weighted normal-derivative congruences: (D_a X D_b^T) with a, b in {t, n}
-// where D_n = sum_m n_m D_m.  SYM: X packed symmetric, else full (TR: X^T).
-template <int DIM, typename T, int MODE>
-__device__ __forceinline__ T cong_any(const KArgs& a, int i, int va, int j, int vb, const T* X, int nb) {
-  if constexpr (MODE == 0) return congruence<DIM, T>(a, i, va, j, vb, X, nb);
-  else if constexpr (MODE == 1) return congruence_full<DIM, T, false>(a, i, va, j, vb, X, nb);
-  else return congruence_full<DIM, T, true>(a, i, va, j, vb, X, nb);
-}
-template <int DIM, typename T, int MODE>
-__device__ __forceinline__ void iface_terms(const KArgs& a, int i, int j, const T* X, int nb, const T* nrm,
-                                            T* ntn, T* ntt, T* ttn, T* nnn) {
-  // ntt = (D_n X D_t^T), ttn = (D_t X D_n^T), nnn = (D_n X D_n^T), ntn unused slot kept for symmetry
-  T a1 = Ar<T>::zero(), a2 = Ar<T>::zero(), a3 = Ar<T>::zero();
-  for (int m = 0; m < DIM; ++m) {
-    a1 = Ar<T>::fma(nrm[m], cong_any<DIM, T, MODE>(a, i, 1 + m, j, 0, X, nb), a1);
-    a2 = Ar<T>::fma(nrm[m], cong_any<DIM, T, MODE>(a, i, 0, j, 1 + m, X, nb), a2);
-    for (int m2 = 0; m2 < DIM; ++m2)
-      a3 = Ar<T>::fma(Ar<T>::mul(nrm[m], nrm[m2]), cong_any<DIM, T, MODE>(a, i, 1 + m, j, 1 + m2, X, nb), a3);
-  }
-  *ntt = a1;
-  *ttn = a2;
-  *nnn = a3;
-  *ntn = cong_any<DIM, T, MODE>(a, i, 0, j, 0, X, nb);   // (D_t X D_t^T)
 }
 
 // One tent per thread-block cluster of CS CTAs (CS = gridDim.x / tents in the
@@ -1556,16 +1493,52 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       __syncthreads();
       T nrm[DIM];
       for (int d = 0; d < DIM; ++d) nrm[d] = R::from(s_fn[f][d]);
-      if (neu) {
-        const double ih2 = ih * ih;
+      // block D_n X W1^T + D_t X W2^T, W = wt D_t + wn D_n (D_n = sum_m n_m D_m), of
+      // a facet Gram X (MODE 0 packed symmetric, 1 full, 2 full transposed) added
+      // to the partial A: first Y = X W^T, then the rows; each entry takes a
+      // few terms instead of the products of both operators' terms
+      // (2D p = 5: a facet's four blocks 80 us before)
+      auto facet_block = [&](auto mode, const T* X, T w1t, T w1n, T w2t, T w2n, int gr, int gcl) {
+        constexpr int MODE = decltype(mode)::value;
+        T *Y1 = sFpm + nb * nb, *Y2 = Y1 + nb * nb;
         for (int id = tid; id < nb * nb; id += blockDim.x) {
-          const int i = id / nb, j = id % nb;
-          T tt_, nt_, tn_, nn_;
-          iface_terms<DIM, T, 0>(a, i, j, sF, nb, nrm, &tt_, &nt_, &tn_, &nn_);
-          const T t = R::fma(R::from(-cp * ih2), nt_, R::mul(R::from(a.beta * ih2), nn_));
-          T* dst = sA + (size_t)(gp * nb + i) * N + gp * nb + j;
+          const int k = id / nb, jj = id - k * nb;
+          T dt = R::zero(), dn = R::zero();
+#pragma unroll
+          for (int v_ = 0; v_ <= DIM; ++v_) {
+            T t = R::zero();
+            for (int e = __ldg(a.rel_ptr + jj * NV + v_), e1_ = __ldg(a.rel_ptr + jj * NV + v_ + 1); e < e1_; ++e) {
+              const int sj = __ldg(a.rel_src + e);
+              const T x = MODE == 0 ? X[pair_index(k, sj, nb)] : MODE == 1 ? X[k * nb + sj] : X[sj * nb + k];
+              t = Fac<T>::add(t, x, a.rel_facf, a.rel_fac, e);
+            }
+            if (v_ == 0) dt = t;
+            else dn = R::fma(nrm[v_ - 1], t, dn);
+          }
+          Y1[id] = R::fma(w1t, dt, R::mul(w1n, dn));
+          Y2[id] = R::fma(w2t, dt, R::mul(w2n, dn));
+        }
+        __syncthreads();
+        for (int id = tid; id < nb * nb; id += blockDim.x) {
+          const int i = id / nb, jj = id - i * nb;
+          T t = R::zero();
+#pragma unroll
+          for (int v_ = 0; v_ <= DIM; ++v_) {
+            const T* Y = v_ == 0 ? Y2 : Y1;
+            T u = R::zero();
+            for (int e = __ldg(a.rel_ptr + i * NV + v_), e1_ = __ldg(a.rel_ptr + i * NV + v_ + 1); e < e1_; ++e)
+              u = Fac<T>::add(u, Y[__ldg(a.rel_src + e) * nb + jj], a.rel_facf, a.rel_fac, e);
+            t = v_ == 0 ? u : R::fma(nrm[v_ - 1], u, t);
+          }
+          T* dst = sA + (size_t)(gr * nb + i) * N + gcl * nb + jj;
           *dst = R::add(*dst, t);
         }
+        __syncthreads();
+      };
+      const double ih2 = ih * ih;
+      if (neu) {
+        facet_block(std::integral_constant<int, 0>{}, sF, R::from(-cp * ih2), R::from(a.beta * ih2), R::zero(), R::zero(), gp,
+                    gp);
         for (int id = tid; id < nrhs * nb; id += blockDim.x) {
           const int r = id / nb, i = id % nb;
           const T* del = sDel + (size_t)r * nb;
@@ -1580,31 +1553,17 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
         __syncthreads();
         continue;
       }
-      {
-        const double ih2 = ih * ih;
-        for (int id = tid; id < 4 * nb * nb; id += blockDim.x) {
-          const int blk = id / (nb * nb), rem = id % (nb * nb), i = rem / nb, j = rem % nb;
-          const int tside = blk >> 1, sside = blk & 1;   // 0: +, 1: -
-          const double st = tside ? -1.0 : 1.0, ss = sside ? -1.0 : 1.0;
-          const double ct = tside ? cm : cp, cs = sside ? cm : cp;
-          T tt_, nt_, tn_, nn_;
-          if (tside == sside) {
-            iface_terms<DIM, T, 0>(a, i, j, tside ? sF2 : sF, nb, nrm, &tt_, &nt_, &tn_, &nn_);
-          } else if (tside == 0) {
-            iface_terms<DIM, T, 1>(a, i, j, sFpm, nb, nrm, &tt_, &nt_, &tn_, &nn_);
-          } else {
-            iface_terms<DIM, T, 2>(a, i, j, sFpm, nb, nrm, &tt_, &nt_, &tn_, &nn_);
-          }
-          T t = R::mul(R::from(-0.5 * st * cs * ih2), nt_);
-          t = R::fma(R::from(-0.5 * st * ct * ih2), tn_, t);
-          t = R::fma(R::from(st * ss * a.alpha * cs * ct * ih2), tt_, t);
-          t = R::fma(R::from(st * ss * a.beta * ih2), nn_, t);
-          const int gr = tside ? gm : gp, gcl = sside ? gm : gp;
-          T* dst = sA + (size_t)(gr * nb + i) * N + gcl * nb + j;
-          *dst = R::add(*dst, t);
-        }
+      for (int blk = 0; blk < 4; ++blk) {
+        const int tside = blk >> 1, sside = blk & 1;   // test and trial side, 0: +, 1: -
+        const double st = tside ? -1.0 : 1.0, ss = sside ? -1.0 : 1.0;
+        const double ct = tside ? cm : cp, cs = sside ? cm : cp;
+        const T w1t = R::from(-0.5 * st * cs * ih2), w1n = R::from(st * ss * a.beta * ih2);
+        const T w2t = R::from(st * ss * a.alpha * cs * ct * ih2), w2n = R::from(-0.5 * st * ct * ih2);
+        const int gr = tside ? gm : gp, gcl = sside ? gm : gp;
+        if (tside == sside) facet_block(std::integral_constant<int, 0>{}, tside ? sF2 : sF, w1t, w1n, w2t, w2n, gr, gcl);
+        else if (tside == 0) facet_block(std::integral_constant<int, 1>{}, sFpm, w1t, w1n, w2t, w2n, gr, gcl);
+        else facet_block(std::integral_constant<int, 2>{}, sFpm, w1t, w1n, w2t, w2n, gr, gcl);
       }
-      __syncthreads();
       for (int id = tid; id < nb * nb; id += blockDim.x) sFpm[id] = R::zero();
       __syncthreads();
     }
@@ -2111,24 +2070,32 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
     __syncthreads();
   }
   {
+    // the C terms of an entry (gamma, (c/h) D_t alpha, -(1/h) D_m beta_m) on
+    // neighbouring lanes, added by shuffles: the chain of dependent tents
+    // waits for the longest of them instead of their sum
     const T mih = R::from(-ih);
-    for (int id = tid; id < nrhs * N; id += blockDim.x) {
-      const int r = id / N, Rw = id % N;
-      const int g = Rw / nb, i = Rw % nb;
-      const T* M = sSM + (size_t)g * nmom + (size_t)r * C * nb;   // gamma, alpha, beta_1..beta_n
-      T t = R::fma(R::from(s_gc[g] * ih), rel_apply<DIM, T>(a, i, 0, M + nb), M[i]);
-      for (int d = 0; d < DIM; ++d) t = R::fma(mih, rel_apply<DIM, T>(a, i, 1 + d, M + (2 + d) * nb), t);
-      // Dirichlet data: b_D = E' delta summed over g's facets,
-      // E' = alpha (c/h) D_t + (1/h) D_n
-      if ((gdir >> g) & 1u) {
-        const T* Dg = sDD + (size_t)g * (DIM + 1) * nrhs * nb + (size_t)r * nb;
-        T dn = rel_apply<DIM, T>(a, i, 1, Dg + (size_t)nrhs * nb);
-        for (int d = 1; d < DIM; ++d) dn = R::add(dn, rel_apply<DIM, T>(a, i, 1 + d, Dg + (size_t)(1 + d) * nrhs * nb));
-        const T ac = R::from(a.alpha * s_gc[g] * ih);
-        t = R::add(t, R::fma(R::from(ih), dn, R::mul(ac, rel_apply<DIM, T>(a, i, 0, Dg))));
+    constexpr int LB = C <= 4 ? 4 : 8;
+    for (int base = 0; base < nrhs * N * LB; base += NT) {
+      const int id = base + tid, it = id / LB, cc = id % LB;
+      const bool live = it < nrhs * N && cc < C;
+      const int r = it / N, Rw = it - r * N, g = Rw / nb, i = Rw - g * nb;
+      T t = R::zero();
+      if (live) {
+        const T* M = sSM + (size_t)g * nmom + ((size_t)r * C + cc) * nb;   // gamma, alpha, beta_1..beta_n
+        t = cc == 0 ? M[i] : R::mul(cc == 1 ? R::from(s_gc[g] * ih) : mih, rel_apply<DIM, T>(a, i, cc - 1, M));
+        // Dirichlet data: b_D = E' delta summed over g's facets,
+        // E' = alpha (c/h) D_t + (1/h) D_n
+        if (cc > 0 && ((gdir >> g) & 1u)) {
+          const T* Dg = sDD + (size_t)(g * (DIM + 1) + cc - 1) * nrhs * nb + (size_t)r * nb;
+          t = R::fma(R::from(cc == 1 ? a.alpha * s_gc[g] * ih : ih), rel_apply<DIM, T>(a, i, cc - 1, Dg), t);
+        }
       }
-      const size_t o = (size_t)r * N + Rw;
-      sb[o] = R::add(sb[o], t);
+#pragma unroll
+      for (int o = 1; o < LB; o <<= 1) t = R::add(t, shfl_xor_t(t, o));
+      if (live && cc == 0) {
+        const size_t o = (size_t)r * N + Rw;
+        sb[o] = R::add(sb[o], t);
+      }
     }
   }
   __syncthreads();
