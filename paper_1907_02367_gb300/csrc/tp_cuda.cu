@@ -1132,7 +1132,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     take(&a.off_tf, rs > 1 ? 0 : (size_t)2 * a.S * a.tf_stride);
     take(&a.off_gd, (size_t)CH * nrg);
     take(&a.off_rd, NB);
-    take(&a.off_rc, NB > 96 ? 4 * NB : 8 * 32 * ((NB + 31) / 32));
+    take(&a.off_rc, std::max((size_t)8 * 32 * std::min<size_t>(3, (NB + 31) / 32), NB > 64 ? 4 * NB : 0));
     take(&a.off_eq, half_nb);
     take(&a.off_keep, (size_t)2 * keep * (nb | 1));   // U-values of the CTA's slice on both faces
     if (share_u) a.off_u = a.off_keep + (2 * keep - 2 * CH) * (nb | 1);
