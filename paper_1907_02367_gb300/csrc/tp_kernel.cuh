@@ -2740,7 +2740,18 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
           __syncthreads();
         }
       }
-      for (int k = tid; k < P; k += blockDim.x) atomicAdd(a.dJdc + s_el[k], s_gel[k]);
+      // one addition per element and tent, the CTAs' shares summed in rank order:
+      // the tents of an element follow one another (each waits for the later
+      // ones of its vertex and neighbours), so the sum's order is fixed
+      csync();
+      for (int k = tid * CS + rank; k < P; k += NT * CS) {
+        double t_ = s_gel[k];
+        if (CS > 1) {
+          t_ = 0.0;
+          for (int r = 0; r < CS; ++r) t_ += cluster.map_shared_rank(s_gel, r)[k];
+        }
+        atomicAdd(a.dJdc + s_el[k], t_);
+      }
       __syncthreads();
     }
   }
