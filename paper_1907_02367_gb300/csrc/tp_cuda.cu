@@ -875,6 +875,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   cudaGetDevice(&ctx->device);
 
   a.nb = ctx->nb;
+  a.nl = basis->nl;
   a.nmono = ctx->nmono;
   a.p = basis->p;
   {
@@ -911,6 +912,12 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
       ev_order.push_back(key[j].second);
     }
     a.ev_off[a.ev_ncls] = basis->nb;
+    a.ev_loff[0] = 0;
+    for (int c = 0; c < a.ev_ncls; ++c) {
+      int k = 0;
+      for (int j = a.ev_off[c]; j < a.ev_off[c + 1]; ++j) k += key[j].second < basis->nl;
+      a.ev_loff[c + 1] = a.ev_loff[c] + k;
+    }
     int* devo = nullptr;
     if ((rc = ctx_upload(ctx, &devo, ev_order))) return fail(rc);
     a.ev_order = devo;
@@ -1036,8 +1043,8 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   a.status_info = ctx->d_info;
   // shared-memory plan: the largest chunk of points that fits
   const int nb = ctx->nb, C = ctx->C;
-  const int npair = nb * (nb + 1) / 2;
-  if (npair > kMaxPairs) {
+  const int nl = basis->nl, npair = nb * (nb + 1) / 2, npl = nl * (nl + 1) / 2;
+  if (npair > kMaxPairs || npl > tp::kMaxLowPairs) {
     tp::set_error("tp_create: dim U^p too large for this kernel (more than 38)");
     return fail(TP_ERR_UNSUPPORTED);
   }
@@ -1073,8 +1080,8 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     // reduced in place, and a partial b (tents with Neumann facets)
     size_t pd = 0, pdd = 0;
     for (const auto& m : facet_mix) {
-      pd = std::max(pd, m[1] > 0 ? (size_t)m[0] * (n + 1) * npair : 0);
-      pdd = std::max(pdd, (m[1] > 0 ? (size_t)m[0] * (n + 1) * nrg * nb : 0) + (m[3] > 0 ? (size_t)nrg * m[0] * nb : 0));
+      pd = std::max(pd, m[1] > 0 ? (size_t)m[0] * (n + 1) * npl : 0);
+      pdd = std::max(pdd, (m[1] > 0 ? (size_t)m[0] * (n + 1) * nrg * nl : 0) + (m[3] > 0 ? (size_t)nrg * m[0] * nb : 0));
     }
     a.ev_rows = std::max(2 * CH, rows);
     const size_t mono = (size_t)a.ev_rows * a.mono_stride;
@@ -1085,16 +1092,16 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     // one region in turn: facet Grams of interface and Neumann facets, the
     // Grams G, H_m, Gbot (contiguous), the float-float inverse
     // (right-hand sides split: the facet Grams have a region of their own)
-    const size_t fg = ifneu ? (size_t)2 * npair + 3 * nb * nb : 0;   // (and two nb x nb products)
+    const size_t fg = ifneu ? (size_t)2 * npl + nl * nl + 2 * nl * nb : 0;   // (and two nl x nb products)
     a.off_f = (int)off;
-    a.off_f2 = a.off_f + npair;
-    a.off_fpm = a.off_f2 + npair;
+    a.off_f2 = a.off_f + npl;
+    a.off_fpm = a.off_f2 + npl;
     if (rs > 1) off += fg;
     a.off_pg = (int)off;
-    a.off_ph = a.off_pg + ngmax * npair;
-    a.off_pgb = a.off_ph + ngmax * n * npair;
+    a.off_ph = a.off_pg + ngmax * npl;
+    a.off_pgb = a.off_ph + ngmax * n * npl;
     a.off_mono = (int)off;
-    take(nullptr, std::max({(size_t)ngmax * (n + 2) * npair, NB * NB, fg, share_mono ? mono : 0}));
+    take(nullptr, std::max({(size_t)ngmax * ((n + 1) * npl + npair), NB * NB, fg, share_mono ? mono : 0}));
     take(&a.off_pm, (size_t)ngmax * nmom);        // moments: partials, summed in place, then the outflow vectors
     a.off_sm = a.off_y = a.off_pm;
     if (!share_mono) take(&a.off_mono, mono);
@@ -1122,7 +1129,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     a.off_raw = (int)off;
     take(&a.off_pd, std::max({pd, raw, tcd > pdd ? tcd - pdd : 0}));
     take(&a.off_dd, pdd);
-    take(&a.off_del, (size_t)nrg * nb);
+    take(&a.off_del, (size_t)nrg * std::max(1, nl));
     if (!share_u) take(&a.off_u, (size_t)2 * CH * (nb | 1));
     take(&a.off_pt, (size_t)a.ev_rows * (n + 2));
     // data coefficients, a row per right-hand side and component: of a chunk

@@ -594,6 +594,34 @@ extern "C" int tp_build_basis(int32_t dim, int32_t p, tp_basis** out) {
     }
   }
   B->nb = (int)funcs.size();
+  // the tables' order: the functions of degree <= p - 1 first.  Every derivative
+  // of a function of U^p is in their span (relations below), so v, sigma, the
+  // moments that are tested with them and the Grams of the faces' derivative
+  // terms run over the first nl functions alone (3D p = 3: 14 of 30)
+  std::vector<int> place(B->nb);   // exported position -> position in the tables
+  {
+    std::vector<int> order;
+    for (int pass = 0; pass < 2; ++pass)
+      for (int j = 0; j < B->nb; ++j) {
+        int deg = ftype[j];
+        for (int d = 1; d <= n; ++d) deg += fbeta[j][d];
+        if ((deg < p) == (pass == 0)) order.push_back(j);
+        if (pass == 0 && deg < p) ++B->nl;
+      }
+    std::vector<std::vector<Term>> f2;
+    std::vector<int> t2;
+    std::vector<Exps> b2;
+    for (int i = 0; i < B->nb; ++i) {
+      const int j = order[i];
+      place[j] = i;
+      f2.push_back(funcs[j]);
+      t2.push_back(ftype[j]);
+      b2.push_back(fbeta[j]);
+    }
+    funcs.swap(f2);
+    ftype.swap(t2);
+    fbeta.swap(b2);
+  }
   // derivative relations (exact identities of the closed form, no rounding):
   //   d/dx_m b_{beta,type} = beta_m b_{beta-e_m,type}
   //   d/dt   b_{beta,1}    = b_{beta,0}
@@ -644,7 +672,7 @@ extern "C" int tp_build_basis(int32_t dim, int32_t p, tp_basis** out) {
     const int nb = B->nb;
     auto pidx = [&](int i, int j) {
       const int lo = std::min(i, j), hi = std::max(i, j);
-      return lo * nb - lo * (lo - 1) / 2 + (hi - lo);
+      return hi * (hi + 1) / 2 + lo;
     };
     auto rel_of = [&](int row, int v, int* b, int* e) {
       *b = B->rel_ptr[(size_t)row * NVAR + v];
@@ -652,8 +680,8 @@ extern "C" int tp_build_basis(int32_t dim, int32_t p, tp_basis** out) {
     };
     B->cg_ptr.assign(1, 0);
     B->ch_ptr.assign(1, 0);
-    for (int i = 0; i < nb; ++i)
-      for (int j = i; j < nb; ++j) {
+    for (int j = 0; j < nb; ++j)
+      for (int i = 0; i <= j; ++i) {
         std::map<int, double> gm, hm;
         for (int va = 0; va < NVAR; ++va) {   // D_t X D_t^T and D_m X D_m^T
           int b0, e0, b1, e1;
@@ -719,8 +747,9 @@ extern "C" int tp_build_basis(int32_t dim, int32_t p, tp_basis** out) {
   }
   B->coef.assign((size_t)B->nb * B->nmono, 0.0);
   B->sp_ptr.assign(B->nb * C + 1, 0);
+  for (int i = 0; i < B->nb; ++i)
+    for (const Term& tm : funcs[place[i]]) B->coef[(size_t)i * B->nmono + index.at(tm.e)] = rat_to_double(tm.num, tm.den);
   for (int j = 0; j < B->nb; ++j) {
-    for (const Term& tm : funcs[j]) B->coef[(size_t)j * B->nmono + index.at(tm.e)] = rat_to_double(tm.num, tm.den);
     for (int comp = 0; comp < C; ++comp) {
       for (const Term& tm : funcs[j]) {
         int var = comp - 1;   // -1: U, 0: t, 1..n: x_m

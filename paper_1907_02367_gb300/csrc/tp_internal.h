@@ -96,11 +96,13 @@ struct tp_tents {
 };
 
 struct tp_basis {
-  int dim = 0, p = 0, nb = 0, nmono = 0;
+  // functions in the order of the tables below: first the nl of degree <= p - 1
+  // (derivatives of U^p lie in their span), then those of degree p
+  int dim = 0, p = 0, nb = 0, nl = 0, nmono = 0;
   std::vector<int32_t> exps;        // nmono * (dim+1): exponents of (that, xhat_1..n)
   std::vector<int32_t> parent;      // monomial g = monomial parent[g] * variable var[g] (g >= 1)
   std::vector<int32_t> var;
-  std::vector<double> coef;         // nb * nmono, U
+  std::vector<double> coef;         // nb * nmono, U, in the exported order (type, degree of the initial polynomial)
   // sparse evaluation table: for basis j and component comp in
   // {U, d/dthat, d/dxhat_1..n}: entries [ptr[j*C+comp], ptr[j*C+comp+1])
   std::vector<int32_t> sp_ptr, sp_mono;
@@ -113,7 +115,8 @@ struct tp_basis {
   std::vector<int32_t> relT_ptr, relT_dst;
   std::vector<double> relT_fac;
   // congruences of the top-face form, merged per entry (i <= j, packed order
-  // p = i nb - i (i - 1) / 2 + j - i):
+  // p = j (j + 1) / 2 + i, so that the pairs of functions < nl come first; no
+  // other pair is referenced by a congruence):
   //   (D_t X D_t^T + sum_m D_m X D_m^T)_ij = sum over [cg_ptr[p], cg_ptr[p+1]) of cg_coef * X[cg_idx]
   //   (sum_m D_m H_m D_t^T + D_t H_m D_m^T)_ij = sum over [ch_ptr[p], ch_ptr[p+1]) of
   //       ch_coef * H_{m}[ch_idx & 0xffff], m = ch_idx >> 16

@@ -20,6 +20,7 @@ namespace tp {
 constexpr int kThreads = 256;      // of a CTA where two share an SM
 constexpr int kThreadsWide = 512;  // where one CTA fills the SM's shared memory (16 warps hide more latency than 8)
 constexpr int kMaxPairs = 768;   // Gram pairs nb (nb+1)/2 (dim U^p <= 38)
+constexpr int kMaxLowPairs = 384;   // the same of the functions of degree <= p - 1 (at most 25: 2D p = 5)
 constexpr int kMaxRefine = 40;   // refinement steps of the mixed path
 constexpr long long kMaxSpin = 1LL << 20;   // bounded dependency wait: 2^20 polls (well under a second), then TP_ERR_TIMEOUT
 
@@ -45,7 +46,10 @@ struct RuleTab {
 
 struct KArgs {
   int geo[Geo::COUNT];
-  int nb, nmono, Q, nrhs, CH, mono_stride, ngmax;
+  // nl: the functions of degree <= p - 1, first in the order; every derivative
+  // lies in their span, so sums that meet the solution through v or sigma alone
+  // (their moments and values, the Grams of the derivative terms) run over them
+  int nb, nl, nmono, Q, nrhs, CH, mono_stride, ngmax;
   int ustride;                    // row stride of the U-values of a point in shared memory (nb rounded up to odd)
   // right-hand sides split over the cluster: CTA r of a tent's cluster owns
   // right-hand sides [r nrhs, (r + 1) nrhs) of the group (nrhs = per CTA) for
@@ -59,6 +63,7 @@ struct KArgs {
   int ev_ncls;
   int ev_off[kMaxEvCls + 1];
   int ev_terms[kMaxEvCls];
+  int ev_loff[kMaxEvCls + 1];     // the same counting functions < nl only (first in each class)
   const int* ev_order;
   int64_t ne, n_bnd;
   double alpha, beta;
@@ -400,15 +405,17 @@ __device__ __forceinline__ dd Ar<dd>::coef(const KArgs& a, int e) {
 // Monomials go to m[q * mono_stride], U-values to u[q * nb].  Callers write pt
 // before the call; the first and last statements that touch shared memory
 // are separated from them by barriers.
-template <int DIM, typename T, bool SCALE = true>
+// LOW: only the functions < nl (degree <= p - 1)
+template <int DIM, typename T, bool SCALE = true, bool LOW = false>
 __device__ __forceinline__ void eval_uvalues_block(const KArgs& a, int npt, const T* pt, T* m, T* u) {
   // Each thread takes one monomial (one basis function) at four points, so
   // that four independent products are in flight per table lookup.
-  const int tid = threadIdx.x, ms = a.mono_stride, nb = a.nb;
+  const int tid = threadIdx.x, ms = a.mono_stride, nfn = LOW ? a.nl : a.nb;
+  const int* const off = LOW ? a.ev_loff : a.ev_off;
   const int nq4 = (npt + 3) >> 2;
   // the constant monomial carries the scale, so every monomial and U-value is scaled
   for (int q = tid; q < npt; q += blockDim.x) m[q * ms] = SCALE ? pt[q * (DIM + 2) + DIM + 1] : Ar<T>::one();
-  for (int d = 1; d <= a.p; ++d) {
+  for (int d = 1; d <= (LOW ? a.p - 1 : a.p); ++d) {
     __syncthreads();   // pt, and the monomials of degree d - 1
     const int g0 = a.mono_lv[d], cnt = a.mono_lv[d + 1] - g0;
     for (int id = tid; id < cnt * nq4; id += blockDim.x) {
@@ -425,11 +432,11 @@ __device__ __forceinline__ void eval_uvalues_block(const KArgs& a, int npt, cons
   __syncthreads();
   // items (function, four points) class after class, so that the lanes of a
   // warp run loops of one length; a one-term function of coefficient 1 is a copy
-  for (int id = tid; id < nb * nq4; id += blockDim.x) {
+  for (int id = tid; id < nfn * nq4; id += blockDim.x) {
     int c = 0;
-    while (id >= a.ev_off[c + 1] * nq4) ++c;
-    const int f0 = a.ev_off[c], nj = a.ev_off[c + 1] - f0, loc = id - f0 * nq4;
-    const int j = __ldg(a.ev_order + f0 + loc % nj), q0 = (loc / nj) << 2;
+    while (id >= off[c + 1] * nq4) ++c;
+    const int nj = off[c + 1] - off[c], loc = id - off[c] * nq4;
+    const int j = __ldg(a.ev_order + a.ev_off[c] + loc % nj), q0 = (loc / nj) << 2;
     const int e0 = __ldg(a.sp_ptr + j * (DIM + 2)), e1 = __ldg(a.sp_ptr + j * (DIM + 2) + 1);
     int qq[4];
     T acc[4];
@@ -501,10 +508,10 @@ __device__ __forceinline__ dd shfl_xor_t(dd v, int o) {
   return {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
 }
 
-// packed upper-triangle index of (i, j), i, j < nb
-__device__ __forceinline__ int pair_index(int i, int j, int nb) {
+// packed index of (i, j), in the order of tp_basis
+__device__ __forceinline__ int pair_index(int i, int j) {
   const int lo = min(i, j), hi = max(i, j);
-  return lo * nb - lo * (lo - 1) / 2 + (hi - lo);
+  return hi * (hi + 1) / 2 + lo;
 }
 
 // (D_var y)_i for a vector y
@@ -621,6 +628,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   static_assert(!TC || (MIXED && !ADJ && SPLIT), "tensor-core contractions: mixed forward sweep, split right-hand sides");
   constexpr int NT = WIDE ? kThreadsWide : kThreads, NW = NT / 32;   // threads and warps of a CTA
   constexpr int kMaxPair = (kMaxPairs + NT - 1) / NT;            // Gram pairs per thread
+  constexpr int kMaxLow = (kMaxLowPairs + NT - 1) / NT;          // of functions < nl
   using T = typename std::conditional<MIXED, dd, double>::type;
   using R = Ar<T>;
   constexpr int NV = DIM + 1;   // vertices per element
@@ -719,26 +727,26 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   } else {
     tent = tent0 + blockIdx.x / CS;
   }
-  const int nb = a.nb, Q = a.Q, nrhs = a.nrhs, CH = a.CH, NG = a.ngmax;
+  const int nb = a.nb, nl = a.nl, Q = a.Q, nrhs = a.nrhs, CH = a.CH, NG = a.ngmax;
   const int us = a.ustride;   // row stride of the U-values in shared memory (odd: no bank conflicts between points)
   // this CTA's right-hand sides (all of the group unless they are split over the cluster)
   constexpr bool rsplit = SPLIT;
   double* const front = a.front + (rsplit ? (size_t)rank * nrhs * a.ne * Q * C : 0);
   const double* const gD = a.gD != nullptr ? a.gD + (rsplit ? (size_t)rank * nrhs * a.n_bnd : 0) : nullptr;
-  const int npair = nb * (nb + 1) / 2;
+  const int npair = nb * (nb + 1) / 2, npl = nl * (nl + 1) / 2;
   const int nmom = nrhs * C * nb;
   T* sA = reinterpret_cast<T*>(sm);                  // N*N        assembled A, then LU factors
   T* sb = reinterpret_cast<T*>(sm + a.off_b);        // nrhs*N     assembled b, then x
-  T* sPG = reinterpret_cast<T*>(sm + a.off_pg);      // NG*npair   this CTA: G (top) per group
-  T* sPH = reinterpret_cast<T*>(sm + a.off_ph);      // NG*DIM*npair  H_m
+  T* sPG = reinterpret_cast<T*>(sm + a.off_pg);      // NG*npl     this CTA: G (top) per group
+  T* sPH = reinterpret_cast<T*>(sm + a.off_ph);      // NG*DIM*npl    H_m
   T* sPGb = reinterpret_cast<T*>(sm + a.off_pgb);    // NG*npair   G (bottom, recovery)
   T* sPM = reinterpret_cast<T*>(sm + a.off_pm);      // NG*nmom    moments (gamma, alpha, beta_m) per rhs, this CTA
   T* sSG = sPG;                                      // the same summed over the cluster, in place
   T* sSM = reinterpret_cast<T*>(sm + a.off_sm);      // NG*nmom    summed moments (in place of sPM)
-  T* sF = reinterpret_cast<T*>(sm + a.off_f);        // npair      facet Gram (+ side)
-  T* sF2 = reinterpret_cast<T*>(sm + a.off_f2);      // npair      facet Gram (- side)
-  T* sFpm = reinterpret_cast<T*>(sm + a.off_fpm);    // nb*nb      facet Gram (+ test, - trial)
-  T* sDel = reinterpret_cast<T*>(sm + a.off_del);    // nrhs*nb    facet moments delta
+  T* sF = reinterpret_cast<T*>(sm + a.off_f);        // npl        facet Gram (+ side)
+  T* sF2 = reinterpret_cast<T*>(sm + a.off_f2);      // npl        facet Gram (- side)
+  T* sFpm = reinterpret_cast<T*>(sm + a.off_fpm);    // nl*nl      facet Gram (+ test, - trial)
+  T* sDel = reinterpret_cast<T*>(sm + a.off_del);    // nrhs*nl    facet moments delta
   T* sU = reinterpret_cast<T*>(sm + a.off_u);        // 2*CH*nb    U-values (scaled) per (side, point)
   T* sPt = reinterpret_cast<T*>(sm + a.off_pt);      // 2*CH*(DIM+2)  (that, xhat, scale) per point
   T* sM = reinterpret_cast<T*>(sm + a.off_mono);     // 2*CH*mono_stride
@@ -977,25 +985,37 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   // moments of the data of the points base .. base + nq - 1 whose U-values are
   // the rows of U, per material (whose elements, of QE points each, are
   // consecutive): one (material, right-hand side, basis function) per group of
-  // ps lanes with its C components as independent sums; the lanes of a group
-  // take every ps-th point and are added by butterfly shuffles (a fixed order)
+  // ps lanes with its C components as independent sums (functions < nl, first)
+  // or gamma alone (the others: alpha and beta are only applied through
+  // derivatives); the lanes of a group take every ps-th point and are added by
+  // butterfly shuffles (a fixed order)
   auto data_moments = [&](int base, int nq, const T* U, int QE) {
-    const int nitem = ng * nrhs * nb;
+    // (the two kinds start at a warp each)
+    const int nlow = ng * nrhs * nl, nhigh = ng * nrhs * (nb - nl);
+    auto high0 = [&](int ps_) { return (nlow * ps_ + 31) & ~31; };
     int ps = 1;
-    while (ps < 8 && nitem * ps * 2 <= NT) ps *= 2;
-    for (int id0 = 0; id0 < nitem * ps; id0 += blockDim.x) {
-      const int id = id0 + tid, item = id / ps, part = id % ps;
-      const int g = item / (nrhs * nb), rest = item % (nrhs * nb), r = rest / nb, i = rest % nb;
+    while (ps < 8 && high0(2 * ps) + nhigh * ps * 2 <= NT) ps *= 2;
+    const int h0_ = high0(ps), nitem = h0_ + nhigh * ps;
+    for (int id0 = 0; id0 < nitem; id0 += blockDim.x) {
+      const int id = id0 + tid;
+      const bool low = id < h0_, live = low ? id < nlow * ps : id < nitem;
+      const int it = (low ? id : id - h0_) / ps, part = (low ? id : id - h0_) % ps, nf = low ? nl : nb - nl;
+      const int g = it / (nrhs * nf), rest = it % (nrhs * nf), r = rest / nf, i = rest % nf + (low ? 0 : nl);
       T t[C];
 #pragma unroll
       for (int cc = 0; cc < C; ++cc) t[cc] = R::zero();
-      if (item < nitem) {
+      if (live) {
         const int l0 = max(0, s_ge0[g] * QE - base), l1 = min(nq, s_ge0[g + 1] * QE - base);
         const T* cb = sCB + (size_t)r * C * cbs;
-        for (int ql = l0 + part; ql < l1; ql += ps) {
-          const T u = U[(size_t)ql * us + i];
+        if (low) {
+          for (int ql = l0 + part; ql < l1; ql += ps) {
+            const T u = U[(size_t)ql * us + i];
 #pragma unroll
-          for (int cc = 0; cc < C; ++cc) t[cc] = R::acc(t[cc], cb[cc * cbs + ql], u);
+            for (int cc = 0; cc < C; ++cc) t[cc] = R::acc(t[cc], cb[cc * cbs + ql], u);
+          }
+        } else {
+#pragma unroll 4
+          for (int ql = l0 + part; ql < l1; ql += ps) t[0] = R::acc(t[0], cb[ql], U[(size_t)ql * us + i]);
         }
       }
 #pragma unroll
@@ -1003,10 +1023,11 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       for (int o = 1; o < ps; o <<= 1)
 #pragma unroll
         for (int cc = 0; cc < C; ++cc) t[cc] = R::add(t[cc], shfl_xor_t(t[cc], o));
-      if (part == 0 && item < nitem) {
+      if (part == 0 && live) {
         T* M = sPM + (size_t)g * nmom + (size_t)r * C * nb + i;
 #pragma unroll
-        for (int cc = 0; cc < C; ++cc) M[cc * nb] = R::add(M[cc * nb], t[cc]);
+        for (int cc = 0; cc < C; ++cc)
+          if (cc == 0 || low) M[cc * nb] = R::add(M[cc * nb], t[cc]);
       }
     }
   };
@@ -1165,7 +1186,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   const bool pblk = nif > 0 || nneu > 0;
   T* sFD = reinterpret_cast<T*>(sm + a.off_pd);      // Dirichlet sums (Grams, then data moments), then Neumann data
   T* sDD = reinterpret_cast<T*>(sm + a.off_dd);
-  const int nfg = nfac > 0 ? ng * (DIM + 1) * npair : 0, nfm = nfac > 0 ? ng * (DIM + 1) * nrhs * nb : 0;
+  const int nfg = nfac > 0 ? ng * (DIM + 1) * npl : 0, nfm = nfac > 0 ? ng * (DIM + 1) * nrhs * nl : 0;
   T* sPBN = sDD + nfm;
   unsigned gdir = 0;   // materials with Dirichlet facets
   for (int f = 0; f < nfac; ++f) gdir |= 1u << s_fg[f];
@@ -1276,24 +1297,30 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
     // sqrt(w) = sqrt(w_ref) sqrt(n! volume) at the facet's points
     s_fsq[f] = sqrt(sqrt(fabs(small_det<DIM>(G))));
   }
-  // Gram pairs owned by this thread (upper triangle, i <= j, row-major order)
-  int pi[kMaxPair], pj[kMaxPair];
-  T aK[kMaxPair], aG[kMaxPair], aH[kMaxPair][DIM], aB[kMaxPair];
+  // Gram pairs owned by this thread: the bottom face's (every function, the
+  // recovery term) from the first thread on, the top face's and the facets'
+  // (functions < nl: they enter through derivatives) from the last thread down,
+  // so that threads without a second pair of the one take the other.  (With
+  // every pair on both faces and the derivative moments over every function:
+  // 3D p = 3, 64 columns binary64, 217 ms a sweep of 3710 tents)
+  int pi[kMaxPair], pj[kMaxPair], li[kMaxLow], lj[kMaxLow];
+  T aK[kMaxLow], aG[kMaxLow], aH[kMaxLow][DIM], aB[kMaxPair];
+  auto unpack = [](int id, int n, int& i, int& j) {
+    i = id;
+    j = 0;
+    if (id >= n) i = 0;
+    else
+      while (i > j) i -= ++j;
+  };
 #pragma unroll
   for (int s = 0; s < kMaxPair; ++s) {
-    const int id = tid + s * NT;
-    int i = 0, j = 0;
-    if (id < npair) {
-      int rem = id;
-      while (rem >= nb - i) {
-        rem -= nb - i;
-        ++i;
-      }
-      j = i + rem;
-    }
-    pi[s] = i;
-    pj[s] = j;
-    aK[s] = aG[s] = aB[s] = R::zero();
+    unpack(tid + s * NT, npair, pi[s], pj[s]);
+    aB[s] = R::zero();
+  }
+#pragma unroll
+  for (int s = 0; s < kMaxLow; ++s) {
+    unpack(NT - 1 - tid + s * NT, npl, li[s], lj[s]);
+    aK[s] = aG[s] = R::zero();
 #pragma unroll
     for (int d = 0; d < DIM; ++d) aH[s][d] = R::zero();
   }
@@ -1307,8 +1334,8 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   // region of the Dirichlet sums)
   // Dirichlet facets, per material g, after the interface blocks: the facet
   // Grams summed over g's facets, G_g, and weighted by the facets' normals,
-  // Gn_g[d] = sum_f n_f[d] F_f (layout [G_g | Gn_g[0..DIM)] of npair each),
-  // then the data moments in the same arrangement (nrhs*nb each).  The
+  // Gn_g[d] = sum_f n_f[d] F_f (layout [G_g | Gn_g[0..DIM)] of npl each),
+  // then the data moments in the same arrangement (nrhs*nl each).  The
   // congruences with the derivative maps are linear, so these sums carry all
   // a tent needs; they are formed after the cluster reduction.
   // Interface and Neumann facets add their blocks to this CTA's partial A
@@ -1320,9 +1347,9 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
     for (int id = tid; id < nfm; id += blockDim.x) sDD[id] = R::zero();
     if (nneu > 0)
       for (int id = tid; id < nrhs * N; id += blockDim.x) sPBN[id] = R::zero();
-    for (int id = tid; id < nrhs * nb; id += blockDim.x) sDel[id] = R::zero();
+    for (int id = tid; id < nrhs * nl; id += blockDim.x) sDel[id] = R::zero();
     if (nif > 0)
-      for (int id = tid; id < nb * nb; id += blockDim.x) sFpm[id] = R::zero();
+      for (int id = tid; id < nl * nl; id += blockDim.x) sFpm[id] = R::zero();
     __syncthreads();
     // (a) Dirichlet facets: the points of all of them (facet after facet) in
     // one pass, split over the cluster; a facet's Gram and moments are folded
@@ -1333,28 +1360,28 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       // the Grams take this CTA's slice [d0, d1); the data moments of split
       // right-hand sides take every point
       const int l0 = rsplit ? 0 : d0, l1 = rsplit ? NPD : d1;
-      T aF[kMaxPair];
+      T aF[kMaxLow];
 #pragma unroll
-      for (int s = 0; s < kMaxPair; ++s) aF[s] = R::zero();
+      for (int s = 0; s < kMaxLow; ++s) aF[s] = R::zero();
       auto fold_gram = [&](int f) {
         if (f >= nfac) return;
-        T* Fg = sFD + (size_t)s_fg[f] * (DIM + 1) * npair;
+        T* Fg = sFD + (size_t)s_fg[f] * (DIM + 1) * npl;
 #pragma unroll
-        for (int s = 0; s < kMaxPair; ++s)
-          if (tid + s * NT < npair) {
-            const int q = tid + s * NT;
+        for (int s = 0; s < kMaxLow; ++s)
+          if (NT - 1 - tid + s * NT < npl) {
+            const int q = NT - 1 - tid + s * NT;
             Fg[q] = R::add(Fg[q], aF[s]);
             for (int d = 0; d < DIM; ++d)
-              Fg[(1 + d) * npair + q] = R::fma(R::from(s_fn[f][d]), aF[s], Fg[(1 + d) * npair + q]);
+              Fg[(1 + d) * npl + q] = R::fma(R::from(s_fn[f][d]), aF[s], Fg[(1 + d) * npl + q]);
             aF[s] = R::zero();
           }
       };
       auto fold_mom = [&](int f, int id, T t) {
         if (f >= nfac) return;
-        T* Dg = sDD + (size_t)s_fg[f] * (DIM + 1) * nrhs * nb;
+        T* Dg = sDD + (size_t)s_fg[f] * (DIM + 1) * nrhs * nl;
         Dg[id] = R::add(Dg[id], t);
         for (int d = 0; d < DIM; ++d)
-          Dg[(1 + d) * nrhs * nb + id] = R::fma(R::from(s_fn[f][d]), t, Dg[(1 + d) * nrhs * nb + id]);
+          Dg[(1 + d) * nrhs * nl + id] = R::fma(R::from(s_fn[f][d]), t, Dg[(1 + d) * nrhs * nl + id]);
       };
       int fc = l0 / Q;   // facet of the points being accumulated (uniform over the CTA)
       for (int base = l0; base < l1; base += CH) {
@@ -1377,18 +1404,18 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
           for (int r = 0; r < nrhs; ++r)
             sGd[id * nrhs + r] = R::from((!ADJ && gD != nullptr) ? sw * gD[(long long)r * a.n_bnd + goff] : 0.0);
         }
-        eval_uvalues_block<DIM, T>(a, nq, sPt, sM, sU);
+        eval_uvalues_block<DIM, T, true, true>(a, nq, sPt, sM, sU);
         const int fc0 = fc;
         for (int ql = 0; ql < nq; ++ql) {
           if (base + ql >= (fc + 1) * Q) fold_gram(fc++);
           if (base + ql < d0 || base + ql >= d1) continue;   // another CTA's Gram points
           const T* u = sU + (size_t)ql * us;
 #pragma unroll
-          for (int s = 0; s < kMaxPair; ++s)
-            if (tid + s * NT < npair) aF[s] = R::fma(u[pi[s]], u[pj[s]], aF[s]);
+          for (int s = 0; s < kMaxLow; ++s)
+            if (NT - 1 - tid + s * NT < npl) aF[s] = R::fma(u[li[s]], u[lj[s]], aF[s]);
         }
-        for (int id = tid; id < nrhs * nb; id += blockDim.x) {
-          const int r = id / nb, i = id % nb;
+        for (int id = tid; id < nrhs * nl; id += blockDim.x) {
+          const int r = id / nl, i = id % nl;
           int f = fc0;
           T t = sDel[id];
           for (int ql = 0; ql < nq; ++ql) {
@@ -1403,7 +1430,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
         __syncthreads();
       }
       fold_gram(fc);
-      for (int id = tid; id < nrhs * nb; id += blockDim.x) {
+      for (int id = tid; id < nrhs * nl; id += blockDim.x) {
         fold_mom(fc, id, sDel[id]);
         sDel[id] = R::zero();
       }
@@ -1422,9 +1449,9 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       const bool neu = NEU && f >= nfac + nif;
       const int gp = s_fg[f], gm = s_fg2[f];
       const double cp = s_gc[gp], cm = s_gc[gm];
-      T aF[kMaxPair], aF2[kMaxPair];
+      T aF[kMaxLow], aF2[kMaxLow];
 #pragma unroll
-      for (int s = 0; s < kMaxPair; ++s) aF[s] = aF2[s] = R::zero();
+      for (int s = 0; s < kMaxLow; ++s) aF[s] = aF2[s] = R::zero();
       // (a Neumann facet's data moments of split right-hand sides take every point)
       const int l0 = (rsplit && neu) ? 0 : f0, l1 = (rsplit && neu) ? Q : f1;
       for (int base = l0; base < l1; base += CH) {
@@ -1455,28 +1482,28 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
           }
         }
         if (!neu) __syncthreads();   // (the - side's rows are read by other threads than wrote them)
-        eval_uvalues_block<DIM, T>(a, npt, sPt, sM, sU);
+        eval_uvalues_block<DIM, T, true, true>(a, npt, sPt, sM, sU);
         for (int ql = 0; ql < nq; ++ql) {
           if (base + ql < f0 || base + ql >= f1) continue;   // another CTA's Gram points
           const T* u = sU + (size_t)ql * us;
           const T* u2 = sU + (size_t)(nq + ql) * us;
 #pragma unroll
-          for (int s = 0; s < kMaxPair; ++s)
-            if (tid + s * NT < npair) {
-              aF[s] = R::fma(u[pi[s]], u[pj[s]], aF[s]);
-              if (!neu) aF2[s] = R::fma(u2[pi[s]], u2[pj[s]], aF2[s]);
+          for (int s = 0; s < kMaxLow; ++s)
+            if (NT - 1 - tid + s * NT < npl) {
+              aF[s] = R::fma(u[li[s]], u[lj[s]], aF[s]);
+              if (!neu) aF2[s] = R::fma(u2[li[s]], u2[lj[s]], aF2[s]);
             }
         }
         if (neu) {
-          for (int id = tid; id < nrhs * nb; id += blockDim.x) {
-            const int r = id / nb, i = id % nb;
+          for (int id = tid; id < nrhs * nl; id += blockDim.x) {
+            const int r = id / nl, i = id % nl;
             T t = sDel[id];
             for (int ql = 0; ql < nq; ++ql) t = R::fma(sGd[ql * nrhs + r], sU[(size_t)ql * us + i], t);
             sDel[id] = t;
           }
         } else {
-          for (int id = tid; id < nb * nb; id += blockDim.x) {
-            const int i = id / nb, j = id % nb;
+          for (int id = tid; id < nl * nl; id += blockDim.x) {
+            const int i = id / nl, j = id % nl;
             T t = sFpm[id];
             for (int ql = 0; ql < nq; ++ql) t = R::fma(sU[(size_t)ql * us + i], sU[(size_t)(nq + ql) * us + j], t);
             sFpm[id] = t;
@@ -1485,10 +1512,10 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
         __syncthreads();
       }
 #pragma unroll
-      for (int s = 0; s < kMaxPair; ++s)
-        if (tid + s * NT < npair) {
-          sF[tid + s * NT] = aF[s];
-          sF2[tid + s * NT] = aF2[s];
+      for (int s = 0; s < kMaxLow; ++s)
+        if (NT - 1 - tid + s * NT < npl) {
+          sF[NT - 1 - tid + s * NT] = aF[s];
+          sF2[NT - 1 - tid + s * NT] = aF2[s];
         }
       __syncthreads();
       T nrm[DIM];
@@ -1500,8 +1527,8 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       // (2D p = 5: a facet's four blocks 80 us before)
       auto facet_block = [&](auto mode, const T* X, T w1t, T w1n, T w2t, T w2n, int gr, int gcl) {
         constexpr int MODE = decltype(mode)::value;
-        T *Y1 = sFpm + nb * nb, *Y2 = Y1 + nb * nb;
-        for (int id = tid; id < nb * nb; id += blockDim.x) {
+        T *Y1 = sFpm + nl * nl, *Y2 = Y1 + nl * nb;
+        for (int id = tid; id < nl * nb; id += blockDim.x) {
           const int k = id / nb, jj = id - k * nb;
           T dt = R::zero(), dn = R::zero();
 #pragma unroll
@@ -1509,7 +1536,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
             T t = R::zero();
             for (int e = __ldg(a.rel_ptr + jj * NV + v_), e1_ = __ldg(a.rel_ptr + jj * NV + v_ + 1); e < e1_; ++e) {
               const int sj = __ldg(a.rel_src + e);
-              const T x = MODE == 0 ? X[pair_index(k, sj, nb)] : MODE == 1 ? X[k * nb + sj] : X[sj * nb + k];
+              const T x = MODE == 0 ? X[pair_index(k, sj)] : MODE == 1 ? X[k * nl + sj] : X[sj * nl + k];
               t = Fac<T>::add(t, x, a.rel_facf, a.rel_fac, e);
             }
             if (v_ == 0) dt = t;
@@ -1541,7 +1568,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
                     gp);
         for (int id = tid; id < nrhs * nb; id += blockDim.x) {
           const int r = id / nb, i = id % nb;
-          const T* del = sDel + (size_t)r * nb;
+          const T* del = sDel + (size_t)r * nl;
           T dn = R::zero();
           for (int d = 0; d < DIM; ++d) dn = R::fma(nrm[d], rel_apply<DIM, T>(a, i, 1 + d, del), dn);
           const T t = R::fma(R::from(-a.beta * ih), dn, R::mul(R::from(-cp * ih), rel_apply<DIM, T>(a, i, 0, del)));
@@ -1549,7 +1576,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
           *dst = R::add(*dst, t);
         }
         __syncthreads();
-        for (int id = tid; id < nrhs * nb; id += blockDim.x) sDel[id] = R::zero();
+        for (int id = tid; id < nrhs * nl; id += blockDim.x) sDel[id] = R::zero();
         __syncthreads();
         continue;
       }
@@ -1564,14 +1591,14 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
         else if (tside == 0) facet_block(std::integral_constant<int, 1>{}, sFpm, w1t, w1n, w2t, w2n, gr, gcl);
         else facet_block(std::integral_constant<int, 2>{}, sFpm, w1t, w1n, w2t, w2n, gr, gcl);
       }
-      for (int id = tid; id < nb * nb; id += blockDim.x) sFpm[id] = R::zero();
+      for (int id = tid; id < nl * nl; id += blockDim.x) sFpm[id] = R::zero();
       __syncthreads();
     }
   }
   };
   if constexpr (!SPLIT) facet_phase();
   if (!kept) {   // (the facets' Grams shared this region)
-    for (int id = tid; id < NG * (DIM + 2) * npair; id += blockDim.x) sPG[id] = R::zero();
+    for (int id = tid; id < NG * ((DIM + 1) * npl + npair); id += blockDim.x) sPG[id] = R::zero();
     if (extra || np == 0) __syncthreads();
   }
 
@@ -1583,7 +1610,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
     T g[DIM];
     for (int d = 0; d < DIM; ++d) g[d] = R::from(s_gt[k][d]);
 #pragma unroll
-    for (int s = 0; s < kMaxPair; ++s) {
+    for (int s = 0; s < kMaxLow; ++s) {
       const T k_ = R::norm(aK[s]);
       aG[s] = R::add(aG[s], k_);
 #pragma unroll
@@ -1593,18 +1620,22 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   };
   auto flush_group = [&](int g) {
 #pragma unroll
-    for (int s = 0; s < kMaxPair; ++s) {
-      const int id = tid + s * NT;
-      if (id < npair) {
-        sPG[g * npair + id] = R::add(sPG[g * npair + id], aG[s]);
+    for (int s = 0; s < kMaxLow; ++s) {
+      const int id = NT - 1 - tid + s * NT;
+      if (id < npl) {
+        sPG[g * npl + id] = R::add(sPG[g * npl + id], aG[s]);
 #pragma unroll
-        for (int d = 0; d < DIM; ++d)
-          sPH[(g * DIM + d) * npair + id] = R::add(sPH[(g * DIM + d) * npair + id], aH[s][d]);
-        sPGb[g * npair + id] = R::add(sPGb[g * npair + id], R::norm(aB[s]));
+        for (int d = 0; d < DIM; ++d) sPH[(g * DIM + d) * npl + id] = R::add(sPH[(g * DIM + d) * npl + id], aH[s][d]);
       }
-      aG[s] = aB[s] = R::zero();
+      aG[s] = R::zero();
 #pragma unroll
       for (int d = 0; d < DIM; ++d) aH[s][d] = R::zero();
+    }
+#pragma unroll
+    for (int s = 0; s < kMaxPair; ++s) {
+      const int id = tid + s * NT;
+      if (id < npair) sPGb[g * npair + id] = R::add(sPGb[g * npair + id], R::norm(aB[s]));
+      aB[s] = R::zero();
     }
   };
   // points pt .. end - 1 (rows of U-values ut at the top, ub at the bottom) added
@@ -1623,20 +1654,44 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
         kend = (k + 1) * QK;
       }
       const int n = min(end, kend) - pt;
-#pragma unroll
-      for (int s = 0; s < kMaxPair; ++s) {
-        if (tid + s * NT < npair) {
-          const T *ti = ut + pi[s], *tj = ut + pj[s], *bi = ub + pi[s], *bj = ub + pj[s];
-          T k_ = aK[s], b_ = aB[s];
+      auto pair_sum = [&](T t, const T* x, const T* y) {
 #pragma unroll 4
-          for (int q = 0; q < n; ++q) {
-            k_ = R::acc(k_, ti[q * us], tj[q * us]);
-            b_ = R::acc(b_, bi[q * us], bj[q * us]);
-          }
-          aK[s] = k_;
-          aB[s] = b_;
+        for (int q = 0; q < n; ++q) t = R::acc(t, x[q * us], y[q * us]);
+        return t;
+      };
+      // a thread's pair on either face in one loop, as independent chains
+      const bool lo0 = NT - 1 - tid < npl;
+      if (tid < npair && lo0) {
+        const T *ti = ut + li[0], *tj = ut + lj[0], *bi = ub + pi[0], *bj = ub + pj[0];
+        T k_ = aK[0], b_ = aB[0];
+#pragma unroll 4
+        for (int q = 0; q < n; ++q) {
+          k_ = R::acc(k_, ti[q * us], tj[q * us]);
+          b_ = R::acc(b_, bi[q * us], bj[q * us]);
         }
+        aK[0] = k_;
+        aB[0] = b_;
+      } else if (lo0) {
+        aK[0] = pair_sum(aK[0], ut + li[0], ut + lj[0]);
+      } else if (kMaxPair > 1 && tid + NT < npair) {
+        const T *bi = ub + pi[0], *bj = ub + pj[0], *ci = ub + pi[1 % kMaxPair], *cj = ub + pj[1 % kMaxPair];
+        T b_ = aB[0], c_ = aB[1 % kMaxPair];
+#pragma unroll 4
+        for (int q = 0; q < n; ++q) {
+          b_ = R::acc(b_, bi[q * us], bj[q * us]);
+          c_ = R::acc(c_, ci[q * us], cj[q * us]);
+        }
+        aB[0] = b_;
+        aB[1 % kMaxPair] = c_;
+      } else if (tid < npair) {
+        aB[0] = pair_sum(aB[0], ub + pi[0], ub + pj[0]);
       }
+#pragma unroll
+      for (int s = 1; s < kMaxPair; ++s)
+        if (tid + s * NT < npair && (s > 1 || lo0)) aB[s] = pair_sum(aB[s], ub + pi[s], ub + pj[s]);
+#pragma unroll
+      for (int s = 1; s < kMaxLow; ++s)
+        if (NT - 1 - tid + s * NT < npl) aK[s] = pair_sum(aK[s], ut + li[s], ut + lj[s]);
       pt += n;
       ut += (size_t)n * us;
       ub += (size_t)n * us;
@@ -1654,7 +1709,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       eval_uvalues_block<DIM, T>(a, n, sPt, sM, sKeep + (size_t)base * us);
     }
     // (the evaluation's buffer may share the Grams' region)
-    for (int id = tid; id < NG * (DIM + 2) * npair; id += blockDim.x) sPG[id] = R::zero();   // PG, PH, PGb contiguous
+    for (int id = tid; id < NG * ((DIM + 1) * npl + npair); id += blockDim.x) sPG[id] = R::zero();   // PG, PH, PGb contiguous
     __syncthreads();
     gram_points(e0 * QK, e1 * QK, ADJ ? sKI : sKeep, ADJ ? sKeep : sKI);
   } else {
@@ -1710,8 +1765,8 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
     real = true;
     if (s_bad) continue;
   }
-  // layout [G (NG*npair) | H_m (NG*DIM*npair) | Gbot (NG*npair)]; unused groups hold zeros
-  if (CS > 1) cluster_reduce(sPG, sPG, NG * (DIM + 2) * npair);
+  // layout [G (NG*npl) | H_m (NG*DIM*npl) | Gbot (NG*npair)]; unused groups hold zeros
+  if (CS > 1) cluster_reduce(sPG, sPG, NG * ((DIM + 1) * npl + npair));
   // (split right-hand sides: each CTA's moments, Dirichlet data sums and
   // Neumann partial b already cover every point for its own right-hand sides)
   // (in place: each entry is read and rewritten by the one thread that owns it)
@@ -1739,14 +1794,15 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
     // i <= j of the packed upper triangle, split over the cluster; each entry
     // is stored with its mirror (the form is symmetric, the Dirichlet and
     // interface parts already in A are not)
-    const int nent = ng * npair, ent0 = (nent * rank) / CS, ent1 = (nent * (rank + 1)) / CS;
+    // (every CS-th entry: those of the high-degree functions, last, have the most terms)
+    const int nent = ng * npair, ment = (nent - rank + CS - 1) / CS;
     if (nfac > 0) {
       // Dirichlet facets, A_D = (c/h) D_t F E^T with E = alpha (c/h) D_t - (1/h) D_n
       // summed over the material's facets, from G_g and Gn_g, added into this
       // CTA's copy of A for the entries this rank forms (each entry and its
       // mirror: one item each)
-      for (int id = tid; id < 2 * (ent1 - ent0); id += blockDim.x) {
-        const int e_ = ent0 + (id >> 1), g = e_ / npair, pp = e_ % npair;
+      for (int id = tid; id < 2 * ment; id += blockDim.x) {
+        const int e_ = rank + (id >> 1) * CS, g = e_ / npair, pp = e_ % npair;
         const int ij = __ldg(a.pair_ij + pp);
         int i = ij >> 16, j = ij & 0xffff;
         if (((id & 1) && i == j) || !((gdir >> g) & 1u)) continue;
@@ -1756,13 +1812,13 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
           j = t_;
         }
         const int e2 = i * nb + j;
-        const T* Fg = sFD + (size_t)g * (DIM + 1) * npair;
+        const T* Fg = sFD + (size_t)g * (DIM + 1) * npl;
         T a0 = R::zero(), am = R::zero();
         for (int e = __ldg(a.ft_ptr + e2), e1 = __ldg(a.ft_ptr + e2 + 1); e < e1; ++e)
           a0 = Fac<T>::acc(a0, Fg[__ldg(a.ft_idx + e)], a.ft_coef, a.ft_coefd, e);
         for (int e = __ldg(a.fm_ptr + e2), e1 = __ldg(a.fm_ptr + e2 + 1); e < e1; ++e) {
           const int c0 = __ldg(a.fm_idx + e);   // (derivative direction << 16) | pair
-          am = Fac<T>::acc(am, Fg[(size_t)(1 + (c0 >> 16)) * npair + (c0 & 0xffff)], a.fm_coef, a.fm_coefd, e);
+          am = Fac<T>::acc(am, Fg[(size_t)(1 + (c0 >> 16)) * npl + (c0 & 0xffff)], a.fm_coef, a.fm_coefd, e);
         }
         const double cf = s_gc[g];
         const T ad = R::mul(R::from(cf * ih), R::fma(mih, R::norm(am), R::mul(R::from(a.alpha * cf * ih), R::norm(a0))));
@@ -1771,12 +1827,12 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       }
       __syncthreads();
     }
-    for (int id = ent0 + tid; id < ent1; id += blockDim.x) {
+    for (int id = rank + tid * CS; id < nent; id += NT * CS) {
       const int g = id / npair, pp = id % npair;
       const int ij = __ldg(a.pair_ij + pp), i = ij >> 16, j = ij & 0xffff;
-      const T* SG = sSG + (size_t)g * npair;
-      const T* SH = sSG + (size_t)(NG + g * DIM) * npair;
-      const T* SGb = sSG + (size_t)(NG * (DIM + 1) + g) * npair;
+      const T* SG = sSG + (size_t)g * npl;
+      const T* SH = sSG + (size_t)(NG + g * DIM) * npl;
+      const T* SGb = sSG + (size_t)NG * (DIM + 1) * npl + (size_t)g * npair;
       T tg0 = R::zero(), tg1 = R::zero(), th0 = R::zero(), th1 = R::zero();
       {
         const int e0 = __ldg(a.cg_ptr + pp), e1 = __ldg(a.cg_ptr + pp + 1);
@@ -1792,12 +1848,12 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
         int e = e0;
         for (; e + 1 < e1; e += 2) {
           const int c0 = __ldg(a.ch_idx + e), c1 = __ldg(a.ch_idx + e + 1);
-          th0 = Fac<T>::acc(th0, SH[(c0 >> 16) * npair + (c0 & 0xffff)], a.ch_coef, a.ch_coefd, e);
-          th1 = Fac<T>::acc(th1, SH[(c1 >> 16) * npair + (c1 & 0xffff)], a.ch_coef, a.ch_coefd, e + 1);
+          th0 = Fac<T>::acc(th0, SH[(c0 >> 16) * npl + (c0 & 0xffff)], a.ch_coef, a.ch_coefd, e);
+          th1 = Fac<T>::acc(th1, SH[(c1 >> 16) * npl + (c1 & 0xffff)], a.ch_coef, a.ch_coefd, e + 1);
         }
         if (e < e1) {
           const int c0 = __ldg(a.ch_idx + e);
-          th0 = Fac<T>::acc(th0, SH[(c0 >> 16) * npair + (c0 & 0xffff)], a.ch_coef, a.ch_coefd, e);
+          th0 = Fac<T>::acc(th0, SH[(c0 >> 16) * npl + (c0 & 0xffff)], a.ch_coef, a.ch_coefd, e);
         }
       }
       const T t = R::fma(R::from(s_gc[g]), R::add(R::norm(th0), R::norm(th1)), R::add(R::norm(tg0), R::norm(tg1)));
@@ -2086,7 +2142,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
         // Dirichlet data: b_D = E' delta summed over g's facets,
         // E' = alpha (c/h) D_t + (1/h) D_n
         if (cc > 0 && ((gdir >> g) & 1u)) {
-          const T* Dg = sDD + (size_t)(g * (DIM + 1) + cc - 1) * nrhs * nb + (size_t)r * nb;
+          const T* Dg = sDD + (size_t)(g * (DIM + 1) + cc - 1) * nrhs * nl + (size_t)r * nl;
           t = R::fma(R::from(cc == 1 ? a.alpha * s_gc[g] * ih : ih), rel_apply<DIM, T>(a, i, cc - 1, Dg), t);
         }
       }
@@ -2386,7 +2442,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       auto fieldv = [&](int g, int r, int cc, const T* u) {   // sqrt(w) times component cc of the solution
         const T* y = sY + (size_t)g * nmom + ((size_t)r * C + cc) * nb;
         T t = R::zero();
-        for (int j = 0; j < nb; ++j) t = R::acc(t, y[j], u[j]);
+        for (int j = 0; j < (cc == 0 ? nb : nl); ++j) t = R::acc(t, y[j], u[j]);
         return R::to(R::norm(t));
       };
       // (a) bottom face: the jump to the stored front and the recovery term
@@ -2567,22 +2623,34 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       __syncthreads();
       coefs(sYxp, sYx + nb, C * nb, nmom);             // x' = y_v(x)
       __syncthreads();
-      // sqrt(w) times the C components of the field of vectors Y at U-values u
-      auto fld = [&](const T* Y, int g, int r, const T* u, double* F) {
-        for (int cc = 0; cc < C; ++cc) {
-          const T* y = Y + (size_t)g * nmom + ((size_t)r * C + cc) * nb;
-          T t = R::zero();
-          for (int j = 0; j < nb; ++j) t = R::acc(t, y[j], u[j]);
-          F[cc] = R::to(R::norm(t));
-        }
-      };
-      // fields of x and mu and their c-derivatives at a point of material g
+      // fields of x and mu and their c-derivatives at a point of material g: sqrt(w)
+      // times the C components of the vectors' fields at U-values u, all of them
+      // in one pass as independent sums (one dependent chain after the other left
+      // the binary64 pipe waiting)
       auto fields4 = [&](int g, int r, const T* u, double tq, double* Fx, double* dFx, double* Fm, double* dFm) {
         const double cg = s_gc[g];
-        fld(sYx, g, r, u, Fx);
-        fld(sYxp, g, r, u, dFx);
-        fld(sY, g, r, u, Fm);
-        fld(sYmp, g, r, u, dFm);
+        const size_t o = (size_t)g * nmom + (size_t)r * C * nb;
+        const T* const Y[4] = {sYx + o, sYxp + o, sY + o, sYmp + o};
+        double* const F[4] = {Fx, dFx, Fm, dFm};
+        T t[4][C];
+#pragma unroll
+        for (int f = 0; f < 4; ++f)
+#pragma unroll
+          for (int cc = 0; cc < C; ++cc) t[f][cc] = R::zero();
+        for (int j = 0; j < nl; ++j) {
+          const T uj = u[j];
+#pragma unroll
+          for (int f = 0; f < 4; ++f)
+#pragma unroll
+            for (int cc = 0; cc < C; ++cc) t[f][cc] = R::acc(t[f][cc], Y[f][cc * nb + j], uj);
+        }
+        for (int j = nl; j < nb; ++j)   // (U of x and mu alone: x' and mu' are derivatives)
+#pragma unroll
+          for (int f = 0; f < 4; f += 2) t[f][0] = R::acc(t[f][0], Y[f][j], u[j]);
+#pragma unroll
+        for (int f = 0; f < 4; ++f)
+#pragma unroll
+          for (int cc = 0; cc < C; ++cc) F[f][cc] = R::to(R::norm(t[f][cc]));
         for (int cc = 0; cc < C; ++cc) {
           dFx[cc] *= tq / cg;
           dFm[cc] *= tq / cg;
@@ -2889,12 +2957,13 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
         const int rc = id / (ne * S), pt = id - rc * (ne * S), k = eb + pt / S;
         const T *u = Ue + (size_t)pt * us, *y = sY + (size_t)s_grp[k] * nmom + (size_t)rc * nb;
         T t0 = R::zero(), t1 = R::zero();
+        const int nj = rc % C == 0 ? nb : nl;
         int j = 0;
-        for (; j + 1 < nb; j += 2) {
+        for (; j + 1 < nj; j += 2) {
           t0 = R::acc(t0, y[j], u[j]);
           t1 = R::acc(t1, y[j + 1], u[j + 1]);
         }
-        if (j < nb) t0 = R::acc(t0, y[j], u[j]);
+        if (j < nj) t0 = R::acc(t0, y[j], u[j]);
         sCB[(size_t)rc * cbs + pt] = R::add(R::norm(t0), R::norm(t1));
       }
       __syncthreads();
@@ -2948,7 +3017,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
           const T* u = kept ? sKeep + (size_t)(base - q0 + ql) * us : sU + (size_t)ql * us;
           const T* y = sY + (size_t)s_grp[k] * nmom + ((size_t)r * C + cc) * nb;
           T t = R::zero();
-          for (int j = 0; j < nb; ++j) t = R::acc(t, y[j], u[j]);
+          for (int j = 0; j < (cc == 0 ? nb : nl); ++j) t = R::acc(t, y[j], u[j]);
           const double val = R::to(R::norm(t));
           front[(((int64_t)r * a.ne + s_el[k]) * Q + q) * C + cc] = kept ? val * (__ldg(a.isqw + q) * s_isdet[k]) : val;
         }
@@ -2963,11 +3032,13 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
         T t[C];
 #pragma unroll
         for (int cc = 0; cc < C; ++cc) t[cc] = R::zero();
-        for (int j = 0; j < nb; ++j) {
+        for (int j = 0; j < nl; ++j) {
           const T uj = u[j];
 #pragma unroll
           for (int cc = 0; cc < C; ++cc) t[cc] = R::acc(t[cc], y[cc * nb + j], uj);
         }
+#pragma unroll 4
+        for (int j = nl; j < nb; ++j) t[0] = R::acc(t[0], y[j], u[j]);   // (v and sigma: zero coefficients)
         double* f = front + (((int64_t)r * a.ne + s_el[k]) * Q + q) * C;
         if (kept) {
           const double sc = __ldg(a.isqw + q) * s_isdet[k];
@@ -2987,7 +3058,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
         for (int cc = 0; cc < C; ++cc) {
           const T* y = sY + (size_t)s_grp[k] * nmom + ((size_t)r * C + cc) * nb;
           T t = R::zero();
-          for (int j = 0; j < nb; ++j) t = R::acc(t, y[j], u[j]);
+          for (int j = 0; j < (cc == 0 ? nb : nl); ++j) t = R::acc(t, y[j], u[j]);
           t = R::norm(t);
           sv[cc] = kept ? R::to(t) * (__ldg(a.isqw + q) * s_isdet[k]) : R::to(t);
         }
