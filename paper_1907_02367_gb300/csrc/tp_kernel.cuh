@@ -1437,16 +1437,18 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       __syncthreads();
     }
     // (b) time-like interface facets, then Neumann facets, one after the
-    // other, each facet's points split over the cluster; their blocks go into
-    // the partial A at once.  Neumann facets (eq. 4.1), with F the facet Gram
+    // other, each taken by one CTA of the cluster (its points split over the
+    // cluster repeated the congruence in every CTA: two thirds of the time of
+    // an interface tent's assembly at 2D p = 5); their blocks go into the
+    // partial A at once.  Neumann facets (eq. 4.1), with F the facet Gram
     // of U-values and delta = sum w g_N u:
     //   A_N = -(c/h^2) D_n F D_t^T + (beta/h^2) D_n F D_n^T,
     //   b_N = -(c/h) D_t delta - (beta/h) D_n delta
     // (v = (c/h) D_t u, sigma.n = -(1/h) D_n u, D_n = sum_m n_m D_m)
-    const int fsl = (Q + CS - 1) / CS;
-    const int f0 = min(Q, rank * fsl), f1 = min(Q, f0 + fsl);
     for (int f = nfac; f < nfac + nif + nneu; ++f) {
-      const bool neu = NEU && f >= nfac + nif;
+      const bool neu = NEU && f >= nfac + nif, mine = (f - nfac) % CS == rank;
+      if (!mine && !(rsplit && neu)) continue;
+      const int f0 = 0, f1 = mine ? Q : 0;
       const int gp = s_fg[f], gm = s_fg2[f];
       const double cp = s_gc[gp], cm = s_gc[gm];
       T aF[kMaxLow], aF2[kMaxLow];
@@ -1490,8 +1492,8 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
 #pragma unroll
           for (int s = 0; s < kMaxLow; ++s)
             if (NT - 1 - tid + s * NT < npl) {
-              aF[s] = R::fma(u[li[s]], u[lj[s]], aF[s]);
-              if (!neu) aF2[s] = R::fma(u2[li[s]], u2[lj[s]], aF2[s]);
+              aF[s] = R::acc(aF[s], u[li[s]], u[lj[s]]);
+              if (!neu) aF2[s] = R::acc(aF2[s], u2[li[s]], u2[lj[s]]);
             }
         }
         if (neu) {
@@ -1505,8 +1507,9 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
           for (int id = tid; id < nl * nl; id += blockDim.x) {
             const int i = id / nl, j = id % nl;
             T t = sFpm[id];
-            for (int ql = 0; ql < nq; ++ql) t = R::fma(sU[(size_t)ql * us + i], sU[(size_t)(nq + ql) * us + j], t);
-            sFpm[id] = t;
+#pragma unroll 4
+            for (int ql = 0; ql < nq; ++ql) t = R::acc(t, sU[(size_t)ql * us + i], sU[(size_t)(nq + ql) * us + j]);
+            sFpm[id] = R::norm(t);
           }
         }
         __syncthreads();
@@ -1514,8 +1517,8 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
 #pragma unroll
       for (int s = 0; s < kMaxLow; ++s)
         if (NT - 1 - tid + s * NT < npl) {
-          sF[NT - 1 - tid + s * NT] = aF[s];
-          sF2[NT - 1 - tid + s * NT] = aF2[s];
+          sF[NT - 1 - tid + s * NT] = R::norm(aF[s]);
+          sF2[NT - 1 - tid + s * NT] = R::norm(aF2[s]);
         }
       __syncthreads();
       T nrm[DIM];
@@ -1564,8 +1567,9 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       };
       const double ih2 = ih * ih;
       if (neu) {
-        facet_block(std::integral_constant<int, 0>{}, sF, R::from(-cp * ih2), R::from(a.beta * ih2), R::zero(), R::zero(), gp,
-                    gp);
+        if (mine)
+          facet_block(std::integral_constant<int, 0>{}, sF, R::from(-cp * ih2), R::from(a.beta * ih2), R::zero(), R::zero(), gp,
+                      gp);
         for (int id = tid; id < nrhs * nb; id += blockDim.x) {
           const int r = id / nb, i = id % nb;
           const T* del = sDel + (size_t)r * nl;
@@ -2624,39 +2628,36 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       coefs(sYxp, sYx + nb, C * nb, nmom);             // x' = y_v(x)
       __syncthreads();
       // fields of x and mu and their c-derivatives at a point of material g: sqrt(w)
-      // times the C components of the vectors' fields at U-values u, all of them
-      // in one pass as independent sums (one dependent chain after the other left
-      // the binary64 pipe waiting)
-      auto fields4 = [&](int g, int r, const T* u, double tq, double* Fx, double* dFx, double* Fm, double* dFm) {
-        const double cg = s_gc[g];
-        const size_t o = (size_t)g * nmom + (size_t)r * C * nb;
-        const T* const Y[4] = {sYx + o, sYxp + o, sY + o, sYmp + o};
-        double* const F[4] = {Fx, dFx, Fm, dFm};
-        T t[4][C];
+      // times the C components of the vectors' fields at U-values u.  Four
+      // neighbouring lanes take a (point, right-hand side): each forms one field,
+      // its components as independent sums, and all receive the four.  (A chunk
+      // has few points: one thread for all left one warp to a sub-partition's
+      // binary64 unit, half of the reverse sweep's time.)
+      auto fields4 = [&](bool live, int g, int r, const T* u, double tq, double* Fx, double* dFx, double* Fm, double* dFm) {
+        const int f_ = lane & 3;
+        const T* const Y = (f_ == 0 ? sYx : f_ == 1 ? sYxp : f_ == 2 ? sY : sYmp) + (size_t)g * nmom + (size_t)r * C * nb;
+        T t[C];
 #pragma unroll
-        for (int f = 0; f < 4; ++f)
+        for (int cc = 0; cc < C; ++cc) t[cc] = R::zero();
+        if (live) {
+          for (int j = 0; j < nl; ++j) {
+            const T uj = u[j];
 #pragma unroll
-          for (int cc = 0; cc < C; ++cc) t[f][cc] = R::zero();
-        for (int j = 0; j < nl; ++j) {
-          const T uj = u[j];
-#pragma unroll
-          for (int f = 0; f < 4; ++f)
-#pragma unroll
-            for (int cc = 0; cc < C; ++cc) t[f][cc] = R::acc(t[f][cc], Y[f][cc * nb + j], uj);
+            for (int cc = 0; cc < C; ++cc) t[cc] = R::acc(t[cc], Y[cc * nb + j], uj);
+          }
+          for (int j = nl; j < nb; ++j) t[0] = R::acc(t[0], Y[j], u[j]);   // (x' and mu' are derivatives: zeros)
         }
-        for (int j = nl; j < nb; ++j)   // (U of x and mu alone: x' and mu' are derivatives)
+        const double rc = s_gc[g] * s_gic2[g], sc = (f_ & 1) ? tq * rc : 1.0;   // 1 / c
 #pragma unroll
-          for (int f = 0; f < 4; f += 2) t[f][0] = R::acc(t[f][0], Y[f][j], u[j]);
-#pragma unroll
-        for (int f = 0; f < 4; ++f)
-#pragma unroll
-          for (int cc = 0; cc < C; ++cc) F[f][cc] = R::to(R::norm(t[f][cc]));
         for (int cc = 0; cc < C; ++cc) {
-          dFx[cc] *= tq / cg;
-          dFm[cc] *= tq / cg;
+          const double own = R::to(R::norm(t[cc])) * sc;
+          Fx[cc] = __shfl_sync(0xffffffffu, own, lane & 28);
+          dFx[cc] = __shfl_sync(0xffffffffu, own, (lane & 28) + 1);
+          Fm[cc] = __shfl_sync(0xffffffffu, own, (lane & 28) + 2);
+          dFm[cc] = __shfl_sync(0xffffffffu, own, (lane & 28) + 3);
         }
-        dFx[1] += Fx[1] / cg;
-        dFm[1] += Fm[1] / cg;
+        dFx[1] = ::fma(Fx[1], rc, dFx[1]);
+        dFm[1] = ::fma(Fm[1], rc, dFm[1]);
       };
       // contributions val[id], id = point * nrhs + right-hand side, added to an
       // element by one warp in a fixed order
@@ -2677,13 +2678,15 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
             map_point(sPt + id * (DIM + 2), qg / Q, qg % Q, side == 0);
           }
           eval_uvalues_block<DIM, T>(a, nq, sPt, sM, sU);
-          for (int id = tid; id < nq * nrhs; id += blockDim.x) {
+          for (int id0 = 0; id0 < nq * nrhs; id0 += NT / 4) {
+            const bool live = id0 + (tid >> 2) < nq * nrhs;
+            const int id = live ? id0 + (tid >> 2) : 0;
             const int ql = id / nrhs, r = id % nrhs, qg = base + ql, k = qg / Q, q = qg % Q, g = s_grp[k];
             double tt = 0.0;
             for (int i = 0; i < NV; ++i) tt = fma(__ldg(a.bary + q * NV + i), side == 0 ? s_tt[k][i] : s_tb[k][i], tt);
             double Fx[C], dFx[C], Fm[C], dFm[C];
-            fields4(g, r, sU + (size_t)ql * us, tt - tc, Fx, dFx, Fm, dFm);
-            const double ic2 = s_gic2[g], dic2 = -2.0 * ic2 / s_gc[g];   // c^-2 and its derivative
+            fields4(live, g, r, sU + (size_t)ql * us, tt - tc, Fx, dFx, Fm, dFm);
+            const double ic2 = s_gic2[g], dic2 = -2.0 * ic2 * (s_gc[g] * ic2);   // c^-2 and its derivative
             const double* gk = side == 0 ? s_gt[k] : s_gb[k];
             // c^-2 a_v b_v + a_s.b_s - a_v (b_s.g) - (a_s.g) b_v: the face form of eq. (4.1)
             auto Qf = [&](const double* A_, const double* B_) {
@@ -2709,7 +2712,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
               for (int cc = 0; cc < C; ++cc) fb[cc] = sw * __ldcg(f0 + cc);
               val = Qf(fb, dFm) + dic2 * fb[1] * Fm[1] + fb[0] * dFm[0] - (dFx[0] * Fm[0] + Fx[0] * dFm[0]);
             }
-            sVal[id] = val;
+            if (live && (lane & 3) == 0) sVal[id] = val;
           }
           __syncthreads();
           for (int k = base / Q + warp; k * Q < base + nq; k += NW)
@@ -2764,12 +2767,14 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
           }
           if (ifc) __syncthreads();   // (the - side's rows are read by other threads than wrote them)
           eval_uvalues_block<DIM, T>(a, ifc ? 2 * nq : nq, sPt, sM, sU);
-          for (int id = tid; id < nq * nrhs; id += blockDim.x) {
+          for (int id0 = 0; id0 < nq * nrhs; id0 += NT / 4) {
+            const bool live = id0 + (tid >> 2) < nq * nrhs, put = live && (lane & 3) == 0;
+            const int id = live ? id0 + (tid >> 2) : 0;
             const int ql = id / nrhs, r = id % nrhs, q = base + ql;
             double tt = 0.0;
             for (int i = 0; i < NV; ++i) tt = fma(__ldg(a.bary + q * NV + i), s_fP[f][i][DIM], tt);
             double Fx[C], dFx[C], Fm[C], dFm[C];
-            fields4(gp, r, sU + (size_t)ql * us, tt - tc, Fx, dFx, Fm, dFm);
+            fields4(live, gp, r, sU + (size_t)ql * us, tt - tc, Fx, dFx, Fm, dFm);
             auto sn = [&](const double* F_) {
               double t_ = 0.0;
               for (int d = 0; d < DIM; ++d) t_ = fma(s_fn[f][d], F_[2 + d], t_);
@@ -2777,7 +2782,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
             };
             if (ifc) {
               double Gx[C], dGx[C], Gm[C], dGm[C], Z[C];
-              fields4(gm, r, sU + (size_t)(nq + ql) * us, tt - tc, Gx, dGx, Gm, dGm);
+              fields4(live, gm, r, sU + (size_t)(nq + ql) * us, tt - tc, Gx, dGx, Gm, dGm);
               for (int cc = 0; cc < C; ++cc) Z[cc] = 0.0;
               // the interface form of eq. (2.5) with trial fields X+-, test fields M+-
               auto I = [&](const double* Xp, const double* Xm, const double* Mp, const double* Mm) {
@@ -2785,8 +2790,11 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
                 return 0.5 * (jm * (Xp[1] + Xm[1]) + dv * (sn(Xp) + sn(Xm))) + a.alpha * dv * (Xp[1] - Xm[1]) +
                        a.beta * jm * (sn(Xp) - sn(Xm));
               };
-              sVal[id] = -(I(dFx, Z, Fm, Gm) + I(Fx, Gx, dFm, Z));
-              sVal[nq * nrhs + id] = -(I(Z, dGx, Fm, Gm) + I(Fx, Gx, Z, dGm));
+              const double vp = -(I(dFx, Z, Fm, Gm) + I(Fx, Gx, dFm, Z)), vm = -(I(Z, dGx, Fm, Gm) + I(Fx, Gx, Z, dGm));
+              if (put) {
+                sVal[id] = vp;
+                sVal[nq * nrhs + id] = vm;
+              }
             } else {
               const double gv = sGdd[id];
               double val;
@@ -2797,7 +2805,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
                 val = gv * (a.alpha * dFm[1] - sn(dFm)) -
                       ((sn(dFx) + a.alpha * dFx[1]) * Fm[1] + (sn(Fx) + a.alpha * Fx[1]) * dFm[1]);
               }
-              sVal[id] = val;
+              if (put) sVal[id] = val;
             }
           }
           __syncthreads();
