@@ -94,7 +94,7 @@ typedef struct tp_params {
   /* rhs_split: how a tent's right-hand sides are shared out over the CTAs of
    * its cluster.  0 = automatic (split when each CTA keeps 16 or more,
    * i.e. nrhs >= 32 and divisible by 2, 4 or 8; binary64 then splits down to
-   * 8 per CTA), 1 = never split
+   * 4 per CTA), 1 = never split
    * (every CTA takes a slice of the points for all right-hand sides), 2, 4
    * or 8 = that many CTAs, each owning nrhs / rhs_split of the right-hand
    * sides at every point of the tent (data moments, solve and outflow),

@@ -1167,13 +1167,14 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     rs = 1;
     for (int r : {8, 4, 2})
       if (rs == 1 && ctx->nrhs % r == 0 && ctx->nrhs / r >= 16) rs = r;
-    // binary64: down to 8 per CTA.  Its moments and outflow are bound by an SM's
+    // binary64: down to 4 per CTA.  Its moments and outflow are bound by an SM's
     // binary64 unit, on small meshes along the chain of dependent tents, where
     // more CTAs per tent shorten it; the U-values that each repeats cost little
     // beside them (3D p = 3, 64 right-hand sides, 4 -> 8 CTAs: 750 elements 218 ->
-    // 132 ms, 6000 elements 271 -> 268 ms).  The mixed path's tensor-core tiles
+    // 132 ms, 6000 elements 271 -> 268 ms; 32, 2 -> 8 CTAs: 150 -> 57, 3072
+    // elements 128 -> 67 ms).  The mixed path's tensor-core tiles
     // want 16 (67 -> 122 ms with 8)
-    while (!ctx->mixed && rs > 1 && rs < 8 && ctx->nrhs % (2 * rs) == 0 && ctx->nrhs / (2 * rs) >= 8) rs *= 2;
+    while (!ctx->mixed && rs > 1 && rs < 8 && ctx->nrhs % (2 * rs) == 0 && ctx->nrhs / (2 * rs) >= 4) rs *= 2;
   }
   if (!(rs == 1 || rs == 2 || rs == 4 || rs == 8) || ctx->nrhs % rs != 0) {
     tp::set_error("tp_create: rhs_split must be 0, 1, 2, 4 or 8 and divide nrhs");

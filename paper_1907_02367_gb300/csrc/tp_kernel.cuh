@@ -621,7 +621,7 @@ __device__ __forceinline__ double recip(double x) {
 // matrix depends on the front times alone, which the tents fix, so the
 // geometry, the U-values, A and its inverse come before the wait: the chain
 // keeps the moments, b, the solve and the outflow.  2D p = 4, 968 triangles,
-// one column: 18.5 -> 10.4 ms binary64, 26.9 -> 8.6 ms mixed (with the S-point
+// one column: 18.5 -> 9.4 ms binary64, 27.0 -> 8.0 ms mixed (with the S-point
 // rule and the float-float inverse below).
 template <int DIM, bool MIXED, bool ADJ, bool PERSIST, bool NEU, bool SPLIT, bool TC, bool WIDE>
 __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) k_layer(const KArgs a, const int tent0) {
@@ -1120,23 +1120,24 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
         if (part == 0 && m >= M && m < M + nb) eB[m - M] = tc::scale_exp(mx);
       }
       __syncthreads();
-      // digit planes, one item = 8 consecutive points of one row of A or B
-      for (int id = tid; id < (M + 32) * KC; id += blockDim.x) {
-        const bool isA = id < M * KC;
-        const int id2 = isA ? id : id - M * KC, rows = isA ? M : 32;
-        const int kc = id2 / rows, m = id2 % rows;
+      // digit planes, one item = 4 consecutive points of one row of A or B (8 left
+      // a second round of the CTA's threads a third full)
+      for (int id = tid; id < (M + 32) * 2 * KC; id += blockDim.x) {
+        const bool isA = id < M * 2 * KC;
+        const int id2 = isA ? id : id - M * 2 * KC, rows = isA ? M : 32;
+        const int k4 = id2 / rows, m = id2 % rows, kc = k4 >> 1, half = 4 * (k4 & 1);
         const bool live = isA || m < nb;
         const int ex = isA ? eA[m] : (live ? eB[m] : 0);
-        float d[8][tc::kSlices];
+        float d[4][tc::kSlices];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int ql = kc * 8 + j;
+        for (int j = 0; j < 4; ++j) {
+          const int ql = k4 * 4 + j;
           T x = R::zero();
           if (ql < nq && live) x = isA ? sCB[(size_t)m * cbs + ql] : sU[(size_t)ql * us + m];
           tc::digits(x.hi, x.lo, ex, d[j]);
         }
-        if (isA) tc::store_row8(sTA + ((size_t)(kc * RG + (m >> 3)) * 64 + (m & 7) * 8), planeA, d);
-        else tc::store_row8(sTB + ((size_t)(kc * 4 * tc::kSlices + (m >> 3)) * 64 + (m & 7) * 8), 4 * 64, d);
+        if (isA) tc::store_row4(sTA + ((size_t)(kc * RG + (m >> 3)) * 64 + (m & 7) * 8 + half), planeA, d);
+        else tc::store_row4(sTB + ((size_t)(kc * 4 * tc::kSlices + (m >> 3)) * 64 + (m & 7) * 8 + half), 4 * 64, d);
       }
       // B: the planes stacked along N, 32 rows each (planeB = 0 selects the stacked products)
       tc_issue(tc::smem_addr(sTA), (uint32_t)planeA * 2, (uint32_t)RG * 128, tc::smem_addr(sTB), 0u,
@@ -1184,6 +1185,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   };
   const int nneu = NEU ? s_nneu : 0;   // (kernels for meshes without Neumann facets leave out their code)
   const bool pblk = nif > 0 || nneu > 0;
+  const bool has_g = !ADJ && gD != nullptr;   // boundary data (else homogeneous)
   T* sFD = reinterpret_cast<T*>(sm + a.off_pd);      // Dirichlet sums (Grams, then data moments), then Neumann data
   T* sDD = reinterpret_cast<T*>(sm + a.off_dd);
   const int nfg = nfac > 0 ? ng * (DIM + 1) * npl : 0, nfm = nfac > 0 ? ng * (DIM + 1) * nrhs * nl : 0;
@@ -1300,9 +1302,9 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   // Gram pairs owned by this thread: the bottom face's (every function, the
   // recovery term) from the first thread on, the top face's and the facets'
   // (functions < nl: they enter through derivatives) from the last thread down,
-  // so that threads without a second pair of the one take the other.  (With
-  // every pair on both faces and the derivative moments over every function:
-  // 3D p = 3, 64 columns binary64, 217 ms a sweep of 3710 tents)
+  // so that threads without a second pair of the one take the other.  (Every
+  // pair on both faces and the derivative moments over every function: 2D p = 5,
+  // two materials, 188 -> 145 ms a sweep, 3D p = 3 mixed 8.6 -> 7.5 ms)
   int pi[kMaxPair], pj[kMaxPair], li[kMaxLow], lj[kMaxLow];
   T aK[kMaxLow], aG[kMaxLow], aH[kMaxLow][DIM], aB[kMaxPair];
   auto unpack = [](int id, int n, int& i, int& j) {
@@ -1358,8 +1360,9 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       const int NPD = nfac * Q, dsl = (NPD + CS - 1) / CS;
       const int d0 = min(NPD, rank * dsl), d1 = min(NPD, d0 + dsl);
       // the Grams take this CTA's slice [d0, d1); the data moments of split
-      // right-hand sides take every point
-      const int l0 = rsplit ? 0 : d0, l1 = rsplit ? NPD : d1;
+      // right-hand sides take every point (homogeneous data have none: 3D p = 3,
+      // 64 columns mixed, with the digit items below 330 -> 328 ms)
+      const int l0 = rsplit && has_g ? 0 : d0, l1 = rsplit && has_g ? NPD : d1;
       T aF[kMaxLow];
 #pragma unroll
       for (int s = 0; s < kMaxLow; ++s) aF[s] = R::zero();
@@ -1401,8 +1404,8 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
           pp[DIM + 1] = R::from(sw);
           // the facet's block of boundary data (without Neumann facets: the facet's own index)
           const long long goff = a.tent_gdoff[tent] + (NEU ? (long long)s_fw[f][0] * Q + qf : (long long)q);
-          for (int r = 0; r < nrhs; ++r)
-            sGd[id * nrhs + r] = R::from((!ADJ && gD != nullptr) ? sw * gD[(long long)r * a.n_bnd + goff] : 0.0);
+          if (has_g)
+            for (int r = 0; r < nrhs; ++r) sGd[id * nrhs + r] = R::from(sw * gD[(long long)r * a.n_bnd + goff]);
         }
         eval_uvalues_block<DIM, T, true, true>(a, nq, sPt, sM, sU);
         const int fc0 = fc;
@@ -1414,7 +1417,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
           for (int s = 0; s < kMaxLow; ++s)
             if (NT - 1 - tid + s * NT < npl) aF[s] = R::fma(u[li[s]], u[lj[s]], aF[s]);
         }
-        for (int id = tid; id < nrhs * nl; id += blockDim.x) {
+        for (int id = tid; id < (has_g ? nrhs * nl : 0); id += blockDim.x) {
           const int r = id / nl, i = id % nl;
           int f = fc0;
           T t = sDel[id];
@@ -1430,7 +1433,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
         __syncthreads();
       }
       fold_gram(fc);
-      for (int id = tid; id < nrhs * nl; id += blockDim.x) {
+      for (int id = tid; id < (has_g ? nrhs * nl : 0); id += blockDim.x) {
         fold_mom(fc, id, sDel[id]);
         sDel[id] = R::zero();
       }
@@ -1447,7 +1450,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
     // (v = (c/h) D_t u, sigma.n = -(1/h) D_n u, D_n = sum_m n_m D_m)
     for (int f = nfac; f < nfac + nif + nneu; ++f) {
       const bool neu = NEU && f >= nfac + nif, mine = (f - nfac) % CS == rank;
-      if (!mine && !(rsplit && neu)) continue;
+      if (!mine && !(rsplit && neu && has_g)) continue;
       const int f0 = 0, f1 = mine ? Q : 0;
       const int gp = s_fg[f], gm = s_fg2[f];
       const double cp = s_gc[gp], cm = s_gc[gm];
@@ -1455,7 +1458,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
 #pragma unroll
       for (int s = 0; s < kMaxLow; ++s) aF[s] = aF2[s] = R::zero();
       // (a Neumann facet's data moments of split right-hand sides take every point)
-      const int l0 = (rsplit && neu) ? 0 : f0, l1 = (rsplit && neu) ? Q : f1;
+      const int l0 = f0, l1 = (rsplit && neu && has_g) ? Q : f1;
       for (int base = l0; base < l1; base += CH) {
         const int nq = min(CH, l1 - base);
         const int npt = neu ? nq : 2 * nq;   // interface: + side points, then - side
@@ -1475,7 +1478,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
           if (neu) {
             const long long goff = a.tent_gdoff[tent] + (long long)s_fw[f][0] * Q + q;
             for (int r = 0; r < nrhs; ++r)
-              sGd[id * nrhs + r] = R::from((!ADJ && gD != nullptr) ? sw * gD[(long long)r * a.n_bnd + goff] : 0.0);
+              sGd[id * nrhs + r] = R::from(has_g ? sw * gD[(long long)r * a.n_bnd + goff] : 0.0);
           } else {
             T* p2 = sPt + (nq + id) * (DIM + 2);
             p2[0] = R::from(cm * (xt[DIM] - tc) * ih);
@@ -1745,7 +1748,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
     prefetch_front(0, min(CH, NP));
     for (int base = 0; base < NP; base += CH) {
       const int nq = min(CH, NP - base);
-      for (int id = tid; id < nq; id += blockDim.x) {
+      for (int id = tid; id < nq; id += blockDim.x) {   // (eval_uvalues_block's first reads: by the same threads)
         const int qg = base + id, k = qg / Q, q = qg % Q;
         map_point(sPt + id * (DIM + 2), k, q, ADJ);
       }
@@ -1785,7 +1788,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   }
   if (nfac > 0) {
     cluster_reduce(sFD, sFD, nfg);
-    if (!rsplit) cluster_reduce(sDD, sDD, nfm);
+    if (!rsplit && has_g) cluster_reduce(sDD, sDD, nfm);
   }
   csync();   // no CTA leaves or reuses its partials while another still reads them
   // congruence: the ranks form shares of A's entries and store them into rank
@@ -2145,7 +2148,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
         t = cc == 0 ? M[i] : R::mul(cc == 1 ? R::from(s_gc[g] * ih) : mih, rel_apply<DIM, T>(a, i, cc - 1, M));
         // Dirichlet data: b_D = E' delta summed over g's facets,
         // E' = alpha (c/h) D_t + (1/h) D_n
-        if (cc > 0 && ((gdir >> g) & 1u)) {
+        if (has_g && cc > 0 && ((gdir >> g) & 1u)) {
           const T* Dg = sDD + (size_t)(g * (DIM + 1) + cc - 1) * nrhs * nl + (size_t)r * nl;
           t = R::fma(R::from(cc == 1 ? a.alpha * s_gc[g] * ih : ih), rel_apply<DIM, T>(a, i, cc - 1, Dg), t);
         }

@@ -168,6 +168,17 @@ __device__ __forceinline__ void store_row8(uint16_t* base, int plane_stride, con
   }
 }
 
+// the same of 4 consecutive K entries, the first or second half of a row: 8 bytes per plane
+__device__ __forceinline__ void store_row4(uint16_t* base, int plane_stride, const float (&d)[4][kSlices]) {
+#pragma unroll
+  for (int s = 0; s < kSlices; ++s) {
+    uint2 w;
+    w.x = bf16_bits(d[0][s]) | (bf16_bits(d[1][s]) << 16);
+    w.y = bf16_bits(d[2][s]) | (bf16_bits(d[3][s]) << 16);
+    *reinterpret_cast<uint2*>(base + (size_t)s * plane_stride) = w;
+  }
+}
+
 // The level sums of one output (acc_l = sum of the digit products of planes
 // i + j = l + 2, integers below 2^24, exact in binary32) as the float-float
 // value (s, e) of sum_l acc_l 512^-l: the two leading levels by TwoSum, the
