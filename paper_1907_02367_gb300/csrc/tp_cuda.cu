@@ -196,7 +196,8 @@ struct tp_ctx {
   std::vector<void*> probe_allocs;
   int* d_inject = nullptr;
   unsigned long long* d_stats = nullptr;   // solve statistics (kMaxRefine + 2 counters)
-  std::map<std::pair<int, int>, cudaGraphExec_t> graphs;
+  // captured sweeps by level range and presence of boundary data (the graphs hold the arguments by value)
+  std::map<std::array<int, 3>, cudaGraphExec_t> graphs;
   int device = 0;
 };
 
@@ -1422,14 +1423,10 @@ extern "C" int tp_set_state(tp_ctx* ctx, const double* d_front, const double* d_
     TP_CUDA_OK(cudaMemsetAsync(ctx->d_probe_out, 0,
                                (size_t)ctx->nrhs * ctx->n_probe_t * ctx->n_probe * sizeof(double), st));
   if (ctx->n_bnd > 0) {
-    if (d_gD) {
+    if (d_gD)
       TP_CUDA_OK(cudaMemcpyAsync(ctx->d_gD, d_gD, (size_t)ctx->nrhs * ctx->n_bnd * sizeof(double),
                                  cudaMemcpyDeviceToDevice, st));
-      ctx->args.gD = ctx->d_gD;
-    } else {
-      TP_CUDA_OK(cudaMemsetAsync(ctx->d_gD, 0, (size_t)ctx->nrhs * ctx->n_bnd * sizeof(double), st));
-      ctx->args.gD = ctx->d_gD;
-    }
+    ctx->args.gD = d_gD ? ctx->d_gD : nullptr;   // (NULL: homogeneous data, whose facet moments are left out)
   }
   ctx->last_stream = st;
   return TP_OK;
@@ -1659,7 +1656,7 @@ extern "C" int tp_advance(tp_ctx* ctx, int32_t level_begin, int32_t level_end, v
     return TP_ERR_ARG;
   }
   if (level_end == level_begin) return TP_OK;
-  auto key = std::make_pair((int)level_begin, (int)level_end);
+  const std::array<int, 3> key = {level_begin, level_end, ctx->args.gD != nullptr};
   auto it = ctx->graphs.find(key);
   if (it == ctx->graphs.end()) {
     cudaGraph_t g = nullptr;
