@@ -1057,6 +1057,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   bool ifneu = false;   // some tent has interface or Neumann facets
   for (const auto& m : facet_mix) ifneu = ifneu || m[2] > 0 || m[3] > 0;
   bool tc_try = false;   // the plan with the tensor-core staging
+  bool tight = false;    // the solve's residual in the data coefficients' buffer (dead from the moments to the outflow)
   // (CH: points per chunk; keep: points whose U-values a CTA keeps; rows: points
   // evaluated at a time into them; rule: the S-point rule of the face integrals)
   const int S_rule = a.S;
@@ -1088,7 +1089,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     const size_t mono = (size_t)a.ev_rows * a.mono_stride;
     take(nullptr, NB * NB);                        // A
     take(&a.off_x, rb);
-    take(&a.off_z, rb);
+    take(&a.off_z, tight ? 0 : rb);
     take(&a.off_b, rb);
     // one region in turn: facet Grams of interface and Neumann facets, the
     // Grams G, H_m, Gbot (contiguous), the float-float inverse
@@ -1136,7 +1137,8 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     // data coefficients, a row per right-hand side and component: of a chunk
     // of points, or of those elements' points
     a.cb_pts = std::max({CH, a.raw_el * QK, keep > 0 && nrg <= 4 ? keep : 0});
-    take(&a.off_cb, (size_t)(a.cb_pts | 1) * nrg * C);
+    take(&a.off_cb, std::max((size_t)(a.cb_pts | 1) * nrg * C, tight ? rb : 0));
+    if (tight) a.off_z = a.off_cb;
     take(&a.off_tf, rs > 1 ? 0 : (size_t)2 * a.S * a.tf_stride);
     take(&a.off_gd, (size_t)CH * nrg);
     take(&a.off_rd, NB);
@@ -1158,7 +1160,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     return off * sizeof(double);
   };
   int CH = 0;
-  size_t bytes = 0, cap_used = 0;
+  size_t bytes = 0;
   size_t max_dyn = 0, two_per_sm = 0;
   if ((rc = max_dyn_smem(n, &max_dyn, &two_per_sm)) != TP_OK) return fail(rc);
   // right-hand sides split over the cluster: rs CTAs, each owning a slice of
@@ -1202,26 +1204,28 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   // (the S-point rule where its points fit the evaluation buffer; right-hand
   // sides not split: U-values evaluated again need whole elements in it)
   // (split right-hand sides keep the front rule, whose U-values their moments and outflow take)
+  // The number of groups comes first, the rule second: a group more assembles
+  // every tent once more (3D p = 3, 750 elements, 29 columns, binary64: 29
+  // groups of one under the S-point rule 65.7 ms, one group 19.2; 26: two
+  // groups 37.3, one 16.6), and the wave-speed gradient takes one group only.  A whole
+  // group that misses by little overlays two buffers, in the last place.
   bool rule = false;
-  for (int pass = 0; pass < 3 && CH == 0; ++pass) {
+  for (int pass = 0; pass < 2 && CH == 0; ++pass) {
     tc_try = tc_want && pass == 0;
     if (!tc_want && pass == 0) continue;
-    rule = S_rule > 0 && rs == 1 && pass < 2;
-    if (pass == 2 && (S_rule == 0 || rs > 1)) continue;
     for (grp = ctx->nrhs; grp >= 1 && CH == 0; --grp) {
       if (ctx->nrhs % grp || grp % rs) continue;
       nrg = grp / rs;
       if (tc_try && nrg * C > 96) continue;
-      for (size_t cap : {two_per_sm, max_dyn}) {
-        for (int ch : {48, 32, 16, 8}) {
-          if (CH != 0 || (rule && 2 * ch < S_rule) || plan(ch, 0, 0, rule) > cap) continue;
-          if (tc_try && (ch % 16 != 0 || ch * tp::kTcSlices * 65536 >= (1 << 24))) continue;
-          CH = ch;
-        }
-        if (CH) {
-          cap_used = cap;
-          break;
-        }
+      for (int form = S_rule > 0 && rs == 1 ? 0 : 1; form < 3 && CH == 0; ++form) {   // S-point rule, front rule, the same tight
+        rule = form == 0;
+        tight = form == 2;
+        for (size_t cap : {two_per_sm, max_dyn})
+          for (int ch : {48, 32, 16, 8}) {
+            if (CH != 0 || (rule && 2 * ch < S_rule) || plan(ch, 0, 0, rule) > cap) continue;
+            if (tc_try && (ch % 16 != 0 || ch * tp::kTcSlices * 65536 >= (1 << 24))) continue;
+            CH = ch;
+          }
       }
       if (CH) break;
     }
@@ -1289,10 +1293,13 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     ctx->max_cs = std::max(cs, keep_cs);
     // dataflow sweep, right-hand sides not split: the smallest cluster that
     // keeps its U-values, doubled while a third of the resident CTAs holds a
-    // level's tents (the others then work ahead) and a CTA keeps 5/4 elements
+    // level's tents (the others then work ahead) and a CTA keeps 5/4 elements.
+    // Where no cluster keeps them, each evaluates its points again after the
+    // wait: the cluster of 32 or more points a CTA (3D p = 3, 16 columns with
+    // checkpoints, 750 elements: 27.6 ms with 2 CTAs, 11.6 with 8)
     const double width = (double)ctx->ntents / std::max(1, ctx->n_levels), star = (double)T.star_el.size() / (double)T.nv;
-    cs = std::max(1, keep_cs);
-    while (cs < 8 && 2.0 * cs * width <= (ctx->wide ? 1 : 2) * ctx->n_sm / 3.0 && star / (2.0 * cs) >= 1.25) cs *= 2;
+    if (keep_cs > 0) cs = keep_cs;
+    while (keep_cs > 0 && cs < 8 && 2.0 * cs * width <= (ctx->wide ? 1 : 2) * ctx->n_sm / 3.0 && star / (2.0 * cs) >= 1.25) cs *= 2;
     ctx->flow_cs = cs;
   }
   {
