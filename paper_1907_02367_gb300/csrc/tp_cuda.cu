@@ -1201,8 +1201,25 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   if ((rc = static_smem(n, &stat_smem)) != TP_OK) return fail(rc);
   const bool tc_want = prm->tensor_cores >= 0 && ctx->mixed && rs > 1 && nb <= 32 &&
                        (ctx->nrhs / rs) * C <= 96;
-  // (the S-point rule where its points fit the evaluation buffer; right-hand
-  // sides not split: U-values evaluated again need whole elements in it)
+  // The S-point rule where it does less work: per element it saves Q - S points
+  // of both faces' U-values (a term counts twice: its table lookups) and Grams,
+  // once, and costs the data of every right-hand side two tables of S x Q
+  // instead of Q - S points of the moments and the outflow.  That is up to 4
+  // columns at 3D p = 3, 3 at 2D p = 4, 5, one at p = 2 and 2D p = 3, none at
+  // p = 1.  Milliseconds a sweep, S-point -> front rule, at and past that line:
+  // 3D p = 3, 1296 elements, mixed 2.4 -> 5.1 with one column, 5.8 -> 6.1 with 4,
+  // 11.5 -> 10.3 with 16; 2D p = 3, 800 triangles, binary64 0.73 -> 0.66 with 2,
+  // 3.7 -> 2.4 with 16 (1.9 with the cluster chosen below); 3D p = 2, 1296
+  // elements, binary64 2.9 -> 2.0 with 4, 10.3 -> 5.8 with 16
+  auto rule_pays = [&](int columns) {
+    if (S_rule == 0 || rs > 1) return false;
+    long long terms = ctx->nmono;
+    for (int j = 0; j < nb; ++j) terms += basis->sp_ptr[(size_t)j * C + 1] - basis->sp_ptr[(size_t)j * C];
+    const long long fewer = Q - S_rule;
+    return columns * (2LL * C * S_rule * Q - 2 * fewer * (nb + (n + 1) * nl)) <= fewer * (npair + npl + 4 * terms);
+  };
+  // (its points fit the evaluation buffer; right-hand sides not split: U-values
+  // evaluated again need whole elements in it)
   // (split right-hand sides keep the front rule, whose U-values their moments and outflow take)
   // The number of groups comes first, the rule second: a group more assembles
   // every tent once more (3D p = 3, 750 elements, 29 columns, binary64: 29
@@ -1217,7 +1234,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
       if (ctx->nrhs % grp || grp % rs) continue;
       nrg = grp / rs;
       if (tc_try && nrg * C > 96) continue;
-      for (int form = S_rule > 0 && rs == 1 ? 0 : 1; form < 3 && CH == 0; ++form) {   // S-point rule, front rule, the same tight
+      for (int form = rule_pays(nrg) ? 0 : 1; form < 3 && CH == 0; ++form) {   // S-point rule, front rule, the same tight
         rule = form == 0;
         tight = form == 2;
         for (size_t cap : {two_per_sm, max_dyn})
@@ -1238,6 +1255,10 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   // nothing is evaluated after the wait.  The smallest cluster for which the
   // slices of the largest patch fit, with two CTAs per SM if any does; the
   // chunks of the other passes shrink for it.
+  // (More than 4 columns: clusters that leave a CTA 3 elements of it, as one
+  // CTA solves for all; 2D p = 5, 800 triangles, 16 columns mixed: 8 CTAs of an
+  // element 6.9 ms, 2 CTAs 3.5.)
+  const bool many = nrg > 4;
   int keep = 0, rows = 0, keep_cs = 0;
   if (rs == 1) {
     const int QK = rule ? S_rule : Q;
@@ -1246,7 +1267,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
       for (int cs : {1, 2, 4, 8})
         for (const auto& c : kChunks) {
           const int want = (pmax + cs - 1) / cs * QK;
-          if (keep_cs != 0 || (rule && 2 * c[0] < S_rule) || plan(c[0], want, c[1], rule) > cap) continue;
+          if (keep_cs != 0 || (cs > 1 && many && pmax < 3 * cs) || (rule && 2 * c[0] < S_rule) || plan(c[0], want, c[1], rule) > cap) continue;
           CH = c[0];
           rows = c[1];
           keep = want;
@@ -1293,13 +1314,21 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     ctx->max_cs = std::max(cs, keep_cs);
     // dataflow sweep, right-hand sides not split: the smallest cluster that
     // keeps its U-values, doubled while a third of the resident CTAs holds a
-    // level's tents (the others then work ahead) and a CTA keeps 5/4 elements.
+    // level's tents (the others then work ahead) and a CTA keeps 5/4 elements;
+    // with more than 4 columns, whose data and outflow the next tents wait for,
+    // also while two thirds hold them and a CTA has 32 points (800 triangles,
+    // p = 3, 16 columns, binary64: 1 -> 2 CTAs 2.4 -> 1.9 ms).
     // Where no cluster keeps them, each evaluates its points again after the
     // wait: the cluster of 32 or more points a CTA (3D p = 3, 16 columns with
     // checkpoints, 750 elements: 27.6 ms with 2 CTAs, 11.6 with 8)
     const double width = (double)ctx->ntents / std::max(1, ctx->n_levels), star = (double)T.star_el.size() / (double)T.nv;
-    if (keep_cs > 0) cs = keep_cs;
-    while (keep_cs > 0 && cs < 8 && 2.0 * cs * width <= (ctx->wide ? 1 : 2) * ctx->n_sm / 3.0 && star / (2.0 * cs) >= 1.25) cs *= 2;
+    if (keep_cs > 0) {
+      const double resident = (ctx->wide ? 1 : 2) * ctx->n_sm;
+      cs = keep_cs;
+      while (cs < 8 && star / (2.0 * cs) >= 1.25 &&
+             (2.0 * cs * width <= resident / 3.0 || (many && 2.0 * cs * width <= resident / 1.5 && avg_pts / (2.0 * cs) >= 32.0)))
+        cs *= 2;
+    }
     ctx->flow_cs = cs;
   }
   {
