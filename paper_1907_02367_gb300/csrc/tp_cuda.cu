@@ -120,6 +120,15 @@ int upload(T** dptr, const std::vector<T>& h) {
 // ===========================================================================
 // context
 // ===========================================================================
+// how the CTAs of a sweep are laid out
+struct SweepPlan {
+  size_t smem = 0;
+  bool wide = false;                // one CTA per SM (its shared-memory plan does not leave room for two): twice the threads
+  int min_cs = 1;                   // smallest cluster whose CTAs keep their U-values (every tent's: the plan counts on it)
+  int max_cs = 1, flow_cs = 1;      // largest cluster of a launch per level; the dataflow sweep's before any tuning
+  int cs = 1, clusters = 0;         // the dataflow sweep's cluster and how many are resident
+};
+
 struct tp_ctx {
   int dim = 0, p = 0, nb = 0, nmono = 0, Q = 0, C = 0, nrhs = 1;
   double alpha = 0.5;
@@ -141,7 +150,6 @@ struct tp_ctx {
   int rhs_groups = 1, nrhs_g = 1;
   double* d_tau_save = nullptr;
   cudaGraphExec_t adj_graph = nullptr;
-  size_t smem_bytes = 0;
   int energy_blocks = 0;
   std::vector<void*> allocs;
   double* d_front = nullptr;
@@ -166,17 +174,15 @@ struct tp_ctx {
   long long* d_info = nullptr;
   cudaStream_t cap_stream = nullptr;
   cudaStream_t last_stream = nullptr;
-  int n_sm = 152, max_cs = 1, flow_cs = 1;   // largest cluster of a launch per level; cluster of the dataflow sweep
+  int n_sm = 152;
+  SweepPlan fwd, rev;     // forward and reverse sweep
+  bool rev_own = false;   // the reverse sweep has a plan of its own (its binary64 sums take the front rule)
   // right-hand sides split over the CTAs of a tent's cluster (1: not split)
   int rsplit_cs = 1;
   bool tc_used = false;   // tensor-core moments and outflow in the forward sweep
-  int min_cs = 1;         // smallest cluster whose CTAs keep their U-values (every tent's: the plan counts on it)
-  bool wide = false;      // one CTA per SM (its shared-memory plan does not leave room for two): twice the threads
   bool mixed = false;
   // persistent dataflow sweep
   bool persistent = true;
-  int persist_clusters = 0, persist_clusters_adj = 0;
-  int persist_cs = 1;
   int tune_key[5] = {0, 0, 0, 0, 0};   // (dim, p, nrhs, mixed, patch bucket) of the autotuner cache
   int* d_queue = nullptr;
   int* d_done = nullptr;
@@ -269,25 +275,29 @@ int forward_kind(const tp_ctx* ctx) { return ctx->tc_used ? kForwardTc : ctx->mi
 
 cudaError_t launch_layer(tp_ctx* ctx, const KArgs& a, int n_cluster, int cs, int t0, cudaStream_t st, int kind,
                          bool persistent) {
-  return kLaunchers[ctx->dim - 1][kind][ctx->neumann].launch(a, n_cluster, cs, t0, ctx->smem_bytes, st, persistent, ctx->wide);
+  const SweepPlan& p = kind == kAdjoint64 ? ctx->rev : ctx->fwd;
+  return kLaunchers[ctx->dim - 1][kind][ctx->neumann].launch(a, n_cluster, cs, t0, p.smem, st, persistent, p.wide);
 }
 
-// resident clusters of the persistent kernel for cluster size cs
+// resident clusters of the dataflow sweep for cluster size cs (of the forward
+// sweep; the reverse takes the same unless it has a plan of its own)
 int set_persist_cs(tp_ctx* ctx, int cs) {
-  if (cs < ctx->min_cs) return TP_ERR_UNSUPPORTED;
+  if (cs < ctx->fwd.min_cs) return TP_ERR_UNSUPPORTED;
+  const int rev_cs = ctx->rev_own ? ctx->rev.flow_cs : cs;
   int nclu = 0, nadj = 0;
   cudaError_t e = kLaunchers[ctx->dim - 1][forward_kind(ctx)][ctx->neumann].max_clusters(
-      cs, ctx->smem_bytes, ctx->rsplit_cs > 1, ctx->wide, &nclu);
+      cs, ctx->fwd.smem, ctx->rsplit_cs > 1, ctx->fwd.wide, &nclu);
   if (e == cudaSuccess)
-    e = kLaunchers[ctx->dim - 1][kAdjoint64][ctx->neumann].max_clusters(cs, ctx->smem_bytes, ctx->rsplit_cs > 1,
-                                                                        ctx->wide, &nadj);
+    e = kLaunchers[ctx->dim - 1][kAdjoint64][ctx->neumann].max_clusters(rev_cs, ctx->rev.smem, ctx->rsplit_cs > 1,
+                                                                        ctx->rev.wide, &nadj);
   if (e != cudaSuccess || nclu < 1 || nadj < 1) {
     cudaGetLastError();
     return TP_ERR_UNSUPPORTED;
   }
-  ctx->persist_cs = cs;
-  ctx->persist_clusters = nclu;
-  ctx->persist_clusters_adj = nadj;
+  ctx->fwd.cs = cs;
+  ctx->fwd.clusters = nclu;
+  ctx->rev.cs = rev_cs;
+  ctx->rev.clusters = nadj;
   return TP_OK;
 }
 
@@ -306,10 +316,11 @@ bool tuned_lookup(const int* key, int* cs, bool* dataflow) {
 
 // cluster size for a level of nt tents: a power of two <= max_cs with
 // nt * cs <= 2 CTAs per SM
-int level_cluster_size(const tp_ctx* ctx, int64_t nt) {
+int level_cluster_size(const tp_ctx* ctx, int64_t nt, bool adj) {
   if (ctx->rsplit_cs > 1) return ctx->rsplit_cs;   // one CTA per slice of the right-hand sides
-  int cs = ctx->min_cs;
-  while (cs * 2 <= ctx->max_cs && nt * cs * 2 <= 2LL * ctx->n_sm) cs *= 2;
+  const SweepPlan& p = adj ? ctx->rev : ctx->fwd;
+  int cs = p.min_cs;
+  while (cs * 2 <= p.max_cs && nt * cs * 2 <= 2LL * ctx->n_sm) cs *= 2;
   return cs;
 }
 
@@ -337,16 +348,17 @@ cudaError_t launch_dataflow(tp_ctx* ctx, KArgs a, int32_t level_begin, int32_t l
                             cudaStream_t st) {
   const int t0 = (int)ctx->level_ptr[level_begin - 1], t1 = (int)ctx->level_ptr[level_end - 1];
   const int lo = adj ? t1 : 0, hi = adj ? (int)ctx->ntents : t0;
+  const SweepPlan& p = adj ? ctx->rev : ctx->fwd;
   a.tent_beg = t0;
   a.tent_end = t1;
   a.done = done;
   a.queue = queue;
   cudaError_t e = cudaMemsetAsync(done, 0, ctx->nv * sizeof(int), st);
   if (e != cudaSuccess) return e;
-  k_sweep_setup<<<std::max(1, std::min(1024, (hi - lo + 255) / 256)), 256, 0, st>>>(ctx->args.tent_v, lo, hi, ctx->persist_cs,
+  k_sweep_setup<<<std::max(1, std::min(1024, (hi - lo + 255) / 256)), 256, 0, st>>>(ctx->args.tent_v, lo, hi, p.cs,
                                                                                      done, queue, t0);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  return launch_layer(ctx, a, adj ? ctx->persist_clusters_adj : ctx->persist_clusters, ctx->persist_cs, 0, st,
+  return launch_layer(ctx, a, p.clusters, p.cs, 0, st,
                       adj ? kAdjoint64 : forward_kind(ctx), true);
 }
 
@@ -356,7 +368,7 @@ int launch_level(tp_ctx* ctx, int32_t L, cudaStream_t st, bool adj = false, int 
   const int64_t t0 = ctx->level_ptr[L - 1], t1 = ctx->level_ptr[L];
   if (t1 <= t0) return TP_OK;
   const int nt = (int)(t1 - t0);
-  const int cs = level_cluster_size(ctx, nt);
+  const int cs = level_cluster_size(ctx, nt, adj);
   const int mode = adj ? kAdjoint64 : forward_kind(ctx);
   double* tau = adj ? ctx->d_tau_adj : ctx->d_tau;
   const int k0 = group < 0 ? 0 : group, k1 = group < 0 ? ctx->rhs_groups : group + 1;
@@ -384,7 +396,7 @@ int launch_range_with(tp_ctx* ctx, int32_t L0, int32_t L1, cudaStream_t st, bool
     const int64_t t0 = ctx->level_ptr[L - 1], t1 = ctx->level_ptr[L];
     if (t1 <= t0) continue;
     const int nt = (int)(t1 - t0);
-    TP_CUDA_OK(launch_layer(ctx, a, nt, level_cluster_size(ctx, nt), (int)t0, st, adj ? kAdjoint64 : forward_kind(ctx), false));
+    TP_CUDA_OK(launch_layer(ctx, a, nt, level_cluster_size(ctx, nt, adj), (int)t0, st, adj ? kAdjoint64 : forward_kind(ctx), false));
     TP_CUDA_OK(cudaGetLastError());
   }
   return TP_OK;
@@ -1066,11 +1078,11 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   // shared: the evaluation's monomials with the Grams, the chunk of U-values of
   // the facet, energy and probe passes with the end of the kept rows, whose
   // owners, the moments' rows, are not yet or no longer needed in those passes)
-  auto plan = [&](int CH, int keep, int rows, bool rule) {
+  auto plan = [&](KArgs& k, int CH, int keep, int rows, bool rule) {
     size_t off = 0;
     const bool share_mono = keep > 0 && ngmax == 1 && !ifneu, share_u = keep >= 2 * CH;
-    a.S = rule ? S_rule : 0;
-    const int QK = a.S > 0 ? a.S : Q;
+    k.S = rule ? S_rule : 0;
+    const int QK = k.S > 0 ? k.S : Q;
     auto take = [&](int* field, size_t count) {
       if (field) *field = (int)off;
       off += count;
@@ -1085,28 +1097,28 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
       pd = std::max(pd, m[1] > 0 ? (size_t)m[0] * (n + 1) * npl : 0);
       pdd = std::max(pdd, (m[1] > 0 ? (size_t)m[0] * (n + 1) * nrg * nl : 0) + (m[3] > 0 ? (size_t)nrg * m[0] * nb : 0));
     }
-    a.ev_rows = std::max(2 * CH, rows);
-    const size_t mono = (size_t)a.ev_rows * a.mono_stride;
+    k.ev_rows = std::max(2 * CH, rows);
+    const size_t mono = (size_t)k.ev_rows * k.mono_stride;
     take(nullptr, NB * NB);                        // A
-    take(&a.off_x, rb);
-    take(&a.off_z, tight ? 0 : rb);
-    take(&a.off_b, rb);
+    take(&k.off_x, rb);
+    take(&k.off_z, tight ? 0 : rb);
+    take(&k.off_b, rb);
     // one region in turn: facet Grams of interface and Neumann facets, the
     // Grams G, H_m, Gbot (contiguous), the float-float inverse
     // (right-hand sides split: the facet Grams have a region of their own)
     const size_t fg = ifneu ? (size_t)2 * npl + nl * nl + 2 * nl * nb : 0;   // (and two nl x nb products)
-    a.off_f = (int)off;
-    a.off_f2 = a.off_f + npl;
-    a.off_fpm = a.off_f2 + npl;
+    k.off_f = (int)off;
+    k.off_f2 = k.off_f + npl;
+    k.off_fpm = k.off_f2 + npl;
     if (rs > 1) off += fg;
-    a.off_pg = (int)off;
-    a.off_ph = a.off_pg + ngmax * npl;
-    a.off_pgb = a.off_ph + ngmax * n * npl;
-    a.off_mono = (int)off;
+    k.off_pg = (int)off;
+    k.off_ph = k.off_pg + ngmax * npl;
+    k.off_pgb = k.off_ph + ngmax * n * npl;
+    k.off_mono = (int)off;
     take(nullptr, std::max({(size_t)ngmax * ((n + 1) * npl + npair), NB * NB, fg, share_mono ? mono : 0}));
-    take(&a.off_pm, (size_t)ngmax * nmom);        // moments: partials, summed in place, then the outflow vectors
-    a.off_sm = a.off_y = a.off_pm;
-    if (!share_mono) take(&a.off_mono, mono);
+    take(&k.off_pm, (size_t)ngmax * nmom);        // moments: partials, summed in place, then the outflow vectors
+    k.off_sm = k.off_y = k.off_pm;
+    if (!share_mono) take(&k.off_mono, mono);
     // tensor-core staging (bf16 digit planes), in the region of the facet
     // sums (dead during the point passes before phase 2 and during the
     // outflow): the moments' A (rows of data coefficients x CH points) and B
@@ -1122,45 +1134,43 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
       tcd = ((std::max(mom, out) + 512 + 3) / 4 + 1) & ~(size_t)1;
     }
     off += off & 1;                                // 16-byte alignment of the staging
-    a.off_tc = (int)off;
+    k.off_tc = (int)off;
     // elements whose front data are taken at a time under the S-point rule (with
     // kept U-values and few right-hand sides: all of the CTA's); the data share
     // the region of the Dirichlet Grams
-    a.raw_el = a.S == 0 || rs > 1 ? 0 : keep > 0 && nrg <= 4 ? keep / QK : std::max(1, (keep > 0 ? CH : 2 * CH) / QK);
-    const size_t raw = (size_t)a.raw_el * Q * nrg * C;
-    a.off_raw = (int)off;
-    take(&a.off_pd, std::max({pd, raw, tcd > pdd ? tcd - pdd : 0}));
-    take(&a.off_dd, pdd);
-    take(&a.off_del, (size_t)nrg * std::max(1, nl));
-    if (!share_u) take(&a.off_u, (size_t)2 * CH * (nb | 1));
-    take(&a.off_pt, (size_t)a.ev_rows * (n + 2));
+    k.raw_el = k.S == 0 || rs > 1 ? 0 : keep > 0 && nrg <= 4 ? keep / QK : std::max(1, (keep > 0 ? CH : 2 * CH) / QK);
+    const size_t raw = (size_t)k.raw_el * Q * nrg * C;
+    k.off_raw = (int)off;
+    take(&k.off_pd, std::max({pd, raw, tcd > pdd ? tcd - pdd : 0}));
+    take(&k.off_dd, pdd);
+    take(&k.off_del, (size_t)nrg * std::max(1, nl));
+    if (!share_u) take(&k.off_u, (size_t)2 * CH * (nb | 1));
+    take(&k.off_pt, (size_t)k.ev_rows * (n + 2));
     // data coefficients, a row per right-hand side and component: of a chunk
     // of points, or of those elements' points
-    a.cb_pts = std::max({CH, a.raw_el * QK, keep > 0 && nrg <= 4 ? keep : 0});
-    take(&a.off_cb, std::max((size_t)(a.cb_pts | 1) * nrg * C, tight ? rb : 0));
-    if (tight) a.off_z = a.off_cb;
-    take(&a.off_tf, rs > 1 ? 0 : (size_t)2 * a.S * a.tf_stride);
-    take(&a.off_gd, (size_t)CH * nrg);
-    take(&a.off_rd, NB);
-    take(&a.off_rc, std::max((size_t)8 * 32 * std::min<size_t>(3, (NB + 31) / 32), NB > 64 ? 4 * NB : 0));
-    take(&a.off_eq, half_nb);
-    take(&a.off_keep, (size_t)2 * keep * (nb | 1));   // U-values of the CTA's slice on both faces
-    if (share_u) a.off_u = a.off_keep + (2 * keep - 2 * CH) * (nb | 1);
+    k.cb_pts = std::max({CH, k.raw_el * QK, keep > 0 && nrg <= 4 ? keep : 0});
+    take(&k.off_cb, std::max((size_t)(k.cb_pts | 1) * nrg * C, tight ? rb : 0));
+    if (tight) k.off_z = k.off_cb;
+    take(&k.off_tf, rs > 1 ? 0 : (size_t)2 * k.S * k.tf_stride);
+    take(&k.off_gd, (size_t)CH * nrg);
+    take(&k.off_rd, NB);
+    take(&k.off_rc, std::max((size_t)8 * 32 * std::min<size_t>(3, (NB + 31) / 32), NB > 64 ? 4 * NB : 0));
+    take(&k.off_eq, half_nb);
+    take(&k.off_keep, (size_t)2 * keep * (nb | 1));   // U-values of the CTA's slice on both faces
+    if (share_u) k.off_u = k.off_keep + (2 * keep - 2 * CH) * (nb | 1);
     {   // the patch (Geo)
       const size_t NVg = n + 1, P_ = pmax, F_ = fmax, M_ = nmax;
-      const size_t dbl[] = {P_ * NVg * n, P_ * NVg * (n + 2), P_ * NVg, P_ * NVg, P_ * n, P_ * n, P_, P_, P_, P_ * NVg,
+      const size_t dbl[] = {P_ * NVg * n, ctx->mixed ? P_ * NVg * (n + 2) : 0, P_ * NVg, P_ * NVg, P_ * n, P_ * n, P_, P_, P_, P_ * NVg,
                             F_ * NVg * NVg, F_, F_ * n, M_};
       const size_t ints[] = {P_, P_, P_ * NVg, F_ * NVg, F_, F_, M_};
       int g = 0;
-      for (size_t c : dbl) take(&a.geo[g++], c);
-      for (size_t c : ints) take(&a.geo[g++], (c + 1) / 2);
+      for (size_t c : dbl) take(&k.geo[g++], c);
+      for (size_t c : ints) take(&k.geo[g++], (c + 1) / 2);
     }
     // wave-speed gradient (reverse sweep): y(x), y(x'), y(mu') per material and the forward solution
-    take(&a.off_yg, prm->ckpt_stride > 0 ? 3 * (size_t)ngmax * nmom + (size_t)nrg * NB : 0);
+    take(&k.off_yg, prm->ckpt_stride > 0 ? 3 * (size_t)ngmax * nmom + (size_t)nrg * NB : 0);
     return off * sizeof(double);
   };
-  int CH = 0;
-  size_t bytes = 0;
   size_t max_dyn = 0, two_per_sm = 0;
   if ((rc = max_dyn_smem(n, &max_dyn, &two_per_sm)) != TP_OK) return fail(rc);
   // right-hand sides split over the cluster: rs CTAs, each owning a slice of
@@ -1210,23 +1220,36 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   // 3D p = 3, 1296 elements, mixed 2.4 -> 5.1 with one column, 5.8 -> 6.1 with 4,
   // 11.5 -> 10.3 with 16; 2D p = 3, 800 triangles, binary64 0.73 -> 0.66 with 2,
   // 3.7 -> 2.4 with 16 (1.9 with the cluster chosen below); 3D p = 2, 1296
-  // elements, binary64 2.9 -> 2.0 with 4, 10.3 -> 5.8 with 16
-  auto rule_pays = [&](int columns) {
-    if (S_rule == 0 || rs > 1) return false;
+  // elements, binary64 2.9 -> 2.0 with 4, 10.3 -> 5.8 with 16.
+  // (Binary64 sums: at 3D p = 3 alone, where its errors are the front rule's; the
+  // kernel's RULE has the figures.)
+  auto rule_pays = [&](int columns, bool binary64) {
+    if (S_rule == 0 || rs > 1 || (binary64 && !(n == 3 && basis->p == 3))) return false;
     long long terms = ctx->nmono;
     for (int j = 0; j < nb; ++j) terms += basis->sp_ptr[(size_t)j * C + 1] - basis->sp_ptr[(size_t)j * C];
     const long long fewer = Q - S_rule;
     return columns * (2LL * C * S_rule * Q - 2 * fewer * (nb + (n + 1) * nl)) <= fewer * (npair + npl + 4 * terms);
   };
-  // (its points fit the evaluation buffer; right-hand sides not split: U-values
-  // evaluated again need whole elements in it)
-  // (split right-hand sides keep the front rule, whose U-values their moments and outflow take)
+  // the largest chunk of points whose plan fits (0: none), with two CTAs per SM if any does
+  // (the rule's points fit the evaluation buffer: U-values evaluated again need
+  // whole elements in it; split right-hand sides keep the front rule, whose
+  // U-values their moments and outflow take)
+  auto chunk = [&](KArgs& k, bool rule) {
+    for (size_t cap : {two_per_sm, max_dyn})
+      for (int ch : {48, 32, 16, 8}) {
+        if ((rule && 2 * ch < S_rule) || plan(k, ch, 0, 0, rule) > cap) continue;
+        if (tc_try && (ch % 16 != 0 || ch * tp::kTcSlices * 65536 >= (1 << 24))) continue;
+        return ch;
+      }
+    return 0;
+  };
   // The number of groups comes first, the rule second: a group more assembles
   // every tent once more (3D p = 3, 750 elements, 29 columns, binary64: 29
   // groups of one under the S-point rule 65.7 ms, one group 19.2; 26: two
   // groups 37.3, one 16.6), and the wave-speed gradient takes one group only.  A whole
   // group that misses by little overlays two buffers, in the last place.
   bool rule = false;
+  int CH = 0;
   for (int pass = 0; pass < 2 && CH == 0; ++pass) {
     tc_try = tc_want && pass == 0;
     if (!tc_want && pass == 0) continue;
@@ -1234,15 +1257,10 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
       if (ctx->nrhs % grp || grp % rs) continue;
       nrg = grp / rs;
       if (tc_try && nrg * C > 96) continue;
-      for (int form = rule_pays(nrg) ? 0 : 1; form < 3 && CH == 0; ++form) {   // S-point rule, front rule, the same tight
+      for (int form = rule_pays(nrg, !ctx->mixed) ? 0 : 1; form < 3 && CH == 0; ++form) {   // S-point rule, front rule, the same tight
         rule = form == 0;
         tight = form == 2;
-        for (size_t cap : {two_per_sm, max_dyn})
-          for (int ch : {48, 32, 16, 8}) {
-            if (CH != 0 || (rule && 2 * ch < S_rule) || plan(ch, 0, 0, rule) > cap) continue;
-            if (tc_try && (ch % 16 != 0 || ch * tp::kTcSlices * 65536 >= (1 << 24))) continue;
-            CH = ch;
-          }
+        CH = chunk(a, rule);
       }
       if (CH) break;
     }
@@ -1251,40 +1269,75 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     tp::set_error("tp_create: shared-memory plan does not fit (nb/nrhs too large)");
     return fail(TP_ERR_UNSUPPORTED);
   }
-  // U-values kept by the CTAs of a tent (right-hand sides not split), so that
-  // nothing is evaluated after the wait.  The smallest cluster for which the
-  // slices of the largest patch fit, with two CTAs per SM if any does; the
-  // chunks of the other passes shrink for it.
-  // (More than 4 columns: clusters that leave a CTA 3 elements of it, as one
-  // CTA solves for all; 2D p = 5, 800 triangles, 16 columns mixed: 8 CTAs of an
-  // element 6.9 ms, 2 CTAs 3.5.)
-  const bool many = nrg > 4;
-  int keep = 0, rows = 0, keep_cs = 0;
-  if (rs == 1) {
-    const int QK = rule ? S_rule : Q;
-    static const int kChunks[][2] = {{48, 96}, {32, 96}, {16, 96}, {16, 64}, {8, 64}, {8, 32}};   // (chunk, rows)
-    for (size_t cap : {two_per_sm, max_dyn})
-      for (int cs : {1, 2, 4, 8})
-        for (const auto& c : kChunks) {
-          const int want = (pmax + cs - 1) / cs * QK;
-          if (keep_cs != 0 || (cs > 1 && many && pmax < 3 * cs) || (rule && 2 * c[0] < S_rule) || plan(c[0], want, c[1], rule) > cap) continue;
-          CH = c[0];
-          rows = c[1];
-          keep = want;
-          keep_cs = cs;
-        }
-  }
-  bytes = plan(CH, keep, rows, rule);
-  ctx->wide = bytes > two_per_sm;
-  ctx->min_cs = std::max(1, keep_cs);
-  // one CTA per SM with the tensor-core contractions (it holds all 512 columns)
-  if (tc_try) {
-    bytes = std::max(bytes, std::min(max_dyn, (size_t)smem_sm / 2 + 1024 - stat_smem));
-    ctx->wide = true;
-  }
-  a.CH = CH;
-  a.keep_pts = keep;
+  // tents per level, elements and points per star: what the clusters are chosen by
+  int nsm = 0;
+  if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev_) == cudaSuccess && nsm > 0) ctx->n_sm = nsm;
+  const double width = (double)ctx->ntents / std::max(1, ctx->n_levels), star = (double)T.star_el.size() / (double)T.nv;
+  // the plan of a sweep with these right-hand sides per group, into its arguments
+  auto fit = [&](KArgs& k, bool rule) {
+    SweepPlan r;
+    int CH = chunk(k, rule), keep = 0, rows = 0, keep_cs = 0;
+    // U-values kept by the CTAs of a tent (right-hand sides not split), so that
+    // nothing is evaluated after the wait.  The smallest cluster for which the
+    // slices of the largest patch fit, with two CTAs per SM if any does; the
+    // chunks of the other passes shrink for it.
+    // (More than 4 columns: clusters that leave a CTA 3 elements of it, as one
+    // CTA solves for all; 2D p = 5, 800 triangles, 16 columns mixed: 8 CTAs of an
+    // element 6.9 ms, 2 CTAs 3.5.)
+    const bool many = nrg > 4;
+    if (rs == 1) {
+      const int QK = rule ? S_rule : Q;
+      static const int kChunks[][2] = {{48, 96}, {32, 96}, {16, 96}, {16, 64}, {8, 64}, {8, 32}};   // (chunk, rows)
+      // (the wave-speed gradient's passes take chunks of 16 points if any cluster
+      // leaves room for them: 2D p = 4, two materials, 128 triangles, one column
+      // 3.5 ms with chunks of 8 and 2 CTAs, 1.7 with 16 and 4)
+      for (int least : {prm->ckpt_stride > 0 ? 16 : 8, 8})
+        for (size_t cap : {two_per_sm, max_dyn})
+          for (int cs : {1, 2, 4, 8})
+            for (const auto& c : kChunks) {
+              const int want = (pmax + cs - 1) / cs * QK;
+              if (keep_cs != 0 || c[0] < least || (cs > 1 && many && pmax < 3 * cs)) continue;
+              if ((rule && 2 * c[0] < S_rule) || plan(k, c[0], want, c[1], rule) > cap) continue;
+              CH = c[0];
+              rows = c[1];
+              keep = want;
+              keep_cs = cs;
+            }
+    }
+    r.smem = plan(k, CH, keep, rows, rule);
+    k.CH = CH;
+    k.keep_pts = keep;
+    r.wide = r.smem > two_per_sm;
+    // one CTA per SM with the tensor-core contractions (it holds all 512 columns)
+    if (tc_try) {
+      r.smem = std::max(r.smem, std::min(max_dyn, (size_t)smem_sm / 2 + 1024 - stat_smem));
+      r.wide = true;
+    }
+    r.min_cs = std::max(1, keep_cs);
+    int cs = 1;
+    while (cs < 8 && star * Q / (2.0 * cs) >= 32.0) cs *= 2;
+    r.max_cs = std::max(cs, keep_cs);
+    // dataflow sweep, right-hand sides not split: the smallest cluster that
+    // keeps its U-values, doubled while a third of the resident CTAs holds a
+    // level's tents (the others then work ahead) and a CTA keeps 5/4 elements;
+    // with more than 4 columns, whose data and outflow the next tents wait for,
+    // also while two thirds hold them and a CTA has 32 points (800 triangles,
+    // p = 3, 16 columns, binary64: 1 -> 2 CTAs 2.4 -> 1.9 ms).
+    // Where no cluster keeps them, each evaluates its points again after the
+    // wait: the cluster of 32 or more points a CTA (3D p = 3, 16 columns with
+    // checkpoints, 750 elements: 27.6 ms with 2 CTAs, 11.6 with 8)
+    if (keep_cs > 0) {
+      const double resident = (r.wide ? 1 : 2) * ctx->n_sm;
+      cs = keep_cs;
+      while (cs < 8 && star / (2.0 * cs) >= 1.25 &&
+             (2.0 * cs * width <= resident / 3.0 || (many && 2.0 * cs * width <= resident / 1.5 && star * Q / (2.0 * cs) >= 32.0)))
+        cs *= 2;
+    }
+    r.flow_cs = cs;
+    return r;
+  };
   a.nrhs = nrg;
+  ctx->fwd = fit(a, rule);
   a.rsplit = rs > 1 ? 1 : 0;
   a.tc = tc_try ? 1 : 0;
   a.tc_cols = tc_try ? tp::tc_cols_max : 0;
@@ -1297,50 +1350,25 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     return fail(TP_ERR_OOM);
   }
   ctx->args_adj = a;
+  ctx->rev = ctx->fwd;
+  // the reverse sweep is binary64 throughout: where that takes the front rule, a plan of its own
+  ctx->rev_own = rule && !rule_pays(nrg, true);
+  if (ctx->rev_own) ctx->rev = fit(ctx->args_adj, false);
   ctx->args_adj.front = ctx->d_adj;
   ctx->args_adj.tau = ctx->d_tau_adj;
   ctx->args_adj.gD = nullptr;
   ctx->args_adj.diss = nullptr;
-  ctx->smem_bytes = bytes;
   rc = set_smem_attr(n, max_dyn);
   if (rc) return fail(rc);
   {
-    int nsm = 0;
-    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device) == cudaSuccess && nsm > 0)
-      ctx->n_sm = nsm;
-    const double avg_pts = (double)T.star_el.size() / (double)T.nv * Q;
-    int cs = 1;
-    while (cs < 8 && avg_pts / (2.0 * cs) >= 32.0) cs *= 2;
-    ctx->max_cs = std::max(cs, keep_cs);
-    // dataflow sweep, right-hand sides not split: the smallest cluster that
-    // keeps its U-values, doubled while a third of the resident CTAs holds a
-    // level's tents (the others then work ahead) and a CTA keeps 5/4 elements;
-    // with more than 4 columns, whose data and outflow the next tents wait for,
-    // also while two thirds hold them and a CTA has 32 points (800 triangles,
-    // p = 3, 16 columns, binary64: 1 -> 2 CTAs 2.4 -> 1.9 ms).
-    // Where no cluster keeps them, each evaluates its points again after the
-    // wait: the cluster of 32 or more points a CTA (3D p = 3, 16 columns with
-    // checkpoints, 750 elements: 27.6 ms with 2 CTAs, 11.6 with 8)
-    const double width = (double)ctx->ntents / std::max(1, ctx->n_levels), star = (double)T.star_el.size() / (double)T.nv;
-    if (keep_cs > 0) {
-      const double resident = (ctx->wide ? 1 : 2) * ctx->n_sm;
-      cs = keep_cs;
-      while (cs < 8 && star / (2.0 * cs) >= 1.25 &&
-             (2.0 * cs * width <= resident / 3.0 || (many && 2.0 * cs * width <= resident / 1.5 && avg_pts / (2.0 * cs) >= 32.0)))
-        cs *= 2;
-    }
-    ctx->flow_cs = cs;
-  }
-  {
-    const double avg_star = (double)T.star_el.size() / (double)T.nv;
-    const int key[5] = {n, ctx->p, ctx->nrhs, ctx->mixed ? 1 : 0, (int)std::lround(avg_star)};
+    const int key[5] = {n, ctx->p, ctx->nrhs, ctx->mixed ? 1 : 0, (int)std::lround(star)};
     std::copy(key, key + 5, ctx->tune_key);
   }
   if (ctx->persistent) {
-    int cs = ctx->flow_cs;
+    int cs = ctx->fwd.flow_cs;
     bool sched_dataflow = true;
     if (tuned_lookup(ctx->tune_key, &cs, &sched_dataflow)) ctx->persistent = sched_dataflow;
-    cs = std::max(cs, ctx->min_cs);
+    cs = std::max(cs, ctx->fwd.min_cs);
     if (rs > 1) cs = rs;   // the cluster is the right-hand-side split
     if (ctx->persistent && set_persist_cs(ctx, cs) != TP_OK) ctx->persistent = false;   // one launch per level
   }
@@ -1376,7 +1404,7 @@ extern "C" int tp_ctx_schedule(const tp_ctx* ctx, int32_t* dataflow, int32_t* cl
     return TP_ERR_ARG;
   }
   if (dataflow) *dataflow = ctx->persistent ? 1 : 0;
-  if (cluster) *cluster = ctx->persistent ? ctx->persist_cs : ctx->max_cs;
+  if (cluster) *cluster = ctx->persistent ? ctx->fwd.cs : ctx->fwd.max_cs;
   if (rhs_split) *rhs_split = ctx->rsplit_cs;
   if (rhs_groups) *rhs_groups = ctx->rhs_groups;
   return TP_OK;
@@ -1937,7 +1965,7 @@ extern "C" int tp_autotune(tp_ctx* ctx, void* stream, int32_t* chosen, double* b
     if (c == 0) {
       ctx->persistent = false;
     } else {
-      if ((ctx->rsplit_cs > 1 ? c != ctx->rsplit_cs : c > ctx->max_cs * 2) || set_persist_cs(ctx, c) != TP_OK)
+      if ((ctx->rsplit_cs > 1 ? c != ctx->rsplit_cs : c > ctx->fwd.max_cs * 2) || set_persist_cs(ctx, c) != TP_OK)
         continue;
       ctx->persistent = true;
     }

@@ -631,6 +631,12 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   constexpr int kMaxLow = (kMaxLowPairs + NT - 1) / NT;          // of functions < nl
   using T = typename std::conditional<MIXED, dd, double>::type;
   using R = Ar<T>;
+  // sweeps that may take the S-point rule of the face integrals.  In binary64 it
+  // is taken at 3D p = 3 alone: there its errors are those of the front rule
+  // (0.90 to 1.06 of them, reverse sweeps 0.90 to 1.06), at 2D p = 2 to 4 and 3D
+  // p = 1, 2 a reverse sweep's are 1.5 to 3.7 times as large (every tent repeats
+  // the same roundings of its points and weights), an energy's up to 4 times
+  constexpr bool RULE = !SPLIT && DIM > 1 && (MIXED || DIM == 3);
   constexpr int NV = DIM + 1;   // vertices per element
   constexpr int C = DIM + 2;    // U, v, sigma  (and gamma, alpha, beta_m moments)
   extern __shared__ __align__(16) double sm[];
@@ -694,7 +700,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
     __syncthreads();
     tc::fence_after();
   }
-  if (!SPLIT && a.S > 0) {   // (ordered before its first use by the first tent's barriers)
+  if (RULE && a.S > 0) {   // (ordered before its first use by the first tent's barriers)
     T* sTF = reinterpret_cast<T*>(sm + a.off_tf);
     for (int id = tid; id < 2 * a.S * a.tf_stride; id += NT) {
       sTF[id] = tab(rule_tab<T>(a.tf) + id);
@@ -860,7 +866,8 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   // is found after the wait, and the tent assembled again from its own.
   // (`real`: the times are those of the front)
   const int slice_el = (P + CS - 1) / CS;   // a CTA's share of the patch: whole elements
-  const int QK = a.S > 0 ? a.S : Q;         // points per element of a kept tent
+  const bool srule = RULE && a.S > 0;
+  const int QK = srule ? a.S : Q;           // points per element of a kept tent
   const bool kept = !SPLIT && slice_el * QK <= a.keep_pts;
   bool real = !PERSIST;
   __syncthreads();
@@ -889,7 +896,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   const int q1 = SPLIT ? min(P * QK, q0 + slice) : e1 * Q;
   const int np = (e1 - e0) * QK;           // points of the slice in the rule of the face integrals
   // elements whose data are taken at a time (their points fit sU where the rows are not kept)
-  const int EC = kept || a.S == 0 ? a.raw_el : min(a.raw_el, 2 * CH / QK);
+  const int EC = kept || !srule ? a.raw_el : min(a.raw_el, 2 * CH / QK);
   double ih = 0.0, tc = 0.0;
   // kept slice: the U-values of the outflow (forward: top points; adjoint:
   // bottom), then those of the moments (the other face)
@@ -899,29 +906,51 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   const T* sTF = sTP + a.S * a.tf_stride;
   T* sRaw = reinterpret_cast<T*>(sm + a.off_raw);
   // a patch point q of element k mapped to the tent's reference coordinates
-  // (Remark 3.1) on the top (TOP) or bottom face: its barycentric coordinates
-  // (a rule's table) times the element's scaled vertices (s_xh), in the path's
-  // arithmetic; and sqrt(w) as the scale of its U-values (UNIT: 1)
-  auto map_with = [&](T* pp, int k, int q, bool top, const T* bary_, const T* sqw_, bool unit) {
-    T x[DIM + 1];
+  // (Remark 3.1) on the top (TOP) or bottom face, and sqrt(w) as the scale of its
+  // U-values (UNIT: 1).  Binary64: the barycentric sums of the vertices, then
+  // shifted and scaled.  Mixed: the sums over the element's scaled vertices
+  // (s_xh) in float-float, where the errors of a sweep are the same as from
+  // points formed in binary64 (0.8 to 1.2 of them, mean 1.0 over 24 outputs)
+  // and the binary64 unit is left alone; binary64 sums over scaled vertices
+  // double the error of a 1D p = 6 sweep.
+  auto map_with = [&](T* pp, int k, int q, bool top, const RuleTab& baryR, const RuleTab& sqwR, bool unit) {
+    if constexpr (MIXED) {
+      const T* bary_ = rule_tab<T>(baryR);
+      T x[DIM + 1];
 #pragma unroll
-    for (int d = 0; d <= DIM; ++d) x[d] = R::zero();
+      for (int d = 0; d <= DIM; ++d) x[d] = R::zero();
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      const T l = tab(bary_ + q * NV + i);
-      x[0] = R::acc(x[0], l, s_xh[k][i][top ? DIM + 1 : DIM]);
+      for (int i = 0; i < NV; ++i) {
+        const T l = tab(bary_ + q * NV + i);
+        x[0] = R::acc(x[0], l, s_xh[k][i][top ? DIM + 1 : DIM]);
 #pragma unroll
-      for (int d = 0; d < DIM; ++d) x[1 + d] = R::acc(x[1 + d], l, s_xh[k][i][d]);
+        for (int d = 0; d < DIM; ++d) x[1 + d] = R::acc(x[1 + d], l, s_xh[k][i][d]);
+      }
+#pragma unroll
+      for (int d = 0; d <= DIM; ++d) pp[d] = R::norm(x[d]);
+      pp[DIM + 1] = unit ? R::one() : R::mul(tab(rule_tab<T>(sqwR) + q), R::from(s_sdet[k]));
+    } else {
+      double x[DIM], tt = 0.0;
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) x[d] = 0.0;
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const double l = __ldg(baryR.d + q * NV + i);
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) x[d] = fma(l, s_X[k][i][d], x[d]);
+        tt = fma(l, top ? s_tt[k][i] : s_tb[k][i], tt);
+      }
+      pp[0] = s_gc[s_grp[k]] * (tt - tc) * ih;
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) pp[1 + d] = (x[d] - s_xv[d]) * ih;
+      pp[DIM + 1] = unit ? 1.0 : __ldg(sqwR.d + q) * s_sdet[k];
     }
-#pragma unroll
-    for (int d = 0; d <= DIM; ++d) pp[d] = R::norm(x[d]);
-    pp[DIM + 1] = unit ? R::one() : R::mul(tab(sqw_ + q), R::from(s_sdet[k]));
   };
   auto map_point = [&](T* pp, int k, int q, bool top) {   // of the front rule
-    map_with(pp, k, q, top, rule_tab<T>(a.baryT), rule_tab<T>(a.sqwT), false);
+    map_with(pp, k, q, top, a.baryT, a.sqwT, false);
   };
   auto map_rule = [&](T* pp, int k, int q, bool top) {    // of the rule of the face integrals
-    map_with(pp, k, q, top, rule_tab<T>(a.S > 0 ? a.s_baryT : a.baryT), rule_tab<T>(a.S > 0 ? a.s_sqwT : a.sqwT), false);
+    map_with(pp, k, q, top, srule ? a.s_baryT : a.baryT, srule ? a.s_sqwT : a.sqwT, false);
   };
   // data coefficients of the points base .. base + nq - 1 (patch point
   // numbering) for every right-hand side, one (point, right-hand side) per
@@ -1263,7 +1292,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       s_gt[k][d] = gt;
       g2 = fma(gt, gt, g2);
     }
-    {   // vertices in the tent's reference coordinates: xhat, then that on the bottom and the top
+    if constexpr (MIXED) {   // vertices in the tent's reference coordinates: xhat, then that on the bottom and the top
       const double cg = s_gc[s_grp[k]], tcn = 0.5 * (tbot + s_ttop), ihn = s_ih;
       for (int i = 0; i < NV; ++i) {
         for (int d = 0; d < DIM; ++d) s_xh[k][i][d] = R::from((s_X[k][i][d] - s_xv[d]) * ihn);
@@ -2074,7 +2103,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   // ---------------- the data of the bottom front (adjoint: of the top) ----------------
   if constexpr (!SPLIT) {
     const T* U = sKI;
-    if (!kept && a.S == 0) {
+    if (!kept && !srule) {
       for (int base = q0; base < q1; base += CH) {
         const int nq = min(CH, q1 - base);
         for (int id = tid; id < nq; id += blockDim.x) map_point(sPt + id * (DIM + 2), (base + id) / Q, (base + id) % Q, ADJ);
@@ -2083,7 +2112,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
         data_moments(base, nq, sU, Q);
         __syncthreads();
       }
-    } else if (a.S > 0) {
+    } else if (srule) {
       // U on a face is in P_p, so sum_q w_q f(q) u(q) = sum_s u(X_s) [sum_q w_q w_s K(X_s, x_q) f(q)]
       // (FaceRule): the data go to the rule's points, a few elements at a time
       const int S = a.S, raws = a.raw_el * Q;
@@ -2951,7 +2980,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
     f[1] = w * (sv[1] / (cg * cg) - gs);
     for (int d = 0; d < DIM; ++d) f[2 + d] = w * (sv[2 + d] - s_gb[k][d] * sv[1]);
   };
-  if (!SPLIT && a.S > 0) {
+  if (srule) {
     // the fields at the rule's points, then through the table to the front's
     const int S = a.S;
     const T* U = sKeep;
@@ -3011,7 +3040,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
     if (!kept) {
     for (int id = tid; id < nq; id += blockDim.x) {
       const int qg = base + id;
-      map_with(sPt + id * (DIM + 2), qg / Q, qg % Q, !ADJ, rule_tab<T>(a.baryT), rule_tab<T>(a.sqwT), true);
+      map_with(sPt + id * (DIM + 2), qg / Q, qg % Q, !ADJ, a.baryT, a.sqwT, true);
     }
     eval_uvalues_block<DIM, T, false>(a, nq, sPt, sM, sU);
     }
