@@ -830,7 +830,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   if ((rc = ctx_upload(ctx, &dX, T.X)) || (rc = ctx_upload(ctx, &dc, T.c)) ||
       (rc = ctx_upload(ctx, &del, T.elems)) || (rc = ctx_upload(ctx, &dbary, ctx->rule.bary)) ||
       (rc = ctx_upload(ctx, &ddp, dep_ptr)) || (rc = ctx_upload(ctx, &dvtp, vt_ptr)) ||
-      (rc = ctx_upload(ctx, &dvtt, vt_tau)) || (rc = ctx_upload(ctx, &dinj, std::vector<int>{-1, 0})) ||
+      (rc = ctx_upload(ctx, &dvtt, vt_tau)) || (rc = ctx_upload(ctx, &dinj, std::vector<int>(ctx->ntents, 0))) ||
       (rc = ctx_upload(ctx, &ddn, dep_need)) || (rc = ctx_upload(ctx, &dqt, queue_tent)) ||
       (rc = ctx_upload(ctx, &dw, ctx->rule.w)) || (rc = ctx_upload(ctx, &dsqw, sqw)) ||
       (rc = ctx_upload(ctx, &dtv, tv)) || (rc = ctx_upload(ctx, &dttop, ttop)) ||
@@ -1686,8 +1686,7 @@ extern "C" int tp_inject_wait(tp_ctx* ctx, int64_t tent, int32_t extra) {
     tp::set_error("tp_inject_wait: tent " + std::to_string(tent) + " waits for no earlier tent");
     return TP_ERR_ARG;
   }
-  const int h[2] = {extra > 0 ? (int)tent : -1, extra};
-  TP_CUDA_OK(cudaMemcpy(ctx->d_inject, h, sizeof(h), cudaMemcpyHostToDevice));
+  TP_CUDA_OK(cudaMemcpy(ctx->d_inject + tent, &extra, sizeof(int), cudaMemcpyHostToDevice));
   return TP_OK;
 }
 

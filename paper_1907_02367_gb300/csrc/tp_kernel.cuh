@@ -148,7 +148,7 @@ struct KArgs {
   const int* dep_need;
   const int* vt_ptr;          // per vertex w: its front times after 0, 1, .. of its tents, vt_tau[vt_ptr[w] ..]
   const double* vt_tau;
-  const int* inject;          // (tent, extra): that tent waits for `extra` completions more (tp_inject_wait)
+  const int* inject;          // per tent: completions that it waits for beyond those that come (tp_inject_wait; 0)
   int tent_beg;               // tents of the sweep's range: [tent_beg, tent_end)
   const int* queue_tent;      // tent at each queue position (level order, critical chains first)
   int tent_end;
@@ -835,7 +835,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   // for (and acquires) the counts itself
   auto wait_deps = [&]() {
     if constexpr (PERSIST) {
-      const int extra_ = !ADJ && __ldg(a.inject) == tent ? __ldg(a.inject + 1) : 0;
+      const int extra_ = ADJ ? 0 : __ldg(a.inject + tent);
       for (int e = tid; e < nn_; e += blockDim.x) {
         const int w = s_nid[e];
         int before = __ldg(a.dep_need + d0_ + e);
