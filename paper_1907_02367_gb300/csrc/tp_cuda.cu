@@ -183,7 +183,7 @@ struct tp_ctx {
   bool mixed = false;
   // persistent dataflow sweep
   bool persistent = true;
-  int tune_key[5] = {0, 0, 0, 0, 0};   // (dim, p, nrhs, mixed, patch bucket) of the autotuner cache
+  std::vector<int> tune_key;   // of the autotuner cache: what the default cluster is chosen by
   int* d_queue = nullptr;
   int* d_done = nullptr;
   int* d_queue_adj = nullptr;   // of the reverse sweep and the gradient's forward sweeps (tp_adjoint)
@@ -305,9 +305,9 @@ int set_persist_cs(tp_ctx* ctx, int cs) {
 std::mutex g_tune_mu;
 std::map<std::vector<int>, std::pair<int, bool>> g_tuned;
 
-bool tuned_lookup(const int* key, int* cs, bool* dataflow) {
+bool tuned_lookup(const std::vector<int>& key, int* cs, bool* dataflow) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  auto it = g_tuned.find(std::vector<int>(key, key + 5));
+  auto it = g_tuned.find(key);
   if (it == g_tuned.end()) return false;
   *cs = it->second.first;
   *dataflow = it->second.second;
@@ -1360,10 +1360,22 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   ctx->args_adj.diss = nullptr;
   rc = set_smem_attr(n, max_dyn);
   if (rc) return fail(rc);
-  {
-    const int key[5] = {n, ctx->p, ctx->nrhs, ctx->mixed ? 1 : 0, (int)std::lround(star)};
-    std::copy(key, key + 5, ctx->tune_key);
-  }
+  // a cluster tuned on one context serves those alike in all that the default is
+  // chosen by; tents per level by powers of two
+  ctx->tune_key = {n,
+                   ctx->p,
+                   ctx->nrhs,
+                   ctx->mixed,
+                   (int)std::lround(star),
+                   (int)std::lround(std::log2(std::max(1.0, width))),
+                   ngmax,
+                   ctx->neumann,
+                   rs,
+                   a.tc,
+                   prm->ckpt_stride > 0,
+                   ctx->fwd.wide,
+                   ctx->fwd.min_cs,
+                   ctx->fwd.flow_cs};
   if (ctx->persistent) {
     int cs = ctx->fwd.flow_cs;
     bool sched_dataflow = true;
@@ -1964,7 +1976,8 @@ extern "C" int tp_autotune(tp_ctx* ctx, void* stream, int32_t* chosen, double* b
     if (c == 0) {
       ctx->persistent = false;
     } else {
-      if ((ctx->rsplit_cs > 1 ? c != ctx->rsplit_cs : c > ctx->fwd.max_cs * 2) || set_persist_cs(ctx, c) != TP_OK)
+      if ((ctx->rsplit_cs > 1 ? c != ctx->rsplit_cs : c > std::max(ctx->fwd.max_cs * 2, ctx->fwd.flow_cs)) ||
+          set_persist_cs(ctx, c) != TP_OK)
         continue;
       ctx->persistent = true;
     }
@@ -1989,7 +2002,7 @@ extern "C" int tp_autotune(tp_ctx* ctx, void* stream, int32_t* chosen, double* b
     ctx->persistent = best > 0;
     if (best > 0) set_persist_cs(ctx, best);
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_tuned[std::vector<int>(ctx->tune_key, ctx->tune_key + 5)] = {best > 0 ? best : 1, best > 0};
+    g_tuned[ctx->tune_key] = {best > 0 ? best : 1, best > 0};
   }
   for (auto& kv : ctx->graphs) cudaGraphExecDestroy(kv.second);
   ctx->graphs.clear();
