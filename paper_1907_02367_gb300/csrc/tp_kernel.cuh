@@ -711,6 +711,9 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
     if (CS > 1) cluster.sync();
     else __syncthreads();
   };
+  // (rank 0 stores the first tent into the other CTAs' shared memory, which
+  // may be written only once they run)
+  if (PERSIST && CS > 1) cluster.sync();
   for (;;) {
   int tent;
   if constexpr (PERSIST) {
