@@ -306,8 +306,11 @@ __device__ __forceinline__ dd dd_split(double x) {
   return {__uint_as_float(hb), lo};
 }
 
-// 1/x of a float-float value: Newton step r + r (1 - x r) from the binary32
-// reciprocal of the leading part (24 -> 48 bits)
+// 1/x of a float-float value: Newton step r + r (1 - x r) from the hardware's
+// approximate binary32 reciprocal of the leading part (about 1 ulp; 24 -> 48
+// bits).  The inverse it serves is refined against A, so its last bits do not
+// matter, and the correctly rounded reciprocal costs several times as long in
+// the elimination's chain of pivots
 __device__ __forceinline__ dd dd_rcp(dd x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x.hi));
@@ -321,8 +324,6 @@ struct Ar;
 template <>
 struct Ar<double> {
   static __device__ __forceinline__ float hi(double x) { return (float)x; }
-  static __device__ __forceinline__ double addf(double a, float f) { return a + (double)f; }
-  static __device__ __forceinline__ double fms(double t, double a, double b) { return ::fma(-a, b, t); }
   static __device__ __forceinline__ double zero() { return 0.0; }
   static __device__ __forceinline__ double one() { return 1.0; }
   static __device__ __forceinline__ double from(double x) { return x; }
@@ -330,8 +331,6 @@ struct Ar<double> {
   static __device__ __forceinline__ double add(double a, double b) { return a + b; }
   static __device__ __forceinline__ double sub(double a, double b) { return a - b; }
   static __device__ __forceinline__ double mul(double a, double b) { return a * b; }
-  static __device__ __forceinline__ double mulf(double a, float f) { return a * (double)f; }
-  static __device__ __forceinline__ double fmac(double a, float f, double c) { return ::fma(a, (double)f, c); }
   // accumulation of a long sum of products (see the float-float version)
   static __device__ __forceinline__ double acc(double s, double a, double b) { return ::fma(a, b, s); }
   static __device__ __forceinline__ double accf(double s, double a, float f) { return ::fma(a, (double)f, s); }
@@ -347,11 +346,6 @@ struct Ar<double> {
 template <>
 struct Ar<dd> {
   static __device__ __forceinline__ float hi(dd x) { return x.hi; }
-  static __device__ __forceinline__ dd addf(dd a, float f) { return dd_add(a, {f, 0.f}); }
-  static __device__ __forceinline__ dd fms(dd t, dd a, dd b) {
-    const dd p = dd_mul(a, b);
-    return dd_add(t, {-p.hi, -p.lo});
-  }
   static __device__ __forceinline__ dd zero() { return {0.f, 0.f}; }
   static __device__ __forceinline__ dd one() { return {1.f, 0.f}; }
   static __device__ __forceinline__ dd from(double x) {
@@ -362,8 +356,6 @@ struct Ar<dd> {
   static __device__ __forceinline__ dd add(dd a, dd b) { return dd_add(a, b); }
   static __device__ __forceinline__ dd sub(dd a, dd b) { return dd_add(a, {-b.hi, -b.lo}); }
   static __device__ __forceinline__ dd mul(dd a, dd b) { return dd_mul(a, b); }
-  static __device__ __forceinline__ dd mulf(dd a, float f) { return dd_mulf(a, f); }
-  static __device__ __forceinline__ dd fmac(dd a, float f, dd c) { return dd_add(dd_mulf(a, f), c); }
   // s += a b for a long sum of products, compensated in the manner of Ogita,
   // Rump and Oishi's Dot2: s = (p, e) holds the running binary32 sum p and
   // the sum e of all rounding errors (of the products, exact by fmaf, and of
@@ -532,15 +524,6 @@ __device__ __forceinline__ T relT_apply(const KArgs& a, int k, int var, const T*
   return s;
 }
 
-// binary32 reciprocal of the hardware's approximate reciprocal instruction
-// (about 1 ulp): the inverse of the solve is refined against A, so its last
-// bits do not matter, and the correctly rounded reciprocal costs several times
-// as long in the elimination's chain of pivots
-__device__ __forceinline__ float rcp_fast(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
 // power of two nearest below 1 / sqrt(d) (within a factor of two; exact scaling)
 __device__ __forceinline__ float pow2_rsqrt(float d) {
   const int e = (int)((__float_as_uint(d) >> 23) & 0xFF) - 127;
