@@ -1289,10 +1289,12 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
       const int QK = rule ? S_rule : Q;
       static const int kChunks[][2] = {{48, 96}, {32, 96}, {16, 96}, {16, 64}, {8, 64}, {8, 32}};   // (chunk, rows)
       // (the wave-speed gradient's passes take chunks of 16 points if any cluster
-      // leaves room for them: 2D p = 4, two materials, 128 triangles, one column
-      // 3.5 ms with chunks of 8 and 2 CTAs, 1.7 with 16 and 4)
-      for (int least : {prm->ckpt_stride > 0 ? 16 : 8, 8})
-        for (size_t cap : {two_per_sm, max_dyn})
+      // leaves room for them, but not one CTA per SM for it: 2D p = 4, two
+      // materials, 128 triangles, one column 3.5 ms with chunks of 8 and 2 CTAs,
+      // 1.7 with 16 and 4; 392 triangles, 4 columns 29.6 ms with chunks of 8 on
+      // narrow CTAs, 31.8 with 16 on wide ones)
+      for (size_t cap : {two_per_sm, max_dyn})
+        for (int least : {prm->ckpt_stride > 0 ? 16 : 8, 8})
           for (int cs : {1, 2, 4, 8})
             for (const auto& c : kChunks) {
               const int want = (pmax + cs - 1) / cs * QK;
