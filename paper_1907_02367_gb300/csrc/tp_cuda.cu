@@ -1173,6 +1173,10 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   };
   size_t max_dyn = 0, two_per_sm = 0;
   if ((rc = max_dyn_smem(n, &max_dyn, &two_per_sm)) != TP_OK) return fail(rc);
+  // tents per level, elements and points per star: what the clusters are chosen by
+  int nsm = 0;
+  if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device) == cudaSuccess && nsm > 0) ctx->n_sm = nsm;
+  const double width = (double)ctx->ntents / std::max(1, ctx->n_levels), star = (double)T.star_el.size() / (double)T.nv;
   // right-hand sides split over the cluster: rs CTAs, each owning a slice of
   // every group's right-hand sides (automatic: 16 or more per CTA; at 3D
   // p = 3 with 64 right-hand sides, 4 CTAs of 16 sweep 1.6x faster than 8 of 8)
@@ -1181,13 +1185,22 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     for (int r : {8, 4, 2})
       if (rs == 1 && ctx->nrhs % r == 0 && ctx->nrhs / r >= 16) rs = r;
     // binary64: down to 4 per CTA.  Its moments and outflow are bound by an SM's
-    // binary64 unit, on small meshes along the chain of dependent tents, where
-    // more CTAs per tent shorten it; the U-values that each repeats cost little
-    // beside them (3D p = 3, 64 right-hand sides, 4 -> 8 CTAs: 750 elements 218 ->
-    // 132 ms, 6000 elements 271 -> 268 ms; 32, 2 -> 8 CTAs: 150 -> 57, 3072
-    // elements 128 -> 67 ms).  The mixed path's tensor-core tiles
-    // want 16 (67 -> 122 ms with 8)
-    while (!ctx->mixed && rs > 1 && rs < 8 && ctx->nrhs % (2 * rs) == 0 && ctx->nrhs / (2 * rs) >= 4) rs *= 2;
+    // binary64 unit, along the chain of dependent tents, where more CTAs per tent
+    // shorten it; the U-values that each repeats cost little beside them.  So
+    // while the tents of a level leave resident CTAs for it, or a CTA keeps 8000
+    // columns times points of a star, below which its fixed work counts.
+    // Milliseconds by columns per sweep and CTAs (1: not split):
+    //   3D p = 3, 750 elements, 14 tents a level, T = 0.6, 64 columns: 1 114, 2 266, 4 212, 8 127; 32: 1 51, 2 210, 8 79
+    //   6000 elements, 76 a level, T = 0.2, 64: 1 484, 2 264, 4 273, 8 260; 32: 1 226, 2 217, 4 148, 8 166
+    //   2D p = 4, 512 triangles, 34 a level, T = 0.2, 64: 1 17.9, 2 24.8, 4 12.1, 8 9.9; 32: 1 8.8, 2 11.2, 4 7.4, 8 7.0
+    //   2048 triangles, 130 a level, T = 0.1, 64: 1 37.0, 2 33.7, 4 28.8, 8 35.5; 32: 1 15.7, 2 16.0, 4 17.9, 8 25.3
+    // (not split is the fastest of all on small 3D meshes, where one cluster of 8
+    // assembles and solves for every column; it is left to rhs_split = 1.)  The
+    // mixed path's tensor-core tiles want 16 columns (750 elements, 64: 67 -> 122 ms with 8).
+    auto apart = [&](int r) {
+      return 2.0 * r * width <= 2.0 * ctx->n_sm || ctx->nrhs / (2 * r) * star * Q >= 8000.0;
+    };
+    while (!ctx->mixed && rs > 1 && rs < 8 && ctx->nrhs % (2 * rs) == 0 && ctx->nrhs / (2 * rs) >= 4 && apart(rs)) rs *= 2;
   }
   if (!(rs == 1 || rs == 2 || rs == 4 || rs == 8) || ctx->nrhs % rs != 0) {
     tp::set_error("tp_create: rhs_split must be 0, 1, 2, 4 or 8 and divide nrhs");
@@ -1269,10 +1282,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     tp::set_error("tp_create: shared-memory plan does not fit (nb/nrhs too large)");
     return fail(TP_ERR_UNSUPPORTED);
   }
-  // tents per level, elements and points per star: what the clusters are chosen by
-  int nsm = 0;
-  if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev_) == cudaSuccess && nsm > 0) ctx->n_sm = nsm;
-  const double width = (double)ctx->ntents / std::max(1, ctx->n_levels), star = (double)T.star_el.size() / (double)T.nv;
+  auto resident = [&](bool narrow) { return (narrow ? 2.0 : 1.0) * ctx->n_sm; };   // CTAs
   // the plan of a sweep with these right-hand sides per group, into its arguments
   auto fit = [&](KArgs& k, bool rule) {
     SweepPlan r;
@@ -1328,11 +1338,12 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     // Where no cluster keeps them, each evaluates its points again after the
     // wait: the cluster of 32 or more points a CTA (3D p = 3, 16 columns with
     // checkpoints, 750 elements: 27.6 ms with 2 CTAs, 11.6 with 8)
+    const double held = resident(!r.wide);
+    const int points_cs = cs;
     if (keep_cs > 0) {
-      const double resident = (r.wide ? 1 : 2) * ctx->n_sm;
       cs = keep_cs;
       while (cs < 8 && star / (2.0 * cs) >= 1.25 &&
-             (2.0 * cs * width <= resident / 3.0 || (many && 2.0 * cs * width <= resident / 1.5 && star * Q / (2.0 * cs) >= 32.0)))
+             (2.0 * cs * width <= held / 3.0 || (many && 2.0 * cs * width <= held / 1.5 && 2 * cs <= points_cs)))
         cs *= 2;
     }
     r.flow_cs = cs;
