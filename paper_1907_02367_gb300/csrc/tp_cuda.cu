@@ -1294,6 +1294,12 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     // (More than 4 columns: clusters that leave a CTA 3 elements of it, as one
     // CTA solves for all; 2D p = 5, 800 triangles, 16 columns mixed: 8 CTAs of an
     // element 6.9 ms, 2 CTAs 3.5.)
+    // (Up to 4 columns in 2D: clusters that leave a fifth of the resident CTAs to
+    // other levels.  Work bounds a wider mesh, and a cluster of half the size
+    // that evaluates its points again after the wait is the faster one: 2D p = 5,
+    // 70 tents a level, two materials, binary64 1038 ms with 4 CTAs, 574 with
+    // one; p = 4 280 and 160.  In 3D, with three times the points, it is not:
+    // p = 3, 34 tents a level 5.9 and 6.8.)
     const bool many = nrg > 4;
     if (rs == 1) {
       const int QK = rule ? S_rule : Q;
@@ -1309,6 +1315,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
             for (const auto& c : kChunks) {
               const int want = (pmax + cs - 1) / cs * QK;
               if (keep_cs != 0 || c[0] < least || (cs > 1 && many && pmax < 3 * cs)) continue;
+              if (n == 2 && cs > 1 && !many && cs * width > 0.8 * resident(cap <= two_per_sm)) continue;
               if ((rule && 2 * c[0] < S_rule) || plan(k, c[0], want, c[1], rule) > cap) continue;
               CH = c[0];
               rows = c[1];
@@ -1336,16 +1343,18 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     // also while two thirds hold them and a CTA has 32 points (800 triangles,
     // p = 3, 16 columns, binary64: 1 -> 2 CTAs 2.4 -> 1.9 ms).
     // Where no cluster keeps them, each evaluates its points again after the
-    // wait: the cluster of 32 or more points a CTA (3D p = 3, 16 columns with
-    // checkpoints, 750 elements: 27.6 ms with 2 CTAs, 11.6 with 8)
+    // wait: doubled while a CTA has 32 points and four fifths of the resident CTAs
+    // hold a level (3D p = 3, 16 columns with checkpoints, 750 elements: 27.6 ms with
+    // 2 CTAs, 11.6 with 8; the 2D meshes above: one CTA)
     const double held = resident(!r.wide);
     const int points_cs = cs;
-    if (keep_cs > 0) {
-      cs = keep_cs;
+    cs = r.min_cs;
+    if (keep_cs > 0)
       while (cs < 8 && star / (2.0 * cs) >= 1.25 &&
              (2.0 * cs * width <= held / 3.0 || (many && 2.0 * cs * width <= held / 1.5 && 2 * cs <= points_cs)))
         cs *= 2;
-    }
+    else
+      while (2 * cs <= points_cs && 2.0 * cs * width <= 0.8 * held) cs *= 2;
     r.flow_cs = cs;
     return r;
   };
