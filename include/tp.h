@@ -94,7 +94,7 @@ typedef struct tp_params {
   /* rhs_split: how a tent's right-hand sides are shared out over the CTAs of
    * its cluster.  0 = automatic (split when each CTA keeps 16 or more,
    * i.e. nrhs >= 32 and divisible by 2, 4 or 8; binary64 then splits down to
-   * 4 per CTA), 1 = never split
+   * 4 per CTA where the mesh's levels leave CTAs for it), 1 = never split
    * (every CTA takes a slice of the points for all right-hand sides), 2, 4
    * or 8 = that many CTAs, each owning nrhs / rhs_split of the right-hand
    * sides at every point of the tent (data moments, solve and outflow),
@@ -261,10 +261,12 @@ int tp_solve_layer(tp_ctx* ctx, int32_t level, void* stream);
 int tp_advance(tp_ctx* ctx, int32_t level_begin, int32_t level_end, void* stream);
 /* Autotuner of the sweep schedule (the paper has no counterpart): times a
  * full forward sweep of this context with one launch per level and with the
- * dataflow schedule at cluster sizes 1, 2, 4 and 8 (state saved and
- * restored), keeps the fastest for later tp_advance calls and caches it for
- * this process under (dim, p, nrhs, precision, rounded mean vertex-star size),
- * so contexts created later with the same key start from it.  *chosen = 0 for
+ * dataflow schedule at cluster sizes 1, 2, 4 and 8 (up to twice the default's
+ * per-level one or the default; state saved and restored), keeps the fastest
+ * for later tp_advance calls and caches it for this process under what the
+ * default is chosen by (dim, p, nrhs, precision, mean vertex-star size, tents
+ * per level by powers of two, materials, Neumann walls, split, checkpoints,
+ * default clusters), so contexts created later with the same key start from it.  *chosen = 0 for
  * one launch per level, else the cluster size; *best_ms = its sweep time.
  * Allocates a scratch copy of the state; synchronises `stream`. */
 int tp_autotune(tp_ctx* ctx, void* stream, int32_t* chosen, double* best_ms);

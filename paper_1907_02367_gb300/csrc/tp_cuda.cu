@@ -159,8 +159,8 @@ struct tp_ctx {
   double* d_diss = nullptr;   // per right-hand side: energy lost in the tents since tp_set_state (tracked contexts)
   // wave-speed gradient (contexts created with ckpt_stride > 0): the initial
   // front of the last tp_set_state, a work front and its times, forward
-  // checkpoints every ckpt_stride levels, the fronts before each level of one
-  // segment, and the forward solutions of one segment's tents
+  // checkpoints every ckpt_stride levels, and of one segment's tents the bottom
+  // fronts and the forward solutions
   int ckpt_stride = 0;
   double* d_front0 = nullptr;
   double* d_work = nullptr;
@@ -1343,9 +1343,9 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
     // also while two thirds hold them and a CTA has 32 points (800 triangles,
     // p = 3, 16 columns, binary64: 1 -> 2 CTAs 2.4 -> 1.9 ms).
     // Where no cluster keeps them, each evaluates its points again after the
-    // wait: doubled while a CTA has 32 points and four fifths of the resident CTAs
-    // hold a level (3D p = 3, 16 columns with checkpoints, 750 elements: 27.6 ms with
-    // 2 CTAs, 11.6 with 8; the 2D meshes above: one CTA)
+    // wait: doubled while a CTA has 32 points and the resident CTAs hold a level, in
+    // 2D four fifths of them (3D p = 3, 16 columns with checkpoints, 750 elements:
+    // 27.6 ms with 2 CTAs, 15.3 with 4, 11.6 with 8; the 2D meshes above: one CTA)
     const double held = resident(!r.wide);
     const int points_cs = cs;
     cs = r.min_cs;
@@ -1354,7 +1354,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
              (2.0 * cs * width <= held / 3.0 || (many && 2.0 * cs * width <= held / 1.5 && 2 * cs <= points_cs)))
         cs *= 2;
     else
-      while (2 * cs <= points_cs && 2.0 * cs * width <= 0.8 * held) cs *= 2;
+      while (2 * cs <= points_cs && 2.0 * cs * width <= (n == 2 ? 0.8 : 1.0) * held) cs *= 2;
     r.flow_cs = cs;
     return r;
   };

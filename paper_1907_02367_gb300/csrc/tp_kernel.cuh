@@ -602,9 +602,10 @@ __device__ __forceinline__ double recip(double x) {
 // tents (levels times what a tent does between its wait and its publication)
 // or, on wide levels, the work of all tents over the resident CTAs.  The tent
 // matrix depends on the front times alone, which the tents fix, so the
-// geometry, the U-values, A and its inverse come before the wait: the chain
-// keeps the moments, b, the solve and the outflow.  2D p = 4, 968 triangles,
-// one column: 18.5 -> 9.4 ms binary64, 27.0 -> 8.0 ms mixed (with the S-point
+// geometry, the U-values, A and its inverse come before the wait (with split
+// right-hand sides the Grams alone): the chain keeps the moments, b, the solve
+// and the outflow.  2D p = 4, 968 triangles,
+// one column: 18.5 -> 9.9 ms binary64, 27.0 -> 7.8 ms mixed (mixed with the S-point
 // rule and the float-float inverse below).
 template <int DIM, bool MIXED, bool ADJ, bool PERSIST, bool NEU, bool SPLIT, bool TC, bool WIDE>
 __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) k_layer(const KArgs a, const int tent0) {
@@ -896,7 +897,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   // U-values (UNIT: 1).  Binary64: the barycentric sums of the vertices, then
   // shifted and scaled.  Mixed: the sums over the element's scaled vertices
   // (s_xh) in float-float, where the errors of a sweep are the same as from
-  // points formed in binary64 (0.8 to 1.2 of them, mean 1.0 over 24 outputs)
+  // points formed in binary64 (0.8 to 1.2 of them, mean 1.0 over 23 outputs)
   // and the binary64 unit is left alone; binary64 sums over scaled vertices
   // double the error of a 1D p = 6 sweep.
   auto map_with = [&](T* pp, int k, int q, bool top, const RuleTab& baryR, const RuleTab& sqwR, bool unit) {
@@ -1136,7 +1137,7 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       }
       __syncthreads();
       // digit planes, one item = 4 consecutive points of one row of A or B (8 left
-      // a second round of the CTA's threads a third full)
+      // a second round of the CTA's threads a third full: 330 -> 328 ms)
       for (int id = tid; id < (M + 32) * 2 * KC; id += blockDim.x) {
         const bool isA = id < M * 2 * KC;
         const int id2 = isA ? id : id - M * 2 * KC, rows = isA ? M : 32;
@@ -1375,8 +1376,9 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
       const int NPD = nfac * Q, dsl = (NPD + CS - 1) / CS;
       const int d0 = min(NPD, rank * dsl), d1 = min(NPD, d0 + dsl);
       // the Grams take this CTA's slice [d0, d1); the data moments of split
-      // right-hand sides take every point (homogeneous data have none: 3D p = 3,
-      // 64 columns mixed, with the digit items below 330 -> 328 ms)
+      // right-hand sides take every point (homogeneous data, a NULL array, have
+      // none: 3D p = 3, 6000 elements, 64 columns mixed 327 -> 300 ms; binary64,
+      // 750 elements, where boundary tents lie on the chain, 130 -> 128)
       const int l0 = rsplit && has_g ? 0 : d0, l1 = rsplit && has_g ? NPD : d1;
       T aF[kMaxLow];
 #pragma unroll
