@@ -1228,8 +1228,10 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   // of both faces' U-values (a term counts twice: its table lookups) and Grams,
   // once, and costs the data of every right-hand side two tables of S x Q
   // instead of Q - S points of the moments and the outflow.  That is up to 4
-  // columns at 3D p = 3, 3 at 2D p = 4, 5, one at p = 2 and 2D p = 3, none at
-  // p = 1.  Milliseconds a sweep, S-point -> front rule, at and past that line:
+  // columns at 3D p = 3, 3 at 2D p = 4, 5, one at 3D p = 2, and none at p = 1.
+  // (At 2D p = 2, 3 one column would break even, 0.90 to 1.01 of its sweep, but a
+  // mixed sweep's error on a graded two-material mesh is 1.4 to 2.1 times that of
+  // the front rule: not taken.)  Milliseconds a sweep, S-point -> front rule, at and past that line:
   // 3D p = 3, 1296 elements, mixed 2.4 -> 5.1 with one column, 5.8 -> 6.1 with 4,
   // 11.5 -> 10.3 with 16; 2D p = 3, 800 triangles, binary64 0.73 -> 0.66 with 2,
   // 3.7 -> 2.4 with 16 (1.9 with the cluster chosen below); 3D p = 2, 1296
@@ -1237,7 +1239,7 @@ extern "C" int tp_create(const tp_mesh_desc* mesh, const tp_tents* tents, const 
   // (Binary64 sums: at 3D p = 3 alone, where its errors are the front rule's; the
   // kernel's RULE has the figures.)
   auto rule_pays = [&](int columns, bool binary64) {
-    if (S_rule == 0 || rs > 1 || (binary64 && !(n == 3 && basis->p == 3))) return false;
+    if (S_rule == 0 || rs > 1 || (n == 2 && basis->p <= 3) || (binary64 && !(n == 3 && basis->p == 3))) return false;
     long long terms = ctx->nmono;
     for (int j = 0; j < nb; ++j) terms += basis->sp_ptr[(size_t)j * C + 1] - basis->sp_ptr[(size_t)j * C];
     const long long fewer = Q - S_rule;

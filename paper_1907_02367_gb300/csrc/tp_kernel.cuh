@@ -617,9 +617,10 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 2) 
   using R = Ar<T>;
   // sweeps that may take the S-point rule of the face integrals.  In binary64 it
   // is taken at 3D p = 3 alone: there its errors are those of the front rule
-  // (0.90 to 1.06 of them, reverse sweeps 0.90 to 1.06), at 2D p = 2 to 4 and 3D
+  // (0.90 to 1.08 of them over 24 outputs, one energy 1.13), at 2D p = 2 to 4 and 3D
   // p = 1, 2 a reverse sweep's are 1.5 to 3.7 times as large (every tent repeats
-  // the same roundings of its points and weights), an energy's up to 4 times
+  // the same roundings of its points and weights), an energy's up to 4 times.  In
+  // float-float at 2D p = 4, 5 and 3D p = 2, 3: 0.6 to 1.2 of the front rule's
   constexpr bool RULE = !SPLIT && DIM > 1 && (MIXED || DIM == 3);
   constexpr int NV = DIM + 1;   // vertices per element
   constexpr int C = DIM + 2;    // U, v, sigma  (and gamma, alpha, beta_m moments)
